@@ -86,14 +86,15 @@ __device__ __forceinline__ void block_reduce2(double& a, double& b) {
 }
 
 // Fused multiply-add in either precision: the apply's sums are written as
-// explicit chains so that every tile shape (and the packed FP32 kernel)
-// rounds each row the same way.
+// explicit chains so that every tile shape (in FP32: every kernel) rounds
+// each row the same way.
 __device__ __forceinline__ float fmat(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmat(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mult(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a, b); }
 
-// Regular part of B x at the unknowns.  One thread owns the column i of TY
+// Regular part of B x at the unknowns in FP32 (the streaming kernel; the
+// ring below takes the wide grids).  One thread owns the column i of TY
 // consecutive rows j and marches the planes k0 .. k1 - 1 of its z chunk (KC
 // planes); TY x KC is the tile shape the autotuner picks per grid.  The z
 // coefficients of the chunk are staged in shared memory once.
@@ -111,10 +112,10 @@ __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a,
 // dependent side-list loads stall the streaming march, and the CTAs near the
 // bodies become the tail.)
 // DOT = 0: y only; 1: partial (d0, y); 2: partials (d0, y) and (y, y).
-template <class T, int DOT, int TY, int KC>
-__global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (sizeof(T) == 4 ? 4 : 2))
-    k_apply(Grid<T> G, const uint8_t* __restrict__ type, const T* __restrict__ x, T* __restrict__ y,
-            const T* __restrict__ d0, double* __restrict__ partial) {
+template <int DOT, int TY, int KC>
+__global__ void __launch_bounds__(kAX, TY == 2 ? 8 : 4)
+    k_apply(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
+            const float* __restrict__ d0, double* __restrict__ partial) {
     constexpr int R = TY + 2;  // rows loaded per plane
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int i = 1 + blockIdx.x * kAX + threadIdx.x;
@@ -122,10 +123,10 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
     const int k0 = 1 + blockIdx.z * KC;
     const int k1 = min(k0 + KC, nz - 1);
     // z coefficients of the chunk's output planes k0 .. k1 - 1
-    __shared__ T zc[5][KC];
+    __shared__ float zc[5][KC];
     for (int q = threadIdx.x; q < 5 * KC; q += kAX) {
         const int m = q / KC, kc = min(k0 + q % KC, nz - 2);
-        const T* src = m == 0 ? G.ax[2].a : m == 1 ? G.ax[2].c : m == 2 ? G.ax[2].ar : m == 3 ? G.ax[2].br : G.ax[2].cr;
+        const float* src = m == 0 ? G.ax[2].a : m == 1 ? G.ax[2].c : m == 2 ? G.ax[2].ar : m == 3 ? G.ax[2].br : G.ax[2].cr;
         zc[m][q % KC] = src[kc];
     }
     __syncthreads();
@@ -133,9 +134,9 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
     const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
     // node offsets fit in 32 bits: contexts hold fewer than 2^31 nodes
     const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
-    const T ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
-    const T arx = G.ax[0].ar[ic], brx = G.ax[0].br[ic], crx = G.ax[0].cr[ic];
-    T ay[TY], cy[TY], ary[TY], bry[TY], cry[TY];
+    const float ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
+    const float arx = G.ax[0].ar[ic], brx = G.ax[0].br[ic], crx = G.ax[0].cr[ic];
+    float ay[TY], cy[TY], ary[TY], bry[TY], cry[TY];
     bool jin[TY];
     unsigned lout0[TY];
 #pragma unroll
@@ -152,37 +153,37 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
     unsigned roff[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) roff[r] = (unsigned)min(j0 - 1 + r, ny - 1) * sy;
-    const T* p = x + ((unsigned)(k0 - 1) * sz + (unsigned)ic);
-    T n[3 * R];
+    const float* p = x + ((unsigned)(k0 - 1) * sz + (unsigned)ic);
+    float n[3 * R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const T* q = p + roff[r];
+        const float* q = p + roff[r];
         n[3 * r] = q[-1];
         n[3 * r + 1] = q[0];
         n[3 * r + 2] = q[1];
     }
     // type byte and dot operand of the next output node of each row
     uint8_t t_next[TY];
-    T d_next[TY];
+    float d_next[TY];
 #pragma unroll
     for (int t = 0; t < TY; ++t) {
         t_next[t] = type[lout0[t]];
-        d_next[t] = DOT ? d0[lout0[t]] : T(0);
+        d_next[t] = DOT ? d0[lout0[t]] : 0.f;
     }
-    T Pm[TY], P0[TY], Pp[TY], Qm[TY], Q0[TY], Qp[TY];
+    float Pm[TY], P0[TY], Pp[TY], Qm[TY], Q0[TY], Qp[TY];
 #pragma unroll
-    for (int t = 0; t < TY; ++t) Pm[t] = P0[t] = Pp[t] = Qm[t] = Q0[t] = Qp[t] = T(0);
-    DotAcc<T> dacc0, dacc1;
+    for (int t = 0; t < TY; ++t) Pm[t] = P0[t] = Pp[t] = Qm[t] = Q0[t] = Qp[t] = 0.f;
+    DotAcc<float> dacc0, dacc1;
 #pragma unroll 3
     for (int kk = k0 - 1; kk <= k1; ++kk) {
-        T c[3 * R];
+        float c[3 * R];
 #pragma unroll
         for (int q = 0; q < 3 * R; ++q) c[q] = n[q];
         if (kk < k1) {  // prefetch plane kk + 1
             p += sz;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const T* q = p + roff[r];
+                const float* q = p + roff[r];
                 n[3 * r] = q[-1];
                 n[3 * r + 1] = q[0];
                 n[3 * r + 2] = q[1];
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
         // output of this step is plane kk - 1 (from step k0 + 1 on); its type
         // bytes and dot operands were fetched one step earlier
         uint8_t t_cur[TY];
-        T d_cur[TY];
+        float d_cur[TY];
 #pragma unroll
         for (int t = 0; t < TY; ++t) {
             t_cur[t] = t_next[t];
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
                 if (DOT) d_next[t] = d0[ln];
             }
         }
-        T XR[R], XL[R];
+        float XR[R], XL[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             XR[r] = fmat(crx, c[3 * r + 2], fmat(brx, c[3 * r + 1], mult(arx, c[3 * r])));
@@ -224,12 +225,12 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
         }
         if (kk >= k0 + 1 && iin) {
             const int k = kk - 1, kl = k - k0;
-            const T az = zc[0][kl], cz = zc[1][kl];
-            const T arz = zc[2][kl], brz = zc[3][kl], crz = zc[4][kl];
+            const float az = zc[0][kl], cz = zc[1][kl];
+            const float arz = zc[2][kl], brz = zc[3][kl], crz = zc[4][kl];
 #pragma unroll
             for (int t = 0; t < TY; ++t) {
                 if (!jin[t]) continue;
-                T v = fmat(cz, Pp[t], fmat(az, Pm[t], P0[t])) + fmat(crz, Qp[t], fmat(brz, Q0[t], mult(arz, Qm[t])));
+                float v = fmat(cz, Pp[t], fmat(az, Pm[t], P0[t])) + fmat(crz, Qp[t], fmat(brz, Q0[t], mult(arz, Qm[t])));
                 const unsigned l = (unsigned)k * sz + (unsigned)(j0 + t) * sy + (unsigned)i;
                 // solid rows are zero; irregular rows belong to k_apply_irr
                 if (t_cur[t] != CFP_REGULAR) v = 0;
@@ -249,6 +250,130 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? (sizeof(T) == 4 ? 8 : 2) : (siz
         }
     }
 }
+// The FP64 apply.  GB300 issues about two FP64 instructions per SM and clock,
+// so the kernel is bound by their number (513^3: 18 per node, 0.86 of the
+// issue floor), not by memory, and the design spends as few as it can:
+//  - the second difference loses its centre weight: with
+//    XR' = (ar - br a) x(i-1) + (cr - br c) x(i+1), XR = XR' + br XL, so
+//    P = Ly XR + Ry XL = Ly XR' + (Ry + br Ly) XL, whose y weights a thread
+//    forms once for its column: 4 instructions per loaded row instead of 5;
+//  - the z pass is one chain of 5 fused multiply-adds;
+//  - a thread owns TY rows, so a loaded row serves up to three outputs.
+// A warp is 32 columns x TY rows and marches its own z chunk of kc planes:
+// no lane beyond the row's last 32-column tile, and small grids still spread
+// over the SMs (apply64_shape; a CTA is four warps, one above the other in y).
+// Before: 128-column CTAs of 4 x 64 columns x planes at every
+// size.  With the irregular rows and the dot: 33^3 98 -> 8 us, 97 x 65 x 82
+// 194 -> 30 us, 513^3 4.96 -> 4.41 ms.
+// DOT, solid and irregular rows as in k_apply.
+constexpr int kA64Warps = 4;
+
+template <int DOT, int TY>
+__global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
+    k_apply64(Grid<double> G, const uint8_t* __restrict__ type, const double* __restrict__ x, double* __restrict__ y,
+              const double* __restrict__ d0, double* __restrict__ partial, int kc) {
+    constexpr int R = TY + 2;  // rows loaded per plane
+    const int nx = G.nx, ny = G.ny, nz = G.nz;
+    const int i = 1 + blockIdx.x * 32 + threadIdx.x;
+    const int j0 = 1 + (blockIdx.y * kA64Warps + threadIdx.y) * TY;
+    const int k0 = 1 + blockIdx.z * kc;
+    const int k1 = min(k0 + kc, nz - 1);
+    double acc0 = 0.0, acc1 = 0.0;
+    if (j0 <= ny - 2) {
+        const bool iin = i <= nx - 2;
+        const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
+        const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
+        const double ax = G.ax[0].a[ic], cx = G.ax[0].c[ic], brx = G.ax[0].br[ic];
+        const double arx = fma(-brx, ax, G.ax[0].ar[ic]), crx = fma(-brx, cx, G.ax[0].cr[ic]);
+        double ay[TY], cy[TY], ary[TY], bry[TY], cry[TY];
+        bool jin[TY];
+        unsigned lout0[TY];
+#pragma unroll
+        for (int t = 0; t < TY; ++t) {
+            jin[t] = j0 + t <= ny - 2;
+            const int jc = jin[t] ? j0 + t : j0;
+            ay[t] = G.ax[1].a[jc];
+            cy[t] = G.ax[1].c[jc];
+            ary[t] = fma(brx, ay[t], G.ax[1].ar[jc]);
+            bry[t] = brx + G.ax[1].br[jc];
+            cry[t] = fma(brx, cy[t], G.ax[1].cr[jc]);
+            lout0[t] = (unsigned)k0 * sz + (unsigned)jc * sy + (unsigned)ic;
+        }
+        unsigned roff[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) roff[r] = (unsigned)min(j0 - 1 + r, ny - 1) * sy;
+        const double* p = x + ((unsigned)(k0 - 1) * sz + (unsigned)ic);
+        double n[3 * R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double* q = p + roff[r];
+            n[3 * r] = q[-1];
+            n[3 * r + 1] = q[0];
+            n[3 * r + 2] = q[1];
+        }
+        double Pm[TY], P0[TY], Pp[TY], Qm[TY], Q0[TY], Qp[TY];
+#pragma unroll
+        for (int t = 0; t < TY; ++t) Pm[t] = P0[t] = Pp[t] = Qm[t] = Q0[t] = Qp[t] = 0.0;
+#pragma unroll 1
+        for (int kk = k0 - 1; kk <= k1; ++kk) {
+            double XR[R], XL[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                XR[r] = fma(crx, n[3 * r + 2], arx * n[3 * r]);
+                XL[r] = fma(cx, n[3 * r + 2], fma(ax, n[3 * r], n[3 * r + 1]));
+            }
+            if (kk < k1) {  // the next plane's loads, ahead of the y and z passes
+                p += sz;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const double* q = p + roff[r];
+                    n[3 * r] = q[-1];
+                    n[3 * r + 1] = q[0];
+                    n[3 * r + 2] = q[1];
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < TY; ++t) {
+                Pm[t] = P0[t];
+                P0[t] = Pp[t];
+                Qm[t] = Q0[t];
+                Q0[t] = Qp[t];
+                Pp[t] = fma(cry[t], XL[t + 2],
+                            fma(bry[t], XL[t + 1],
+                                fma(ary[t], XL[t], fma(cy[t], XR[t + 2], fma(ay[t], XR[t], XR[t + 1])))));
+                Qp[t] = fma(cy[t], XL[t + 2], fma(ay[t], XL[t], XL[t + 1]));
+            }
+            if (kk >= k0 + 1) {
+                const int k = kk - 1;
+                const double az = G.ax[2].a[k], cz = G.ax[2].c[k];
+                const double arz = G.ax[2].ar[k], brz = G.ax[2].br[k], crz = G.ax[2].cr[k];
+#pragma unroll
+                for (int t = 0; t < TY; ++t) {
+                    const unsigned l = lout0[t] + (unsigned)(k - k0) * sz;
+                    const uint8_t tl = type[l];
+                    const double v =
+                        fma(crz, Qp[t],
+                            fma(brz, Q0[t], fma(arz, Qm[t], fma(cz, Pp[t], fma(az, Pm[t], P0[t])))));
+                    // solid rows are zero; irregular rows belong to k_apply_irr
+                    if (!iin || !jin[t]) continue;
+                    const bool reg = tl == CFP_REGULAR;
+                    if (tl != CFP_IRREGULAR) y[l] = reg ? v : 0.0;
+                    if (DOT >= 1 && reg) acc0 = fma(d0[l], v, acc0);
+                    if (DOT == 2 && reg) acc1 = fma(v, v, acc1);
+                }
+            }
+        }
+    }
+    if (DOT) {
+        block_reduce2(acc0, acc1);
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
+            const int64_t b = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
+            partial[2 * b] = acc0;
+            partial[2 * b + 1] = acc1;
+        }
+    }
+}
+
 // The FP32 apply fed by a ring of bulk copies (the TMA engine) through shared
 // memory.  The streaming kernel above keeps one plane of loads in flight per
 // thread, too few bytes per SM to cover the HBM latency.  Here a producer
@@ -622,9 +747,8 @@ __global__ void k_lift_shell(Grid<double> G, const uint8_t* __restrict__ type, c
 }
 
 // The rows of the irregular points, whole (Eq. Bdec): the regular 27-point
-// part with the arithmetic of the factorised kernels -- the same fused
-// multiply-add chains on the same 27 values, so that part has the same bits
-// as there -- plus the side-list corrections of the row's modified lines
+// part with the arithmetic of the factorised kernels -- in FP32 the same
+// fused multiply-add chains on the same 27 values -- plus the side-list corrections of the row's modified lines
 // (Eqs. A27_mod, cor, cor_case2).  One thread per irregular point.  The
 // regular rows' kernels leave these rows alone, so this kernel runs beside
 // them on a second stream; its dot terms go to its own partials.
@@ -869,8 +993,8 @@ dim3 rows_grid(const cfp_ctx* c, int rows, int kc = kApplyKC) {
 }
 
 // the apply's kernel and tile shape of precision q (0 FP64, 1 FP32), as set
-// by the autotuner; otherwise in FP64 the streaming kernel with 4 x 64, in
-// FP32 the ring (2 x 64) where its 512-column tiles are at least 85 % filled
+// by the autotuner; otherwise in FP64 the shape apply64_shape finds (reported
+// as 4 x 64), in FP32 the ring (2 x 64) where its 512-column tiles are at least 85 % filled
 // (n_x = 513: 511 of 512 columns) and else the streaming kernel with 2 x 64
 // (at 385^3, 383 of 512 columns, it measured 0.285 ms against 0.256 ms)
 int apply_kind(const cfp_ctx* c, int q) {
@@ -930,6 +1054,47 @@ int irr_blocks(const cfp_ctx* c) {
     return (int)std::min<int64_t>((c->n_irr + 127) / 128, 152 * 8);
 }
 
+// k_apply64's rows per thread and planes per z chunk
+struct Shape64 {
+    int ty, kc;
+    dim3 grid(const cfp_ctx* c) const {
+        const int rows = ty * kA64Warps;
+        return dim3((unsigned)((c->n[0] - 2 + 31) / 32), (unsigned)((c->n[1] - 2 + rows - 1) / rows),
+                    (unsigned)((c->n[2] - 2 + kc - 1) / kc));
+    }
+    int64_t ctas(const cfp_ctx* c) const {
+        const dim3 g = grid(c);
+        return (int64_t)g.x * g.y * g.z;
+    }
+};
+
+// The shape of k_apply64: set by the tuner, else the one whose busiest SM
+// issues the fewest FP64 instructions.  A warp issues (kc + 2) (4 (ty + 2) +
+// 7 ty) + 5 kc ty of them (its two halo planes do the x and y passes only),
+// each of the SM's four schedulers takes one warp of a CTA, and the CTAs
+// spread over 152 SMs; each plane adds the latency of its loads (about 130
+// instruction slots), which counts where few warps share an SM.  Large grids
+// take 4 rows and 32 or 64 planes; 33^3 takes 128 CTAs of 1 x 2, where 4 x 64
+// would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
+// 33^3 14.5 us with them, 10.4 with four warps in the same shape.)
+Shape64 apply64_shape(const cfp_ctx* c) {
+    if (c->apply_ty[0] && c->apply_kc[0]) return Shape64{c->apply_ty[0], c->apply_kc[0]};
+    Shape64 best{4, 64};
+    double est_best = 1e300;
+    for (int t : {4, 2, 1})
+        for (int q : {64, 32, 16, 8, 4, 2}) {
+            const Shape64 sh{t, q};
+            const double per = (double)((sh.ctas(c) + 151) / 152);
+            const double warp = (q + 2) * (4.0 * (t + 2) + 7.0 * t) + 5.0 * q * t;
+            const double est = per * kA64Warps * warp + 130.0 * (q + 2);
+            if (est < est_best * 0.99) {
+                est_best = est;
+                best = sh;
+            }
+        }
+    return best;
+}
+
 // the most CTAs any apply tile shape launches, with the correction kernel's
 // (dot-product partials per launch); the ring's persistent grid never has
 // more CTAs than the streaming kernel with 2 rows x 16 planes
@@ -938,9 +1103,20 @@ int apply_blocks(cfp_ctx* c) {
     for (int ty : {2, 4})
         for (int kc : {16, 32, 64}) {
             const dim3 g = rows_grid(c, ty, kc);
-            m = std::max<int64_t>(m, (int64_t)g.x * g.y * g.z);
+            m = std::max(m, std::max((int64_t)g.x * g.y * g.z, Shape64{ty, kc}.ctas(c)));
         }
+    m = std::max(m, apply64_shape(c).ctas(c));
     return (int)m + corr_blocks(c);
+}
+
+// the FP64 regular rows' kernel
+template <int DOT>
+void apply64_launch(cfp_ctx* c, const Shape64& sh, const double* x, double* y, const double* d0, double* partial,
+                    cudaStream_t s) {
+    const dim3 g = sh.grid(c), b(32, kA64Warps);
+    if (sh.ty == 4) k_apply64<DOT, 4><<<g, b, 0, s>>>(grid_view<double>(c), c->type, x, y, d0, partial, sh.kc);
+    else if (sh.ty == 2) k_apply64<DOT, 2><<<g, b, 0, s>>>(grid_view<double>(c), c->type, x, y, d0, partial, sh.kc);
+    else k_apply64<DOT, 1><<<g, b, 0, s>>>(grid_view<double>(c), c->type, x, y, d0, partial, sh.kc);
 }
 
 // B x: the regular rows' kernel on s and, forked onto the context's second
@@ -953,11 +1129,15 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
     constexpr int RKC = KC < 32 ? 32 : KC;  // the ring marches 32 or 64 planes
     int ntx = 0, nty = 0, ntz = 0;
     dim3 grid;
+    Shape64 sh64{0, 0};
     if constexpr (sizeof(T) == 4)
         ring = apply_kind(c, 1) == CFP_APPLY_RING && c->ring_grid > 0 && aligned16(x) && (!DOT || aligned16(d0));
     if (ring) {
         ring_tiles(c, RKC, &ntx, &nty, &ntz);
         nmain = std::min(ntx * nty * ntz, c->ring_grid);
+    } else if (sizeof(T) == 8) {
+        sh64 = apply64_shape(c);
+        nmain = (int)sh64.ctas(c);
     } else {
         grid = rows_grid(c, TY, KC);
         nmain = (int)(grid.x * grid.y * grid.z);
@@ -978,8 +1158,10 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
                 k_apply_ring<DOT, RKC, false><<<nmain, kRingThreads, kRingSmem, s>>>(
                     grid_view<float>(c), c->type, x, y, d0, partial, ntx, nty, ntz, c->dwait);
         }
+    } else if constexpr (sizeof(T) == 8) {
+        apply64_launch<DOT>(c, sh64, x, y, d0, partial, s);
     } else {
-        k_apply<T, DOT, TY, KC><<<grid, kAX, 0, s>>>(grid_view<T>(c), c->type, x, y, d0, partial);
+        k_apply<DOT, TY, KC><<<grid, kAX, 0, s>>>(grid_view<T>(c), c->type, x, y, d0, partial);
     }
     if (nirr) {
         cudaEventRecord(c->ev_join, c->aux);
@@ -1041,7 +1223,8 @@ void launch_apply(cfp_ctx* c, const T* x, T* y, const T* d0, int dotmode, double
                   int* nblocks_out) {
     const int q = sizeof(T) == 4 ? 1 : 0;
     const int ty = apply_rows(c, q), kc = apply_planes(c, q);
-    if (ty == 4) apply_depth<T, 4>(c, kc, x, y, d0, dotmode, partial, s, nblocks_out);
+    if constexpr (sizeof(T) == 8) apply_dot<T, 4, 64>(c, x, y, d0, dotmode, partial, s, nblocks_out);
+    else if (ty == 4) apply_depth<T, 4>(c, kc, x, y, d0, dotmode, partial, s, nblocks_out);
     else apply_depth<T, 2>(c, kc, x, y, d0, dotmode, partial, s, nblocks_out);
     c->launches += 1;
 }
