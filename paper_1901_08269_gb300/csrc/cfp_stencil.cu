@@ -86,8 +86,8 @@ __device__ __forceinline__ void block_reduce2(double& a, double& b) {
 }
 
 // Fused multiply-add in either precision: the apply's sums are written as
-// explicit chains so that every tile shape (in FP32: every kernel) rounds
-// each row the same way.
+// explicit chains so that every kernel and tile shape rounds each row the same
+// way.
 __device__ __forceinline__ float fmat(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmat(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mult(float a, float b) { return __fmul_rn(a, b); }
@@ -251,20 +251,18 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? 8 : 4)
     }
 }
 // The FP64 apply.  GB300 issues about two FP64 instructions per SM and clock,
-// so the kernel is bound by their number (513^3: 18 per node, 0.86 of the
-// issue floor), not by memory, and the design spends as few as it can:
-//  - the second difference loses its centre weight: with
-//    XR' = (ar - br a) x(i-1) + (cr - br c) x(i+1), XR = XR' + br XL, so
-//    P = Ly XR + Ry XL = Ly XR' + (Ry + br Ly) XL, whose y weights a thread
-//    forms once for its column: 4 instructions per loaded row instead of 5;
-//  - the z pass is one chain of 5 fused multiply-adds;
-//  - a thread owns TY rows, so a loaded row serves up to three outputs.
+// so the kernel is bound by their number (20.5 per node with four rows to a
+// thread: 5 per loaded row, 7 and 6 per output in y and z), not by memory.
+// (Folding the x operator's centre weight into the y weights would save one
+// per loaded row, and one chain for the z pass one per output, but both round
+// worse: 1.4 to 2.3 times the error on smooth fields of stretched grids for
+// the first.)
 // A warp is 32 columns x TY rows and marches its own z chunk of kc planes:
 // no lane beyond the row's last 32-column tile, and small grids still spread
 // over the SMs (apply64_shape; a CTA is four warps, one above the other in y).
 // Before: 128-column CTAs of 4 x 64 columns x planes at every
 // size.  With the irregular rows and the dot: 33^3 98 -> 8 us, 97 x 65 x 82
-// 194 -> 30 us, 513^3 4.96 -> 4.41 ms.
+// 194 -> 36 us, 129^3 199 -> 110 us; 513^3 is as before (5.0 ms).
 // DOT, solid and irregular rows as in k_apply.
 constexpr int kA64Warps = 4;
 
@@ -283,8 +281,8 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
         const bool iin = i <= nx - 2;
         const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
         const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
-        const double ax = G.ax[0].a[ic], cx = G.ax[0].c[ic], brx = G.ax[0].br[ic];
-        const double arx = fma(-brx, ax, G.ax[0].ar[ic]), crx = fma(-brx, cx, G.ax[0].cr[ic]);
+        const double ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
+        const double arx = G.ax[0].ar[ic], brx = G.ax[0].br[ic], crx = G.ax[0].cr[ic];
         double ay[TY], cy[TY], ary[TY], bry[TY], cry[TY];
         bool jin[TY];
         unsigned lout0[TY];
@@ -294,9 +292,9 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
             const int jc = jin[t] ? j0 + t : j0;
             ay[t] = G.ax[1].a[jc];
             cy[t] = G.ax[1].c[jc];
-            ary[t] = fma(brx, ay[t], G.ax[1].ar[jc]);
-            bry[t] = brx + G.ax[1].br[jc];
-            cry[t] = fma(brx, cy[t], G.ax[1].cr[jc]);
+            ary[t] = G.ax[1].ar[jc];
+            bry[t] = G.ax[1].br[jc];
+            cry[t] = G.ax[1].cr[jc];
             lout0[t] = (unsigned)k0 * sz + (unsigned)jc * sy + (unsigned)ic;
         }
         unsigned roff[R];
@@ -319,8 +317,8 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
             double XR[R], XL[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                XR[r] = fma(crx, n[3 * r + 2], arx * n[3 * r]);
-                XL[r] = fma(cx, n[3 * r + 2], fma(ax, n[3 * r], n[3 * r + 1]));
+                XR[r] = fmat(crx, n[3 * r + 2], fmat(brx, n[3 * r + 1], mult(arx, n[3 * r])));
+                XL[r] = fmat(cx, n[3 * r + 2], fmat(ax, n[3 * r], n[3 * r + 1]));
             }
             if (kk < k1) {  // the next plane's loads, ahead of the y and z passes
                 p += sz;
@@ -338,10 +336,10 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
                 P0[t] = Pp[t];
                 Qm[t] = Q0[t];
                 Q0[t] = Qp[t];
-                Pp[t] = fma(cry[t], XL[t + 2],
-                            fma(bry[t], XL[t + 1],
-                                fma(ary[t], XL[t], fma(cy[t], XR[t + 2], fma(ay[t], XR[t], XR[t + 1])))));
-                Qp[t] = fma(cy[t], XL[t + 2], fma(ay[t], XL[t], XL[t + 1]));
+                Pp[t] = fmat(cry[t], XL[t + 2],
+                             fmat(bry[t], XL[t + 1],
+                                  fmat(ary[t], XL[t], fmat(cy[t], XR[t + 2], fmat(ay[t], XR[t], XR[t + 1])))));
+                Qp[t] = fmat(cy[t], XL[t + 2], fmat(ay[t], XL[t], XL[t + 1]));
             }
             if (kk >= k0 + 1) {
                 const int k = kk - 1;
@@ -351,15 +349,14 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
                 for (int t = 0; t < TY; ++t) {
                     const unsigned l = lout0[t] + (unsigned)(k - k0) * sz;
                     const uint8_t tl = type[l];
-                    const double v =
-                        fma(crz, Qp[t],
-                            fma(brz, Q0[t], fma(arz, Qm[t], fma(cz, Pp[t], fma(az, Pm[t], P0[t])))));
+                    const double v = fmat(cz, Pp[t], fmat(az, Pm[t], P0[t])) +
+                                     fmat(crz, Qp[t], fmat(brz, Q0[t], mult(arz, Qm[t])));
                     // solid rows are zero; irregular rows belong to k_apply_irr
                     if (!iin || !jin[t]) continue;
                     const bool reg = tl == CFP_REGULAR;
                     if (tl != CFP_IRREGULAR) y[l] = reg ? v : 0.0;
-                    if (DOT >= 1 && reg) acc0 = fma(d0[l], v, acc0);
-                    if (DOT == 2 && reg) acc1 = fma(v, v, acc1);
+                    if (DOT >= 1 && reg) acc0 = fmat(d0[l], v, acc0);
+                    if (DOT == 2 && reg) acc1 = fmat(v, v, acc1);
                 }
             }
         }
@@ -747,8 +744,9 @@ __global__ void k_lift_shell(Grid<double> G, const uint8_t* __restrict__ type, c
 }
 
 // The rows of the irregular points, whole (Eq. Bdec): the regular 27-point
-// part with the arithmetic of the factorised kernels -- in FP32 the same
-// fused multiply-add chains on the same 27 values -- plus the side-list corrections of the row's modified lines
+// part with the arithmetic of the factorised kernels -- the same fused
+// multiply-add chains on the same 27 values, so that part has the same bits
+// as there -- plus the side-list corrections of the row's modified lines
 // (Eqs. A27_mod, cor, cor_case2).  One thread per irregular point.  The
 // regular rows' kernels leave these rows alone, so this kernel runs beside
 // them on a second stream; its dot terms go to its own partials.
@@ -1068,14 +1066,15 @@ struct Shape64 {
     }
 };
 
-// The shape of k_apply64: set by the tuner, else the one whose busiest SM
-// issues the fewest FP64 instructions.  A warp issues (kc + 2) (4 (ty + 2) +
-// 7 ty) + 5 kc ty of them (its two halo planes do the x and y passes only),
-// each of the SM's four schedulers takes one warp of a CTA, and the CTAs
-// spread over 152 SMs; each plane adds the latency of its loads (about 130
-// instruction slots), which counts where few warps share an SM.  Large grids
-// take 4 rows and 32 or 64 planes; 33^3 takes 128 CTAs of 1 x 2, where 4 x 64
-// would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
+// The shape of k_apply64: set by the tuner, else the one with the smallest
+// estimate.  A warp issues w = (kc + 2) (5 (ty + 2) + 7 ty) + 6 kc ty FP64
+// instructions (its two halo planes do the x and y passes only), a CTA 4 w;
+// the estimate is the busiest of 152 SMs, the latency of a plane's loads
+// (about 130 slots per plane), which counts where few CTAs share an SM, and,
+// past four CTAs per SM, half of a last one that runs alone.  Large grids
+// take 4 rows and 64 planes, 129^3 and 257^3 4 x 16 (109 and 712 us; 4 x 64
+// 250 and 895), 97 x 65 x 82 2 x 8; 33^3 takes 128 CTAs of 1 x 2, where 4 x
+// 64 would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
 // 33^3 14.5 us with them, 10.4 with four warps in the same shape.)
 Shape64 apply64_shape(const cfp_ctx* c) {
     if (c->apply_ty[0] && c->apply_kc[0]) return Shape64{c->apply_ty[0], c->apply_kc[0]};
@@ -1084,9 +1083,9 @@ Shape64 apply64_shape(const cfp_ctx* c) {
     for (int t : {4, 2, 1})
         for (int q : {64, 32, 16, 8, 4, 2}) {
             const Shape64 sh{t, q};
+            const double cta = kA64Warps * ((q + 2) * (5.0 * (t + 2) + 7.0 * t) + 6.0 * q * t);
             const double per = (double)((sh.ctas(c) + 151) / 152);
-            const double warp = (q + 2) * (4.0 * (t + 2) + 7.0 * t) + 5.0 * q * t;
-            const double est = per * kA64Warps * warp + 130.0 * (q + 2);
+            const double est = per * cta + 130.0 * (q + 2) + (per > 4 ? 0.5 * cta : 0.0);
             if (est < est_best * 0.99) {
                 est_best = est;
                 best = sh;
