@@ -152,7 +152,7 @@ struct MgLevel {
                                // in FP32: TMA tensor maps need 16-byte row strides)
     int64_t Nh = 0;            // entries per colour array: hp * n[1] * n[2]
     uint8_t* stype = nullptr;  // split type, colour c at stype + c * Nh
-    double* s64 = nullptr;     // split e0 e1 b0 b1 r0 (Nh each), FP64
+    double* s64 = nullptr;     // split e0 e1 b0 b1 r0 and the reciprocal diagonals of both colours (Nh each), FP64
     float* s32 = nullptr;      // the same in FP32; b holds NaN at every entry that is not an unknown
     void* pk64 = nullptr;      // packed (ka, kb, kc, 0) per index, x then y then z, FP64
     void* pk32 = nullptr;      // the same in FP32

@@ -106,6 +106,7 @@ struct SLev {
     T* e[2];                    // the iterate per colour
     T* b[2];                    // the right-hand side per colour
     T* r0;                      // the red residual
+    const T* rd[2];             // FP64: reciprocal diagonals per colour (see times_rd)
 };
 
 // the arrays one half-sweep of colour c touches (chosen on the host)
@@ -117,6 +118,7 @@ struct Half {
     T* bown;             // b of colour c
     T* both;             // b of the other colour (written in MODE 2)
     const uint8_t* tyo;  // type of the other colour (MODE 2)
+    const T* rd;         // FP64: reciprocal diagonals of colour c
 };
 
 // FP32 levels hold NaN in b at every entry that is not an unknown (the TMA
@@ -127,55 +129,83 @@ enum { kSplitVecs = 5 };  // e0 e1 b0 b1 r0
 
 __device__ __forceinline__ bool is_unknown(uint8_t t) { return t == CFP_REGULAR || t == CFP_IRREGULAR; }
 
-// x * (1 / d).  FP64: a correctly rounded reciprocal (two roundings instead
-// of the division's one, several times cheaper than an IEEE division).  FP32:
-// the hardware reciprocal approximation (rcp.approx.ftz.f32, within 1 ulp of
-// 1 / d; the diagonal of K is a normal number), a single instruction where the
-// correctly rounded one costs a short sequence: the FP32 smoother is the inner
-// preconditioner of the mixed solve, whose FP64 refinement removes the error.
-// The off-diagonal sum of a half-sweep node,
-//   (cx_lo xm + cx_hi xp) + (cy_lo ym + cy_hi yp) + (cz_lo zm + cz_hi zp),
-// each pair one product and one fused multiply-add in this order: written
-// out so that every kernel that updates a node (one launch per half-sweep,
-// the TMA pipeline, the single-CTA smoothing) rounds it the same way.
-__device__ __forceinline__ float rb_pair(float a, float x, float b, float y) { return __fmaf_rn(b, y, __fmul_rn(a, x)); }
-__device__ __forceinline__ double rb_pair(double a, double x, double b, double y) {
-    return __fma_rn(b, y, __dmul_rn(a, x));
+// What a half-sweep divides by its diagonal: b minus the off-diagonal sum, as
+// one chain of six fused multiply-adds in the order x, y, z (low neighbour
+// first).  Every kernel that updates a node uses this chain, so all give the
+// same bits.
+__device__ __forceinline__ float rb_rest(float b, float cxl, float cxh, float cyl, float cyh, float czl, float czh,
+                                         float xm, float xp, float ym, float yp, float zm, float zp) {
+    float v = __fmaf_rn(-cxl, xm, b);
+    v = __fmaf_rn(-cxh, xp, v);
+    v = __fmaf_rn(-cyl, ym, v);
+    v = __fmaf_rn(-cyh, yp, v);
+    v = __fmaf_rn(-czl, zm, v);
+    return __fmaf_rn(-czh, zp, v);
 }
-template <class T>
-__device__ __forceinline__ T rb_sum(T cxl, T cxh, T cyl, T cyh, T czl, T czh, T xm, T xp, T ym, T yp, T zm, T zp) {
-    return (rb_pair(cxl, xm, cxh, xp) + rb_pair(cyl, ym, cyh, yp)) + rb_pair(czl, zm, czh, zp);
+__device__ __forceinline__ double rb_rest(double b, double cxl, double cxh, double cyl, double cyh, double czl,
+                                          double czh, double xm, double xp, double ym, double yp, double zm,
+                                          double zp) {
+    double v = __fma_rn(-cxl, xm, b);
+    v = __fma_rn(-cxh, xp, v);
+    v = __fma_rn(-cyl, ym, v);
+    v = __fma_rn(-cyh, yp, v);
+    v = __fma_rn(-czl, zm, v);
+    return __fma_rn(-czh, zp, v);
 }
 
+// FP32: x * (1 / d) with the hardware reciprocal approximation
+// (rcp.approx.ftz.f32, within 1 ulp of 1 / d; the diagonal of K is a normal
+// number), a single instruction where the correctly rounded one costs a short
+// sequence: the FP32 smoother is the inner preconditioner of the mixed solve,
+// whose FP64 refinement removes the error.
 __device__ __forceinline__ float times_rcp(float x, float d) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
     return x * r;
 }
-__device__ __forceinline__ double times_rcp(double x, double d) { return x * __drcp_rn(d); }
 
-// One red-black half-sweep of colour `colour` on a split level, with K's
-// regular coefficients at every node.  Thread (m, j, k0 + q), q <
-// kSweepPlanes, owns the pair of nodes i = 2m, 2m + 1 of rows (j, k0 + q);
-// its node of this colour is i = 2m + par.  Its x-neighbours (the other
-// colour) sit at entries m - 1 + par and m + par of the other colour's row.
-// Every load is in bounds for every thread that passes the first test (rows
-// j, k and the pair are interior, entry m - 1 exists for m = 0 because the
-// row is not the first; planes past the last interior one repeat plane k0
-// and store nothing), so the loads of all kSweepPlanes nodes are issued
-// before any value is stored: three independent nodes per thread keep more
-// loads in flight.  The Shortley-Weller rows of the fine level's irregular
-// nodes are applied afterwards by k_sweep_fix (no node reads another of its
-// own colour, so the order within the half-sweep does not matter).
+// FP64: a level keeps the correctly rounded reciprocal of every node's
+// diagonal (SLev::rd, k_fill_rd), because GB300 issues about two FP64
+// instructions per SM and clock and the reciprocal is eight of them, the
+// diagonal's sum two: with the array a node update is six fused
+// multiply-adds and one product (7 instead of about 20) for 8 more bytes
+// read: a half-sweep of 129^3 nodes 42 -> 21 us, of 513^3 2.06 -> 1.08 ms.  An entry is 0
+// where the node is not an unknown, the reciprocal (negative, as K's
+// diagonal) at a node with K's regular coefficients, and the reciprocal's
+// magnitude where the node is irregular (its Shortley-Weller row comes from
+// the side list): it also stands for the type.
+__device__ __forceinline__ double times_rd(double x, double rd) { return -(x * fabs(rd)); }
+
+// The off-diagonal coefficients of one node, in rb_rest's order; with a
+// Shortley-Weller row, from the side list.
+template <class T>
+struct Off {
+    T xl, xh, yl, yh, zl, zh;
+};
+
+// One red-black half-sweep of colour `colour` on a split level.  Thread (m,
+// j, k0 + q), q < kSweepPlanes, owns the pair of nodes i = 2m, 2m + 1 of rows
+// (j, k0 + q); its node of this colour is i = 2m + par.  Its x-neighbours
+// (the other colour) sit at entries m - 1 + par and m + par of the other
+// colour's row.  Every load is in bounds for every thread that passes the
+// first test (rows j, k and the pair are interior, entry m - 1 exists for
+// m = 0 because the row is not the first; planes past the last interior one
+// repeat plane k0 and store nothing), so the loads of all kSweepPlanes nodes
+// are issued before any value is stored: three independent nodes per thread
+// keep more loads in flight.  FINE: the fine level, whose irregular nodes
+// take their Shortley-Weller rows (Eq. A7_mod) from the side list: few
+// nodes (0.3 % at 513^3), whose dependent loads other warps cover, for one
+// launch less per half-sweep than a follow-up kernel.
 // MODE 0: plain; 1: from zero (the other colour is taken as zero);
 // 2: from zero, and b of both colours is first read from the natural-layout
 //    rho; 3: plain, and both nodes of the pair are written to the
 //    natural-layout phi (the own node's new value is not stored).
 constexpr int kSweepPlanes = 3;
 
-template <class T, int MODE>
+template <class T, int MODE, bool FINE>
 __global__ void __launch_bounds__(kSplitThreads)
-    k_sweep_split(SLev<T> L, Half<T> H, int colour, const T* __restrict__ rho, T* __restrict__ phi) {
+    k_sweep_split(SLev<T> L, Half<T> H, Side<T> S, int colour, const T* __restrict__ rho, T* __restrict__ phi) {
+    constexpr bool F64 = sizeof(T) == 8, READ = MODE == 0 || MODE == 3;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes * blockIdx.z;
@@ -194,17 +224,20 @@ __global__ void __launch_bounds__(kSplitThreads)
         const int i = 2 * m + par, io = 2 * m + 1 - par;
         const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
         const int64_t row = ((int64_t)k * L.ny + j) * nx;
-        const uint8_t t = H.ty[o];
+        // which nodes are unknowns (and irregular): FP64 from the reciprocal
+        // diagonal, FP32 from the type
+        const T rd = F64 ? H.rd[o] : T(0);
+        const uint8_t t = F64 ? (uint8_t)CFP_REGULAR : H.ty[o];
         bv[q] = MODE == 2 ? rho[row + i] : H.bown[o];
         if (MODE == 2) {
             bo[q] = rho[row + io];
-            if (sizeof(T) == 4) {  // the NaN marks of the FP32 levels
+            if (!F64) {  // the NaN marks of the FP32 levels
                 if (!is_unknown(t)) bv[q] = T(b_mark());
                 if (!is_unknown(H.tyo[o])) bo[q] = T(b_mark());
             }
         }
         T xm = T(0), xp = T(0), ym = T(0), yp = T(0), zm = T(0), zp = T(0);
-        if (MODE == 0 || MODE == 3) {
+        if (READ) {
             xm = eoth[o - 1 + par];
             xp = eoth[o + par];
             ym = eoth[o - hp];
@@ -213,12 +246,18 @@ __global__ void __launch_bounds__(kSplitThreads)
             zp = eoth[o + hs];
         }
         const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-        const T dg = ckx.y + (cky.y + ckz.y);
-        live[q] = inz[q] && i >= 1 && i <= nx - 2 && is_unknown(t);
+        live[q] = inz[q] && i >= 1 && i <= nx - 2 && (F64 ? rd != T(0) : is_unknown(t));
+        Off<T> f{ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z};
+        T dg = F64 ? T(0) : ckx.y + (cky.y + ckz.y);
+        if (FINE && live[q] && (F64 ? rd > T(0) : t == CFP_IRREGULAR)) {
+            const T* kr = S.krow + 7 * (int64_t)S.slot[row + i];
+            f = Off<T>{kr[1], kr[2], kr[3], kr[4], kr[5], kr[6]};
+            dg = kr[0];
+        }
         T v = bv[q];
-        if (MODE == 0 || MODE == 3)
-            v -= rb_sum(ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z, xm, xp, ym, yp, zm, zp);
-        val[q] = times_rcp(v, dg);
+        if (READ) v = rb_rest(v, f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, xm, xp, ym, yp, zm, zp);
+        if constexpr (F64) val[q] = times_rd(v, rd);
+        else val[q] = times_rcp(v, dg);
         xo[q] = par ? xm : xp;  // MODE 3: the other node of the pair
         oo[q] = o;
     }
@@ -243,13 +282,32 @@ __global__ void __launch_bounds__(kSplitThreads)
     }
 }
 
+// FP64: the reciprocal diagonals of a level (times_rd); S.krow null below
+// the fine level
+__global__ void k_fill_rd(SLev<double> L, Side<double> S, double* __restrict__ rd, int64_t Nh) {
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 2 * Nh; q += (int64_t)gridDim.x * blockDim.x) {
+        const int c = q >= Nh;
+        const int64_t e = q - c * Nh;
+        const uint8_t t = L.ty[c][e];
+        double r = 0.0;
+        if (is_unknown(t)) {  // an interior node
+            const int m = (int)(e % L.hp);
+            const int64_t rowi = e / L.hp;
+            const int j = (int)(rowi % L.ny), k = (int)(rowi / L.ny), i = 2 * m + ((c + j + k) & 1);
+            if (t == CFP_IRREGULAR && S.krow) r = fabs(__drcp_rn(S.krow[7 * (int64_t)S.slot[rowi * L.nx + i]]));
+            else r = __drcp_rn(L.cx[i].y + (L.cy[j].y + L.cz[k].y));
+        }
+        rd[q] = r;
+    }
+}
+
 // All the red-black sweeps of one smoothing of a small level (at most
 // kCoarseMaxNodes nodes: the coarsest level's 16 sweeps, a 17^3 level's
 // pre- or post-smoothing) in one CTA, with a CTA barrier between
 // half-sweeps, where separate launches would cost a few microseconds each
 // for a few thousand nodes.  The node update is k_sweep_split's (MODE 1 for
-// a first red half-sweep from zero, MODE 0 otherwise) with the same rb_sum
-// and reciprocal: the results are bitwise equal.
+// a first red half-sweep from zero, MODE 0 otherwise): the results are
+// bitwise equal.
 // CLUSTER: the same with the CTAs of one thread-block cluster (up to 16,
 // one per SM) and a cluster barrier, whose release / acquire order the
 // global writes of one half-sweep before the reads of the next, for levels
@@ -277,6 +335,7 @@ __global__ void __launch_bounds__(CLUSTER ? kClusterThreads : kCoarseThreads)
         T* eown = colour ? L.e[1] : L.e[0];
         const T* eoth = colour ? L.e[0] : L.e[1];
         const T* bown = colour ? L.b[1] : L.b[0];
+        const T* rdc = colour ? L.rd[1] : L.rd[0];
         const uint8_t* ty = colour ? L.ty[1] : L.ty[0];
         for (int64_t it = t0; it < items; it += nt) {
             const int m = (int)(it % mp);
@@ -285,8 +344,9 @@ __global__ void __launch_bounds__(CLUSTER ? kClusterThreads : kCoarseThreads)
             const int par = (colour + j + k) & 1;
             const int i = 2 * m + par;
             const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
-            const uint8_t t = ty[o];
+            const T rd = sizeof(T) == 8 ? rdc[o] : T(0);
             T v = bown[o];
+            const bool unk = sizeof(T) == 8 ? rd != T(0) : is_unknown(ty[o]);
             T xm = T(0), xp = T(0), ym = T(0), yp = T(0), zm = T(0), zp = T(0);
             if (!zero) {
                 xm = eoth[o - 1 + par];
@@ -297,10 +357,11 @@ __global__ void __launch_bounds__(CLUSTER ? kClusterThreads : kCoarseThreads)
                 zp = eoth[o + hs];
             }
             const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-            const T dg = ckx.y + (cky.y + ckz.y);
-            if (!zero) v -= rb_sum(ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z, xm, xp, ym, yp, zm, zp);
-            const T val = times_rcp(v, dg);
-            if (i >= 1 && i <= nx - 2 && is_unknown(t)) eown[o] = val;
+            if (!zero) v = rb_rest(v, ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z, xm, xp, ym, yp, zm, zp);
+            T val;
+            if constexpr (sizeof(T) == 8) val = times_rd(v, rd);
+            else val = times_rcp(v, ckx.y + (cky.y + ckz.y));
+            if (i >= 1 && i <= nx - 2 && unk) eown[o] = val;
         }
         if (CLUSTER) cooperative_groups::this_cluster().sync();
         else __syncthreads();
@@ -522,12 +583,10 @@ __global__ void __launch_bounds__(kTmaThreads)
                 const bool in = (ly & 1) ? ino : ine;  // the node of this colour is an interior column
                 if (KIND == 1) {
                     const float e0 = Es[ly * kTmaTX];
-                    const float ke =
-                        dg * e0 + (cx.x * xm + cx.z * xp) + (cya[ly] * ym + cyc[ly] * yp) + (cz.x * zm + cz.z * zp);
-                    if (in && jin[ly] && unk) ep[ly * hp] = b - ke;
+                    const float v = rb_rest(b, cx.x, cx.z, cya[ly], cyc[ly], cz.x, cz.z, xm, xp, ym, yp, zm, zp);
+                    if (in && jin[ly] && unk) ep[ly * hp] = __fmaf_rn(-dg, e0, v);
                 } else {
-                    float v = b;
-                    v -= rb_sum(cx.x, cx.z, cya[ly], cyc[ly], cz.x, cz.z, xm, xp, ym, yp, zm, zp);
+                    const float v = rb_rest(b, cx.x, cx.z, cya[ly], cyc[ly], cz.x, cz.z, xm, xp, ym, yp, zm, zp);
                     if (KIND == 0) {
                         if (in && jin[ly] && unk) ep[ly * hp] = times_rcp(v, dg);
                     } else if (jin[ly]) {
@@ -651,24 +710,21 @@ __global__ void k_fix_rows(const FixPt* __restrict__ list, int n, int nx, int64_
     }
 }
 
-// The half-sweep's update at the fine level's irregular nodes of colour
-// `colour` (the list of that colour), with their Shortley-Weller rows
-// (Eq. A7_mod); one thread per node.  Runs right after the half-sweep of the
-// same colour and mode, overwriting what it stored there.
-template <class T, int MODE>
-__global__ void k_sweep_fix(SLev<T> L, Side<T> S, Half<T> H, const FixPt* __restrict__ list, int64_t n,
-                            T* __restrict__ phi) {
+// The update at the fine level's irregular nodes of colour `colour` (the
+// list of that colour) after a TMA-fed FP32 half-sweep, with their
+// Shortley-Weller rows (Eq. A7_mod); one thread per node, overwriting what
+// the half-sweep stored there (MODE 0, or 3: in phi).
+template <int MODE>
+__global__ void k_sweep_fix(SLev<float> L, Side<float> S, Half<float> H, const FixPt* __restrict__ list, int64_t n,
+                            float* __restrict__ phi) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         const FixPt p = list[q];
         const int par = p.par;
         const unsigned o = p.o;
-        const T* kr = S.krow + 7 * (int64_t)p.slot;
-        T v = H.bown[o];
-        if (MODE == 0 || MODE == 3) {
-            const T* __restrict__ eoth = H.eoth;
-            v -= rb_sum(kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], eoth[o - 1 + par], eoth[o + par], eoth[o - L.hp],
-                        eoth[o + L.hp], eoth[o - L.hs], eoth[o + L.hs]);
-        }
+        const float* kr = S.krow + 7 * (int64_t)p.slot;
+        const float* __restrict__ eoth = H.eoth;
+        float v = rb_rest(H.bown[o], kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], eoth[o - 1 + par], eoth[o + par],
+                          eoth[o - L.hp], eoth[o + L.hp], eoth[o - L.hs], eoth[o + L.hs]);
         v = times_rcp(v, kr[0]);
         if (MODE == 3) phi[p.lin] = v;
         else H.eown[o] = v;
@@ -725,8 +781,8 @@ __device__ __forceinline__ void pair_bar() { asm volatile("bar.sync 1, %0;" ::"n
 // an unknown interior node (live false or b NaN), as the black array holds
 __device__ __forceinline__ float pair_node(const float* Ym, const float* Y0, const float* Yp, float b, int c, int par,
                                            float4 cx, float4 cy, float4 cz, bool live) {
-    const float v = b - rb_sum(cx.x, cx.z, cy.x, cy.z, cz.x, cz.z, Y0[c - 1 + par], Y0[c + par], Y0[c - kPairOX],
-                               Y0[c + kPairOX], Ym[c], Yp[c]);
+    const float v = rb_rest(b, cx.x, cx.z, cy.x, cy.z, cz.x, cz.z, Y0[c - 1 + par], Y0[c + par], Y0[c - kPairOX],
+                            Y0[c + kPairOX], Ym[c], Yp[c]);
     const float dg = cx.y + (cy.y + cz.y);
     return live && b == b ? times_rcp(v, dg) : 0.f;
 }
@@ -894,8 +950,8 @@ __global__ void __launch_bounds__(kPairThreads, 4)
                         if (mm < -1 || mm > kPairTX) continue;
                         const float* kr = F.krow + 7 * (int64_t)p.slot;
                         const int cb = (r + 1) * kPairOX + mm + 4, c = cb + kPairOX, par = p.par;
-                        const float v = Bx[cb] - rb_sum(kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], Y0[c - 1 + par],
-                                                        Y0[c + par], Y0[c - kPairOX], Y0[c + kPairOX], Ym[c], Yp[c]);
+                        const float v = rb_rest(Bx[cb], kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], Y0[c - 1 + par],
+                                                Y0[c + par], Y0[c - kPairOX], Y0[c + kPairOX], Ym[c], Yp[c]);
                         xb[cb] = times_rcp(v, kr[0]);
                     }
                 }
@@ -914,8 +970,8 @@ __global__ void __launch_bounds__(kPairThreads, 4)
                     const float4 cx = par ? c1 : c0;
                     const int c = (r0 + ly + 1) * kPairOX + lx + 4;
                     const float b = By[(r0 + ly) * kPairTX + lx];
-                    const float v = b - rb_sum(cx.x, cx.z, cyo[ly].x, cyo[ly].z, cz.x, cz.z, X0[c - 1 + par],
-                                               X0[c + par], X0[c - kPairOX], X0[c + kPairOX], Xm[c], xb[c]);
+                    const float v = rb_rest(b, cx.x, cx.z, cyo[ly].x, cyo[ly].z, cz.x, cz.z, X0[c - 1 + par],
+                                            X0[c + par], X0[c - kPairOX], X0[c + kPairOX], Xm[c], xb[c]);
                     const float dg = cx.y + (cyo[ly].y + cz.y);
                     const unsigned o = (unsigned)kr * hs + (unsigned)((j0 + r0 + ly) * hp + m);
                     if ((par ? in1 : in0) && jin[ly] && b == b) red_out[o] = times_rcp(v, dg);
@@ -932,9 +988,9 @@ __global__ void __launch_bounds__(kPairThreads, 4)
                             if (mm < 0 || mm >= kPairTX) continue;
                             const float* kr7 = F.krow + 7 * (int64_t)p.slot;
                             const int c = (r + 1) * kPairOX + mm + 4, par = p.par;
-                            const float v = By[r * kPairTX + mm] -
-                                            rb_sum(kr7[1], kr7[2], kr7[3], kr7[4], kr7[5], kr7[6], X0[c - 1 + par],
-                                                   X0[c + par], X0[c - kPairOX], X0[c + kPairOX], Xm[c], xb[c]);
+                            const float v = rb_rest(By[r * kPairTX + mm], kr7[1], kr7[2], kr7[3], kr7[4], kr7[5], kr7[6],
+                                                    X0[c - 1 + par], X0[c + par], X0[c - kPairOX], X0[c + kPairOX], Xm[c],
+                                                    xb[c]);
                             red_out[p.o] = times_rcp(v, kr7[0]);
                         }
                     }
@@ -952,12 +1008,14 @@ __global__ void __launch_bounds__(kPairThreads, 4)
     }
 }
 
-// r0 = b0 - K e at the red unknowns with K's regular coefficients (black
-// residuals are zero after a black half-sweep; r0 stays zero at the other
-// red entries); three planes per thread with all loads first, as in the
-// half-sweep.  k_resid_fix then redoes the fine level's irregular red nodes.
-template <class T>
-__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L) {
+// r0 = b0 - K e at the red unknowns (black residuals are zero after a black
+// half-sweep; r0 stays zero at the other red entries): the half-sweep's chain
+// and one more product with the diagonal; three planes per thread with all
+// loads first, and the fine level's Shortley-Weller rows, as in the
+// half-sweep.
+template <class T, bool FINE>
+__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S) {
+    constexpr bool F64 = sizeof(T) == 8;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes * blockIdx.z;
@@ -980,10 +1038,17 @@ __global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L) {
         const T xm = e1[o - 1 + par], xp = e1[o + par], ym = e1[o - hp], yp = e1[o + hp], zm = e1[o - hs],
                 zp = e1[o + hs];
         const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-        const T dg = ckx.y + (cky.y + ckz.y);
-        const T ke = dg * e0 + (ckx.x * xm + ckx.z * xp) + (cky.x * ym + cky.z * yp) + (ckz.x * zm + ckz.z * zp);
-        rv[q] = b0 - ke;
         live[q] = inz && i >= 1 && i <= nx - 2 && is_unknown(t);
+        Off<T> f{ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z};
+        T dg = ckx.y + (cky.y + ckz.y);
+        if (FINE && live[q] && t == CFP_IRREGULAR) {
+            const T* kr = S.krow + 7 * (int64_t)S.slot[((int64_t)k * L.ny + j) * nx + i];
+            f = Off<T>{kr[1], kr[2], kr[3], kr[4], kr[5], kr[6]};
+            dg = kr[0];
+        }
+        const T v = rb_rest(b0, f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, xm, xp, ym, yp, zm, zp);
+        if constexpr (F64) rv[q] = __fma_rn(-dg, e0, v);
+        else rv[q] = __fmaf_rn(-dg, e0, v);
         oo[q] = o;
     }
 #pragma unroll
@@ -992,18 +1057,17 @@ __global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L) {
 }
 
 // the red residual at the fine level's irregular red nodes with their
-// Shortley-Weller rows (after k_resid_split)
-template <class T>
-__global__ void k_resid_fix(SLev<T> L, Side<T> S, const FixPt* __restrict__ red, int64_t n) {
+// Shortley-Weller rows, after the TMA-fed FP32 residual
+__global__ void k_resid_fix(SLev<float> L, Side<float> S, const FixPt* __restrict__ red, int64_t n) {
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         const FixPt p = red[q];
         const int par = p.par;
         const unsigned o = p.o;
-        const T* kr = S.krow + 7 * (int64_t)p.slot;
-        const T* __restrict__ e1 = L.e[1];
-        const T ke = kr[0] * L.e[0][o] + (kr[1] * e1[o - 1 + par] + kr[2] * e1[o + par]) +
-                     (kr[3] * e1[o - L.hp] + kr[4] * e1[o + L.hp]) + (kr[5] * e1[o - L.hs] + kr[6] * e1[o + L.hs]);
-        L.r0[o] = L.b[0][o] - ke;
+        const float* kr = S.krow + 7 * (int64_t)p.slot;
+        const float* __restrict__ e1 = L.e[1];
+        const float v = rb_rest(L.b[0][o], kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], e1[o - 1 + par], e1[o + par],
+                                e1[o - L.hp], e1[o + L.hp], e1[o - L.hs], e1[o + L.hs]);
+        L.r0[o] = __fmaf_rn(-kr[0], L.e[0][o], v);
     }
 }
 
@@ -1301,6 +1365,7 @@ SLev<T> slev(cfp_ctx* c, int l) {
         v.b[q] = sv + (2 + q) * L.Nh;
     }
     v.r0 = sv + 4 * L.Nh;
+    for (int q = 0; q < 2; ++q) v.rd[q] = sizeof(T) == 8 ? sv + (kSplitVecs + q) * L.Nh : nullptr;
     if (std::is_same<T, float>::value && L.red_cur) v.e[0] = sv + 5 * L.Nh;  // after an odd number of fused passes
     return v;
 }
@@ -1379,36 +1444,47 @@ void reset_red(cfp_ctx* c) {
     for (MgLevel& M : c->mg) M.red_cur = 0;
 }
 
+template <class T, int MODE>
+void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Half<T>& H, const Side<T>& S, int colour,
+                        const T* rho, T* phi, cudaStream_t s) {
+    const dim3 g = plane_grid(c->mg[l].n), blk = plane_block(c->mg[l].n);
+    if (l == 0 && c->n_irr > 0) k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
+    else k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
+}
+
+// the fine level's Shortley-Weller rows after a TMA-fed half-sweep (MODE 0 or 3)
+template <int MODE>
+void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, const Side<float>& S, int colour,
+                      float* phi, cudaStream_t s) {
+    const MgLevel& M0 = c->mg[0];
+    const int64_t n = M0.nfix[colour];
+    if (n <= 0) return;
+    k_sweep_fix<MODE><<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
+        L, S, H, static_cast<const FixPt*>(M0.fix) + colour * c->n_irr, n, phi);
+    c->launches += 1;
+}
+
 template <class T>
 void half_sweep(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colour, int mode, const T* rho, T* phi,
                 cudaStream_t s) {
-    const dim3 g = plane_grid(c->mg[l].n), blk = plane_block(c->mg[l].n);
-    const Half<T> H{L.ty[colour], L.e[colour], L.e[1 - colour], L.b[colour], L.b[1 - colour], L.ty[1 - colour]};
-    switch (mode) {
-        case 0:
-            if (!sweep_tma(c, l, L, 0, colour, phi, s))
-                k_sweep_split<T, 0><<<g, blk, 0, s>>>(L, H, colour, rho, phi);
-            break;
-        case 1: k_sweep_split<T, 1><<<g, blk, 0, s>>>(L, H, colour, rho, phi); break;
-        case 2: k_sweep_split<T, 2><<<g, blk, 0, s>>>(L, H, colour, rho, phi); break;
-        default:  // the last black half-sweep of the fine level
-            if (colour != 1 || !sweep_tma(c, l, L, 2, colour, phi, s))
-                k_sweep_split<T, 3><<<g, blk, 0, s>>>(L, H, colour, rho, phi);
-            break;
-    }
+    const Half<T> H{L.ty[colour], L.e[colour], L.e[1 - colour], L.b[colour], L.b[1 - colour], L.ty[1 - colour],
+                    L.rd[colour]};
     c->launches += 1;
-    const MgLevel& M0 = c->mg[0];
-    if (l == 0 && M0.nfix[colour] > 0) {  // the Shortley-Weller rows of the irregular nodes
-        const int64_t n = M0.nfix[colour];
-        const FixPt* list = static_cast<const FixPt*>(M0.fix) + colour * c->n_irr;
-        const unsigned nb = (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8);
-        switch (mode) {
-            case 0: k_sweep_fix<T, 0><<<nb, 256, 0, s>>>(L, S, H, list, n, phi); break;
-            case 1: k_sweep_fix<T, 1><<<nb, 256, 0, s>>>(L, S, H, list, n, phi); break;
-            case 2: k_sweep_fix<T, 2><<<nb, 256, 0, s>>>(L, S, H, list, n, phi); break;
-            default: k_sweep_fix<T, 3><<<nb, 256, 0, s>>>(L, S, H, list, n, phi); break;
+    // the TMA-fed pass: plain, or the last black half-sweep of the fine level
+    if (mode == 0 || (mode == 3 && colour == 1)) {
+        if (sweep_tma(c, l, L, mode == 0 ? 0 : 2, colour, phi, s)) {
+            if constexpr (sizeof(T) == 4) {
+                if (l == 0 && mode == 0) launch_sweep_fix<0>(c, L, H, S, colour, phi, s);
+                else if (l == 0) launch_sweep_fix<3>(c, L, H, S, colour, phi, s);
+            }
+            return;
         }
-        c->launches += 1;
+    }
+    switch (mode) {
+        case 0: launch_sweep_split<T, 0>(c, l, L, H, S, colour, rho, phi, s); break;
+        case 1: launch_sweep_split<T, 1>(c, l, L, H, S, colour, rho, phi, s); break;
+        case 2: launch_sweep_split<T, 2>(c, l, L, H, S, colour, rho, phi, s); break;
+        default: launch_sweep_split<T, 3>(c, l, L, H, S, colour, rho, phi, s); break;
     }
 }
 
@@ -1766,8 +1842,13 @@ cfp_status ensure_mg(cfp_ctx* c, int prec) {
     for (MgLevel& L : c->mg) {
         const size_t n = (size_t)kSplitVecs * L.Nh;
         if (prec == 0 && !L.s64) {
-            CFP_CUDA(pool_malloc(&L.s64, sizeof(double) * n, c->stream));
+            // + the reciprocal diagonals of both colours
+            CFP_CUDA(pool_malloc(&L.s64, sizeof(double) * (n + 2 * L.Nh), c->stream));
             CFP_CUDA(cudaMemsetAsync(L.s64, 0, sizeof(double) * n, c->stream));
+            const int l = (int)(&L - c->mg.data());
+            const Side<double> S = l == 0 ? side_view<double>(c) : Side<double>{nullptr, nullptr, nullptr, nullptr, nullptr};
+            k_fill_rd<<<flat_blocks(2 * L.Nh), 256, 0, c->stream>>>(slev<double>(c, l), S, L.s64 + n, L.Nh);
+            CFP_CUDA(cudaGetLastError());
         }
         if (prec == 1 && !L.s32) {  // + the second red array of the fused pass
             CFP_CUDA(pool_malloc(&L.s32, sizeof(float) * (n + L.Nh), c->stream));
@@ -1814,12 +1895,19 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
         const Side<T>& S = l == 0 ? S0 : Sc;
         smooth<T>(c, l, S, nu, l == 0 ? 2 : 1, 0, rho, phi, s);
         const SLev<T> F = slev<T>(c, l), C = slev<T>(c, l + 1);
-        if (!sweep_tma(c, l, F, 1, 0, phi, s)) k_resid_split<T><<<plane_grid(c->mg[l].n), plane_block(c->mg[l].n), 0, s>>>(F);
-        if (l == 0 && c->mg[0].nfix[0] > 0) {
-            const int64_t n = c->mg[0].nfix[0];
-            k_resid_fix<T><<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
-                F, S, static_cast<const FixPt*>(c->mg[0].fix), n);
-            c->launches += 1;
+        if (sweep_tma(c, l, F, 1, 0, phi, s)) {
+            if constexpr (sizeof(T) == 4) {
+                const int64_t n = c->mg[0].nfix[0];
+                if (l == 0 && n > 0) {
+                    k_resid_fix<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
+                        F, S, static_cast<const FixPt*>(c->mg[0].fix), n);
+                    c->launches += 1;
+                }
+            }
+        } else {
+            const dim3 g = plane_grid(c->mg[l].n), blk = plane_block(c->mg[l].n);
+            if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(F, S);
+            else k_resid_split<T, false><<<g, blk, 0, s>>>(F, S);
         }
         const MgLevel& Cn = c->mg[l + 1];
         const dim3 gr((unsigned)((Cn.n[0] - 2 + 127) / 128), (unsigned)(Cn.n[1] - 2), (unsigned)(Cn.n[2] - 2));
