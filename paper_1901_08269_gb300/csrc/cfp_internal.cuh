@@ -171,6 +171,7 @@ struct MgLevel {
     // the red e at tm32[4]; per pass kind (half-sweep, red residual, last
     // black half-sweep) the persistent grid (resident CTAs x SMs)
     int tma = 0;
+    int tma_planes = 32;       // planes per tile (even)
     int tma_grid[3] = {0, 0, 0};
     CUtensorMap tm32[5];
     // The fused black-then-red pass (FP32, TMA levels) writes the red iterate

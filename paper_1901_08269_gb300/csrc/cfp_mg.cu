@@ -371,29 +371,37 @@ __global__ void __launch_bounds__(CLUSTER ? kClusterThreads : kCoarseThreads)
 // ---------------------------------------------------------------- TMA path
 // Three FP32 passes of a large level with the access pattern of a half-sweep
 // (a node of one colour reads its six neighbours of the other colour and its
-// b, NaN where the node is not an unknown), run as a pipeline.  KIND 0: the plain half-sweep (MODE 0)
-// into e of its colour; KIND 1: the red residual r0 = b0 - K e (k_resid_split;
-// the stage also holds the red e of the tile); KIND 2: the fine level's last
-// black half-sweep into the natural-layout phi, both nodes of each pair
-// (MODE 3).  Per CTA
-// one producer thread streams planes of a tile through a ring of shared-memory
-// stages with cp.async.bulk.tensor (completion counted on an mbarrier per
-// stage), and kTmaRows consumer warps update the tile's nodes from shared
-// memory and release each plane through a second mbarrier.  A tile is
-// kTmaTX pairs x kTmaRows rows x kTmaPlanes planes of colour `colour`; a
-// stage holds, for one plane k, the other colour's pairs m0 - 4 .. m0 +
-// kTmaTX + 3 of rows j0 - 1 .. j0 + kTmaRows (the one-node halo in x and y;
-// the x start is a multiple of 4 entries, 16 bytes) and b of the tile's own
-// rows; the output of plane k reads the stages of planes k - 1, k, k + 1.
+// b, NaN where the node is not an unknown), run as a pipeline.  KIND 0: the
+// plain half-sweep (MODE 0) into e of its colour; KIND 1: the red residual r0
+// = b0 - K e (k_resid_split; the stage also holds the red e of the tile);
+// KIND 2: the fine level's last black half-sweep into the natural-layout phi,
+// both nodes of each pair (MODE 3).  Per CTA one producer thread streams
+// planes of a tile through a ring of shared-memory stages with
+// cp.async.bulk.tensor (completion counted on an mbarrier per stage), and
+// kTmaRows consumer warps update the tile's nodes and release each plane
+// through a second mbarrier.  A tile is kTmaTX pairs x kTmaRows rows x an
+// even number of planes (tma_planes) of colour COLOUR; a stage holds, for one
+// plane k, the other colour's pairs m0 - 4 .. m0 + kTmaTX + 3 of rows j0 - 1
+// .. j0 + kTmaRows (the one-node halo in x and y; the x start is a multiple of
+// 4 entries, 16 bytes) and b of the tile's own rows.
+// The traffic is near its floor (1.01 of 6 bytes per node), so what bounds
+// the pass next is instruction issue, and a consumer spends few: it marches z
+// with its column of the other colour (its pair, its four rows and one either
+// side) in registers, where entry m of planes k - 1, k + 1 and of rows j - 1,
+// j + 1 is the z and y neighbour and entry m of plane k one of the two x
+// neighbours; per plane it loads the six entries of plane k + 1, per node the
+// other x neighbour and b.  The parity of a row's node is the same in every
+// tile (j0 and k0 are odd), so planes alternate between two compiled bodies
+// with the neighbours and coefficients fixed.  About 25 instructions per node
+// where loading all seven values at computed parities took 75.
 // Copies outside the array (row j0 + kTmaRows past the last, pair -4 .. -1)
-// fill zeros and feed only nodes that are not updated.  The CTAs
-// are persistent: CTA q takes tiles q, q + grid, ... with the x tile varying
+// fill zeros and feed only nodes that are not updated.  The CTAs are
+// persistent: CTA q takes tiles q, q + grid, ... with the x tile varying
 // fastest, then y, then the z chunk, so the CTAs at work at one time share
 // their halo rows through L2.  Same arithmetic as k_sweep_split<float, 0>:
 // the results are bitwise equal.
 constexpr int kTmaTX = 128;     // pairs per tile row: one consumer thread each
 constexpr int kTmaRows = 8;     // rows per tile: consumer warps 0-3 take rows 0-3, warps 4-7 rows 4-7
-constexpr int kTmaPlanes = 32;  // output planes per tile
 constexpr int kTmaMinPairs = 96;  // levels with fewer pairs per row use k_sweep_split
 constexpr int kTmaOX = kTmaTX + 8;                                   // other-colour row in a stage
 constexpr int kTmaOBytes = kTmaOX * (kTmaRows + 2) * 4;              // other-colour tile
@@ -463,21 +471,72 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
 // shared memory; a consumer whose wait ran out stops waiting: every index
 // stays in bounds whatever the stages hold, so the launch still ends, and
 // the host reports the error.
-// out: e of `colour` (KIND 0), r0 (KIND 1, colour 0), phi (KIND 2, colour 1).
-template <int KIND>
-__global__ void __launch_bounds__(kTmaThreads)
+// out: e of COLOUR (KIND 0), r0 (KIND 1, COLOUR 0), phi (KIND 2, COLOUR 1).
+struct TmaTile {
+    int ntx, nty, ntz, planes;  // tiles per axis, planes per tile (even)
+};
+
+// what a consumer keeps across the planes of a tile
+struct TmaCol {
+    float m[4], c[6], n[6];          // the other colour at entry m: plane k - 1 (rows 0..3), k, k + 1 (rows -1..4)
+    float xl[2], xc[2], xh[2];       // x coefficients of the pair's nodes 2m, 2m + 1
+    float yl[4], yc[4], yh[4];       // y coefficients of the rows
+    float zl, zc, zh;                // z coefficients of plane k
+    int rows;                        // rows of the thread inside the grid (0: its pair is outside)
+    bool in0, in1;                   // KIND 2: nodes 2m, 2m + 1 are interior columns
+};
+
+// One output plane.  P: the parity of row 0's node (row ly's is P ^ (ly & 1)).
+// x0: the other colour at the thread's pair and row 0 in the plane's stage;
+// bs, es: b and (KIND 1) the own e there; o: the node's output offset (KIND
+// 2: of the natural-layout pair), step: from one row to the next.
+template <int KIND, int P>
+__device__ __forceinline__ void tma_plane(const TmaCol& T, const float* x0, const float* bs, const float* es,
+                                          float* __restrict__ out, unsigned o, unsigned step) {
+    float side[4], b[4], e[4];
+#pragma unroll
+    for (int ly = 0; ly < 4; ++ly) {
+        const int par = P ^ (ly & 1);
+        side[ly] = x0[ly * kTmaOX + (par ? 1 : -1)];
+        b[ly] = bs[ly * kTmaTX];
+        e[ly] = KIND == 1 ? es[ly * kTmaTX] : 0.f;
+    }
+#pragma unroll
+    for (int ly = 0; ly < 4; ++ly) {
+        const int par = P ^ (ly & 1);
+        const float own = T.c[ly + 1];
+        const float v = rb_rest(b[ly], T.xl[par], T.xh[par], T.yl[ly], T.yh[ly], T.zl, T.zh, par ? own : side[ly],
+                                par ? side[ly] : own, T.c[ly], T.c[ly + 2], T.m[ly], T.n[ly + 1]);
+        const float dg = T.xc[par] + (T.yc[ly] + T.zc);
+        const bool unk = b[ly] == b[ly];  // not NaN: an unknown
+        float* q = out + (o + (unsigned)ly * step);
+        if (KIND == 0) {
+            if (unk && ly < T.rows) *q = times_rcp(v, dg);
+        } else if (KIND == 1) {
+            if (unk && ly < T.rows) *q = __fmaf_rn(-dg, e[ly], v);
+        } else if (ly < T.rows) {
+            // this colour's node 2m + par gets its new value (0 off the
+            // unknowns), the pair's other node keeps the other colour's
+            if (par ? T.in1 : T.in0) q[par] = unk ? times_rcp(v, dg) : 0.f;
+            if (par ? T.in0 : T.in1) q[1 - par] = own;
+        }
+    }
+}
+
+template <int KIND, int COLOUR>
+__global__ void __launch_bounds__(kTmaThreads, 3)
     k_sweep_tma(const __grid_constant__ CUtensorMap t_oth, const __grid_constant__ CUtensorMap t_b,
-                const __grid_constant__ CUtensorMap t_own, SLev<float> L,
-                float* __restrict__ out, int colour, int ntx, int nty, int ntz, int* __restrict__ wait_err) {
-    constexpr int kTmaStages = tma_stages(KIND), kTmaStage = tma_stage(KIND);
+                const __grid_constant__ CUtensorMap t_own, SLev<float> L, float* __restrict__ out, TmaTile G,
+                int* __restrict__ wait_err) {
+    constexpr int S = tma_stages(KIND), kTmaStage = tma_stage(KIND);
     constexpr int kEOff = kTmaOPad + kTmaBBytes;  // KIND 1: own e of the tile
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    uint64_t* full = (uint64_t*)(base + kTmaStages * kTmaStage);  // stage filled (tx bytes landed)
-    uint64_t* empty = full + kTmaStages;                           // stage released by every consumer warp
+    uint64_t* full = (uint64_t*)(base + S * kTmaStage);  // stage filled (tx bytes landed)
+    uint64_t* empty = full + S;                          // stage released by every consumer warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int q = 0; q < kTmaStages; ++q) {
+        for (int q = 0; q < S; ++q) {
             mbar_init(&full[q], 1);
             mbar_init(&empty[q], kTmaRows);
         }
@@ -486,21 +545,21 @@ __global__ void __launch_bounds__(kTmaThreads)
     }
     __syncthreads();
     const int nx = L.nx, ny = L.ny, nz = L.nz;
-    const int ntiles = ntx * nty * ntz;
+    const int ntiles = G.ntx * G.nty * G.ntz;
     if (warp == kTmaRows) {  // producer
         if (lane != 0) return;
-        unsigned g = 0;  // planes issued by this CTA; plane g uses stage g % kTmaStages
+        unsigned g = 0;  // planes issued by this CTA; plane g uses stage g % S
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-            const int tx = tile % ntx, rest = tile / ntx, tyi = rest % nty, tz = rest / nty;
-            const int m0 = tx * kTmaTX, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * kTmaPlanes;
-            const int k1 = min(k0 + kTmaPlanes, nz - 1);
+            const int tx = tile % G.ntx, rest = tile / G.ntx, tyi = rest % G.nty, tz = rest / G.nty;
+            const int m0 = tx * kTmaTX, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * G.planes;
+            const int k1 = min(k0 + G.planes, nz - 1);
             for (int k = k0 - 1; k <= k1; ++k, ++g) {
-                const int st = g % kTmaStages;
+                const int st = g % S;
                 // a stage is refilled only once every consumer warp released
                 // it; if that wait runs out, nothing more is issued (the
                 // consumers may still read the stage)
-                if (g >= kTmaStages && !mbar_wait(&empty[st], ((g / kTmaStages) - 1) & 1)) {
+                if (g >= S && !mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
                     ok = false;
                     atomicExch(wait_err, 1);
                     break;
@@ -513,101 +572,99 @@ __global__ void __launch_bounds__(kTmaThreads)
             }
         }
         // Every copy issued has landed before the CTA may end, after a
-        // timeout too: planes g - kTmaStages .. g - 1 are the only ones whose
-        // stage was not released (an older plane's stage was waited free
-        // before it was refilled), and each of their full phases is the
-        // latest of its barrier.  Each wait is bounded again.
-        for (unsigned q = g > (unsigned)kTmaStages ? g - kTmaStages : 0; q < g; ++q)
-            if (!mbar_wait(&full[q % kTmaStages], (q / kTmaStages) & 1)) atomicExch(wait_err, 2);
+        // timeout too: planes g - S .. g - 1 are the only ones whose stage
+        // was not released (an older plane's stage was waited free before it
+        // was refilled), and each of their full phases is the latest of its
+        // barrier.  Each wait is bounded again.
+        for (unsigned q = g > (unsigned)S ? g - S : 0; q < g; ++q)
+            if (!mbar_wait(&full[q % S], (q / S) & 1)) atomicExch(wait_err, 2);
         return;
     }
     // consumers: thread (lx, group) owns pair m0 + lx of the rows r0 .. r0 + 3
     const int lx = threadIdx.x & (kTmaTX - 1), r0 = 4 * (threadIdx.x / kTmaTX);
-    const unsigned hs = L.hs;
-    const int hp = L.hp;
-    unsigned g = 0;
+    const int at = (r0 + 1) * kTmaOX + lx + 4;  // the thread's pair and row 0 in a stage
+    const unsigned step = KIND == 2 ? (unsigned)nx : (unsigned)L.hp;
+    const unsigned plane = KIND == 2 ? (unsigned)nx * (unsigned)ny : L.hs;
+    TmaCol T;
+    int st = 0;       // stage of the next plane to wait for
+    unsigned ph = 0;  // and its phase
     bool ok = true;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int tx = tile % ntx, rest = tile / ntx, tyi = rest % nty, tz = rest / nty;
-        const int m = tx * kTmaTX + lx, j0 = 1 + tyi * kTmaRows + r0, k0 = 1 + tz * kTmaPlanes;
-        const int nk = min(k0 + kTmaPlanes, nz - 1) - k0;
-        // the pair's two nodes: coefficients and whether each is an interior column
-        const float4 c0 = L.cx[min(2 * m, nx - 1)], c1 = L.cx[min(2 * m + 1, nx - 1)];
-        const bool in0 = 2 * m >= 1 && 2 * m <= nx - 2, in1 = 2 * m + 1 <= nx - 2;
-        float cya[4], cyb[4], cyc[4];
-        bool jin[4];
-#pragma unroll
-        for (int ly = 0; ly < 4; ++ly) {
-            const float4 cy = L.cy[min(j0 + ly, ny - 1)];
-            cya[ly] = cy.x;
-            cyb[ly] = cy.y;
-            cyc[ly] = cy.z;
-            jin[ly] = j0 + ly <= ny - 2;
+    auto wait_next = [&](int code) -> const float* {  // the next plane's stage
+        if (ok && !mbar_wait(&full[st], ph)) {
+            ok = false;
+            atomicExch(wait_err, code);
         }
-        for (int q = 0; q < 2; ++q)
-            if (ok && !mbar_wait(&full[(g + q) % kTmaStages], ((g + q) / kTmaStages) & 1)) {
-                ok = false;
-                atomicExch(wait_err, 3);
-            }
-        for (int kk = 0; kk < nk; ++kk) {
-            const unsigned gp = g + kk;  // stage of plane k - 1
-            if (ok && !mbar_wait(&full[(gp + 2) % kTmaStages], ((gp + 2) / kTmaStages) & 1)) {
-                ok = false;
-                atomicExch(wait_err, 4);
-            }
-            const int at = (r0 + 1) * kTmaOX + lx + 4;  // the thread's first row, centre entry
-            const unsigned char* s0 = base + ((gp + 1) % kTmaStages) * kTmaStage;
-            const float* Om = (const float*)(base + (gp % kTmaStages) * kTmaStage) + at;
-            const float* O0 = (const float*)s0 + at;
-            const float* Op = (const float*)(base + ((gp + 2) % kTmaStages) * kTmaStage) + at;
-            const float* Bs = (const float*)(s0 + kTmaOPad) + r0 * kTmaTX + lx;
-            const float* Es = (const float*)(s0 + kEOff) + r0 * kTmaTX + lx;  // KIND 1 only
-            const int k = k0 + kk;
-            const float4 cz = L.cz[k];
-            const int p0 = (colour + j0 + k) & 1;  // parity of row r0; rows alternate
-            const float4 ce = p0 ? c1 : c0, co = p0 ? c0 : c1;
-            const bool ine = p0 ? in1 : in0, ino = p0 ? in0 : in1;
-            float* ep = out + ((unsigned)k * hs + (unsigned)(j0 * hp + m));  // KIND 0, 1
-            // KIND 2: natural-layout row of (j0, k) and the pair's first node
-            float* pp = out + ((unsigned)k * (unsigned)ny + (unsigned)j0) * (unsigned)nx + 2u * (unsigned)m;
+        const float* p = (const float*)(base + st * kTmaStage);
+        if (++st == S) {
+            st = 0;
+            ph ^= 1u;
+        }
+        return p;
+    };
+    auto release = [&](int stage) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[stage]);
+    };
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int tx = tile % G.ntx, rest = tile / G.ntx, tyi = rest % G.nty, tz = rest / G.nty;
+        const int m = tx * kTmaTX + lx, j0 = 1 + tyi * kTmaRows + r0, k0 = 1 + tz * G.planes;
+        const int nk = min(k0 + G.planes, nz - 1) - k0;
+        {  // coefficients (indices clamped into the tables)
+            const float4 c0 = L.cx[min(2 * m, nx - 1)], c1 = L.cx[min(2 * m + 1, nx - 1)];
+            T.xl[0] = c0.x, T.xc[0] = c0.y, T.xh[0] = c0.z;
+            T.xl[1] = c1.x, T.xc[1] = c1.y, T.xh[1] = c1.z;
+            T.in0 = 2 * m >= 1 && 2 * m <= nx - 2, T.in1 = 2 * m + 1 <= nx - 2;
 #pragma unroll
             for (int ly = 0; ly < 4; ++ly) {
-                const int par = p0 ^ (ly & 1);
-                const float4 cx = (ly & 1) ? co : ce;
-                const int o = ly * kTmaOX;
-                const float xm = O0[o - 1 + par], xp = O0[o + par], ym = O0[o - kTmaOX], yp = O0[o + kTmaOX];
-                const float zm = Om[o], zp = Op[o];
-                const float b = Bs[ly * kTmaTX];
-                const bool unk = b == b;  // not NaN: an unknown
-                const float dg = cx.y + (cyb[ly] + cz.y);
-                const bool in = (ly & 1) ? ino : ine;  // the node of this colour is an interior column
-                if (KIND == 1) {
-                    const float e0 = Es[ly * kTmaTX];
-                    const float v = rb_rest(b, cx.x, cx.z, cya[ly], cyc[ly], cz.x, cz.z, xm, xp, ym, yp, zm, zp);
-                    if (in && jin[ly] && unk) ep[ly * hp] = __fmaf_rn(-dg, e0, v);
-                } else {
-                    const float v = rb_rest(b, cx.x, cx.z, cya[ly], cyc[ly], cz.x, cz.z, xm, xp, ym, yp, zm, zp);
-                    if (KIND == 0) {
-                        if (in && jin[ly] && unk) ep[ly * hp] = times_rcp(v, dg);
-                    } else if (jin[ly]) {
-                        // this colour's node i = 2m + par gets its new value (0 off
-                        // the unknowns), the pair's other node keeps the other colour's
-                        float* row = pp + (unsigned)ly * (unsigned)nx;
-                        const bool ino2 = (ly & 1) ? ine : ino;  // the other node is an interior column
-                        if (in) row[par] = unk ? times_rcp(v, dg) : 0.f;
-                        if (ino2) row[1 - par] = par ? xm : xp;
-                    }
-                }
+                const float4 cy = L.cy[min(j0 + ly, ny - 1)];
+                T.yl[ly] = cy.x, T.yc[ly] = cy.y, T.yh[ly] = cy.z;
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[gp % kTmaStages]);
+            // b is NaN at the box, so within the arrays it tells the
+            // unknowns; pairs and rows past them read zeros and are left out
+            T.rows = T.in0 || T.in1 ? max(0, min(4, ny - 1 - j0)) : 0;
         }
-        __syncwarp();
-        if (lane == 0) {  // the tile's last two planes
-            mbar_arrive(&empty[(g + nk) % kTmaStages]);
-            mbar_arrive(&empty[(g + nk + 1) % kTmaStages]);
+        unsigned o = KIND == 2 ? (unsigned)k0 * plane + (unsigned)j0 * step + 2u * (unsigned)m
+                               : (unsigned)k0 * plane + (unsigned)j0 * step + (unsigned)m;
+        const int sm = st;
+        const float* pm = wait_next(3);  // plane k0 - 1
+#pragma unroll
+        for (int ly = 0; ly < 4; ++ly) T.m[ly] = pm[at + ly * kTmaOX];
+        release(sm);
+        int s0 = st;                     // stage of plane k
+        const float* p0 = wait_next(3);  // plane k0
+#pragma unroll
+        for (int q = 0; q < 6; ++q) T.c[q] = p0[at + (q - 1) * kTmaOX];
+        float4 cz = L.cz[k0];
+        auto advance = [&](int kk, auto body) {
+            const float4 czn = L.cz[min(k0 + kk + 1, nz - 1)];  // the next plane's, ahead of use
+            T.zl = cz.x, T.zc = cz.y, T.zh = cz.z;
+            const int s1 = st;
+            const float* p1 = wait_next(4);  // plane k + 1
+#pragma unroll
+            for (int q = 0; q < 6; ++q) T.n[q] = p1[at + (q - 1) * kTmaOX];
+            const float* bs = p0 + kTmaOPad / 4 + r0 * kTmaTX + lx;
+            body(p0 + at, bs, bs + kTmaBBytes / 4);
+            release(s0);
+#pragma unroll
+            for (int ly = 0; ly < 4; ++ly) T.m[ly] = T.c[ly + 1];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) T.c[q] = T.n[q];
+            cz = czn;
+            p0 = p1;
+            s0 = s1;
+            o += plane;
+        };
+        // colour + j0 + k is COLOUR + even in the first plane of every tile
+        for (int kk = 0; kk < nk; kk += 2) {
+            advance(kk, [&](const float* x, const float* bs, const float* es) {
+                tma_plane<KIND, COLOUR>(T, x, bs, es, out, o, step);
+            });
+            if (kk + 1 < nk)
+                advance(kk + 1, [&](const float* x, const float* bs, const float* es) {
+                    tma_plane<KIND, 1 - COLOUR>(T, x, bs, es, out, o, step);
+                });
         }
-        g += nk + 2;
+        release(s0);  // the tile's last plane
     }
 }
 
@@ -734,7 +791,7 @@ __global__ void k_sweep_fix(SLev<float> L, Side<float> S, Half<float> H, const F
 // ------------------------------------------------ fused black + red pass
 // The black half-sweep of one red-black sweep and the red half-sweep of the
 // next (both plain, MODE 0) in one TMA-fed pass over an FP32 level.  Per tile
-// (kPairTX pairs x kTmaRows rows x up to kTmaPlanes planes) the CTA marches in
+// (kPairTX pairs x kTmaRows rows x up to kPairPlanes planes) the CTA marches in
 // z: at step k it forms the new black values of plane k on the tile and on a
 // ring one pair (x) or one row (y) wide around it, from the old red values
 // staged with a two-node halo, keeps them in a ring of kPairRing planes in
@@ -747,6 +804,7 @@ __global__ void k_sweep_fix(SLev<float> L, Side<float> S, Half<float> H, const F
 // lists.  Every node is formed by the arithmetic of k_sweep_tma<0> or
 // k_sweep_fix<float, 0>, so the pass is bitwise the two half-sweeps.
 constexpr int kPairTX = 64;                                       // pairs per tile row
+constexpr int kPairPlanes = 32;                                   // output planes per tile
 constexpr int kPairOX = kPairTX + 8;                              // staged row: entries m0 - 4 .. m0 + kPairTX + 3
 constexpr int kPairWarps = kPairTX * kTmaRows / (4 * 32);          // consumer warps: four rows per thread
 constexpr int kPairThreads = 32 * (kPairWarps + 1);               // + the producer warp
@@ -819,8 +877,8 @@ __global__ void __launch_bounds__(kPairThreads, 4)
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             const int tx = tile % ntx, rest = tile / ntx, tyi = rest % nty, tz = rest / nty;
-            const int m0 = tx * kPairTX, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * kTmaPlanes;
-            const int k1 = min(k0 + kTmaPlanes, nz - 1);
+            const int m0 = tx * kPairTX, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * kPairPlanes;
+            const int k1 = min(k0 + kPairPlanes, nz - 1);
             for (int k = k0 - 2; k <= k1 + 1; ++k, ++g) {
                 const int st = g % S;
                 if (g >= (unsigned)S && !mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
@@ -846,11 +904,11 @@ __global__ void __launch_bounds__(kPairThreads, 4)
     // ring's coefficients and the irregular lists' ranges of every plane are
     // first staged in shared memory: within the pass the CTA's warps meet at
     // a barrier every plane, so a global load in the loop would stall them all.
-    __shared__ float4 czs[kTmaPlanes + 2];  // planes k0 - 1 .. k1
+    __shared__ float4 czs[kPairPlanes + 2];  // planes k0 - 1 .. k1
     __shared__ float4 cyt[kTmaRows + 2];    // rows j0 - 1 .. j0 + kTmaRows
     __shared__ float4 cxt[4];               // ring pairs m0 - 1, m0 + kPairTX: nodes 2m, 2m + 1
-    __shared__ int2 xr[kTmaPlanes + 2];     // black irregular nodes of rows j0 - 1 .. j0 + kTmaRows, per plane
-    __shared__ int2 yr[kTmaPlanes + 2];     // red irregular nodes of rows j0 .. j0 + kTmaRows - 1, per plane
+    __shared__ int2 xr[kPairPlanes + 2];     // black irregular nodes of rows j0 - 1 .. j0 + kTmaRows, per plane
+    __shared__ int2 yr[kPairPlanes + 2];     // red irregular nodes of rows j0 .. j0 + kTmaRows - 1, per plane
     const int lx = threadIdx.x & (kPairTX - 1), grp = threadIdx.x / kPairTX, r0 = 4 * grp;
     const unsigned hs = L.hs;
     const int hp = L.hp;
@@ -859,8 +917,8 @@ __global__ void __launch_bounds__(kPairThreads, 4)
     bool ok = true;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int tx = tile % ntx, rest = tile / ntx, tyi = rest % nty, tz = rest / nty;
-        const int m0 = tx * kPairTX, m = m0 + lx, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * kTmaPlanes;
-        const int nk = min(k0 + kTmaPlanes, nz - 1) - k0;
+        const int m0 = tx * kPairTX, m = m0 + lx, j0 = 1 + tyi * kTmaRows, k0 = 1 + tz * kPairPlanes;
+        const int nk = min(k0 + kPairPlanes, nz - 1) - k0;
         pair_bar();  // the previous tile's tables are no longer read
         {
             const int t = threadIdx.x;
@@ -1391,6 +1449,33 @@ Transfer<float> transfer<float>(MgLevel& F) {
     return X;
 }
 
+TmaTile tma_tile(const int n[3], int planes) {
+    return TmaTile{(n[0] / 2 + kTmaTX - 1) / kTmaTX, (n[1] - 2 + kTmaRows - 1) / kTmaRows,
+                   (n[2] - 2 + planes - 1) / planes, planes};
+}
+
+// Planes per tile of a level's TMA passes: even (the kernel's parities), and
+// so that the SM with the most tiles (tiles spread evenly over nsm) streams
+// the fewest planes, its tiles' two halo planes and about one plane's time of
+// start-up included; at least two tiles per SM, so that one tile's loads
+// cover another's arithmetic.  513^3: 74 planes, 257^3: 30 (288 tiles on 152
+// SMs, where 32 planes made 256).
+int tma_planes(const int n[3], int nsm) {
+    int best = 32;
+    int64_t est_best = INT64_MAX;
+    for (int p = 8; p <= 128; p += 2) {
+        const TmaTile G = tma_tile(n, p);
+        const int64_t tiles = (int64_t)G.ntx * G.nty * G.ntz;
+        if (tiles < 2 * nsm && p > 8) continue;
+        const int64_t est = (tiles + nsm - 1) / nsm * (p + 3);
+        if (est < est_best) {
+            est_best = est;
+            best = p;
+        }
+    }
+    return best;
+}
+
 // The TMA-fed pass where it applies (FP32, a level with maps): kind 0 the
 // plain half-sweep of `colour`, kind 1 the red residual, kind 2 the last
 // black half-sweep into phi (natural layout).  False: use the plain kernel.
@@ -1398,21 +1483,20 @@ bool sweep_tma(cfp_ctx*, int, const SLev<double>&, int, int, double*, cudaStream
 bool sweep_tma(cfp_ctx* c, int l, const SLev<float>& L, int kind, int colour, float* phi, cudaStream_t s) {
     const MgLevel& M = c->mg[l];
     if (!M.tma || !c->mg_tma) return false;
-    const int ntx = (M.n[0] / 2 + kTmaTX - 1) / kTmaTX, nty = (M.n[1] - 2 + kTmaRows - 1) / kTmaRows;
-    const int ntz = (M.n[2] - 2 + kTmaPlanes - 1) / kTmaPlanes;
+    const TmaTile G = tma_tile(M.n, M.tma_planes);
     // other colour's e (the red one from the array that holds it), b of `colour`
     const CUtensorMap& t_oth = colour == 1 && M.red_cur ? M.tmalt[0] : M.tm32[2 * colour];
     const CUtensorMap& t_b = M.tm32[2 * colour + 1];
     const unsigned grid = (unsigned)M.tma_grid[kind];
-    if (kind == 0)
-        k_sweep_tma<0><<<grid, kTmaThreads, tma_smem(0), s>>>(t_oth, t_b, t_oth, L, L.e[colour], colour, ntx, nty,
-                                                               ntz, c->dwait);
+    if (kind == 0 && colour == 0)
+        k_sweep_tma<0, 0><<<grid, kTmaThreads, tma_smem(0), s>>>(t_oth, t_b, t_oth, L, L.e[0], G, c->dwait);
+    else if (kind == 0)
+        k_sweep_tma<0, 1><<<grid, kTmaThreads, tma_smem(0), s>>>(t_oth, t_b, t_oth, L, L.e[1], G, c->dwait);
     else if (kind == 1)
-        k_sweep_tma<1><<<grid, kTmaThreads, tma_smem(1), s>>>(t_oth, t_b, M.red_cur ? M.tmalt[1] : M.tm32[4], L,
-                                                               L.r0, 0, ntx, nty, ntz, c->dwait);
+        k_sweep_tma<1, 0><<<grid, kTmaThreads, tma_smem(1), s>>>(t_oth, t_b, M.red_cur ? M.tmalt[1] : M.tm32[4], L,
+                                                                 L.r0, G, c->dwait);
     else
-        k_sweep_tma<2><<<grid, kTmaThreads, tma_smem(2), s>>>(t_oth, t_b, t_oth, L, phi, 1, ntx, nty, ntz,
-                                                               c->dwait);
+        k_sweep_tma<2, 1><<<grid, kTmaThreads, tma_smem(2), s>>>(t_oth, t_b, t_oth, L, phi, G, c->dwait);
     return true;
 }
 
@@ -1426,7 +1510,7 @@ bool sweep_pair(cfp_ctx* c, int l, const Side<float>& S, cudaStream_t s, bool al
     if (!M.tma || !M.pair || !(always || (c->mg_tma && c->mg_fuse))) return false;
     const SLev<float> L = slev<float>(c, l);
     const int ntx = (M.n[0] / 2 + kPairTX - 1) / kPairTX, nty = (M.n[1] - 2 + kTmaRows - 1) / kTmaRows;
-    const int ntz = (M.n[2] - 2 + kTmaPlanes - 1) / kTmaPlanes;
+    const int ntz = (M.n[2] - 2 + kPairPlanes - 1) / kPairPlanes;
     PairFix F{nullptr, nullptr, nullptr, 0, 0};
     if (l == 0 && M.fix && M.fixrows && S.krow)
         F = PairFix{static_cast<const FixPt*>(M.fix), M.fixrows, S.krow, c->n_irr, (int64_t)M.n[1] * M.n[2]};
@@ -1781,20 +1865,23 @@ cfp_status pair_occupancy(int* per) {
     return CFP_OK;
 }
 
-template <int KIND>
+template <int KIND, int COLOUR>
 cfp_status tma_occupancy(int* per) {
     static_assert(tma_smem(KIND) <= 227 * 1024, "shared memory per CTA");
-    CFP_CUDA(cudaFuncSetAttribute(k_sweep_tma<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, tma_smem(KIND)));
-    CFP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, k_sweep_tma<KIND>, kTmaThreads, tma_smem(KIND)));
+    CFP_CUDA(cudaFuncSetAttribute(k_sweep_tma<KIND, COLOUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, tma_smem(KIND)));
+    int p = 0;
+    CFP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_sweep_tma<KIND, COLOUR>, kTmaThreads, tma_smem(KIND)));
+    *per = *per ? std::min(*per, p) : p;
     return CFP_OK;
 }
 
 cfp_status setup_tma(cfp_ctx* c) {
     int per[3] = {0, 0, 0}, per_pair = 0, nsm = 0;
     CFP_TRY(pair_occupancy(&per_pair));
-    CFP_TRY(tma_occupancy<0>(&per[0]));
-    CFP_TRY(tma_occupancy<1>(&per[1]));
-    CFP_TRY(tma_occupancy<2>(&per[2]));
+    CFP_TRY((tma_occupancy<0, 0>(&per[0])));
+    CFP_TRY((tma_occupancy<0, 1>(&per[0])));
+    CFP_TRY((tma_occupancy<1, 0>(&per[1])));
+    CFP_TRY((tma_occupancy<2, 1>(&per[2])));
     CFP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
     for (MgLevel& L : c->mg) {
         L.tma = 0;
@@ -1813,11 +1900,12 @@ cfp_status setup_tma(cfp_ctx* c) {
         CFP_TRY(tile_map(&L.tmp[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, red2, L, kPairOX, kPairYRows));
         CFP_TRY(tile_map(&L.tmp[2], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L.s32 + 3 * L.Nh, L, kPairOX, kPairXRows));
         CFP_TRY(tile_map(&L.tmp[3], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, L.s32 + 2 * L.Nh, L, kPairTX, kTmaRows));
-        const int64_t tiles = (int64_t)((L.n[0] / 2 + kTmaTX - 1) / kTmaTX) * ((L.n[1] - 2 + kTmaRows - 1) / kTmaRows) *
-                              ((L.n[2] - 2 + kTmaPlanes - 1) / kTmaPlanes);
+        L.tma_planes = tma_planes(L.n, nsm);
+        const TmaTile G = tma_tile(L.n, L.tma_planes);
+        const int64_t tiles = (int64_t)G.ntx * G.nty * G.ntz;
         for (int q = 0; q < 3; ++q) L.tma_grid[q] = (int)std::min<int64_t>(tiles, (int64_t)per[q] * nsm);
         const int64_t ptiles = (int64_t)((L.n[0] / 2 + kPairTX - 1) / kPairTX) *
-                               ((L.n[1] - 2 + kTmaRows - 1) / kTmaRows) * ((L.n[2] - 2 + kTmaPlanes - 1) / kTmaPlanes);
+                               ((L.n[1] - 2 + kTmaRows - 1) / kTmaRows) * ((L.n[2] - 2 + kPairPlanes - 1) / kPairPlanes);
         L.pair_grid = (int)std::min<int64_t>(ptiles, (int64_t)per_pair * nsm);
         L.pair = per_pair >= 1;
         L.tma = 1;
