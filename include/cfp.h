@@ -103,8 +103,9 @@ typedef struct {
                           multigrid levels (and of the fine level's sweeps)
                           with at least 192 nodes per row stream their tiles
                           through shared memory with TMA bulk-tensor copies,
-                          a coarse level of at most 2^15 nodes does all
-                          sweeps of a smoothing in one single-CTA launch,
+                          the coarse levels from the first of at most 2^16
+                          nodes down run as one launch of a thread-block
+                          cluster that holds them in shared memory,
                           and the prolongation runs one thread per coarse
                           cell; 0: plain loads, one launch per half-sweep,
                           one prolongation thread per fine pair; 2: as 1,

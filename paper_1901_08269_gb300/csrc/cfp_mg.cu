@@ -301,73 +301,6 @@ __global__ void k_fill_rd(SLev<double> L, Side<double> S, double* __restrict__ r
     }
 }
 
-// All the red-black sweeps of one smoothing of a small level (at most
-// kCoarseMaxNodes nodes: the coarsest level's 16 sweeps, a 17^3 level's
-// pre- or post-smoothing) in one CTA, with a CTA barrier between
-// half-sweeps, where separate launches would cost a few microseconds each
-// for a few thousand nodes.  The node update is k_sweep_split's (MODE 1 for
-// a first red half-sweep from zero, MODE 0 otherwise): the results are
-// bitwise equal.
-// CLUSTER: the same with the CTAs of one thread-block cluster (up to 16,
-// one per SM) and a cluster barrier, whose release / acquire order the
-// global writes of one half-sweep before the reads of the next, for levels
-// of up to kClusterMaxNodes nodes (33^3; at 65^3, eight nodes per thread
-// and half-sweep, separate launches on the whole GPU measured faster).
-constexpr int kCoarseThreads = 512;
-constexpr int64_t kCoarseMaxNodes = int64_t(1) << 15;
-constexpr int kClusterThreads = 1024;
-constexpr int64_t kClusterMaxNodes = int64_t(1) << 16;
-
-template <class T, bool CLUSTER>
-__global__ void __launch_bounds__(CLUSTER ? kClusterThreads : kCoarseThreads)
-    k_smooth_cta(SLev<T> L, int sweeps, int first_red_zero) {
-    const int nx = L.nx, ny = L.ny, nz = L.nz, hp = L.hp;
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
-    const unsigned hs = L.hs;
-    const int mp = (nx - 2) / 2 + 1;  // pairs m with 2 m <= nx - 2
-    const int64_t items = (int64_t)mp * (ny - 2) * (nz - 2);
-    for (int q = 0; q < 2 * sweeps; ++q) {
-        const int colour = q & 1;
-        const bool zero = q == 0 && first_red_zero;
-        // plain pointers: the e arrays are written by this launch's earlier
-        // half-sweeps, so their loads must not take the non-coherent
-        // read-only path that a const __restrict__ pointer allows
-        T* eown = colour ? L.e[1] : L.e[0];
-        const T* eoth = colour ? L.e[0] : L.e[1];
-        const T* bown = colour ? L.b[1] : L.b[0];
-        const T* rdc = colour ? L.rd[1] : L.rd[0];
-        const uint8_t* ty = colour ? L.ty[1] : L.ty[0];
-        for (int64_t it = t0; it < items; it += nt) {
-            const int m = (int)(it % mp);
-            const int64_t rest = it / mp;
-            const int j = 1 + (int)(rest % (ny - 2)), k = 1 + (int)(rest / (ny - 2));
-            const int par = (colour + j + k) & 1;
-            const int i = 2 * m + par;
-            const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
-            const T rd = sizeof(T) == 8 ? rdc[o] : T(0);
-            T v = bown[o];
-            const bool unk = sizeof(T) == 8 ? rd != T(0) : is_unknown(ty[o]);
-            T xm = T(0), xp = T(0), ym = T(0), yp = T(0), zm = T(0), zp = T(0);
-            if (!zero) {
-                xm = eoth[o - 1 + par];
-                xp = eoth[o + par];
-                ym = eoth[o - hp];
-                yp = eoth[o + hp];
-                zm = eoth[o - hs];
-                zp = eoth[o + hs];
-            }
-            const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-            if (!zero) v = rb_rest(v, ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z, xm, xp, ym, yp, zm, zp);
-            T val;
-            if constexpr (sizeof(T) == 8) val = times_rd(v, rd);
-            else val = times_rcp(v, ckx.y + (cky.y + ckz.y));
-            if (i >= 1 && i <= nx - 2 && unk) eown[o] = val;
-        }
-        if (CLUSTER) cooperative_groups::this_cluster().sync();
-        else __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------- TMA path
 // Three FP32 passes of a large level with the access pattern of a half-sweep
 // (a node of one colour reads its six neighbours of the other colour and its
@@ -1129,6 +1062,44 @@ __global__ void k_resid_fix(SLev<float> L, Side<float> S, const FixPt* __restric
     }
 }
 
+__device__ __forceinline__ float mg_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mg_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// (P^T r) / (P^T 1) of a coarse node from its 27 fine neighbours' red
+// residuals, r(a, b, c) that of fine node (2I - 1 + a, 2J - 1 + b, 2K - 1 + c).
+// That node is red, (i + j + k) even, exactly where a + b + c is odd: a
+// pattern fixed at compile time, so only those 13 of the 27 terms are formed.
+// P^T 1, the sum of all 27 weights, is separable per axis.  Written out in
+// fused multiply-adds so that every kernel rounds it the same way.
+template <class T, class F>
+__device__ __forceinline__ T restrict_sum(const RwPk<T>& rx, const RwPk<T>& ry, const RwPk<T>& rz, F r) {
+    const T* wx = rx.w;
+    const T* wy = ry.w;
+    const T* wz = rz.w;
+    T s = T(0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const T wyz = wy[b] * wz[c];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if ((a + b + c) & 1) s = mg_fma(wx[a] * wyz, r(a, b, c), s);
+        }
+    return s / (((wx[0] + wx[1]) + wx[2]) * ((wy[0] + wy[1]) + wy[2]) * ((wz[0] + wz[1]) + wz[2]));
+}
+
+// f plus the trilinear interpolation of the cell's corners e[c][b][a], in
+// fused multiply-adds for the same reason
+template <class T>
+__device__ __forceinline__ T prolong_value(T f, const IpPk<T>& px, const IpPk<T>& py, const IpPk<T>& pz, T e000,
+                                           T e001, T e010, T e011, T e100, T e101, T e110, T e111) {
+    const T x00 = mg_fma(px.whi, e001, px.wlo * e000), x01 = mg_fma(px.whi, e011, px.wlo * e010);
+    const T x10 = mg_fma(px.whi, e101, px.wlo * e100), x11 = mg_fma(px.whi, e111, px.wlo * e110);
+    const T y0 = mg_fma(py.whi, x01, py.wlo * x00), y1 = mg_fma(py.whi, x11, py.wlo * x10);
+    return mg_fma(pz.whi, y1, mg_fma(pz.wlo, y0, f));
+}
+
 // b_c = (P^T r_f) / (P^T 1) at the coarse unknowns; r_f is the fine red
 // residual (zero on black nodes).  One thread per coarse node (I, J, K);
 // interior coarse nodes sit on fine node (2I, 2J, 2K).
@@ -1146,32 +1117,11 @@ __global__ void k_restrict_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
     const int nfy = F.ny;
     const int fi = 2 * I, fj = 2 * J, fk = 2 * K;
     const RwPk<T> rx = X.rw[0][I], ry = X.rw[1][J], rz = X.rw[2][K];
-    const T* wx = rx.w;
-    const T* wy = ry.w;
-    const T* wz = rz.w;
     const T* __restrict__ r0 = F.r0;
-    T s = 0;
-    // fine node (2I - 1 + a, 2J - 1 + b, 2K - 1 + c) is red, (i + j + k) even,
-    // exactly where a + b + c is odd: a pattern fixed at compile time, so
-    // only those 13 of the 27 terms are formed
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const int k = fk - 1 + c;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int j = fj - 1 + b;
-            const T wyz = wy[b] * wz[c];
-            const unsigned rowo = (unsigned)(k * nfy + j) * (unsigned)F.hp;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const int i = fi - 1 + a;
-                if ((a + b + c) & 1) s += (wx[a] * wyz) * r0[rowo + (unsigned)(i >> 1)];
-            }
-        }
-    }
-    // P^T 1 at the node: the sum of all 27 weights, separable per axis
-    const T w = ((wx[0] + wx[1]) + wx[2]) * ((wy[0] + wy[1]) + wy[2]) * ((wz[0] + wz[1]) + wz[2]);
-    if (is_unknown(tc)) (cc ? C.b[1] : C.b[0])[oc] = s / w;
+    const T v = restrict_sum(rx, ry, rz, [&](int a, int b, int c) {
+        return r0[(unsigned)((fk - 1 + c) * nfy + fj - 1 + b) * (unsigned)F.hp + (unsigned)((fi - 1 + a) >> 1)];
+    });
+    if (is_unknown(tc)) (cc ? C.b[1] : C.b[0])[oc] = v;
 }
 
 // e1 += P e_c at the fine black unknowns (the red values are overwritten by
@@ -1185,7 +1135,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, 
     const unsigned hc = (unsigned)C.hp;
     const IpPk<T> py = X.ip[1][j];
     const int J = py.ilo;
-    const T ay0 = py.wlo, ay1 = py.whi;
     T* __restrict__ e1 = F.e[1];
     T val[kSweepPlanes];
     bool live[kSweepPlanes];
@@ -1200,8 +1149,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, 
         const uint8_t t = F.ty[1][o];
         const IpPk<T> px = X.ip[0][ic], pz = X.ip[2][k];
         const int I = px.ilo, K = pz.ilo;
-        const T ax0 = px.wlo, ax1 = px.whi;
-        const T az0 = pz.wlo, az1 = pz.whi;
         // coarse (I + a, J + b, K + c): colour (I + a + J + b + K + c) & 1,
         // entry ((K + c) * ncy + J + b) * hc + (I + a) >> 1
         const int p = (I + J + K) & 1;
@@ -1212,8 +1159,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, 
         const T e000 = ea[r00 + x0], e001 = eb[r00 + x1], e010 = eb[r01 + x0], e011 = ea[r01 + x1];
         const T e100 = eb[r10 + x0], e101 = ea[r10 + x1], e110 = ea[r11 + x0], e111 = eb[r11 + x1];
         const T f0 = e1[o];
-        val[q] = f0 + (az0 * (ay0 * (ax0 * e000 + ax1 * e001) + ay1 * (ax0 * e010 + ax1 * e011)) +
-                       az1 * (ay0 * (ax0 * e100 + ax1 * e101) + ay1 * (ax0 * e110 + ax1 * e111)));
+        val[q] = prolong_value(f0, px, py, pz, e000, e001, e010, e011, e100, e101, e110, e111);
         live[q] = inz && i >= 1 && i <= nx - 2 && is_unknown(t);
         oo[q] = o;
     }
@@ -1222,7 +1168,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, 
         if (live[q]) e1[oo[q]] = val[q];
 }
 
-// packed (ka, kb, kc) per index of each axis from a level's metric arrays
 // The same e1 += P e_c with one thread per coarse cell (I, J, K): the fine
 // nodes 2I .. 2I + 1 x 2J .. 2J + 1 x 2K .. 2K + 1 interpolate between the
 // cell's eight corners (every interior fine node's lower table index is its
@@ -1270,20 +1215,18 @@ __global__ void __launch_bounds__(128) k_prolong_cell(Transfer<T> X, SLev<T> F, 
     }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-        const T az0 = pzv[c].wlo, az1 = pzv[c].whi;
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             if (!live[c][b] || !is_unknown(t[c][b])) continue;
-            const T ay0 = pyv[b].wlo, ay1 = pyv[b].whi;
             const IpPk<T>& px = ((1 + 2 * J + b + 2 * K + c) & 1) ? px1 : px0;
-            const T ax0 = px.wlo, ax1 = px.whi;
-            const T f0 = f[c][b];
-            e1[o[c][b]] = f0 + (az0 * (ay0 * (ax0 * e000 + ax1 * e001) + ay1 * (ax0 * e010 + ax1 * e011)) +
-                                az1 * (ay0 * (ax0 * e100 + ax1 * e101) + ay1 * (ax0 * e110 + ax1 * e111)));
+            e1[o[c][b]] = prolong_value(f[c][b], px, pyv[b], pzv[c], e000, e001, e010, e011, e100, e101, e110, e111);
         }
     }
 }
 
+#include "cfp_mg_coarse.cuh"
+
+// packed (ka, kb, kc) per index of each axis from a level's metric arrays
 template <class T>
 __global__ void k_pack_coefs(Grid<T> G, PkT<T>* __restrict__ out) {
     const int n[3] = {G.nx, G.ny, G.nz};
@@ -1572,30 +1515,122 @@ void half_sweep(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colou
     }
 }
 
-// The cluster of k_smooth_cta<T, true>: 16 CTAs where the device schedules
-// such a cluster (a non-portable size), else 8, else 0 (not used); found once.
+// The cluster of k_coarse with shared levels: 16 CTAs where the device
+// schedules such a cluster (a non-portable size) with kCoarseSmem bytes each,
+// else 8, else 0 (not used); found once.
 template <class T>
-int smooth_cluster_size() {
+int coarse_cluster_size() {
     static const int size = []() {
-        cudaFuncSetAttribute(k_smooth_cta<T, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        for (int cl : {16, 8}) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)cl);
-            cfg.blockDim = dim3(kClusterThreads);
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = (unsigned)cl;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k_smooth_cta<T, true>, &cfg) == cudaSuccess && n >= 1) return cl;
-            cudaGetLastError();
-        }
-        return 0;
+        int found = 0;
+        if (cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem) == cudaSuccess)
+            for (int cl : {16, 8}) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)cl);
+                cfg.blockDim = dim3(kCoarseThreads);
+                cfg.dynamicSmemBytes = kCoarseSmem;
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeClusterDimension;
+                at[0].val.clusterDim.x = (unsigned)cl;
+                at[0].val.clusterDim.y = 1;
+                at[0].val.clusterDim.z = 1;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                int n = 0;
+                if (cudaOccupancyMaxActiveClusters(&n, k_coarse<T>, &cfg) == cudaSuccess && n >= 1) {
+                    found = cl;
+                    break;
+                }
+            }
+        cudaGetLastError();
+        return found;
     }();
     return size;
+}
+
+// k_coarse's arguments with level `first` as its first level; false where
+// they do not fit (too many nodes, levels or bytes).  *smem: bytes per CTA,
+// *cl: CTAs.
+template <class T>
+bool coarse_args(cfp_ctx* c, int first, CoarseArgs<T>* A, size_t* smem, int* cl) {
+    const int nl = (int)c->mg.size() - first;
+    const int size = coarse_cluster_size<T>();
+    if (size == 0 || nl < 1 || nl > kCoarseLevels || c->mg[first].N > kCoarseMaxNodes) return false;
+    A->nl = nl;
+    A->ndist = 0;
+    A->pre = std::max(1, c->mg_smooth);
+    A->post = std::max(1, c->mg_post);
+    size_t bytes = 0;
+    for (int q = 0; q < nl; ++q) {  // coefficients first: they want the wider alignment
+        CoarseLevel<T>& V = A->V[q];
+        const MgLevel& M = c->mg[first + q];
+        V.L = slev<T>(c, first + q);
+        if (q + 1 < nl) V.X = transfer<T>(c->mg[first + q]);
+        V.cof = (unsigned)(bytes / sizeof(PkT<T>));
+        bytes += sizeof(PkT<T>) * (size_t)(M.n[0] + M.n[1] + M.n[2]);
+        V.dist = M.N > kCoarseSolo<T>;
+        A->ndist += V.dist;
+    }
+    for (int q = 0; q < nl; ++q) {
+        CoarseLevel<T>& V = A->V[q];
+        const MgLevel& M = c->mg[first + q];
+        V.hps = (M.n[0] + 1) / 2;
+        V.mp = (M.n[0] - 2) / 2 + 1;
+        V.rows = M.n[1] * M.n[2];
+        V.halo = V.dist ? M.n[1] + 1 : 0;  // the restriction reads row R - n_y - 1
+        V.rpc = V.dist ? std::max((V.rows + size - 1) / size, V.halo) : V.rows;
+        V.inv_hps = 1.0f / (float)V.hps;
+        V.inv_mp = 1.0f / (float)V.mp;
+        V.inv_ny = 1.0f / (float)M.n[1];
+        V.inv_rpc = 1.0f / (float)V.rpc;
+        V.vec = (unsigned)(bytes / sizeof(T));
+        bytes += sizeof(T) * (2 * (size_t)(V.rpc + 2 * V.halo) + 4 * (size_t)V.rpc) * V.hps;
+    }
+    for (int q = 0; q < nl; ++q) {
+        CoarseLevel<T>& V = A->V[q];
+        bytes = (bytes + 7) / 8 * 8;
+        V.itm = (unsigned)(bytes / 8);
+        bytes += sizeof(CoarseItem) * (size_t)V.rpc * V.mp;
+        if ((int64_t)V.rpc * V.hps > 65535) return false;  // CoarseItem::o
+    }
+    *smem = bytes;
+    *cl = A->ndist ? size : 1;
+    return bytes <= (size_t)kCoarseSmem;
+}
+
+// the first level k_coarse takes (the finest below the fine grid that fits),
+// or the number of levels if none
+template <class T>
+int coarse_first(cfp_ctx* c) {
+    const int nl = (int)c->mg.size();
+    CoarseArgs<T> A;
+    size_t smem = 0;
+    int cl = 0;
+    for (int l = 1; c->mg_tma && l < nl; ++l)
+        if (coarse_args<T>(c, l, &A, &smem, &cl)) return l;
+    return nl;
+}
+
+template <class T>
+void launch_coarse(cfp_ctx* c, int first, cudaStream_t s) {
+    CoarseArgs<T> A;
+    size_t smem = 0;
+    int cl = 0;
+    if (!coarse_args<T>(c, first, &A, &smem, &cl)) return;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cl);
+    cfg.blockDim = dim3(kCoarseThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_coarse<T>, A);
+    c->launches += 1;
 }
 
 // `sweeps` red-black sweeps at level l.  first_red / last_black: the modes of
@@ -1604,33 +1639,6 @@ template <class T>
 void smooth(cfp_ctx* c, int l, const Side<T>& S, int sweeps, int first_red, int last_black, const T* rho, T* phi,
             cudaStream_t s) {
     const SLev<T> L = slev<T>(c, l);
-    // a small coarse level (no irregular rows, plain or from-zero modes):
-    // one CTA does every half-sweep
-    if (c->mg_tma && l > 0 && c->mg[l].N <= kCoarseMaxNodes && (first_red == 0 || first_red == 1) &&
-        last_black == 0) {
-        k_smooth_cta<T, false><<<1, kCoarseThreads, 0, s>>>(L, sweeps, first_red);
-        c->launches += 1;
-        return;
-    }
-    // a mid-size coarse level: one thread-block cluster does every half-sweep
-    const int cl = smooth_cluster_size<T>();
-    if (cl > 0 && c->mg_tma && l > 0 && c->mg[l].N <= kClusterMaxNodes && (first_red == 0 || first_red == 1) &&
-        last_black == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)cl);
-        cfg.blockDim = dim3(kClusterThreads);
-        cfg.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)cl;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, k_smooth_cta<T, true>, L, sweeps, first_red);
-        c->launches += 1;
-        return;
-    }
     // red of sweep 0, then per sweep q its black half-sweep and the red one of
     // sweep q + 1: one fused pass where the level has one, else two launches
     half_sweep<T>(c, l, L, S, 0, first_red, rho, phi, s);
@@ -1978,8 +1986,10 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
         smooth<T>(c, 0, S0, 16, 2, 3, rho, phi, s);
         return;
     }
+    // the levels k_coarse takes (none: lc = nl)
+    const int lc = coarse_first<T>(c);
     // downward leg: smooth from zero, red residual, restrict to b of l + 1
-    for (int l = 0; l < nl - 1; ++l) {
+    for (int l = 0; l < std::min(lc, nl - 1); ++l) {
         const Side<T>& S = l == 0 ? S0 : Sc;
         smooth<T>(c, l, S, nu, l == 0 ? 2 : 1, 0, rho, phi, s);
         const SLev<T> F = slev<T>(c, l), C = slev<T>(c, l + 1);
@@ -2002,10 +2012,11 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
         k_restrict_split<T><<<gr, 128, 0, s>>>(transfer<T>(c->mg[l]), F, C);
         c->launches += 2;
     }
-    smooth<T>(c, nl - 1, Sc, 16, 1, 0, rho, phi, s);  // coarsest level
+    if (lc < nl) launch_coarse<T>(c, lc, s);
+    else smooth<T>(c, nl - 1, Sc, 16, 1, 0, rho, phi, s);  // coarsest level
     // upward leg: black coarse correction, smooth; the last half-sweep of the
     // fine level writes phi
-    for (int l = nl - 2; l >= 0; --l) {
+    for (int l = std::min(lc, nl - 1) - 1; l >= 0; --l) {
         const SLev<T> F = slev<T>(c, l), C = slev<T>(c, l + 1);
         launch_prolong<T>(c, l, F, C, s);
         c->launches += 1;
