@@ -292,10 +292,15 @@ cfp_status cfp::assemble_rhs(cfp_ctx* c, const double* f, const double* g, const
     double* bg = c->v64 + V_TMP2 * vstride(c);
     double* qf = c->v64 + V_T * vstride(c);
     if (rhs == gb || rhs == bg || rhs == qf) return fail(CFP_EINVAL, "rhs aliases the context's work space");
-    launch_boundary_lift(c, g, gb, c->stream);
-    launch_apply_lift(c, gb, bg, c->stream);
-    launch_qf(c, f, qf, c->stream);
-    launch_rhs_finish(c, qf, bg, c->n_ibi ? gi : c->ibi_xyz, rhs, c->stream);
+    // rhs may share memory with an input: then through a work field
+    auto overlaps = [&](const double* p, int64_t n) {
+        const uintptr_t a = (uintptr_t)p, b = (uintptr_t)rhs;
+        return a < b + sizeof(double) * (uintptr_t)c->N && b < a + sizeof(double) * (uintptr_t)n;
+    };
+    const bool shared = overlaps(f, c->N) || overlaps(g, c->N) || (c->n_ibi && overlaps(gi, c->n_ibi));
+    launch_rhs(c, f, g, c->n_ibi ? gi : c->ibi_xyz, gb, shared ? qf : rhs, c->stream);
+    if (shared)
+        CFP_CUDA(cudaMemcpyAsync(rhs, qf, sizeof(double) * c->N, cudaMemcpyDeviceToDevice, c->stream));
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
 }

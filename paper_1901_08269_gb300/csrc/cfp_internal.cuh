@@ -133,7 +133,7 @@ enum { DETAIL_OFFGRID = 1, DETAIL_FEWPOINTS = 2, DETAIL_SINGULAR = 3, DETAIL_BOX
        DETAIL_OVERFLOW = 5, DETAIL_MISSINGIBI = 6 };
 
 constexpr int kAX = 128;           // apply CTA: columns (threads) along x
-constexpr int kApplyKC = 32;       // planes per apply CTA
+
 constexpr int kUpdBlocks = 152 * 8;   // grid of the vector-update kernels
 constexpr int kUpdThreads = 256;
 
@@ -358,7 +358,8 @@ template <>
 Side<double> side_view<double>(cfp_ctx* c);
 template <>
 Side<float> side_view<float>(cfp_ctx* c);
-void launch_apply_lift(cfp_ctx* c, const double* gb, double* y, cudaStream_t s);
+void launch_rhs(cfp_ctx* c, const double* f, const double* g, const double* g_ibi, double* gb, double* rhs,
+                cudaStream_t s);
 template <class T>
 void launch_apply(cfp_ctx* c, const T* x, T* y, const T* d0, int dotmode, double* partial,
                   cudaStream_t s, int* nblocks_out);
@@ -388,14 +389,10 @@ bool launch_mg_transfer(cfp_ctx* c, bool prolong, cudaStream_t s);
 // the fused black-then-red pass on the fine level; false where it does not apply
 template <class T>
 bool launch_mg_pair(cfp_ctx* c, cudaStream_t s);
-void launch_qf(cfp_ctx* c, const double* f, double* out, cudaStream_t s);
-void launch_rhs_finish(cfp_ctx* c, const double* qf, const double* bg, const double* g_ibi,
-                       double* rhs, cudaStream_t s);
 void launch_boundary_lift(cfp_ctx* c, const double* g, double* gb, cudaStream_t s);
 void launch_finish_solution(cfp_ctx* c, const double* x, const double* g, double* u, cudaStream_t s);
 void launch_mask_unknowns(cfp_ctx* c, const double* in, double* out, cudaStream_t s);
 int apply_blocks(cfp_ctx* c);  // partial pairs written by one launch_apply
-int corr_blocks(const cfp_ctx* c);
 void launch_metrics(cfp_ctx* c);  // Eq. app_xxx and Eq. 2ndorder_coef per axis
 
 // Krylov (cfp_krylov.cu)

@@ -916,17 +916,12 @@ cfp_status capture_device_solve(cfp_ctx* c, cudaStream_t s, const double* f, con
     double* tmp = c->v64 + V_TMP * vstride(c);
     double* X = c->v64 + V_X * vstride(c);
     double* gb = c->v64 + V_TMP * vstride(c);
-    double* bg = c->v64 + V_TMP2 * vstride(c);
-    double* qf = c->v64 + V_T * vstride(c);
     float* b32 = c->v32 + kNV32 * vstride(c);
     float* e32 = c->v32;
     KState* st = c->kst + 1;
     use_aux(c, 0);
     // the right-hand side (cfp_assemble_rhs), the masked initial iterate, ||rhs||^2, the first residual
-    launch_boundary_lift(c, g, gb, s);
-    launch_apply_lift(c, gb, bg, s);
-    launch_qf(c, f, qf, s);
-    launch_rhs_finish(c, qf, bg, c->n_ibi ? gi : c->ibi_xyz, rhs, s);
+    launch_rhs(c, f, g, c->n_ibi ? gi : c->ibi_xyz, gb, rhs, s);
     launch_mask_unknowns(c, u, X, s);
     k_dot<<<kUpdBlocks, kUpdThreads, 0, s>>>(rhs, rhs, c->partial, N);
     k_fin_store<<<1, 256, 0, s>>>(c->partial, kUpdBlocks, scalar_slot(c, 7));

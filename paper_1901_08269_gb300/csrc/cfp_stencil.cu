@@ -3,13 +3,11 @@
 //    rebuilt on the fly from the 1D metrics, sum-factorised as
 //      A x = sum_r Lz[r] (sum_q Ly[q] XR + Ry[q] XL) + Rz[r] (sum_q Ly[q] XL),
 //      XR = sum_p Rx[p] x,  XL = sum_p Lx[p] x,
-//    with the x-pass of each z-plane staged in shared memory and the y-pass
-//    results of three planes kept in registers while a CTA marches in z;
-//    rows of irregular points get their modified-stencil corrections from the
-//    side list in the same pass; solid rows are zero.
-//  - red-black Gauss-Seidel half-sweeps on K (Eqs. A7 / A7_mod, Sec. 3.3).
-//  - the source term of Eq. q with solid weights dropped, and helpers of the
-//    right-hand side of Eq. Bu=q.
+//    with the y-pass results of three planes kept in registers while a thread
+//    (FP64, narrow FP32 grids) or a shared-memory ring's consumer (wide FP32
+//    grids) marches in z; the rows of irregular points, with their
+//    modified-stencil corrections, in a kernel beside it; solid rows are zero.
+//  - the right-hand side of Eq. Bu=q and helpers of the solves.
 #include <algorithm>
 
 #include "cfp_internal.cuh"
@@ -688,58 +686,238 @@ __global__ void __launch_bounds__(kRingThreads, 2)
     }
 }
 
-constexpr int kQfRows = 2;  // rows per thread of k_qf
+// ---- the right-hand side of Eq. Bu=q: k_rhs_box gathers the Dirichlet
+// values of the box, k_rhs_source writes Q-bar f at every interior node,
+// k_rhs_shell subtracts the box values times their matrix entries from the
+// rows next to the box, and k_rhs_irr finishes the irregular rows.  Each node
+// of f is read once and each of rhs written once, plus the shell and the
+// irregular points; as separate full-grid passes (lift, B times the lift, Q,
+// difference) it took 685 us at 321 x 257 x 289, now 345.
 
-// B gb for a field gb that is zero away from the box (the boundary lift of
-// the right-hand side): its regular rows can be nonzero only on the shell of
-// interior nodes next to the box, so only those rows are evaluated, with the
-// 27 weights of Eq. A27 (Rx Ly Lz + Lx Ry Lz + Lx Ly Rz); every other
-// interior row is zero (the caller clears y).  Solid rows are zero; the
-// irregular rows get their corrections from k_apply_corr.  Thread q walks
-// the shell as two z-planes, then two y-rows of each inner plane, then the
-// two x-ends of each inner row.
-__global__ void k_lift_shell(Grid<double> G, const uint8_t* __restrict__ type, const double* __restrict__ gb,
-                             double* __restrict__ y) {
-    const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const int64_t ax = nx - 2, ay = ny - 2, az = nz - 2;
-    const int64_t bz = az - 2 > 0 ? az - 2 : 0, by = ay - 2 > 0 ? ay - 2 : 0;
-    const int64_t nA = 2 * ax * ay, nB = 2 * bz * ax, nC = 2 * bz * by;
-    const int64_t sy = nx, sz = (int64_t)nx * ny;
+// gb = g at the box nodes and rhs = 0 there; the other entries of gb are never
+// read.  Thread q walks the two z faces, the y faces without their z edges,
+// the x faces without theirs.
+__global__ void k_rhs_box(const double* __restrict__ g, double* __restrict__ gb, double* __restrict__ rhs, int nx, int ny,
+                          int nz) {
+    const int64_t sz = (int64_t)nx * ny;
+    const int64_t nA = 2 * sz, nB = 2 * (int64_t)(nz - 2) * nx, nC = 2 * (int64_t)(nz - 2) * (ny - 2);
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nA + nB + nC;
          q += (int64_t)gridDim.x * blockDim.x) {
-        int i, j, k;
+        int64_t l;
         if (q < nA) {
-            const int64_t r = q % (ax * ay);
-            k = q < ax * ay ? 1 : nz - 2;
-            i = 1 + (int)(r % ax);
-            j = 1 + (int)(r / ax);
+            l = q < sz ? q : (int64_t)(nz - 1) * sz + (q - sz);
         } else if (q < nA + nB) {
-            const int64_t r = (q - nA) % (bz * ax);
-            j = q - nA < bz * ax ? 1 : ny - 2;
-            i = 1 + (int)(r % ax);
-            k = 2 + (int)(r / ax);
+            const int64_t t = (q - nA) >> 1;
+            l = (1 + t / nx) * sz + ((q - nA) & 1 ? (int64_t)(ny - 1) * nx : 0) + t % nx;
         } else {
-            const int64_t r = (q - nA - nB) % (bz * by);
-            i = q - nA - nB < bz * by ? 1 : nx - 2;
-            j = 2 + (int)(r % by);
-            k = 2 + (int)(r / by);
+            const int64_t t = (q - nA - nB) >> 1;
+            l = (1 + t / (ny - 2)) * sz + (1 + t % (ny - 2)) * nx + ((q - nA - nB) & 1 ? nx - 1 : 0);
+        }
+        gb[l] = g[l];
+        rhs[l] = 0.0;
+    }
+}
+
+// The source term of Eq. q with the weights of solid points set to zero
+// (Q-bar): the tensor product Q = Lx Ly Lz applied to f with its solid
+// entries replaced by zero (SOLID: there are bodies), sum-factorised and
+// marched in z like k_apply64, whose launch shape it shares: 7 FP64
+// instructions per node with four rows per thread, which is what bounds it
+// (265 us at 321 x 257 x 289).  Interior solid nodes get 0.
+template <int TY, bool SOLID>
+__global__ void __launch_bounds__(32 * kA64Warps)
+    k_rhs_source(Grid<double> G, const uint8_t* __restrict__ type, const double* __restrict__ f,
+                 double* __restrict__ rhs, int kc) {
+    constexpr int R = TY + 2;
+    const int nx = G.nx, ny = G.ny, nz = G.nz;
+    const int i = 1 + blockIdx.x * 32 + threadIdx.x;
+    const int j0 = 1 + (blockIdx.y * kA64Warps + threadIdx.y) * TY;
+    const int k0 = 1 + blockIdx.z * kc;
+    const int k1 = min(k0 + kc, nz - 1);
+    if (j0 > ny - 2) return;
+    const bool iin = i <= nx - 2;
+    const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
+    const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
+    const double ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
+    double ay[TY], cy[TY];
+    bool jin[TY];
+#pragma unroll
+    for (int t = 0; t < TY; ++t) {
+        jin[t] = j0 + t <= ny - 2;
+        const int jc = jin[t] ? j0 + t : j0;
+        ay[t] = G.ax[1].a[jc];
+        cy[t] = G.ax[1].c[jc];
+    }
+    unsigned roff[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) roff[r] = (unsigned)min(j0 - 1 + r, ny - 1) * sy + (unsigned)ic;
+    double n[3 * R];
+    uint8_t own[R], prev[R] = {};  // type of (i, row) in the plane just loaded, and in the one before
+    auto load = [&](int k) {
+        const unsigned pz = (unsigned)k * sz;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const unsigned q = pz + roff[r];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const uint8_t t = SOLID ? type[q + d - 1] : (uint8_t)CFP_REGULAR;
+                n[3 * r + d] = SOLID && t == CFP_SOLID ? 0.0 : f[q + d - 1];
+                if (d == 1) own[r] = t;
+            }
+        }
+    };
+    load(k0 - 1);
+    double Qm[TY], Q0[TY], Qp[TY];
+#pragma unroll
+    for (int t = 0; t < TY; ++t) Qm[t] = Q0[t] = Qp[t] = 0.0;
+#pragma unroll 1
+    for (int kk = k0 - 1; kk <= k1; ++kk) {
+        double XL[R];
+        uint8_t tout[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            XL[r] = fmat(cx, n[3 * r + 2], fmat(ax, n[3 * r], n[3 * r + 1]));
+            tout[r] = prev[r];
+            prev[r] = own[r];
+        }
+        if (kk < k1) load(kk + 1);  // ahead of the y and z passes
+#pragma unroll
+        for (int t = 0; t < TY; ++t) {
+            Qm[t] = Q0[t];
+            Q0[t] = Qp[t];
+            Qp[t] = fmat(cy[t], XL[t + 2], fmat(ay[t], XL[t], XL[t + 1]));
+        }
+        if (kk >= k0 + 1 && iin) {
+            const int k = kk - 1;
+            const double az = G.ax[2].a[k], cz = G.ax[2].c[k];
+#pragma unroll
+            for (int t = 0; t < TY; ++t)
+                if (jin[t])
+                    rhs[(unsigned)k * sz + (unsigned)(j0 + t) * sy + (unsigned)i] =
+                        SOLID && tout[t + 1] == CFP_SOLID ? 0.0 : fmat(cz, Qp[t], fmat(az, Qm[t], Q0[t]));
+        }
+    }
+}
+
+// One axis' operators at a node: L = (a, 1, c), R = (ar, br, cr)
+struct Ops3 {
+    double L[3], R[3];
+    __device__ __forceinline__ Ops3(const Axis<double>& A, int i) : L{A.a[i], 1.0, A.c[i]}, R{A.ar[i], A.br[i], A.cr[i]} {}
+};
+
+// The row of B at a node of exactly one face shell, applied to the box values
+// of that face: nine nodes, a tensor product of the face's two axes (u, v)
+// times entry s of the normal axis (w): Lw[s] (Lv Ru + Rv Lu) + Rw[s] Lv Lu.
+__device__ __forceinline__ double face_lift(const Ops3& U, const Ops3& V, const Ops3& W, int s, const double* p,
+                                            int64_t su, int64_t sv) {
+    double P = 0.0, Q = 0.0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const double* x = p + (q - 1) * sv;
+        const double xr = U.R[0] * x[-su] + U.R[1] * x[0] + U.R[2] * x[su];
+        const double xl = U.L[0] * x[-su] + x[0] + U.L[2] * x[su];
+        P += V.L[q] * xr + V.R[q] * xl;
+        Q += V.L[q] * xl;
+    }
+    return W.L[s] * P + W.R[s] * Q;
+}
+
+// rhs -= B gb on the shell of interior nodes next to the box, the only rows
+// that reach it (solid rows stay zero; irregular rows get their corrections
+// from k_rhs_irr).  The inner nodes of each face (face_lift) and the nodes
+// next to two or three faces (27 weights, the box nodes among them read) are
+// separate ranges of q, so that a warp takes one path: 24 to 30 FP64
+// instructions per node instead of 135.  An axis with fewer than three
+// interior nodes has no inner ones: every shell node then takes the second.
+__global__ void k_rhs_shell(Grid<double> G, const uint8_t* __restrict__ type, const double* __restrict__ gb,
+                            double* __restrict__ rhs) {
+    const int nx = G.nx, ny = G.ny, nz = G.nz;
+    const int64_t ax = nx - 2, ay = ny - 2, az = nz - 2;  // interior nodes per axis
+    const bool thin = ax < 3 || ay < 3 || az < 3;
+    const int64_t bx = ax - 2, by = ay - 2, bz = az - 2;
+    const int64_t nA = thin ? 0 : 2 * bx * by, nB = thin ? 0 : 2 * bx * bz, nC = thin ? 0 : 2 * by * bz;
+    // edges: 4 lines along z (corners included), 4 along y, 4 along x; thin: the whole interior
+    const int64_t nE = thin ? ax * ay * az : 4 * az + 4 * by + 4 * bx;
+    const int64_t sy = nx, sz = (int64_t)nx * ny;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nA + nB + nC + nE;
+         q += (int64_t)gridDim.x * blockDim.x) {
+        int i, j, k, face = -1;
+        if (q < nA) {
+            const int64_t t = q % (bx * by);
+            i = 2 + (int)(t % bx), j = 2 + (int)(t / bx), k = q < bx * by ? 1 : nz - 2, face = 2;
+        } else if (q < nA + nB) {
+            const int64_t u = q - nA, t = u % (bx * bz);
+            i = 2 + (int)(t % bx), k = 2 + (int)(t / bx), j = u < bx * bz ? 1 : ny - 2, face = 1;
+        } else if (q < nA + nB + nC) {
+            const int64_t u = q - nA - nB, t = u % (by * bz);
+            j = 2 + (int)(t % by), k = 2 + (int)(t / by), i = u < by * bz ? 1 : nx - 2, face = 0;
+        } else {
+            const int64_t u = q - nA - nB - nC;
+            if (thin) {
+                i = 1 + (int)(u % ax), j = 1 + (int)((u / ax) % ay), k = 1 + (int)(u / (ax * ay));
+                if (i > 1 && i < nx - 2 && j > 1 && j < ny - 2 && k > 1 && k < nz - 2) continue;
+            } else if (u < 4 * az) {
+                i = u & 1 ? nx - 2 : 1, j = u & 2 ? ny - 2 : 1, k = 1 + (int)(u >> 2);
+            } else if (u < 4 * az + 4 * by) {
+                const int64_t t = u - 4 * az;
+                i = t & 1 ? nx - 2 : 1, k = t & 2 ? nz - 2 : 1, j = 2 + (int)(t >> 2);
+            } else {
+                const int64_t t = u - 4 * az - 4 * by;
+                j = t & 1 ? ny - 2 : 1, k = t & 2 ? nz - 2 : 1, i = 2 + (int)(t >> 2);
+            }
         }
         const int64_t l = (int64_t)k * sz + (int64_t)j * sy + i;
-        if (type[l] == CFP_SOLID) {
-            y[l] = 0.0;
-            continue;
-        }
-        const double Lx[3] = {G.ax[0].a[i], 1.0, G.ax[0].c[i]}, Rx[3] = {G.ax[0].ar[i], G.ax[0].br[i], G.ax[0].cr[i]};
-        const double Ly[3] = {G.ax[1].a[j], 1.0, G.ax[1].c[j]}, Ry[3] = {G.ax[1].ar[j], G.ax[1].br[j], G.ax[1].cr[j]};
-        const double Lz[3] = {G.ax[2].a[k], 1.0, G.ax[2].c[k]}, Rz[3] = {G.ax[2].ar[k], G.ax[2].br[k], G.ax[2].cr[k]};
+        if (type[l] == CFP_SOLID) continue;
+        const Ops3 X(G.ax[0], i), Y(G.ax[1], j), Z(G.ax[2], k);
         double v = 0.0;
-        for (int r = 0; r < 3; ++r)
-            for (int p = 0; p < 3; ++p)
-                for (int o = 0; o < 3; ++o) {
-                    const double w = Rx[o] * Ly[p] * Lz[r] + Lx[o] * Ry[p] * Lz[r] + Lx[o] * Ly[p] * Rz[r];
-                    v += w * gb[l + (o - 1) + (p - 1) * sy + (r - 1) * sz];
-                }
-        y[l] = v;
+        if (face == 2) {
+            const int s = k == 1 ? 0 : 2;
+            v = face_lift(X, Y, Z, s, gb + l + (s - 1) * sz, 1, sy);
+        } else if (face == 1) {
+            const int s = j == 1 ? 0 : 2;
+            v = face_lift(X, Z, Y, s, gb + l + (s - 1) * sy, 1, sz);
+        } else if (face == 0) {
+            const int s = i == 1 ? 0 : 2;
+            v = face_lift(Y, Z, X, s, gb + l + (s - 1), sy, sz);
+        } else {
+            for (int c = 0; c < 3; ++c)
+                for (int b = 0; b < 3; ++b)
+                    for (int a = 0; a < 3; ++a) {
+                        const int ii = i + a - 1, jj = j + b - 1, kk = k + c - 1;
+                        if (ii > 0 && jj > 0 && kk > 0 && ii < nx - 1 && jj < ny - 1 && kk < nz - 1) continue;
+                        const double w = X.R[a] * Y.L[b] * Z.L[c] + X.L[a] * Y.R[b] * Z.L[c] + X.L[a] * Y.L[b] * Z.R[c];
+                        v += w * gb[l + (a - 1) + (b - 1) * sy + (c - 1) * sz];
+                    }
+        }
+        rhs[l] -= v;
+    }
+}
+
+// The irregular rows' share: the corrections of the modified lines (the C
+// part of Eq. Bdec) times the box values they reach, and the IBI term of Eqs.
+// bc / qb_case2; one thread per irregular point.  A correction lies at most
+// six nodes away (a line of the 3 x 3 x 3 block, then at most five grid nodes
+// along it), so only points that near to the box look for box nodes.
+__global__ void __launch_bounds__(128)
+    k_rhs_irr(Side<double> S, const uint8_t* __restrict__ type, const int32_t* __restrict__ irr_lin, int64_t n_irr,
+              const int32_t* __restrict__ bib_ptr, const int32_t* __restrict__ bib_idx,
+              const double* __restrict__ bib_val, const double* __restrict__ gb, const double* __restrict__ g_ibi,
+              double* __restrict__ rhs, int nx, int ny, int nz) {
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_irr;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const int l = irr_lin[s];
+        const int k = l / (nx * ny), rem = l - k * nx * ny, j = rem / nx, i = rem - j * nx;
+        double v = rhs[l];
+        if (min(min(min(i, nx - 1 - i), min(j, ny - 1 - j)), min(k, nz - 1 - k)) <= 6) {
+            double cor = 0.0;
+            for (int e = S.corr_ptr[s]; e < S.corr_ptr[s + 1]; ++e) {
+                const int m = l + S.corr_off[e];
+                if (type[m] == CFP_BOUNDARY) cor += S.corr_val[e] * gb[m];
+            }
+            v -= cor;
+        }
+        for (int e = bib_ptr[s]; e < bib_ptr[s + 1]; ++e) v -= bib_val[e] * g_ibi[bib_idx[e]];
+        rhs[l] = v;
     }
 }
 
@@ -805,134 +983,12 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-// Side-list corrections of the irregular rows (the modified stencils of
-// Secs. 2.2-2.3, the C part of Eq. Bdec) added to a y that holds their
-// regular part, one warp per irregular point: the lanes gather the merged
-// entries in parallel, lane 0 adds the sum to y and updates the dot partials:
-// (d0, y) gains d0 c, (y, y) gains 2 v c + c^2 where v is the row's regular
-// part.  Used for the boundary lift (after k_lift_shell), one pair of
-// partials per CTA.
-template <class T, int DOT>
-__global__ void __launch_bounds__(256)
-    k_apply_corr(Side<T> S, const int32_t* __restrict__ irr_lin, int64_t n_irr, const T* __restrict__ x,
-                 T* __restrict__ y, const T* __restrict__ d0, double* __restrict__ partial) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    double acc0 = 0.0, acc1 = 0.0;
-    for (int64_t s = warp; s < n_irr; s += nwarps) {
-        const int64_t l = irr_lin[s];
-        const int e0 = S.corr_ptr[s], e1 = S.corr_ptr[s + 1];
-        T c = T(0);
-        for (int e = e0 + lane; e < e1; e += 32) c += S.corr_val[e] * x[l + S.corr_off[e]];
-        for (int o = 16; o; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-        if (lane == 0) {
-            const T v = y[l];
-            y[l] = v + c;
-            if (DOT >= 1) acc0 += (double)d0[l] * (double)c;
-            if (DOT == 2) acc1 += 2.0 * (double)v * (double)c + (double)c * (double)c;
-        }
-    }
-    if (DOT) {
-        block_reduce2(acc0, acc1);
-        if (threadIdx.x == 0) {
-            partial[2 * blockIdx.x] = acc0;
-            partial[2 * blockIdx.x + 1] = acc1;
-        }
-    }
-}
-
-
 template <class T>
 __global__ void k_mask_copy(const uint8_t* __restrict__ type, const T* __restrict__ in, T* __restrict__ out,
                             int64_t N) {
     for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < N; l += (int64_t)gridDim.x * blockDim.x) {
         const uint8_t t = type[l];
         out[l] = (t == CFP_REGULAR || t == CFP_IRREGULAR) ? in[l] : T(0);
-    }
-}
-
-// Eq. q with the weights of solid points set to zero (Q-bar), i.e. the
-// tensor product Q = Lx Ly Lz applied to f with its solid entries replaced
-// by zero, sum-factorised like the apply: each thread owns the columns
-// (i, j0) and (i, j0 + 1) and marches kApplyKC planes in z; per plane it
-// loads rows j0-1 .. j0+2 of the masked f, forms the x-pass XL = Lx f of
-// each row and the y-pass Q = Ly XL of its two rows, and keeps Q of three
-// planes for the z-pass out = Lz Q.  Interior non-unknowns get 0.
-__global__ void __launch_bounds__(kAX) k_qf(Grid<double> G, const uint8_t* __restrict__ type,
-                                            const double* __restrict__ f, double* __restrict__ out) {
-    constexpr int TY = kQfRows, R = TY + 2;
-    const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const int i = 1 + blockIdx.x * kAX + threadIdx.x;
-    const int j0 = 1 + blockIdx.y * TY;
-    const int k0 = 1 + blockIdx.z * kApplyKC;
-    const int k1 = min(k0 + kApplyKC, nz - 1);
-    const bool iin = i <= nx - 2;
-    const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
-    const int64_t sy = nx, sz = (int64_t)nx * ny;
-    const double ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
-    double ay[TY], cy[TY];
-    bool jin[TY];
-#pragma unroll
-    for (int t = 0; t < TY; ++t) {
-        jin[t] = j0 + t <= ny - 2;
-        const int jc = jin[t] ? j0 + t : j0;
-        ay[t] = G.ax[1].a[jc];
-        cy[t] = G.ax[1].c[jc];
-    }
-    int64_t roff[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) roff[r] = (int64_t)min(j0 - 1 + r, ny - 1) * sy + ic;
-    double Qm[TY], Q0[TY], Qp[TY];
-#pragma unroll
-    for (int t = 0; t < TY; ++t) Qm[t] = Q0[t] = Qp[t] = 0.0;
-    for (int kk = k0 - 1; kk <= k1; ++kk) {
-        const int64_t pz = (int64_t)kk * sz;
-        double XL[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int64_t q = pz + roff[r];
-            const double fm = type[q - 1] == CFP_SOLID ? 0.0 : f[q - 1];
-            const double f0 = type[q] == CFP_SOLID ? 0.0 : f[q];
-            const double fp = type[q + 1] == CFP_SOLID ? 0.0 : f[q + 1];
-            XL[r] = ax * fm + f0 + cx * fp;
-        }
-#pragma unroll
-        for (int t = 0; t < TY; ++t) {
-            Qm[t] = Q0[t];
-            Q0[t] = Qp[t];
-            Qp[t] = ay[t] * XL[t] + XL[t + 1] + cy[t] * XL[t + 2];
-        }
-        if (kk >= k0 + 1 && iin) {
-            const int k = kk - 1;
-            const double az = G.ax[2].a[k], cz = G.ax[2].c[k];
-#pragma unroll
-            for (int t = 0; t < TY; ++t) {
-                if (!jin[t]) continue;
-                const int64_t l = (int64_t)k * sz + (int64_t)(j0 + t) * sy + i;
-                const uint8_t tl = type[l];
-                out[l] = (tl == CFP_REGULAR || tl == CFP_IRREGULAR) ? az * Qm[t] + Q0[t] + cz * Qp[t] : 0.0;
-            }
-        }
-    }
-}
-
-__global__ void k_rhs_finish(const uint8_t* __restrict__ type, const int32_t* __restrict__ slot,
-                             const int32_t* __restrict__ bib_ptr, const int32_t* __restrict__ bib_idx,
-                             const double* __restrict__ bib_val, const double* __restrict__ qf,
-                             const double* __restrict__ bg, const double* __restrict__ g_ibi,
-                             double* __restrict__ rhs, int64_t N) {
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < N; l += (int64_t)gridDim.x * blockDim.x) {
-        const uint8_t t = type[l];
-        double v = 0.0;
-        if (t == CFP_REGULAR || t == CFP_IRREGULAR) {
-            v = qf[l] - bg[l];
-            if (t == CFP_IRREGULAR) {
-                const int s = slot[l];
-                for (int e = bib_ptr[s]; e < bib_ptr[s + 1]; ++e) v -= bib_val[e] * g_ibi[bib_idx[e]];
-            }
-        }
-        rhs[l] = v;
     }
 }
 
@@ -985,7 +1041,7 @@ unsigned flat_grid(int64_t n) {
 
 namespace {
 
-dim3 rows_grid(const cfp_ctx* c, int rows, int kc = kApplyKC) {
+dim3 rows_grid(const cfp_ctx* c, int rows, int kc) {
     return dim3((unsigned)((c->n[0] - 2 + kAX - 1) / kAX), (unsigned)((c->n[1] - 2 + rows - 1) / rows),
                 (unsigned)((c->n[2] - 2 + kc - 1) / kc));
 }
@@ -1039,14 +1095,8 @@ void launch_metrics(cfp_ctx* c) {
     c->launches += 3;
 }
 
-// CTAs of the correction kernel (8 irregular points per CTA, at most 152 x 16)
-int corr_blocks(const cfp_ctx* c) {
-    if (c->n_irr <= 0) return 0;
-    return (int)std::min<int64_t>((c->n_irr + 7) / 8, 152 * 16);
-}
-
 // CTAs of k_apply_irr (128 threads, one irregular point each per pass; at
-// most 152 x 8, never more than corr_blocks)
+// most 152 x 8)
 int irr_blocks(const cfp_ctx* c) {
     if (c->n_irr <= 0) return 0;
     return (int)std::min<int64_t>((c->n_irr + 127) / 128, 152 * 8);
@@ -1066,24 +1116,24 @@ struct Shape64 {
     }
 };
 
-// The shape of k_apply64: set by the tuner, else the one with the smallest
-// estimate.  A warp issues w = (kc + 2) (5 (ty + 2) + 7 ty) + 6 kc ty FP64
-// instructions (its two halo planes do the x and y passes only), a CTA 4 w;
-// the estimate is the busiest of 152 SMs, the latency of a plane's loads
+// The launch shape of k_apply64 (where the tuner set none) and k_rhs_source:
+// the one with the smallest estimate.  A warp issues w = (kc + 2) (row (ty +
+// 2) + yout ty) + zout kc ty FP64 instructions (row per loaded row, yout and
+// zout per output row in y and z: 5, 7, 6 in the apply; its two halo planes do
+// the x and y passes only), a CTA 4 w; the estimate is the busiest of 152 SMs, the latency of a plane's loads
 // (about 130 slots per plane), which counts where few CTAs share an SM, and,
 // past four CTAs per SM, half of a last one that runs alone.  Large grids
 // take 4 rows and 64 planes, 129^3 and 257^3 4 x 16 (109 and 712 us; 4 x 64
 // 250 and 895), 97 x 65 x 82 2 x 8; 33^3 takes 128 CTAs of 1 x 2, where 4 x
 // 64 would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
 // 33^3 14.5 us with them, 10.4 with four warps in the same shape.)
-Shape64 apply64_shape(const cfp_ctx* c) {
-    if (c->apply_ty[0] && c->apply_kc[0]) return Shape64{c->apply_ty[0], c->apply_kc[0]};
+Shape64 shape64(const cfp_ctx* c, double row, double yout, double zout) {
     Shape64 best{4, 64};
     double est_best = 1e300;
     for (int t : {4, 2, 1})
         for (int q : {64, 32, 16, 8, 4, 2}) {
             const Shape64 sh{t, q};
-            const double cta = kA64Warps * ((q + 2) * (5.0 * (t + 2) + 7.0 * t) + 6.0 * q * t);
+            const double cta = kA64Warps * ((q + 2) * (row * (t + 2) + yout * t) + zout * q * t);
             const double per = (double)((sh.ctas(c) + 151) / 152);
             const double est = per * cta + 130.0 * (q + 2) + (per > 4 ? 0.5 * cta : 0.0);
             if (est < est_best * 0.99) {
@@ -1093,8 +1143,12 @@ Shape64 apply64_shape(const cfp_ctx* c) {
         }
     return best;
 }
+Shape64 apply64_shape(const cfp_ctx* c) {
+    if (c->apply_ty[0] && c->apply_kc[0]) return Shape64{c->apply_ty[0], c->apply_kc[0]};
+    return shape64(c, 5.0, 7.0, 6.0);
+}
 
-// the most CTAs any apply tile shape launches, with the correction kernel's
+// the most CTAs any apply tile shape launches, with the irregular rows' kernel's
 // (dot-product partials per launch); the ring's persistent grid never has
 // more CTAs than the streaming kernel with 2 rows x 16 planes
 int apply_blocks(cfp_ctx* c) {
@@ -1105,7 +1159,7 @@ int apply_blocks(cfp_ctx* c) {
             m = std::max(m, std::max((int64_t)g.x * g.y * g.z, Shape64{ty, kc}.ctas(c)));
         }
     m = std::max(m, apply64_shape(c).ctas(c));
-    return (int)m + corr_blocks(c);
+    return (int)m + irr_blocks(c);
 }
 
 // the FP64 regular rows' kernel
@@ -1249,34 +1303,39 @@ void launch_precond(cfp_ctx* c, int sweeps, const T* rho, T* phi, cudaStream_t s
     else launch_precond_rbgs<T>(c, sweeps, rho, phi, s);
 }
 
-// y = B gb for the boundary lift gb (zero away from the box), FP64
-void launch_apply_lift(cfp_ctx* c, const double* gb, double* y, cudaStream_t s) {
-    cudaMemsetAsync(y, 0, sizeof(double) * c->N, s);
-    k_lift_shell<<<flat_grid(c->N), 256, 0, s>>>(grid_view<double>(c), c->type, gb, y);
-    c->launches += 1;
-    if (corr_blocks(c)) {
-        k_apply_corr<double, 0><<<corr_blocks(c), 256, 0, s>>>(side_view<double>(c), c->irr_lin, c->n_irr, gb, y,
-                                                               nullptr, nullptr);
-        c->launches += 1;
-    }
-}
-
 template void launch_apply<double>(cfp_ctx*, const double*, double*, const double*, int, double*, cudaStream_t,
                                    int*);
 template void launch_apply<float>(cfp_ctx*, const float*, float*, const float*, int, double*, cudaStream_t, int*);
 template void launch_precond<double>(cfp_ctx*, int, const double*, double*, cudaStream_t);
 template void launch_precond<float>(cfp_ctx*, int, const float*, float*, cudaStream_t);
 
-void launch_qf(cfp_ctx* c, const double* f, double* out, cudaStream_t s) {
-    c->launches += 1;
-    k_qf<<<rows_grid(c, kQfRows), kAX, 0, s>>>(grid_view<double>(c), c->type, f, out);
-}
-
-void launch_rhs_finish(cfp_ctx* c, const double* qf, const double* bg, const double* g_ibi, double* rhs,
-                       cudaStream_t s) {
-    c->launches += 1;
-    k_rhs_finish<<<flat_grid(c->N), 256, 0, s>>>(c->type, c->slot, c->bib_ptr, c->bib_idx, c->bib_val, qf, bg, g_ibi,
-                                                 rhs, c->N);
+// rhs (at every node) from f, g and g_ibi; gb: work field, overwritten at the
+// box nodes; rhs overlaps neither f nor gb
+void launch_rhs(cfp_ctx* c, const double* f, const double* g, const double* g_ibi, double* gb, double* rhs,
+                cudaStream_t s) {
+    const int nx = c->n[0], ny = c->n[1], nz = c->n[2];
+    const Grid<double> G = grid_view<double>(c);
+    const int64_t box = 2 * ((int64_t)nx * ny + (int64_t)nx * nz + (int64_t)ny * nz);
+    k_rhs_box<<<flat_grid(box), 256, 0, s>>>(g, gb, rhs, nx, ny, nz);
+    const Shape64 sh = shape64(c, 2.0, 2.0, 2.0);
+    const dim3 gr = sh.grid(c), b(32, kA64Warps);
+    const bool solid = !c->bodies.empty();
+#define CFP_SOURCE(TY)                                                                                     \
+    (solid ? k_rhs_source<TY, true><<<gr, b, 0, s>>>(G, c->type, f, rhs, sh.kc)                            \
+           : k_rhs_source<TY, false><<<gr, b, 0, s>>>(G, c->type, f, rhs, sh.kc))
+    if (sh.ty == 4) CFP_SOURCE(4);
+    else if (sh.ty == 2) CFP_SOURCE(2);
+    else CFP_SOURCE(1);
+#undef CFP_SOURCE
+    const bool thin = nx < 5 || ny < 5 || nz < 5;
+    k_rhs_shell<<<flat_grid(thin ? c->N : box), 256, 0, s>>>(G, c->type, gb, rhs);
+    c->launches += 3;
+    if (c->n_irr > 0) {
+        k_rhs_irr<<<(unsigned)std::min<int64_t>((c->n_irr + 127) / 128, 152 * 16), 128, 0, s>>>(
+            side_view<double>(c), c->type, c->irr_lin, c->n_irr, c->bib_ptr, c->bib_idx, c->bib_val, gb, g_ibi, rhs, nx,
+            ny, nz);
+        c->launches += 1;
+    }
 }
 
 void launch_boundary_lift(cfp_ctx* c, const double* g, double* gb, cudaStream_t s) {
