@@ -448,16 +448,18 @@ enum { CFP_APPLY_STREAM = 1,  /* each thread streams its column of `rows`
  * mixed solve's inner iterations): the kernel (CFP_APPLY_STREAM with 2 or 4
  * rows per thread and 16, 32 or 64 planes a CTA marches in z;
  * CFP_APPLY_RING, FP32 only, 2 rows per tile and 32 or 64 planes).
- * kernel = rows = planes = 0: every candidate (6 in FP64 and the context's own
- * shape by grid size, 8 in FP32) is timed (CUDA events, 5 launches after two untimed, on the context's work
- * vectors) and the fastest is kept by the context for its later solves;
+ * kernel = rows = planes = 0: every candidate (the context's own shape by grid
+ * size, 6 others in FP64, 8 in FP32) is timed (CUDA events, 5 launches after
+ * two untimed, on the context's work vectors) and the fastest is kept by the context for its later solves;
  * otherwise that choice is set and timed.  The rows of B x do not depend on the choice (the same fused
  * multiply-add chain per row in every kernel); the dot products fused into
  * the apply are summed per CTA, so their rounding does.  Without a call the
  * context uses CFP_APPLY_STREAM in FP64, in a shape that spreads the grid over
  * the SMs (cfp_apply_shape reports it as 4 rows x 64 planes); in FP32
  * CFP_APPLY_RING with 64 planes where its 512-column tiles are at least 85 %
- * filled by the n_x - 2 interior columns, else CFP_APPLY_STREAM with 2 x 64.
+ * filled by the n_x - 2 interior columns, else CFP_APPLY_STREAM with 2 x 64
+ * (fewer planes, down to 4, where 64 would leave the SMs fewer than four CTAs
+ * each; cfp_apply_shape reports at least 16).
  *   ms  NULL or the chosen candidate's mean time per launch.
  * Requires classification.  Synchronises.  Errors: CFP_ESTATE, CFP_EINVAL
  * (a choice outside those values, or CFP_APPLY_RING with CFP_PREC_FP64 or

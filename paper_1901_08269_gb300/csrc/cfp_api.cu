@@ -312,7 +312,7 @@ cfp_status cfp_apply(cfp_ctx* c, const double* x, double* y) {
     CFP_TRY(need_field(x, "x_dev"));
     CFP_TRY(need_field(y, "y_dev"));
     if (x == y) return fail(CFP_EINVAL, "x and y must not overlap");
-    CFP_CUDA(cudaMemsetAsync(y, 0, sizeof(double) * c->N, c->stream));
+    launch_zero_box(c, y, c->stream);
     launch_apply<double>(c, x, y, nullptr, 0, nullptr, c->stream, nullptr);
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
@@ -324,7 +324,7 @@ cfp_status cfp_apply_f32(cfp_ctx* c, const float* x, float* y) {
     CFP_TRY(need_field(y, "y_dev"));
     if (x == y) return fail(CFP_EINVAL, "x and y must not overlap");
     setup_apply_ring(c);
-    CFP_CUDA(cudaMemsetAsync(y, 0, sizeof(float) * c->N, c->stream));
+    launch_zero_box(c, y, c->stream);
     launch_apply<float>(c, x, y, nullptr, 0, nullptr, c->stream, nullptr);
     CFP_CUDA(cudaGetLastError());
     return check_waits(c);

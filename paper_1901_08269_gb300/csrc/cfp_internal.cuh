@@ -363,6 +363,9 @@ void launch_rhs(cfp_ctx* c, const double* f, const double* g, const double* g_ib
 template <class T>
 void launch_apply(cfp_ctx* c, const T* x, T* y, const T* d0, int dotmode, double* partial,
                   cudaStream_t s, int* nblocks_out);
+// y = 0 at the box nodes (with launch_apply: y = B x at every node)
+template <class T>
+void launch_zero_box(cfp_ctx* c, T* y, cudaStream_t s);
 template <class T>
 void launch_precond(cfp_ctx* c, int sweeps, const T* rho, T* phi, cudaStream_t s);
 

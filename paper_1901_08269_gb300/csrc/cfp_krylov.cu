@@ -507,7 +507,7 @@ cfp_status tune_apply(cfp_ctx* c, int prec, int kind, int rows, int planes, int 
             return fail(CFP_EINVAL, "apply ring: FP32 only, and its launch could not be set up");
         cand.push_back({kind, rows, planes});
     } else {
-        if (q == 0) cand.push_back({0, 0, 0});  // the shape by grid size that FP64 uses unless one is set
+        cand.push_back({0, 0, 0});  // the shape by grid size used unless one is set
         for (int r : {2, 4})
             for (int k : {16, 32, 64}) cand.push_back({CFP_APPLY_STREAM, r, k});
         if (ring)

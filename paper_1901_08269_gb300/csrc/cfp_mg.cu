@@ -153,6 +153,9 @@ __device__ __forceinline__ double rb_rest(double b, double cxl, double cxh, doub
     return __fma_rn(-czh, zp, v);
 }
 
+__device__ __forceinline__ float mg_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mg_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // FP32: x * (1 / d) with the hardware reciprocal approximation
 // (rcp.approx.ftz.f32, within 1 ulp of 1 / d; the diagonal of K is a normal
 // number), a single instruction where the correctly rounded one costs a short
@@ -200,7 +203,10 @@ struct Off {
 // 2: from zero, and b of both colours is first read from the natural-layout
 //    rho; 3: plain, and both nodes of the pair are written to the
 //    natural-layout phi (the own node's new value is not stored).
-constexpr int kSweepPlanes = 3;
+// kSweepPlanes: three in FP32; two in FP64, which is bound by issue rather than
+// by loads in flight and whose registers cost it warps (129^3: 20.8 us).
+template <class T>
+constexpr int kSweepPlanes = sizeof(T) == 8 ? 2 : 3;
 
 template <class T, int MODE, bool FINE>
 __global__ void __launch_bounds__(kSplitThreads)
@@ -208,61 +214,73 @@ __global__ void __launch_bounds__(kSplitThreads)
     constexpr bool F64 = sizeof(T) == 8, READ = MODE == 0 || MODE == 3;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
     const T* __restrict__ eoth = H.eoth;
-    T val[kSweepPlanes], bv[kSweepPlanes], bo[kSweepPlanes], xo[kSweepPlanes];
-    bool inz[kSweepPlanes], live[kSweepPlanes];
-    unsigned oo[kSweepPlanes];
+    T bv[kSweepPlanes<T>], bo[kSweepPlanes<T>], rdv[kSweepPlanes<T>], nb[kSweepPlanes<T>][6];
+    uint8_t ty[kSweepPlanes<T>], tyo[kSweepPlanes<T>];
+    bool inz[kSweepPlanes<T>];
+    unsigned oo[kSweepPlanes<T>];
+    // every load first (a branch between two nodes' loads would order them)
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q) {
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
         inz[q] = k0 + q <= L.nz - 2;
         const int k = inz[q] ? k0 + q : k0;
         const int par = (colour + j + k) & 1;
-        const int i = 2 * m + par, io = 2 * m + 1 - par;
         const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
-        const int64_t row = ((int64_t)k * L.ny + j) * nx;
+        oo[q] = o;
         // which nodes are unknowns (and irregular): FP64 from the reciprocal
         // diagonal, FP32 from the type
-        const T rd = F64 ? H.rd[o] : T(0);
-        const uint8_t t = F64 ? (uint8_t)CFP_REGULAR : H.ty[o];
-        bv[q] = MODE == 2 ? rho[row + i] : H.bown[o];
+        rdv[q] = F64 ? H.rd[o] : T(0);
+        ty[q] = F64 ? (uint8_t)CFP_REGULAR : H.ty[o];
         if (MODE == 2) {
-            bo[q] = rho[row + io];
-            if (!F64) {  // the NaN marks of the FP32 levels
-                if (!is_unknown(t)) bv[q] = T(b_mark());
-                if (!is_unknown(H.tyo[o])) bo[q] = T(b_mark());
-            }
+            const T* pair = rho + (((int64_t)k * L.ny + j) * nx + 2 * m);
+            bv[q] = pair[par];
+            bo[q] = pair[1 - par];
+            tyo[q] = F64 ? (uint8_t)CFP_REGULAR : H.tyo[o];
+        } else {
+            bv[q] = H.bown[o];
         }
-        T xm = T(0), xp = T(0), ym = T(0), yp = T(0), zm = T(0), zp = T(0);
         if (READ) {
-            xm = eoth[o - 1 + par];
-            xp = eoth[o + par];
-            ym = eoth[o - hp];
-            yp = eoth[o + hp];
-            zm = eoth[o - hs];
-            zp = eoth[o + hs];
+            nb[q][0] = eoth[o - 1 + par];
+            nb[q][1] = eoth[o + par];
+            nb[q][2] = eoth[o - hp];
+            nb[q][3] = eoth[o + hp];
+            nb[q][4] = eoth[o - hs];
+            nb[q][5] = eoth[o + hs];
         }
-        const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-        live[q] = inz[q] && i >= 1 && i <= nx - 2 && (F64 ? rd != T(0) : is_unknown(t));
+    }
+    const PkT<T> cx0 = L.cx[2 * m], cx1 = L.cx[2 * m + 1], cky = L.cy[j];
+    T val[kSweepPlanes<T>];
+    bool live[kSweepPlanes<T>];
+#pragma unroll
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
+        const int k = inz[q] ? k0 + q : k0;
+        const int par = (colour + j + k) & 1;
+        const int i = 2 * m + par;
+        const PkT<T> ckx = par ? cx1 : cx0, ckz = L.cz[k];
+        live[q] = inz[q] && i >= 1 && i <= nx - 2 && (F64 ? rdv[q] != T(0) : is_unknown(ty[q]));
+        if (MODE == 2 && !F64) {  // the NaN marks of the FP32 levels
+            if (!is_unknown(ty[q])) bv[q] = T(b_mark());
+            if (!is_unknown(tyo[q])) bo[q] = T(b_mark());
+        }
         Off<T> f{ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z};
         T dg = F64 ? T(0) : ckx.y + (cky.y + ckz.y);
-        if (FINE && live[q] && (F64 ? rd > T(0) : t == CFP_IRREGULAR)) {
-            const T* kr = S.krow + 7 * (int64_t)S.slot[row + i];
-            f = Off<T>{kr[1], kr[2], kr[3], kr[4], kr[5], kr[6]};
+        if (FINE && live[q] && (F64 ? rdv[q] > T(0) : ty[q] == CFP_IRREGULAR)) {
+            const T* kr = S.krow + 7 * (int64_t)S.slot[((int64_t)k * L.ny + j) * nx + i];
+            if (READ) f = Off<T>{kr[1], kr[2], kr[3], kr[4], kr[5], kr[6]};
             dg = kr[0];
         }
         T v = bv[q];
-        if (READ) v = rb_rest(v, f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, xm, xp, ym, yp, zm, zp);
-        if constexpr (F64) val[q] = times_rd(v, rd);
+        if (READ)
+            v = rb_rest(v, f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, nb[q][0], nb[q][1], nb[q][2], nb[q][3], nb[q][4], nb[q][5]);
+        if constexpr (F64) val[q] = times_rd(v, rdv[q]);
         else val[q] = times_rcp(v, dg);
-        xo[q] = par ? xm : xp;  // MODE 3: the other node of the pair
-        oo[q] = o;
     }
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q) {
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
         if (!inz[q]) continue;
         const unsigned o = oo[q];
         if (MODE == 2) {
@@ -275,7 +293,8 @@ __global__ void __launch_bounds__(kSplitThreads)
             const int i = 2 * m + par, io = 2 * m + 1 - par;
             const int64_t row = ((int64_t)k * L.ny + j) * nx;
             if (i >= 1 && i <= nx - 2) phi[row + i] = live[q] ? val[q] : T(0);
-            if (io >= 1 && io <= nx - 2) phi[row + io] = xo[q];
+            // the other node of the pair
+            if (io >= 1 && io <= nx - 2) phi[row + io] = par ? nb[q][0] : nb[q][1];
         } else if (live[q]) {
             H.eown[o] = val[q];
         }
@@ -701,9 +720,9 @@ __global__ void k_fix_rows(const FixPt* __restrict__ list, int n, int nx, int64_
 }
 
 // The update at the fine level's irregular nodes of colour `colour` (the
-// list of that colour) after a TMA-fed FP32 half-sweep, with their
+// list of that colour) after an FP32 half-sweep of a large grid, with their
 // Shortley-Weller rows (Eq. A7_mod); one thread per node, overwriting what
-// the half-sweep stored there (MODE 0, or 3: in phi).
+// the half-sweep stored there (MODE 0 and 2, or 3: in phi).
 template <int MODE>
 __global__ void k_sweep_fix(SLev<float> L, Side<float> S, Half<float> H, const FixPt* __restrict__ list, int64_t n,
                             float* __restrict__ phi) {
@@ -713,8 +732,10 @@ __global__ void k_sweep_fix(SLev<float> L, Side<float> S, Half<float> H, const F
         const unsigned o = p.o;
         const float* kr = S.krow + 7 * (int64_t)p.slot;
         const float* __restrict__ eoth = H.eoth;
-        float v = rb_rest(H.bown[o], kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], eoth[o - 1 + par], eoth[o + par],
-                          eoth[o - L.hp], eoth[o + L.hp], eoth[o - L.hs], eoth[o + L.hs]);
+        float v = H.bown[o];
+        if (MODE != 2)
+            v = rb_rest(v, kr[1], kr[2], kr[3], kr[4], kr[5], kr[6], eoth[o - 1 + par], eoth[o + par], eoth[o - L.hp],
+                        eoth[o + L.hp], eoth[o - L.hs], eoth[o + L.hs]);
         v = times_rcp(v, kr[0]);
         if (MODE == 3) phi[p.lin] = v;
         else H.eown[o] = v;
@@ -1006,44 +1027,55 @@ __global__ void __launch_bounds__(kPairThreads, 4)
 // half-sweep.
 template <class T, bool FINE>
 __global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S) {
-    constexpr bool F64 = sizeof(T) == 8;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
     const T* __restrict__ e1 = L.e[1];
-    T rv[kSweepPlanes];
-    bool live[kSweepPlanes];
-    unsigned oo[kSweepPlanes];
+    T b0[kSweepPlanes<T>], e0[kSweepPlanes<T>], nb[kSweepPlanes<T>][6], rv[kSweepPlanes<T>];
+    uint8_t ty[kSweepPlanes<T>];
+    bool inz[kSweepPlanes<T>], live[kSweepPlanes<T>];
+    unsigned oo[kSweepPlanes<T>];
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q) {
-        const bool inz = k0 + q <= L.nz - 2;
-        const int k = inz ? k0 + q : k0;
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
+        inz[q] = k0 + q <= L.nz - 2;
+        const int k = inz[q] ? k0 + q : k0;
+        const int par = (j + k) & 1;
+        const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
+        oo[q] = o;
+        ty[q] = L.ty[0][o];
+        e0[q] = L.e[0][o];
+        b0[q] = L.b[0][o];
+        nb[q][0] = e1[o - 1 + par];
+        nb[q][1] = e1[o + par];
+        nb[q][2] = e1[o - hp];
+        nb[q][3] = e1[o + hp];
+        nb[q][4] = e1[o - hs];
+        nb[q][5] = e1[o + hs];
+    }
+    const PkT<T> cx0 = L.cx[2 * m], cx1 = L.cx[2 * m + 1], cky = L.cy[j];
+#pragma unroll
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
+        const int k = inz[q] ? k0 + q : k0;
         const int par = (j + k) & 1;
         const int i = 2 * m + par;
-        const unsigned o = (unsigned)k * hs + (unsigned)(j * hp + m);
-        const uint8_t t = L.ty[0][o];
-        const T e0 = L.e[0][o], b0 = L.b[0][o];
-        const T xm = e1[o - 1 + par], xp = e1[o + par], ym = e1[o - hp], yp = e1[o + hp], zm = e1[o - hs],
-                zp = e1[o + hs];
-        const PkT<T> ckx = L.cx[i], cky = L.cy[j], ckz = L.cz[k];
-        live[q] = inz && i >= 1 && i <= nx - 2 && is_unknown(t);
+        const PkT<T> ckx = par ? cx1 : cx0, ckz = L.cz[k];
+        live[q] = inz[q] && i >= 1 && i <= nx - 2 && is_unknown(ty[q]);
         Off<T> f{ckx.x, ckx.z, cky.x, cky.z, ckz.x, ckz.z};
         T dg = ckx.y + (cky.y + ckz.y);
-        if (FINE && live[q] && t == CFP_IRREGULAR) {
+        if (FINE && live[q] && ty[q] == CFP_IRREGULAR) {
             const T* kr = S.krow + 7 * (int64_t)S.slot[((int64_t)k * L.ny + j) * nx + i];
             f = Off<T>{kr[1], kr[2], kr[3], kr[4], kr[5], kr[6]};
             dg = kr[0];
         }
-        const T v = rb_rest(b0, f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, xm, xp, ym, yp, zm, zp);
-        if constexpr (F64) rv[q] = __fma_rn(-dg, e0, v);
-        else rv[q] = __fmaf_rn(-dg, e0, v);
-        oo[q] = o;
+        const T v = rb_rest(b0[q], f.xl, f.xh, f.yl, f.yh, f.zl, f.zh, nb[q][0], nb[q][1], nb[q][2], nb[q][3], nb[q][4],
+                            nb[q][5]);
+        rv[q] = mg_fma(-dg, e0[q], v);
     }
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q)
+    for (int q = 0; q < kSweepPlanes<T>; ++q)
         if (live[q]) L.r0[oo[q]] = rv[q];
 }
 
@@ -1062,8 +1094,6 @@ __global__ void k_resid_fix(SLev<float> L, Side<float> S, const FixPt* __restric
     }
 }
 
-__device__ __forceinline__ float mg_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double mg_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // (P^T r) / (P^T 1) of a coarse node from its 27 fine neighbours' red
 // residuals, r(a, b, c) that of fine node (2I - 1 + a, 2J - 1 + b, 2K - 1 + c).
@@ -1130,17 +1160,17 @@ template <class T>
 __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
     const int nx = F.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > F.ny - 2) return;
     const unsigned hc = (unsigned)C.hp;
     const IpPk<T> py = X.ip[1][j];
     const int J = py.ilo;
     T* __restrict__ e1 = F.e[1];
-    T val[kSweepPlanes];
-    bool live[kSweepPlanes];
-    unsigned oo[kSweepPlanes];
+    T val[kSweepPlanes<T>];
+    bool live[kSweepPlanes<T>];
+    unsigned oo[kSweepPlanes<T>];
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q) {
+    for (int q = 0; q < kSweepPlanes<T>; ++q) {
         const bool inz = k0 + q <= F.nz - 2;
         const int k = inz ? k0 + q : k0;
         const int i = 2 * m + ((1 + j + k) & 1);
@@ -1164,7 +1194,7 @@ __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, 
         oo[q] = o;
     }
 #pragma unroll
-    for (int q = 0; q < kSweepPlanes; ++q)
+    for (int q = 0; q < kSweepPlanes<T>; ++q)
         if (live[q]) e1[oo[q]] = val[q];
 }
 
@@ -1292,10 +1322,11 @@ dim3 plane_block(const int n[3]) {
     const int bx = std::min(kSplitThreads, (n[0] / 2 + 31) / 32 * 32);
     return dim3((unsigned)bx, (unsigned)(kSplitThreads / bx));
 }
+template <class T>
 dim3 plane_grid(const int n[3]) {
     const dim3 b = plane_block(n);
     return dim3((unsigned)((n[0] / 2 + b.x - 1) / b.x), (unsigned)((n[1] - 2 + b.y - 1) / b.y),
-                (unsigned)((n[2] - 2 + kSweepPlanes - 1) / kSweepPlanes));
+                (unsigned)((n[2] - 2 + kSweepPlanes<T> - 1) / kSweepPlanes<T>));
 }
 
 template <class T>
@@ -1471,15 +1502,7 @@ void reset_red(cfp_ctx* c) {
     for (MgLevel& M : c->mg) M.red_cur = 0;
 }
 
-template <class T, int MODE>
-void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Half<T>& H, const Side<T>& S, int colour,
-                        const T* rho, T* phi, cudaStream_t s) {
-    const dim3 g = plane_grid(c->mg[l].n), blk = plane_block(c->mg[l].n);
-    if (l == 0 && c->n_irr > 0) k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
-    else k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
-}
-
-// the fine level's Shortley-Weller rows after a TMA-fed half-sweep (MODE 0 or 3)
+// the fine level's Shortley-Weller rows after a half-sweep of a large FP32 grid
 template <int MODE>
 void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, const Side<float>& S, int colour,
                       float* phi, cudaStream_t s) {
@@ -1489,6 +1512,24 @@ void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, co
     k_sweep_fix<MODE><<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
         L, S, H, static_cast<const FixPt*>(M0.fix) + colour * c->n_irr, n, phi);
     c->launches += 1;
+}
+
+// The plain-load half-sweep, with the fine level's Shortley-Weller rows: taken
+// inside the kernel, except by the first red half-sweep of a large FP32 grid,
+// which is bound by HBM and pays more for the branch (513^3: 289 us against
+// 233 and a follow-up of 5).
+template <class T, int MODE>
+void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Half<T>& H, const Side<T>& S, int colour,
+                        const T* rho, T* phi, cudaStream_t s) {
+    const dim3 g = plane_grid<T>(c->mg[l].n), blk = plane_block(c->mg[l].n);
+    const bool after = MODE == 2 && sizeof(T) == 4 && c->mg[l].tma;
+    if (l == 0 && c->n_irr > 0 && !after) {
+        k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
+        return;
+    }
+    k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
+    if constexpr (MODE == 2 && sizeof(T) == 4)
+        if (l == 0) launch_sweep_fix<2>(c, L, H, S, colour, phi, s);
 }
 
 template <class T>
@@ -1970,7 +2011,7 @@ void launch_prolong(cfp_ctx* c, int l, const SLev<T>& F, const SLev<T>& C, cudaS
         const dim3 g((unsigned)((Cn.n[0] - 1 + 127) / 128), (unsigned)(Cn.n[1] - 1), (unsigned)(Cn.n[2] - 1));
         k_prolong_cell<T><<<g, 128, 0, s>>>(transfer<T>(c->mg[l]), F, C);
     } else {
-        k_prolong_split<T><<<plane_grid(c->mg[l].n), plane_block(c->mg[l].n), 0, s>>>(transfer<T>(c->mg[l]), F, C);
+        k_prolong_split<T><<<plane_grid<T>(c->mg[l].n), plane_block(c->mg[l].n), 0, s>>>(transfer<T>(c->mg[l]), F, C);
     }
 }
 
@@ -2003,7 +2044,7 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
                 }
             }
         } else {
-            const dim3 g = plane_grid(c->mg[l].n), blk = plane_block(c->mg[l].n);
+            const dim3 g = plane_grid<T>(c->mg[l].n), blk = plane_block(c->mg[l].n);
             if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(F, S);
             else k_resid_split<T, false><<<g, blk, 0, s>>>(F, S);
         }

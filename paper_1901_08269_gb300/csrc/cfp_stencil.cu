@@ -93,8 +93,9 @@ __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a,
 
 // Regular part of B x at the unknowns in FP32 (the streaming kernel; the
 // ring below takes the wide grids).  One thread owns the column i of TY
-// consecutive rows j and marches the planes k0 .. k1 - 1 of its z chunk (KC
-// planes); TY x KC is the tile shape the autotuner picks per grid.  The z
+// consecutive rows j and marches the planes k0 .. k1 - 1 of its z chunk (kc
+// planes, at most kMaxPlanes); TY x kc is the tile shape (apply32_planes, or
+// the autotuner's choice).  The z
 // coefficients of the chunk are staged in shared memory once.
 // Per plane it loads the values x(i-1..i+1, j) of the rows j0-1 .. j0+TY (the
 // x and y neighbours come from L1/L2; the loads of the next plane are issued
@@ -110,22 +111,23 @@ __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a,
 // dependent side-list loads stall the streaming march, and the CTAs near the
 // bodies become the tail.)
 // DOT = 0: y only; 1: partial (d0, y); 2: partials (d0, y) and (y, y).
-template <int DOT, int TY, int KC>
+constexpr int kMaxPlanes = 64;
+template <int DOT, int TY>
 __global__ void __launch_bounds__(kAX, TY == 2 ? 8 : 4)
     k_apply(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
-            const float* __restrict__ d0, double* __restrict__ partial) {
+            const float* __restrict__ d0, double* __restrict__ partial, int kc) {
     constexpr int R = TY + 2;  // rows loaded per plane
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int i = 1 + blockIdx.x * kAX + threadIdx.x;
     const int j0 = 1 + blockIdx.y * TY;
-    const int k0 = 1 + blockIdx.z * KC;
-    const int k1 = min(k0 + KC, nz - 1);
+    const int k0 = 1 + blockIdx.z * kc;
+    const int k1 = min(k0 + kc, nz - 1);
     // z coefficients of the chunk's output planes k0 .. k1 - 1
-    __shared__ float zc[5][KC];
-    for (int q = threadIdx.x; q < 5 * KC; q += kAX) {
-        const int m = q / KC, kc = min(k0 + q % KC, nz - 2);
+    __shared__ float zc[5][kMaxPlanes];
+    for (int q = threadIdx.x; q < 5 * kMaxPlanes; q += kAX) {
+        const int m = q / kMaxPlanes, kq = min(k0 + q % kMaxPlanes, nz - 2);
         const float* src = m == 0 ? G.ax[2].a : m == 1 ? G.ax[2].c : m == 2 ? G.ax[2].ar : m == 3 ? G.ax[2].br : G.ax[2].cr;
-        zc[m][q % KC] = src[kc];
+        zc[m][q % kMaxPlanes] = src[kq];
     }
     __syncthreads();
     const bool iin = i <= nx - 2;
@@ -470,10 +472,10 @@ struct DotAcc2 {
     }
 };
 
-template <int DOT, int KC, bool SPAN>
+template <int DOT, bool SPAN>
 __global__ void __launch_bounds__(kRingThreads, 2)
     k_apply_ring(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
-                 const float* __restrict__ d0, double* __restrict__ partial, int ntx, int nty, int ntz,
+                 const float* __restrict__ d0, double* __restrict__ partial, int ntx, int nty, int ntz, int kc,
                  int* __restrict__ wait_err) {
     using namespace tc;
     // indexed from the __shared__ array itself, so that every stage access
@@ -513,8 +515,8 @@ __global__ void __launch_bounds__(kRingThreads, 2)
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             const int tyi = tile % nty, rest = tile / nty, tx = rest % ntx, tz = rest / ntx;
-            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * KC;
-            const int k1 = min(k0 + KC, nz - 1);
+            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
+            const int k1 = min(k0 + kc, nz - 1);
             int64_t rowe;  // the copy's first element within a plane
             int w;         // elements wanted
             if (SPAN) {
@@ -555,12 +557,13 @@ __global__ void __launch_bounds__(kRingThreads, 2)
         // consumer: columns i0 + lx (low half) and i0 + 256 + lx (high half)
         // of the rows j0, j0 + 1
         const int lx = threadIdx.x;
-        unsigned g = 0;
+        int st = 0;       // stage of the next plane
+        unsigned ph = 0;  // and its phase
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const int tyi = tile % nty, rest = tile / nty, tx = rest % ntx, tz = rest / ntx;
-            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * KC;
-            const int k1 = min(k0 + KC, nz - 1);
+            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
+            const int k1 = min(k0 + kc, nz - 1);
             const int c = i0 + lx;  // the low half's column; the high half's is c + 256
             const bool in0 = c <= nx - 2, in1 = c + kRingCons <= nx - 2;
             const int c0i = in0 ? c : nx - 2, c1i = in1 ? c + kRingCons : nx - 2;
@@ -568,10 +571,9 @@ __global__ void __launch_bounds__(kRingThreads, 2)
             const float2 ARX = f2(G.ax[0].ar[c0i], G.ax[0].ar[c1i]), BRX = f2(G.ax[0].br[c0i], G.ax[0].br[c1i]);
             const float2 CRX = f2(G.ax[0].cr[c0i], G.ax[0].cr[c1i]);
             float2 AY[2], CY[2], ARY[2], BRY[2], CRY[2];
-            bool jin[2];
+            const bool jin1 = j0 + 1 <= ny - 2;  // row j0 always is
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
-                jin[t] = j0 + t <= ny - 2;
                 const int jc = min(j0 + t, ny - 2);
                 AY[t] = f2b(G.ax[1].a[jc]);
                 CY[t] = f2b(G.ax[1].c[jc]);
@@ -581,50 +583,44 @@ __global__ void __launch_bounds__(kRingThreads, 2)
             }
             // stage positions: element (row q, column col) of a plane at
             // xb[q] + ((kp + xa[q]) & 3) + col, kp = the plane's first element
-            // (SPAN: one offset for all rows); likewise for the output rows
-            int xb[4], db[2], tb[2];
-            unsigned xa[4], da[2], ta[2];
+            // (SPAN: rows n_x apart, one offset for all); likewise for the
+            // output rows.  kx, ko carry kp of the plane being read and of the
+            // one being written, kept below 16 (only their low bits count).
+            const int xrow = SPAN ? nx : kRingXRow, drow = SPAN ? nx : kRingDRow, trow = SPAN ? nx : kRingTRow;
+            const int xcol = SPAN ? c : c - (i0 - 1), ocol = SPAN ? c : c - i0;
+            unsigned xa[4], oa[2];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                xb[q] = SPAN ? q * nx : q * kRingXRow - (i0 - 1);
+            for (int q = 0; q < 4; ++q)
                 xa[q] = SPAN ? ((unsigned)(j0 - 1) * sy) & 3u
                              : ((unsigned)min(j0 - 1 + q, ny - 1) * sy + (unsigned)(i0 - 1)) & 3u;
-            }
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const unsigned jr = SPAN ? (unsigned)j0 : (unsigned)min(j0 + t, ny - 2);
-                db[t] = SPAN ? t * nx : t * kRingDRow - i0;
-                tb[t] = SPAN ? t * nx : t * kRingTRow - i0;
-                da[t] = (jr * sy + (SPAN ? 0u : (unsigned)i0)) & 3u;
-                ta[t] = (jr * sy + (SPAN ? 0u : (unsigned)i0)) & 15u;
-            }
+            for (int t = 0; t < 2; ++t)
+                oa[t] = ((SPAN ? (unsigned)j0 : (unsigned)min(j0 + t, ny - 2)) * sy + (SPAN ? 0u : (unsigned)i0)) & 15u;
+            unsigned kx = ((unsigned)(k0 - 1) * sz) & 15u, ko = 0;
             float2 Pm[2], P0[2], Pp[2], Qm[2], Q0[2], Qp[2];
 #pragma unroll
             for (int t = 0; t < 2; ++t) Pm[t] = P0[t] = Pp[t] = Qm[t] = Q0[t] = Qp[t] = f2b(0.f);
             // z coefficients of the plane the next step outputs, loaded a step ahead
+            const float* zp = G.ax[2].a + k0;  // a, c, ar, br, cr follow at n_z
             float zn[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            float* yr = y + ((unsigned)k0 * sz + (unsigned)j0 * sy + (unsigned)c);
+            int sprev = 0;  // stage of the plane before
             for (int kk = k0 - 1; kk <= k1; ++kk) {
                 const float2 AZ = f2b(zn[0]), CZ = f2b(zn[1]), ARZ = f2b(zn[2]), BRZ = f2b(zn[3]), CRZ = f2b(zn[4]);
-                if (kk < k1) {
-                    const int kn = max(kk, 1);
-                    zn[0] = G.ax[2].a[kn];
-                    zn[1] = G.ax[2].c[kn];
-                    zn[2] = G.ax[2].ar[kn];
-                    zn[3] = G.ax[2].br[kn];
-                    zn[4] = G.ax[2].cr[kn];
+                if (kk >= k0 && kk < k1) {
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) zn[q] = zp[q * nz];
+                    ++zp;
                 }
-                const unsigned gp = g + (unsigned)(kk - (k0 - 1));
-                const unsigned st = gp % kRingStages;
-                if (ok && !mbar_wait(&full[st], (gp / kRingStages) & 1)) {
+                if (ok && !mbar_wait(&full[st], ph)) {
                     ok = false;
                     atomicExch(wait_err, 33);
                 }
-                const unsigned kp = (unsigned)kk * sz;
-                const float* xs = sf + st * (kRingStage / 4) + c;
+                const float* xs = sf + st * (kRingStage / 4) + xcol + (SPAN ? (int)((kx + xa[0]) & 3u) : 0);
                 float2 XR[4], XL[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const float* row = xs + xb[q] + (int)((kp + xa[SPAN ? 0 : q]) & 3u);
+                    const float* row = xs + q * xrow + (SPAN ? 0 : (int)((kx + xa[q]) & 3u));
                     const float2 xm = f2(row[-1], row[kRingCons - 1]), x0 = f2(row[0], row[kRingCons]),
                                  xp = f2(row[1], row[kRingCons + 1]);
                     XR[q] = fma2(CRX, xp, fma2(BRX, x0, mul2(ARX, xm)));
@@ -641,39 +637,48 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                                       fma2(ARY[t], XL[t], fma2(CY[t], XR[t + 2], fma2(AY[t], XR[t], XR[t + 1])))));
                     Qp[t] = fma2(CY[t], XL[t + 2], fma2(AY[t], XL[t], XL[t + 1]));
                 }
-                if (kk >= k0) {
-                    const unsigned sq = (gp - 1) % kRingStages;  // plane kk - 1: output (from kk = k0 + 1 on), then released
-                    if (kk >= k0 + 1 && in0) {
-                        const unsigned kq = (unsigned)(kk - 1) * sz;
-                        const unsigned char* ts = ring_smem + sq * kRingStage + kRingTOff + c;
-                        const float* ds = sf + sq * (kRingStage / 4) + kRingDOff / 4 + c;
+                if (kk >= k0) {  // plane kk - 1 (stage sprev): output (from kk = k0 + 1 on), then released
+                    if (kk >= k0 + 1) {
+                        if (in0) {
+                            const unsigned char* ts =
+                                ring_smem + sprev * kRingStage + kRingTOff + ocol + (SPAN ? (int)((ko + oa[0]) & 15u) : 0);
+                            const float* ds =
+                                sf + sprev * (kRingStage / 4) + kRingDOff / 4 + ocol + (SPAN ? (int)((ko + oa[0]) & 3u) : 0);
 #pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            if (!jin[t]) continue;
-                            float2 v = add2(fma2(CZ, Pp[t], fma2(AZ, Pm[t], P0[t])),
-                                            fma2(CRZ, Qp[t], fma2(BRZ, Q0[t], mul2(ARZ, Qm[t]))));
-                            const unsigned char* tr = ts + tb[t] + (int)((kq + ta[SPAN ? 0 : t]) & 15u);
-                            // solid rows are zero; irregular rows belong to k_apply_irr
-                            const uint8_t t0 = tr[0], t1 = in1 ? tr[kRingCons] : (uint8_t)CFP_SOLID;
-                            if (t0 != CFP_REGULAR) v.x = 0.f;
-                            if (t1 != CFP_REGULAR) v.y = 0.f;
-                            float* yr = y + (kq + (unsigned)(j0 + t) * sy + (unsigned)c);
-                            if (t0 != CFP_IRREGULAR) yr[0] = v.x;
-                            if (in1 && t1 != CFP_IRREGULAR) yr[kRingCons] = v.y;
-                            if (DOT >= 1) {
-                                const float* dr = ds + db[t] + (int)((kq + da[SPAN ? 0 : t]) & 3u);
-                                dacc0.add(f2(dr[0], in1 ? dr[kRingCons] : 0.f), v);
+                            for (int t = 0; t < 2; ++t) {
+                                if (t && !jin1) continue;
+                                float2 v = add2(fma2(CZ, Pp[t], fma2(AZ, Pm[t], P0[t])),
+                                                fma2(CRZ, Qp[t], fma2(BRZ, Q0[t], mul2(ARZ, Qm[t]))));
+                                const unsigned char* tr = ts + t * trow + (SPAN ? 0 : (int)((ko + oa[t]) & 15u));
+                                // solid rows are zero; irregular rows belong to k_apply_irr
+                                const uint8_t t0 = tr[0], t1 = in1 ? tr[kRingCons] : (uint8_t)CFP_SOLID;
+                                if (t0 != CFP_REGULAR) v.x = 0.f;
+                                if (t1 != CFP_REGULAR) v.y = 0.f;
+                                float* yt = yr + t * nx;
+                                if (t0 != CFP_IRREGULAR) yt[0] = v.x;
+                                if (in1 && t1 != CFP_IRREGULAR) yt[kRingCons] = v.y;
+                                if (DOT >= 1) {
+                                    const float* dr = ds + t * drow + (SPAN ? 0 : (int)((ko + oa[t]) & 3u));
+                                    dacc0.add(f2(dr[0], in1 ? dr[kRingCons] : 0.f), v);
+                                }
+                                if (DOT == 2) dacc1.add(v, v);
                             }
-                            if (DOT == 2) dacc1.add(v, v);
                         }
+                        yr += sz;
                     }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&empty[sq]);
+                    if (lane == 0) mbar_arrive(&empty[sprev]);
+                }
+                ko = kx;
+                kx = (kx + sz) & 15u;
+                sprev = st;
+                if (++st == kRingStages) {
+                    st = 0;
+                    ph ^= 1u;
                 }
             }
             __syncwarp();
-            g += (unsigned)(k1 - k0 + 2);
-            if (lane == 0) mbar_arrive(&empty[(g - 1) % kRingStages]);  // the tile's last plane
+            if (lane == 0) mbar_arrive(&empty[sprev]);  // the tile's last plane
         }
     }
     if (DOT) {
@@ -694,28 +699,39 @@ __global__ void __launch_bounds__(kRingThreads, 2)
 // irregular points; as separate full-grid passes (lift, B times the lift, Q,
 // difference) it took 685 us at 321 x 257 x 289, now 345.
 
-// gb = g at the box nodes and rhs = 0 there; the other entries of gb are never
-// read.  Thread q walks the two z faces, the y faces without their z edges,
-// the x faces without theirs.
-__global__ void k_rhs_box(const double* __restrict__ g, double* __restrict__ gb, double* __restrict__ rhs, int nx, int ny,
-                          int nz) {
+// f(l) at every box node l: the two z faces, the y faces without their z
+// edges, the x faces without theirs
+template <class F>
+__device__ __forceinline__ void for_box(int nx, int ny, int nz, F f) {
     const int64_t sz = (int64_t)nx * ny;
     const int64_t nA = 2 * sz, nB = 2 * (int64_t)(nz - 2) * nx, nC = 2 * (int64_t)(nz - 2) * (ny - 2);
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nA + nB + nC;
          q += (int64_t)gridDim.x * blockDim.x) {
-        int64_t l;
         if (q < nA) {
-            l = q < sz ? q : (int64_t)(nz - 1) * sz + (q - sz);
+            f(q < sz ? q : (int64_t)(nz - 1) * sz + (q - sz));
         } else if (q < nA + nB) {
             const int64_t t = (q - nA) >> 1;
-            l = (1 + t / nx) * sz + ((q - nA) & 1 ? (int64_t)(ny - 1) * nx : 0) + t % nx;
+            f((1 + t / nx) * sz + ((q - nA) & 1 ? (int64_t)(ny - 1) * nx : 0) + t % nx);
         } else {
             const int64_t t = (q - nA - nB) >> 1;
-            l = (1 + t / (ny - 2)) * sz + (1 + t % (ny - 2)) * nx + ((q - nA - nB) & 1 ? nx - 1 : 0);
+            f((1 + t / (ny - 2)) * sz + (1 + t % (ny - 2)) * nx + ((q - nA - nB) & 1 ? nx - 1 : 0));
         }
+    }
+}
+
+// gb = g at the box nodes and rhs = 0 there; the other entries of gb are never read
+__global__ void k_rhs_box(const double* __restrict__ g, double* __restrict__ gb, double* __restrict__ rhs, int nx, int ny,
+                          int nz) {
+    for_box(nx, ny, nz, [=](int64_t l) {
         gb[l] = g[l];
         rhs[l] = 0.0;
-    }
+    });
+}
+
+// y = 0 at the box nodes: what an apply does not write itself
+template <class T>
+__global__ void k_zero_box(T* __restrict__ y, int nx, int ny, int nz) {
+    for_box(nx, ny, nz, [=](int64_t l) { y[l] = T(0); });
 }
 
 // The source term of Eq. q with the weights of solid points set to zero
@@ -1048,7 +1064,7 @@ dim3 rows_grid(const cfp_ctx* c, int rows, int kc) {
 
 // the apply's kernel and tile shape of precision q (0 FP64, 1 FP32), as set
 // by the autotuner; otherwise in FP64 the shape apply64_shape finds (reported
-// as 4 x 64), in FP32 the ring (2 x 64) where its 512-column tiles are at least 85 % filled
+// as 4 x 64), in FP32 (apply32_planes; reported with at least 16 planes) the ring (2 x 64) where its 512-column tiles are at least 85 % filled
 // (n_x = 513: 511 of 512 columns) and else the streaming kernel with 2 x 64
 // (at 385^3, 383 of 512 columns, it measured 0.285 ms against 0.256 ms)
 int apply_kind(const cfp_ctx* c, int q) {
@@ -1062,13 +1078,28 @@ int apply_kind(const cfp_ctx* c, int q) {
 int apply_rows(const cfp_ctx* c, int q) { return c->apply_ty[q] ? c->apply_ty[q] : (q ? 2 : 4); }
 int apply_planes(const cfp_ctx* c, int q) { return c->apply_kc[q] ? c->apply_kc[q] : 64; }
 
+// planes per z chunk of the FP32 streaming kernel: the tuner's, else 64, less
+// on grids that 64 would leave with fewer than four CTAs per SM (33^3 with 64
+// is 16 CTAs and takes 12.4 us, with 4 it is 128)
+int apply32_planes(const cfp_ctx* c) {
+    int kc = apply_planes(c, 1);
+    if (!c->apply_kc[1])
+        while (kc > 4) {
+            const dim3 g = rows_grid(c, apply_rows(c, 1), kc);
+            if ((int64_t)g.x * g.y * g.z >= 4 * 152) break;
+            kc /= 2;
+        }
+    return kc;
+}
+
 }  // namespace
 
-// the kernel and tile shape the apply of precision q runs with
+// the kernel and tile shape the apply of precision q runs with, as a shape
+// that can be set
 void apply_shape(const cfp_ctx* c, int q, int* kernel, int* rows, int* planes) {
     *kernel = apply_kind(c, q);
     *rows = *kernel == CFP_APPLY_RING ? 2 : apply_rows(c, q);
-    *planes = apply_planes(c, q);
+    *planes = q ? std::max(16, apply32_planes(c)) : apply_planes(c, q);
     if (*kernel == CFP_APPLY_RING && *planes < 32) *planes = 32;
 }
 
@@ -1159,6 +1190,8 @@ int apply_blocks(cfp_ctx* c) {
             m = std::max(m, std::max((int64_t)g.x * g.y * g.z, Shape64{ty, kc}.ctas(c)));
         }
     m = std::max(m, apply64_shape(c).ctas(c));
+    const dim3 g = rows_grid(c, apply_rows(c, 1), apply32_planes(c));
+    m = std::max(m, (int64_t)g.x * g.y * g.z);
     return (int)m + irr_blocks(c);
 }
 
@@ -1175,25 +1208,26 @@ void apply64_launch(cfp_ctx* c, const Shape64& sh, const double* x, double* y, c
 // B x: the regular rows' kernel on s and, forked onto the context's second
 // stream and joined back before anything later on s, the irregular rows'
 // kernel; dot partials: the main kernel's CTAs, then k_apply_irr's.
-template <class T, int DOT, int TY, int KC>
+template <class T, int DOT>
 void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cudaStream_t s, int* nb) {
-    int nmain = 0;
+    int nmain = 0, ntx = 0, nty = 0, ntz = 0, kc = 0;
     bool ring = false;
-    constexpr int RKC = KC < 32 ? 32 : KC;  // the ring marches 32 or 64 planes
-    int ntx = 0, nty = 0, ntz = 0;
     dim3 grid;
     Shape64 sh64{0, 0};
-    if constexpr (sizeof(T) == 4)
-        ring = apply_kind(c, 1) == CFP_APPLY_RING && c->ring_grid > 0 && aligned16(x) && (!DOT || aligned16(d0));
-    if (ring) {
-        ring_tiles(c, RKC, &ntx, &nty, &ntz);
-        nmain = std::min(ntx * nty * ntz, c->ring_grid);
-    } else if (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8) {
         sh64 = apply64_shape(c);
         nmain = (int)sh64.ctas(c);
     } else {
-        grid = rows_grid(c, TY, KC);
-        nmain = (int)(grid.x * grid.y * grid.z);
+        ring = apply_kind(c, 1) == CFP_APPLY_RING && c->ring_grid > 0 && aligned16(x) && (!DOT || aligned16(d0));
+        if (ring) {
+            kc = std::max(32, apply_planes(c, 1));  // the ring marches 32 or 64 planes
+            ring_tiles(c, kc, &ntx, &nty, &ntz);
+            nmain = std::min(ntx * nty * ntz, c->ring_grid);
+        } else {
+            kc = apply32_planes(c);
+            grid = rows_grid(c, apply_rows(c, 1), kc);
+            nmain = (int)(grid.x * grid.y * grid.z);
+        }
     }
     const int nirr = irr_blocks(c);
     if (nirr) {
@@ -1202,19 +1236,20 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
         k_apply_irr<T, DOT><<<nirr, 128, 0, c->aux>>>(grid_view<T>(c), side_view<T>(c), c->irr_lin, c->n_irr, x, y,
                                                       d0, partial ? partial + 2 * (int64_t)nmain : nullptr);
     }
-    if (ring) {
-        if constexpr (sizeof(T) == 4) {
-            if (c->n[0] <= kRingSpanNx)
-                k_apply_ring<DOT, RKC, true><<<nmain, kRingThreads, kRingSmem, s>>>(
-                    grid_view<float>(c), c->type, x, y, d0, partial, ntx, nty, ntz, c->dwait);
-            else
-                k_apply_ring<DOT, RKC, false><<<nmain, kRingThreads, kRingSmem, s>>>(
-                    grid_view<float>(c), c->type, x, y, d0, partial, ntx, nty, ntz, c->dwait);
-        }
-    } else if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8) {
         apply64_launch<DOT>(c, sh64, x, y, d0, partial, s);
+    } else if (ring) {
+        const Grid<float> G = grid_view<float>(c);
+        if (c->n[0] <= kRingSpanNx)
+            k_apply_ring<DOT, true><<<nmain, kRingThreads, kRingSmem, s>>>(G, c->type, x, y, d0, partial, ntx, nty, ntz,
+                                                                           kc, c->dwait);
+        else
+            k_apply_ring<DOT, false><<<nmain, kRingThreads, kRingSmem, s>>>(G, c->type, x, y, d0, partial, ntx, nty, ntz,
+                                                                            kc, c->dwait);
+    } else if (apply_rows(c, 1) == 4) {
+        k_apply<DOT, 4><<<grid, kAX, 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, kc);
     } else {
-        k_apply<DOT, TY, KC><<<grid, kAX, 0, s>>>(grid_view<T>(c), c->type, x, y, d0, partial);
+        k_apply<DOT, 2><<<grid, kAX, 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, kc);
     }
     if (nirr) {
         cudaEventRecord(c->ev_join, c->aux);
@@ -1224,38 +1259,18 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
     if (nb) *nb = nmain + nirr;
 }
 
-template <class T, int TY, int KC>
-void apply_dot(cfp_ctx* c, const T* x, T* y, const T* d0, int dotmode, double* partial, cudaStream_t s, int* nb) {
-    if (dotmode == 0) apply_launch<T, 0, TY, KC>(c, x, y, d0, partial, s, nb);
-    else if (dotmode == 1) apply_launch<T, 1, TY, KC>(c, x, y, d0, partial, s, nb);
-    else apply_launch<T, 2, TY, KC>(c, x, y, d0, partial, s, nb);
-}
-
-template <class T, int TY>
-void apply_depth(cfp_ctx* c, int kc, const T* x, T* y, const T* d0, int dotmode, double* partial, cudaStream_t s,
-                 int* nb) {
-    if (kc == 16) apply_dot<T, TY, 16>(c, x, y, d0, dotmode, partial, s, nb);
-    else if (kc == 64) apply_dot<T, TY, 64>(c, x, y, d0, dotmode, partial, s, nb);
-    else apply_dot<T, TY, 32>(c, x, y, d0, dotmode, partial, s, nb);
-}
-
 namespace {
-template <int DOT, int KC, bool SPAN>
+template <int DOT, bool SPAN>
 bool ring_attr(int* per) {
-    if (cudaFuncSetAttribute(k_apply_ring<DOT, KC, SPAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmem) !=
+    if (cudaFuncSetAttribute(k_apply_ring<DOT, SPAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmem) !=
         cudaSuccess)
         return false;
     int p = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_apply_ring<DOT, KC, SPAN>, kRingThreads, kRingSmem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_apply_ring<DOT, SPAN>, kRingThreads, kRingSmem) !=
         cudaSuccess)
         return false;
     *per = std::min(*per, p);
     return true;
-}
-template <int DOT>
-bool ring_attr_kc(int* per) {
-    return ring_attr<DOT, 32, true>(per) && ring_attr<DOT, 64, true>(per) && ring_attr<DOT, 32, false>(per) &&
-           ring_attr<DOT, 64, false>(per);
 }
 }  // namespace
 
@@ -1264,7 +1279,8 @@ bool ring_attr_kc(int* per) {
 bool setup_apply_ring(cfp_ctx* c) {
     if (c->ring_grid) return c->ring_grid > 0;
     int per = 1 << 20, nsm = 0;
-    const bool ok = ring_attr_kc<0>(&per) && ring_attr_kc<1>(&per) && ring_attr_kc<2>(&per) &&
+    const bool ok = ring_attr<0, true>(&per) && ring_attr<1, true>(&per) && ring_attr<2, true>(&per) &&
+                    ring_attr<0, false>(&per) && ring_attr<1, false>(&per) && ring_attr<2, false>(&per) &&
                     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess;
     cudaGetLastError();
     c->ring_grid = ok && per >= 1 ? per * nsm : -1;
@@ -1274,13 +1290,21 @@ bool setup_apply_ring(cfp_ctx* c) {
 template <class T>
 void launch_apply(cfp_ctx* c, const T* x, T* y, const T* d0, int dotmode, double* partial, cudaStream_t s,
                   int* nblocks_out) {
-    const int q = sizeof(T) == 4 ? 1 : 0;
-    const int ty = apply_rows(c, q), kc = apply_planes(c, q);
-    if constexpr (sizeof(T) == 8) apply_dot<T, 4, 64>(c, x, y, d0, dotmode, partial, s, nblocks_out);
-    else if (ty == 4) apply_depth<T, 4>(c, kc, x, y, d0, dotmode, partial, s, nblocks_out);
-    else apply_depth<T, 2>(c, kc, x, y, d0, dotmode, partial, s, nblocks_out);
+    if (dotmode == 0) apply_launch<T, 0>(c, x, y, d0, partial, s, nblocks_out);
+    else if (dotmode == 1) apply_launch<T, 1>(c, x, y, d0, partial, s, nblocks_out);
+    else apply_launch<T, 2>(c, x, y, d0, partial, s, nblocks_out);
     c->launches += 1;
 }
+
+template <class T>
+void launch_zero_box(cfp_ctx* c, T* y, cudaStream_t s) {
+    const int nx = c->n[0], ny = c->n[1], nz = c->n[2];
+    const int64_t box = 2 * ((int64_t)nx * ny + (int64_t)nx * nz + (int64_t)ny * nz);
+    k_zero_box<T><<<flat_grid(box), 256, 0, s>>>(y, nx, ny, nz);
+    c->launches += 1;
+}
+template void launch_zero_box<double>(cfp_ctx*, double*, cudaStream_t);
+template void launch_zero_box<float>(cfp_ctx*, float*, cudaStream_t);
 
 // `sweeps` red-black sweeps from phi = 0 (sweeps = 0: masked copy).  The
 // sweeps run on the fine level's red/black split arrays of the multigrid
