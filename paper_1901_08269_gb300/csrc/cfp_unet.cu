@@ -26,8 +26,6 @@
 #include <math.h>
 #include <string.h>
 
-#include <cudaTypedefs.h>
-
 #include <random>
 #include <vector>
 
@@ -61,36 +59,6 @@ int64_t param_count() {
     return n;
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            return nullptr;
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }();
-    return fn;
-}
-
-// Activation (Np x C BF16) as a 2D tensor (channels innermost) with a box of
-// 8 channels x rows; rows outside [0, Np) read as zero.
-cfp_status act_map(CUtensorMap* m, const void* base, int C, int Np, int rows) {
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encoder();
-    if (!enc) return fail(CFP_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    if (((uintptr_t)base & 15) != 0) return fail(CFP_EINVAL, "activation arrays must be 16-byte aligned");
-    const cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)Np};
-    const cuuint64_t strides[1] = {(cuuint64_t)C * 2};
-    const cuuint32_t box[2] = {8, (cuuint32_t)rows};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return fail(CFP_ECUDA, "cuTensorMapEncodeTiled failed for an activation");
-    return CFP_OK;
-}
-
 Pad make_pad(int nx, int ny, int nz) {
     Pad P;
     P.nx = nx;
@@ -118,6 +86,12 @@ unsigned blocks(int64_t n, int per = 256) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 152 * 32));
 }
 
+// the producers copy 16 bytes at a time
+cfp_status aligned_act(const void* p) {
+    if (((uintptr_t)p & 15) != 0) return fail(CFP_EINVAL, "activation arrays must be 16-byte aligned");
+    return CFP_OK;
+}
+
 // ------------------------------------------------------ launch dispatch
 template <int CIN, int COUT>
 cfp_status prep_conv() {
@@ -137,14 +111,8 @@ cfp_status prep_conv() {
 
 template <int CIN, int COUT>
 int conv_grid(const Pad& P) {
-    using C = ConvCfg<CIN, COUT>;
-    static int per = []() {
-        int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_conv_tc<CIN, COUT>, kConvThreads, C::SMEM);
-        return v > 0 ? v : 1;
-    }();
     const int ntiles = (P.Np + 127) / 128;
-    return std::max(1, std::min(ntiles, per * num_sms()));
+    return std::max(1, std::min(ntiles, ConvCfg<CIN, COUT>::PER * num_sms()));
 }
 
 template <int CIN, int COUT>
@@ -152,69 +120,96 @@ cfp_status conv_t(cudaStream_t s, const uint16_t* in, const uint16_t* wsrc, bool
                   const float* bias, const uint16_t* act, const Pad& P, int flags, void* out, int* err) {
     using C = ConvCfg<CIN, COUT>;
     { const cfp_status ps_ = prep_conv<CIN, COUT>(); if (ps_ != CFP_OK) return ps_; }
-    CUtensorMap m;
-    CFP_TRY(act_map(&m, in, CIN, P.Np, kWin));
+    CFP_TRY(aligned_act(in));
     const int nw = COUT * 27 * CIN;
     if (flip) k_wpack<CIN, COUT, true><<<blocks(nw), 256, 0, s>>>(wsrc, wpk);
     else k_wpack<CIN, COUT, false><<<blocks(nw), 256, 0, s>>>(wsrc, wpk);
     k_conv_tc<CIN, COUT><<<conv_grid<CIN, COUT>(P), kConvThreads, C::SMEM, s>>>(
-        m, wpk, bias, act, P, flags, (flags & F_OUT_F32) ? nullptr : (uint16_t*)out,
+        in, wpk, bias, act, P, flags, (flags & F_OUT_F32) ? nullptr : (uint16_t*)out,
         (flags & F_OUT_F32) ? (float*)out : nullptr, err);
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
 }
 
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int nchunks, int cin, int cout,
-                               float* __restrict__ dw) {
-    const int n = 27 * cin * cout;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+// dw += the chunks' partials; 64 entries per block, four threads an entry (each
+// a quarter of the chunks), added in a fixed order
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part, int nchunks, int cin, int cout,
+                                                      float* __restrict__ dw) {
+    const int n = 27 * cin * cout, sub = threadIdx.x >> 6, per = (nchunks + 3) / 4;
+    const int e = blockIdx.x * 64 + (threadIdx.x & 63);
+    __shared__ float red[3][64];
+    float s = 0.f;
+    if (e < n)
+#pragma unroll 8
+        for (int q = sub * per; q < min(nchunks, (sub + 1) * per); ++q) s += part[(size_t)q * n + e];
+    if (sub) red[sub - 1][threadIdx.x & 63] = s;
+    __syncthreads();
+    if (sub == 0 && e < n) {
         const int co = e % cout, r = e / cout, ci = r % cin, t = r / cin;
-        float s = 0.f;
-        for (int q = 0; q < nchunks; ++q) s += part[(size_t)q * n + e];
+        for (int k = 0; k < 3; ++k) s += red[k][threadIdx.x];
         dw[((size_t)co * 27 + t) * cin + ci] += s;
     }
 }
 
-// column sums of a (Np x C) BF16 matrix: per-block partials, then a fixed-order sum
-__global__ void k_colsum_part(const uint16_t* __restrict__ g, int Np, int C, float* __restrict__ part) {
-    const int c = threadIdx.x % C, lanes = blockDim.x / C, l = threadIdx.x / C;
+// column sums of a (Np x C) BF16 matrix (16-byte aligned, C = 16 .. 128): a
+// thread adds the same 8 channels of every (256 / (C / 8))-th row of its
+// block's share, then per-block partials and sums in a fixed order
+__global__ void __launch_bounds__(256) k_colsum_part(const uint16_t* __restrict__ g, int Np, int C,
+                                                     float* __restrict__ part) {
+    const int c8 = C / 8, lanes = 256 / c8, c = threadIdx.x % c8, l = threadIdx.x / c8;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int r = blockIdx.x * lanes + l; r < Np; r += gridDim.x * lanes) {
+        const uint4 v = reinterpret_cast<const uint4*>(g + (size_t)r * C)[c];
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s[2 * q] += __uint_as_float(w[q] << 16);
+            s[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
+        }
+    }
+    __shared__ float red[256][8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) red[threadIdx.x][q] = s[q];
+    __syncthreads();
+    for (int e = threadIdx.x; e < C; e += 256) {  // channel e = 8 c + q
+        float t = 0.f;
+        for (int k = 0; k < lanes; ++k) t += red[k * c8 + e / 8][e % 8];
+        part[blockIdx.x * C + e] = t;
+    }
+}
+__global__ void __launch_bounds__(1024) k_colsum_final(const float* __restrict__ part, int nb, int C,
+                                                       float* __restrict__ db) {
+    __shared__ float red[1024];
+    const int lanes = 1024 / C, c = threadIdx.x % C, l = threadIdx.x / C;
     float s = 0.f;
-    for (int r = blockIdx.x * lanes + l; r < Np; r += gridDim.x * lanes) s += bf2f(g[(size_t)r * C + c]);
-    __shared__ float red[256];
+    for (int b = l; b < nb; b += lanes) s += part[b * C + c];
     red[threadIdx.x] = s;
     __syncthreads();
     if (l == 0) {
-        for (int q = 1; q < lanes; ++q) s += red[q * C + c];
-        part[blockIdx.x * C + c] = s;
+        for (int k = 1; k < lanes; ++k) s += red[k * C + c];
+        db[c] += s;
     }
 }
-__global__ void k_colsum_final(const float* __restrict__ part, int nb, int C, float* __restrict__ db) {
-    const int c = threadIdx.x;
-    if (c >= C) return;
-    float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part[b * C + c];
-    db[c] += s;
-}
-constexpr int kColBlocks = 256;
+constexpr int kColBlocks = 304;
 
 template <int CIN, int COUT>
 cfp_status wgrad_t(cudaStream_t s, const uint16_t* x, const uint16_t* g, const Pad& P, float* part, int64_t part_cap,
                    float* dw, float* db, float* bpart, int* err) {
     using W = WgCfg<CIN, COUT>;
     { const cfp_status ps_ = prep_conv<CIN, COUT>(); if (ps_ != CFP_OK) return ps_; }
-    CUtensorMap mx, mg;
-    CFP_TRY(act_map(&mx, x, CIN, P.Np, kWin));
-    CFP_TRY(act_map(&mg, g, COUT, P.Np, 128));
+    CFP_TRY(aligned_act(x));
+    CFP_TRY(aligned_act(g));
     const int ntiles = (P.Np + 127) / 128;
     int nch = std::max(1, std::min(ntiles, num_sms() / W::NSETS));
     while ((int64_t)nch * 27 * CIN * COUT > part_cap && nch > 1) --nch;
     const int tpc = (ntiles + nch - 1) / nch;
     nch = (ntiles + tpc - 1) / tpc;
-    k_wgrad_tc<CIN, COUT><<<dim3(W::NSETS, nch), kConvThreads, W::SMEM, s>>>(mx, mg, P, tpc, part, err);
-    k_wgrad_reduce<<<blocks(27 * CIN * COUT), 256, 0, s>>>(part, nch, CIN, COUT, dw);
+    k_wgrad_tc<CIN, COUT><<<dim3(W::NSETS, nch), kConvThreads, W::SMEM, s>>>(x, g, P, tpc, part, err);
+    k_wgrad_reduce<<<(27 * CIN * COUT + 63) / 64, 256, 0, s>>>(part, nch, CIN, COUT, dw);
     if (db) {
-        k_colsum_part<<<kColBlocks, 256 / COUT * COUT, 0, s>>>(g, P.Np, COUT, bpart);
-        k_colsum_final<<<1, 128, 0, s>>>(bpart, kColBlocks, COUT, db);
+        k_colsum_part<<<kColBlocks, 256, 0, s>>>(g, P.Np, COUT, bpart);
+        k_colsum_final<<<1, 1024, 0, s>>>(bpart, kColBlocks, COUT, db);
     }
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
@@ -1051,7 +1046,7 @@ cfp_status cfp_nn_conv3d(cfp_ctx* ctx, int nx, int ny, int nz, int cin, int cout
         CFP_CUDA(cudaMemsetAsync(ctx->dwait, 0, sizeof(int), ctx->stream));
     }
     void* wpk = nullptr;
-    CFP_CUDA(cudaMallocAsync(&wpk, (size_t)27 * cin * cout * 2, ctx->stream));
+    CFP_CUDA(pool_malloc(&wpk, (size_t)27 * cin * cout * 2, ctx->stream));
     const int f = (flags & CFP_NN_RELU ? F_RELU : 0) | (flags & CFP_NN_MASK ? F_MASK : 0) |
                   (flags & CFP_NN_OUT_F32 ? F_OUT_F32 : 0) | (flags & CFP_NN_ACCUM ? F_ACCUM : 0);
     cfp_status st = conv_any(ctx->stream, cin, cout, in_dev, w_dev, (flags & CFP_NN_DGRAD) != 0, (uint16_t*)wpk,
@@ -1074,8 +1069,8 @@ cfp_status cfp_nn_conv3d_wgrad(cfp_ctx* ctx, int nx, int ny, int nz, int cin, in
     }
     const int64_t cap = (int64_t)num_sms() * 27 * cin * cout;
     void *part = nullptr, *bpart = nullptr;
-    CFP_CUDA(cudaMallocAsync(&part, cap * 4, ctx->stream));
-    CFP_CUDA(cudaMallocAsync(&bpart, kColBlocks * 128 * 4, ctx->stream));
+    CFP_CUDA(pool_malloc(&part, cap * 4, ctx->stream));
+    CFP_CUDA(pool_malloc(&bpart, kColBlocks * 128 * 4, ctx->stream));
     cfp_status st = wgrad_any(ctx->stream, cin, cout, in_dev, gout_dev, P, (float*)part, cap, dw_dev, db_dev,
                               (float*)bpart, ctx->dwait);
     cudaFreeAsync(part, ctx->stream);

@@ -13,15 +13,23 @@
 //     out[v][co] = bias[co] + sum_t sum_ci W[co][t][ci] in[v + off(t)][ci].
 //
 // Forward convolution (k_conv_tc): the implicit GEMM D (128 voxels x Cout) =
-// sum over taps of A_t (128 x Cin) B_t^T.  For each (dy, dz) pair one TMA
-// window of 130 rows (the 128 outputs and one row either side) serves the
-// three taps dx = -1, 0, 1, whose A operands start 0, 16 and 32 bytes into
-// it (K-major, no swizzle).  The weights of the three taps come with it, in
-// the operand layout (k_wpack).  The input gradient is the same kernel on
-// flipped, transposed weights.  Weight gradient (k_wgrad_tc): D_t (Cin x
+// sum over taps of A_t (128 x Cin) B_t^T.  For each (dy, dz) pair one window
+// of 130 rows (the 128 outputs and one row either side) serves the three taps
+// dx = -1, 0, 1, whose A operands start 0, 16 and 32 bytes into it (K-major,
+// no swizzle).  The weights of the three taps come with it, in the operand
+// layout (k_wpack), as one bulk copy.  The input gradient is the same kernel
+// on flipped, transposed weights.
+// The windows are copied by four producer warps with 16-byte cp.async: the
+// operand layout scatters a row's 8-channel pieces over planes, which the TMA
+// engine does 16 bytes at a time (about two cycles each: 2340 pieces per tile
+// bound the 16-channel layers to 5 % of the tensor pipe), while the copies of
+// 128 threads run at the shared-memory write rate.  Weight gradient (k_wgrad_tc): D_t (Cin x
 // Cout) = sum over voxels of X(v + off_t)^T G(v), both operands MN-major, the
-// voxel shift again a start-address offset; per-chunk partials are summed in
-// a fixed order (deterministic).
+// voxel shift again a start-address offset.  The windows of 128 / Cin (dy, dz)
+// pairs lie one after the other in a stage, so one MMA's 128 rows are that
+// many pairs' channels (with 16 channels a single pair would leave seven of
+// eight rows idle, and reading the operand is what an MMA of 16 columns
+// costs).  Per-chunk partials are summed in a fixed order (deterministic).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -39,10 +47,43 @@ struct Pad {
 
 enum { F_RELU = 1, F_MASK = 2, F_OUT_F32 = 4, F_ACCUM = 8 };
 
-constexpr int kWin = 130;             // rows of a TMA window: 128 outputs + one either side
-constexpr int kPlane = 136 * 16;      // bytes of one 8-channel plane of a window (128-byte multiple)
-constexpr int kGPlane = 128 * 16;     // bytes of one 8-channel plane of a 128-voxel gradient tile
-constexpr int kConvThreads = 192;     // warps 0-3 epilogue, 4 TMA producer, 5 MMA issuer
+constexpr int kWin = 130;             // rows of a window: 128 outputs + one either side
+// bytes of one 8-channel plane of a window / of a 128-voxel gradient tile: an
+// odd number of 16-byte rows, so that the pieces of a voxel row, written
+// together, fall into different banks
+constexpr int kPlane = 137 * 16;
+constexpr int kGPlane = 129 * 16;
+constexpr int kConvThreads = 288;     // warps 0-3 epilogue, 4-7 producers, 8 MMA issuer
+constexpr int kProd = 128;            // producer threads
+
+// 16 bytes global -> shared, asynchronous; zeros where ok is false (src is then
+// not read)
+__device__ __forceinline__ void copy16(unsigned dst, const void* src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+// one arrival on bar when every copy this thread has issued so far has landed.
+// The thread goes on to the next stage at once; the MMA thread, which waits on
+// bar, orders the copies before the tensor core's reads (async_after).  (With
+// the fence on the producer's side a stage took the whole latency of its
+// copies: the fence waits for the later stages' copies too.)
+__device__ __forceinline__ void copy_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void async_after() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// producer thread p's share of rows row0 .. row0 + nrows - 1 of an (Np x C)
+// activation, channels 8 c0 .. 8 c0 + 8 NPL - 1, into NPL planes of PLANE bytes;
+// rows outside [0, Np) become zeros
+template <int NPL, int PLANE>
+__device__ __forceinline__ void copy_rows(unsigned dst, const uint16_t* __restrict__ a, int C, int c0, int row0,
+                                          int nrows, int Np, int p) {
+#pragma unroll 4
+    for (int q = p; q < nrows * NPL; q += kProd) {
+        const int r = q / NPL, c = q % NPL, row = row0 + r;  // NPL is a power of two
+        const bool ok = row >= 0 && row < Np;
+        copy16(dst + c * PLANE + r * 16, a + (size_t)(ok ? row : 0) * C + 8 * (c0 + c), ok);
+    }
+}
 
 __host__ __device__ constexpr int pow2ceil(int v) {
     int p = 32;
@@ -74,11 +115,15 @@ struct ConvCfg {
     static constexpr int W_BYTES = 3 * W_TAP;
     static constexpr int STAGE = rup(A_BYTES + W_BYTES, 128);
     static constexpr int S0 = (196 * 1024) / STAGE;
-    static constexpr int STAGES = S0 < 2 ? 2 : (S0 > 8 ? 8 : S0);
+    static constexpr int STAGES = S0 > 8 ? 8 : S0;
+    static_assert(STAGES >= 2, "shared memory");
     static constexpr int SPT = 9 * NKB;             // stages per 128-voxel tile
     static constexpr int TCOLS = pow2ceil(2 * COUT);  // two accumulators
     static constexpr int SMEM = 128 + STAGES * STAGE + (2 * STAGES + 5) * 8 + 16;
-    static constexpr unsigned TX = NCH * kWin * 16 + W_BYTES;
+    // CTAs per SM: shared memory, tensor-memory columns and registers permitting, up to three
+    static constexpr int PER0 = (220 * 1024) / SMEM;
+    static constexpr int PER1 = 512 / TCOLS < PER0 ? 512 / TCOLS : PER0;
+    static constexpr int PER = PER1 < 1 ? 1 : PER1 > 3 ? 3 : PER1;
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 128, "channel counts");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
@@ -117,8 +162,8 @@ __global__ void k_wpack(const uint16_t* __restrict__ w, uint16_t* __restrict__ o
 // a code in *err and that role stops issuing; every issued copy and MMA is
 // waited for (bounded) before the tensor memory is released.
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kConvThreads, 1)
-    k_conv_tc(const __grid_constant__ CUtensorMap t_in, const uint16_t* __restrict__ wpk,
+__global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
+    k_conv_tc(const uint16_t* __restrict__ in, const uint16_t* __restrict__ wpk,
               const float* __restrict__ bias, const uint16_t* __restrict__ act, Pad P, int flags,
               uint16_t* __restrict__ out_bf, float* __restrict__ out_f, int* __restrict__ err) {
     using C = ConvCfg<CIN, COUT>;
@@ -134,7 +179,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int q = 0; q < S; ++q) {
-            tc::mbar_init(&full[q], 1);
+            tc::mbar_init(&full[q], 1 + kProd);  // the weights' bytes; the producer threads
             tc::mbar_init(&empty[q], 1);
         }
         for (int q = 0; q < 2; ++q) {
@@ -151,28 +196,35 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     const unsigned tmem = *tslot;
     const int ntiles = (P.Np + 127) / 128;
 
-    if (warp == 4 && lane == 0) {  // TMA producer
+    if (warp >= 4 && warp < 8) {  // producers
+        const int p = threadIdx.x - 128;
         unsigned g = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             for (int s = 0; s < C::SPT; ++s, ++g) {
                 const int kb = s / 9, gi = s % 9, st = g % S;
-                if (g >= S && !tc::mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
-                    ok = false;
+                int free = 1;
+                if (g >= S && lane == 0 && !tc::mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
+                    free = 0;
                     atomicExch(err, 11);
-                    break;
                 }
+                ok = __shfl_sync(0xffffffffu, free, 0);
+                if (!ok) break;
                 unsigned char* buf = base + st * C::STAGE;
-                tc::mbar_arrive_expect_tx(&full[st], C::TX);
+                if (p == 0) {
+                    tc::mbar_arrive_expect_tx(&full[st], C::W_BYTES);
+                    tc::bulk_load(buf + C::A_BYTES, wpk + (size_t)(kb * 9 + gi) * (C::W_BYTES / 2), C::W_BYTES, &full[st]);
+                }
                 const int row0 = tile * 128 + ((gi / 3 - 1) * P.nyp + (gi % 3 - 1)) * P.nxp - 1;
-#pragma unroll
-                for (int c = 0; c < C::NCH; ++c) tc::tma_load_2d(buf + c * kPlane, &t_in, &full[st], (kb * C::NCH + c) * 8, row0);
-                tc::bulk_load(buf + C::A_BYTES, wpk + (size_t)(kb * 9 + gi) * (C::W_BYTES / 2), C::W_BYTES, &full[st]);
+                copy_rows<C::NCH, kPlane>(tc::smem_u32(buf), in, CIN, kb * C::NCH, row0, kWin, P.Np, p);
+                copy_arrive(&full[st]);
             }
         }
-        for (unsigned q = g > (unsigned)S ? g - S : 0; q < g; ++q)
-            if (!tc::mbar_wait(&full[q % S], (q / S) & 1)) atomicExch(err, 12);
-    } else if (warp == 5 && lane == 0) {  // MMA issuer
+        copy_wait_all();
+        if (p == 0)  // every bulk copy issued has landed before the CTA may end
+            for (unsigned q = g > (unsigned)S ? g - S : 0; q < g; ++q)
+                if (!tc::mbar_wait(&full[q % S], (q / S) & 1)) atomicExch(err, 12);
+    } else if (warp == 8 && lane == 0) {  // MMA issuer
         constexpr unsigned idesc = tc::idesc_bf16(128, COUT, 0, 0);
         unsigned g = 0, tl = 0;
         bool ok = true;
@@ -192,6 +244,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
                     atomicExch(err, 14);
                     break;
                 }
+                async_after();
                 tc::fence_after();
                 const unsigned ab = tc::smem_u32(base + st * C::STAGE), wb = ab + C::A_BYTES;
 #pragma unroll
@@ -293,54 +346,56 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 // ------------------------------------------------------- weight gradient
 template <int CIN, int COUT>
 struct WgCfg {
-    static constexpr int NCA = CIN / 8;                    // planes of the X window
+    static constexpr int NCA = CIN / 8;                    // planes of one X window
     static constexpr int NCB = COUT / 8;                   // planes of the gradient tile
-    static constexpr int A_BYTES = NCA * kPlane;
+    static constexpr int GP = 16 / NCA;                    // (dy, dz) pairs of a unit: 128 rows of an MMA
+    static constexpr int NU = (9 + GP - 1) / GP;           // units of the nine pairs
+    static constexpr int A_BYTES = 16 * kPlane;
     static constexpr int B_BYTES = NCB * kGPlane;
     static constexpr int STAGE = rup(A_BYTES + B_BYTES, 128);
-    static constexpr int G0 = 512 / (3 * COUT);
-    static constexpr int GMAX = G0 > 9 ? 9 : G0;           // (dy, dz) pairs per CTA
-    static constexpr int NSETS = (9 + GMAX - 1) / GMAX;
-    static constexpr int TCOLS = pow2ceil(3 * GMAX * COUT);
-    // the MMA reads all 16 M planes of a window (128 rows; rows >= CIN are
-    // discarded): the space after the last stage is reserved for them
-    static constexpr int OVER = 16 * kPlane > STAGE ? 16 * kPlane - STAGE : 0;
-    static constexpr int S0 = (190 * 1024 - OVER) / STAGE;
-    static constexpr int STAGES = S0 < 2 ? 2 : (S0 > 8 ? 8 : S0);
-    static constexpr int SMEM0 = 128 + STAGES * STAGE + OVER + (2 * STAGES + 3) * 8 + 16;
-    // at least half an SM's shared memory: one CTA per SM, as it takes all
+    static constexpr int U0 = 512 / (3 * COUT);
+    static constexpr int UMAX = U0 > NU ? NU : U0;         // units per CTA
+    static constexpr int NSETS = (NU + UMAX - 1) / UMAX;
+    static constexpr int TCOLS = pow2ceil(3 * UMAX * COUT);
+    static constexpr int S0 = (200 * 1024) / STAGE;
+    static constexpr int STAGES = S0 > 8 ? 8 : S0;
+    static_assert(STAGES >= 2, "shared memory");
+    static constexpr int SMEM0 = 128 + STAGES * STAGE + (2 * STAGES + 3) * 8 + 16;
+    // at least half an SM's shared memory: one CTA per SM, as it may take all
     // 512 tensor-memory columns
     static constexpr int SMEM = SMEM0 > 116 * 1024 ? SMEM0 : 116 * 1024;
-    static constexpr unsigned TX = NCA * kWin * 16 + NCB * 128 * 16;
+    static_assert(CIN % 16 == 0 && CIN <= 128, "channel counts");
     static_assert(SMEM <= 227 * 1024, "shared memory");
     static_assert(TCOLS <= 512, "tensor memory");
 };
 
-// Partial weight gradient of one voxel chunk and one set of (dy, dz) pairs:
+// Partial weight gradient of one voxel chunk and one set of units:
 // part[chunk][t][ci][co] = sum over the chunk's 128-voxel tiles of
 // X[v + off(t)][ci] G[v][co].  Grid: (NSETS, nchunks); chunk q owns tiles
-// [q * tpc, min((q + 1) * tpc, ntiles)).
+// [q * tpc, min((q + 1) * tpc, ntiles)).  A stage holds one tile's windows of
+// one unit and its gradient tile; the rows of an MMA past the ninth pair are
+// whatever the stage holds there, and are not read back.
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kConvThreads, 1)
-    k_wgrad_tc(const __grid_constant__ CUtensorMap t_x, const __grid_constant__ CUtensorMap t_g, Pad P, int tpc,
+    k_wgrad_tc(const uint16_t* __restrict__ x, const uint16_t* __restrict__ gr, Pad P, int tpc,
                float* __restrict__ part, int* __restrict__ err) {
     using C = WgCfg<CIN, COUT>;
     constexpr int S = C::STAGES;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-    uint64_t* full = (uint64_t*)(base + S * C::STAGE + C::OVER);
+    uint64_t* full = (uint64_t*)(base + S * C::STAGE);
     uint64_t* empty = full + S;
     uint64_t* accf = empty + S;
     uint64_t* fin = accf + 1;
     unsigned* tslot = (unsigned*)(fin + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int set = blockIdx.x, chunk = blockIdx.y;
-    const int g0 = set * C::GMAX, g1 = min(9, g0 + C::GMAX), ng = g1 - g0;
+    const int u0 = set * C::UMAX, nu = min(C::NU - u0, C::UMAX);
     const int ntiles = (P.Np + 127) / 128;
     const int t0 = chunk * tpc, t1 = min(ntiles, t0 + tpc);
     if (threadIdx.x == 0) {
         for (int q = 0; q < S; ++q) {
-            tc::mbar_init(&full[q], 1);
+            tc::mbar_init(&full[q], kProd);
             tc::mbar_init(&empty[q], 1);
         }
         tc::mbar_init(accf, 1);
@@ -352,41 +407,46 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     __syncthreads();
     tc::fence_after();
     const unsigned tmem = *tslot;
-    const int nst = (t1 > t0 ? t1 - t0 : 0) * ng;
+    const int nst = (t1 > t0 ? t1 - t0 : 0) * nu;
 
-    if (warp == 4 && lane == 0) {  // TMA producer
+    if (warp >= 4 && warp < 8) {  // producers
+        const int p = threadIdx.x - 128;
         unsigned g = 0;
         for (; (int)g < nst; ++g) {
-            const int tile = t0 + (int)g / ng, gi = g0 + (int)g % ng, st = g % S;
-            if (g >= (unsigned)S && !tc::mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
+            const int tile = t0 + (int)g / nu, u = u0 + (int)g % nu, st = g % S;
+            int free = 1;
+            if (g >= (unsigned)S && lane == 0 && !tc::mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
+                free = 0;
                 atomicExch(err, 21);
-                break;
             }
-            unsigned char* buf = base + st * C::STAGE;
-            tc::mbar_arrive_expect_tx(&full[st], C::TX);
-            const int row0 = tile * 128 + ((gi / 3 - 1) * P.nyp + (gi % 3 - 1)) * P.nxp - 1;
+            if (!__shfl_sync(0xffffffffu, free, 0)) break;
+            const unsigned buf = tc::smem_u32(base + st * C::STAGE);
 #pragma unroll
-            for (int c = 0; c < C::NCA; ++c) tc::tma_load_2d(buf + c * kPlane, &t_x, &full[st], 8 * c, row0);
-#pragma unroll
-            for (int c = 0; c < C::NCB; ++c)
-                tc::tma_load_2d(buf + C::A_BYTES + c * kGPlane, &t_g, &full[st], 8 * c, tile * 128);
+            for (int q = 0; q < C::GP; ++q) {
+                const int gi = u * C::GP + q;
+                if (gi < 9)
+                    copy_rows<C::NCA, kPlane>(buf + q * C::NCA * kPlane, x, CIN, 0,
+                                              tile * 128 + ((gi / 3 - 1) * P.nyp + (gi % 3 - 1)) * P.nxp - 1, kWin, P.Np, p);
+            }
+            copy_rows<C::NCB, kGPlane>(buf + C::A_BYTES, gr, COUT, 0, tile * 128, 128, P.Np, p);
+            copy_arrive(&full[st]);
         }
-        for (unsigned q = g > (unsigned)S ? g - S : 0; q < g; ++q)
-            if (!tc::mbar_wait(&full[q % S], (q / S) & 1)) atomicExch(err, 22);
-    } else if (warp == 5 && lane == 0) {  // MMA issuer
+        copy_wait_all();
+    } else if (warp == 8 && lane == 0) {  // MMA issuer
         constexpr unsigned idesc = tc::idesc_bf16(128, COUT, 1, 1);
         for (int g = 0; g < nst; ++g) {
-            const int st = g % S, first = g < ng;  // the chunk's first tile: the accumulators start
-            const int gl = g % ng;
+            const int st = g % S, first = g < nu;  // the chunk's first tile: the accumulators start
+            const int ul = g % nu;
             if (!tc::mbar_wait(&full[st], (g / S) & 1)) {
                 atomicExch(err, 23);
                 break;
             }
+            async_after();
             tc::fence_after();
             const unsigned ab = tc::smem_u32(base + st * C::STAGE), bb = ab + C::A_BYTES;
 #pragma unroll
             for (int dx = 0; dx < 3; ++dx) {
-                const unsigned d = tmem + (unsigned)((gl * 3 + dx) * COUT);
+                const unsigned d = tmem + (unsigned)((ul * 3 + dx) * COUT);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const uint64_t da = tc::sdesc(ab + dx * 16 + q * 256, 128, kPlane);
@@ -399,7 +459,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         tc::mma_commit(accf);
         tc::mma_commit(fin);
         if (!tc::mbar_wait(fin, 0)) atomicExch(err, 24);
-    } else if (warp < 4 && 32 * warp < CIN) {  // epilogue: lane = input channel
+    } else if (warp < 4) {  // epilogue: row 32 warp + lane is channel ci of pair `pair` of a unit
         int ok = 1;
         if (nst > 0) {
             if (lane == 0 && !tc::mbar_wait(accf, 0)) {
@@ -410,15 +470,15 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         }
         if (ok) {
             tc::fence_after();
-            const int ci = 32 * warp + lane;
-            for (int gl = 0; gl < ng; ++gl)
+            const int row = 32 * warp + lane, pair = row / CIN, ci = row % CIN;
+            for (int ul = 0; ul < nu; ++ul)
                 for (int dx = 0; dx < 3; ++dx) {
-                    const int t = 3 * (g0 + gl) + dx;
+                    const int gi = (u0 + ul) * C::GP + pair, t = 3 * gi + dx;
 #pragma unroll 1
                     for (int c16 = 0; c16 < COUT / 16; ++c16) {
                         float v[16];
-                        tc::tmem_ld16(tmem + ((unsigned)(32 * warp) << 16) + (unsigned)((gl * 3 + dx) * COUT + 16 * c16), v);
-                        if (ci < CIN) {
+                        tc::tmem_ld16(tmem + ((unsigned)(32 * warp) << 16) + (unsigned)((ul * 3 + dx) * COUT + 16 * c16), v);
+                        if (gi < 9) {
                             float4* op = reinterpret_cast<float4*>(
                                 part + (((size_t)chunk * 27 + t) * CIN + ci) * COUT + 16 * c16);
 #pragma unroll
