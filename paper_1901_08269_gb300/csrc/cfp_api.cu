@@ -161,7 +161,7 @@ cfp_status cfp_ctx_create(const double* x, int nx, const double* y, int ny, cons
     chk(cudaMalloc(&c->dwait, sizeof(int)), "cudaMalloc");
     if (c->dwait) chk(cudaMemsetAsync(c->dwait, 0, sizeof(int), c->stream), "cudaMemsetAsync");
     chk(cudaMalloc(&c->kst, sizeof(KState) * 2), "cudaMalloc");
-    chk(cudaMallocHost(&c->hkst, sizeof(KState) * 2), "cudaMallocHost");
+    chk(cudaMallocHost(&c->hkst, sizeof(KState) * 3), "cudaMallocHost");
     chk(cudaMalloc(&c->rst, sizeof(RState)), "cudaMalloc");
     chk(cudaMallocHost(&c->hrst, sizeof(RState)), "cudaMallocHost");
     for (int q = 0; q < 3; ++q) {

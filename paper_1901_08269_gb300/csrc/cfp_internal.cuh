@@ -266,7 +266,7 @@ struct cfp_ctx {
     double* partial = nullptr;
     int64_t partial_cap = 0;
     cfp::KState* kst = nullptr;   // [0]: FP64 run, [1]: FP32 run
-    cfp::KState* hkst = nullptr;  // pinned host mirror
+    cfp::KState* hkst = nullptr;  // pinned host mirror; a third entry receives dwait
     cfp::RState* rst = nullptr;   // device-driven refinement loop
     cfp::RState* hrst = nullptr;  // pinned host mirror
 

@@ -557,9 +557,11 @@ int mg_key(const cfp_ctx* c) {
 }
 
 cfp_status check_waits(cfp_ctx* c) {
-    int w = 0;
-    CFP_CUDA(cudaMemcpyAsync(&w, c->dwait, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    // through page-locked memory: a copy to the stack is staged by the driver
+    int* hw = reinterpret_cast<int*>(c->hkst + 2);
+    CFP_CUDA(cudaMemcpyAsync(hw, c->dwait, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CFP_CUDA(cudaStreamSynchronize(c->stream));
+    const int w = *hw;
     if (w == 0) return CFP_OK;
     CFP_CUDA(cudaMemsetAsync(c->dwait, 0, sizeof(int), c->stream));
     CFP_CUDA(cudaStreamSynchronize(c->stream));
