@@ -124,10 +124,12 @@ __device__ int body_sign32(const Body32& b, float x, float y, float z) {
 // lie inside its bounding sphere (outside it phi > 0 holds with a margin far
 // above rounding); that test runs in FP32 against a threshold above the
 // FP32 squared distance of every point within the sphere (set on the host
-// from a bound on the rounding), so it skips only points outside.
-__device__ bool node_solid(const GeoArgs& g, double x, double y, double z) {
+// from a bound on the rounding), so it skips only points outside.  far: bits
+// of bodies (of the first 32) known to lie outside their spheres.
+__device__ bool node_solid(const GeoArgs& g, double x, double y, double z, unsigned far = 0) {
     const float xf = (float)x, yf = (float)y, zf = (float)z;
     for (int m = 0; m < g.nb; ++m) {
+        if (m < 32 && (far >> m & 1)) continue;
         const Body32& b = g.b32[m];
         if (!g.inside) {
             const float dx = __fsub_rn(xf, b.c[0]), dy = __fsub_rn(yf, b.c[1]), dz = __fsub_rn(zf, b.c[2]);
@@ -145,20 +147,34 @@ __device__ bool node_solid(const GeoArgs& g, double x, double y, double z) {
 }
 
 // ------------------------------------------------------------ classification
-__global__ void k_classify_solid(GeoArgs g, uint8_t* type, int64_t N) {
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < N;
-         l += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(l % nx);
-        const int j = (int)((l / nx) % ny);
-        const int k = (int)(l / ((int64_t)nx * ny));
-        uint8_t t;
-        if (i == 0 || j == 0 || k == 0 || i == nx - 1 || j == ny - 1 || k == nz - 1) {
-            t = CFP_BOUNDARY;
-        } else {
-            t = node_solid(g, g.X[0][i], g.X[1][j], g.X[2][k]) ? CFP_SOLID : CFP_REGULAR;
+// One warp per grid row (j, k) at a time.  A body whose sphere the row's line
+// misses is left out for the whole row: the FP32 squared distance of each of
+// its nodes is at least the rounded dy^2 + dz^2 (rounding is monotone), so the
+// node's own test would skip it too.  Most rows meet no body and are only
+// written.  (Per node, with its 64-bit divisions: 0.80 ms at 513^3, now 0.27.)
+__global__ void __launch_bounds__(256) k_classify_solid(GeoArgs g, uint8_t* type, int nrows) {
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], lane = threadIdx.x & 31;
+    for (int row = (blockIdx.x * 256 + threadIdx.x) >> 5; row < nrows; row += (gridDim.x * 256) >> 5) {
+        const int k = row / ny, j = row - k * ny;
+        uint8_t* t = type + (int64_t)row * nx;
+        const bool edge = j == 0 || k == 0 || j == ny - 1 || k == nz - 1;
+        const double y = g.X[1][j], z = g.X[2][k];
+        unsigned far = 0;
+        if (!g.inside) {
+            const float yf = (float)y, zf = (float)z;
+            for (int m = 0; m < min(g.nb, 32); ++m) {
+                const Body32& b = g.b32[m];
+                const float dy = __fsub_rn(yf, b.c[1]), dz = __fsub_rn(zf, b.c[2]);
+                if (__fadd_rn(__fmul_rn(dy, dy), __fmul_rn(dz, dz)) > b.thr) far |= 1u << m;
+            }
         }
-        type[l] = t;
+        const bool none = !g.inside && g.nb <= 32 && far == (g.nb == 32 ? ~0u : (1u << g.nb) - 1u);
+        for (int i = lane; i < nx; i += 32) {
+            uint8_t v = CFP_REGULAR;
+            if (edge || i == 0 || i == nx - 1) v = CFP_BOUNDARY;
+            else if (!none && node_solid(g, g.X[0][i], y, z, far)) v = CFP_SOLID;
+            t[i] = v;
+        }
     }
 }
 
@@ -174,6 +190,7 @@ __global__ void k_classify_solid(GeoArgs g, uint8_t* type, int64_t N) {
 // race.
 constexpr int kIrrPlanes = 16;  // planes per thread
 constexpr int kIrrWarps = 8;    // warps per block
+constexpr int kIrrBatch = 8;    // planes loaded at a time
 
 __global__ void __launch_bounds__(32 * kIrrWarps) k_classify_irregular(uint8_t* type, int nx, int ny, int nz) {
     const int lane = threadIdx.x & 31;
@@ -185,26 +202,37 @@ __global__ void __launch_bounds__(32 * kIrrWarps) k_classify_irregular(uint8_t* 
     const int64_t row = (int64_t)nx;
     uint8_t* col = type + ((int64_t)j * nx + (inx ? i : 0));  // node (i, j) of plane 0
     const int64_t pl = (int64_t)nx * ny;
-    // the dilated solid flag of plane k at (i, j), and the node's own type
-    auto dil = [&](int k, uint8_t& own) -> bool {
-        bool s = false;
-        own = CFP_SOLID;
-        if (inx) {
-            const uint8_t* c = col + k * pl;
-            own = c[0];
-            s = c[-row] == CFP_SOLID || own == CFP_SOLID || c[row] == CFP_SOLID;
-        }
-        const unsigned b = s ? 1u : 0u;
-        return (b | __shfl_up_sync(0xffffffffu, b, 1) | __shfl_down_sync(0xffffffffu, b, 1)) != 0u;
+    // a plane's three types at (i, j - 1 .. j + 1), and from them the dilated
+    // solid flag at (i, j)
+    auto dil = [&](uint8_t a, uint8_t own, uint8_t b) -> bool {
+        const unsigned f = inx && (a == CFP_SOLID || own == CFP_SOLID || b == CFP_SOLID) ? 1u : 0u;
+        return (f | __shfl_up_sync(0xffffffffu, f, 1) | __shfl_down_sync(0xffffffffu, f, 1)) != 0u;
     };
-    uint8_t tm, t0, tp;
-    bool dm = dil(k0 - 1, tm), d0 = dil(k0, t0);
-    for (int k = k0; k < k1; ++k) {
-        const bool dp = dil(k + 1, tp);
-        if (mine && t0 == CFP_REGULAR && (dm || d0 || dp)) col[k * pl] = CFP_IRREGULAR;
-        dm = d0;
-        d0 = dp;
-        t0 = tp;
+    const uint8_t* c0 = col + (k0 - 1) * pl;
+    const uint8_t* c1 = col + k0 * pl;
+    uint8_t t0 = c1[0];
+    bool dm = dil(c0[-row], c0[0], c0[row]), d0 = dil(c1[-row], t0, c1[row]);
+    // the loads of kIrrBatch planes before any of their stores, which the
+    // compiler must take for possible overwrites of what is still to be read
+    for (int kb = k0; kb < k1; kb += kIrrBatch) {
+        uint8_t a[kIrrBatch], own[kIrrBatch], b[kIrrBatch];
+#pragma unroll
+        for (int q = 0; q < kIrrBatch; ++q) {
+            const uint8_t* c = col + min(kb + 1 + q, nz - 1) * pl;
+            a[q] = c[-row];
+            own[q] = c[0];
+            b[q] = c[row];
+        }
+#pragma unroll
+        for (int q = 0; q < kIrrBatch; ++q) {
+            const int k = kb + q;
+            if (k >= k1) break;
+            const bool dp = dil(a[q], own[q], b[q]);
+            if (mine && t0 == CFP_REGULAR && (dm || d0 || dp)) col[k * pl] = CFP_IRREGULAR;
+            dm = d0;
+            d0 = dp;
+            t0 = own[q];
+        }
     }
 }
 
@@ -237,21 +265,9 @@ __device__ int block_excl_scan(int v, int* total) {
     return before + x - v;
 }
 
-struct FlagIrregular {
-    const uint8_t* type;
-    __device__ int operator()(int64_t i) const { return type[i] == CFP_IRREGULAR; }
-};
 struct FetchInt {
     const int* a;
     __device__ int operator()(int64_t i) const { return a[i]; }
-};
-struct SinkSlots {
-    int32_t* slot;
-    int32_t* irr_lin;
-    __device__ void operator()(int64_t i, int off, int v) const {
-        slot[i] = v ? off : -1;
-        if (v) irr_lin[off] = (int32_t)i;
-    }
 };
 struct SinkOffsets {
     int32_t* out;
@@ -306,6 +322,64 @@ __global__ void k_scan_scatter(F f, S sink, int64_t n, const int* boff) {
             sink(base + q, off, v[q]);
             off += v[q];
         }
+    }
+}
+
+// The irregular nodes' list and slots, in ascending index: 16 bytes of types per
+// load, kListLoads loads per thread, the flags of a chunk counted and, with the
+// chunks' offsets, stored.  The slot array is -1 everywhere else (set before).
+constexpr int kListLoads = 4;
+constexpr int kListChunk = kScanThreads * 16 * kListLoads;
+
+// bit b: byte b of the 16 types at node l0 (a multiple of 16) is irregular
+__device__ __forceinline__ unsigned irregular_bits(const uint8_t* type, int64_t l0, int64_t N) {
+    unsigned m = 0;
+    if (l0 + 16 <= N) {
+        const uint4 v = *reinterpret_cast<const uint4*>(type + l0);
+        const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned e = __vcmpeq4(w[q], 0x01010101u * CFP_IRREGULAR) & 0x08040201u;
+            m |= ((e | e >> 8 | e >> 16 | e >> 24) & 15u) << (4 * q);
+        }
+    } else {
+        for (int q = 0; q < 16; ++q)
+            if (l0 + q < N && type[l0 + q] == CFP_IRREGULAR) m |= 1u << q;
+    }
+    return m;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_list_count(const uint8_t* __restrict__ type, int64_t N, int* bsum) {
+    const int64_t base = (int64_t)blockIdx.x * kListChunk;
+    int s = 0;
+#pragma unroll
+    for (int q = 0; q < kListLoads; ++q)
+        s += __popc(irregular_bits(type, base + 16 * (int64_t)(q * kScanThreads + threadIdx.x), N));
+    int tot;
+    block_excl_scan(s, &tot);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
+}
+
+__global__ void __launch_bounds__(kScanThreads)
+    k_list_store(const uint8_t* __restrict__ type, int64_t N, const int* __restrict__ boff, int32_t* __restrict__ slot,
+                 int32_t* __restrict__ irr_lin) {
+    const int64_t base = (int64_t)blockIdx.x * kListChunk;
+    int off = boff[blockIdx.x];
+    unsigned m[kListLoads];
+#pragma unroll
+    for (int q = 0; q < kListLoads; ++q)
+        m[q] = irregular_bits(type, base + 16 * (int64_t)(q * kScanThreads + threadIdx.x), N);
+#pragma unroll
+    for (int q = 0; q < kListLoads; ++q) {
+        int tot;
+        int at = off + block_excl_scan(__popc(m[q]), &tot);
+        const int64_t l0 = base + 16 * (int64_t)(q * kScanThreads + threadIdx.x);
+        for (unsigned f = m[q]; f; f &= f - 1, ++at) {
+            const int64_t l = l0 + __ffs(f) - 1;
+            slot[l] = at;
+            irr_lin[at] = (int32_t)l;
+        }
+        off += tot;
     }
 }
 
@@ -364,7 +438,11 @@ __global__ void k_ibi_count(IrrArgs a, int* cnt) {
 // bisection steps; the solid end of the last bracket is returned.  Only the
 // sign of phi decides each step, so node_solid (which skips bodies whose
 // bounding sphere excludes the point, those have phi > 0) gives the same
-// decisions as the full union of the bodies.
+// decisions as the full union of the bodies.  And the sign depends on the
+// coordinate alone, so a midpoint whose coordinate rounds to an end's takes
+// that end's sign (a cell is far shorter than its distance from the origin,
+// so the coordinate's resolution runs out before t's), and once the midpoint
+// is an end itself the remaining steps change nothing (513^3: 2.30 -> 2.05 ms).
 __device__ double ibi_root(const GeoArgs& g, int d, const double pa[3], double xb) {
     double q[3] = {pa[0], pa[1], pa[2]};
     double lo = 0.0, hi = 1.0;
@@ -377,11 +455,23 @@ __device__ double ibi_root(const GeoArgs& g, int d, const double pa[3], double x
         }
         lo = ts;
     }
+    // the ends' coordinates, where their signs are known: fluid at lo > 0,
+    // solid at hi < 1 (t = 0 and 1 are the nodes, evaluated from their own
+    // coordinates); NaN compares unequal
+    double xlo = lo > 0.0 ? edge_pos(pa[d], xb, lo) : nan("");
+    double xhi = hi < 1.0 ? edge_pos(pa[d], xb, hi) : nan("");
     for (int it = 0; it < 60; ++it) {
         const double mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
+        if (mid == lo || mid == hi) break;
         q[d] = edge_pos(pa[d], xb, mid);
-        if (!node_solid(g, q[0], q[1], q[2])) lo = mid;
-        else hi = mid;
+        const bool solid = q[d] == xhi || (q[d] != xlo && node_solid(g, q[0], q[1], q[2]));
+        if (!solid) {
+            lo = mid;
+            xlo = q[d];
+        } else {
+            hi = mid;
+            xhi = q[d];
+        }
     }
     return hi;
 }
@@ -423,35 +513,6 @@ __global__ void k_ibi_roots(IrrArgs a, GeoArgs g, const int32_t* src, int64_t n_
 // ------------------------------------------------------------- side list
 constexpr int kMaxRaw = 320;   // correction adds per row before merging (27 lines x <= 11)
 constexpr int kMaxBib = 64;
-
-// Correction adds of one row, appended in order to the row's slice of the
-// global scratch (no merging here: k_side_merge merges them afterwards).
-struct RawAcc {
-    int n;
-    int32_t* off;
-    double* val;
-    __device__ bool add(int o, double v) {
-        if (n == kMaxRaw) return false;
-        off[n] = o;
-        val[n] = v;
-        ++n;
-        return true;
-    }
-};
-
-// IBI weights of one row, appended to its scratch slice.
-struct BibAcc {
-    int n;
-    int32_t* idx;
-    double* val;
-    __device__ bool add(int i, double v) {
-        if (n == kMaxBib) return false;
-        idx[n] = i;
-        val[n] = v;
-        ++n;
-        return true;
-    }
-};
 
 struct SideArgs {
     IrrArgs a;
@@ -669,13 +730,6 @@ __device__ void op_walk(const SideArgs& S, const Line& ln, const OpSpec& o, int6
     W.deg = W.ng < o.G || W.nib > 1;
 }
 
-// An operator whose moments are still to be matched: the slot of its
-// point, its line and operator index (code = 2 L + k), and where its
-// correction adds and IBI weights go in the point's scratch slices.
-struct SideTask {
-    int slot, code, cpos, bpos;
-};
-
 // The first error of a row in the order of its lines, operators and steps:
 // key (2 L + k) x 4 + step (0: the R subtraction overflows the slice; 1:
 // the walk fails; 2: the moment matrix is singular; 3: the operator's adds
@@ -686,112 +740,250 @@ __device__ __forceinline__ int side_err(int L, int k, int step, int detail) {
 }
 constexpr int kSideNoErr = 0x7fffffff;
 
-// Plans the row of every irregular point (one thread per point), walking its
-// 27 lines in order up to its first error: the R subtraction of every line
-// with a solid node (Eq. cor: minus the regular R operator at the line's
-// fluid nodes) and the walk of its modified operator(s).  COUNT: only the
-// number of operators; otherwise the R subtraction's adds are stored, each
-// operator becomes a task at its place (task_off[s] onwards) with the
-// positions of its adds, and the row's counts, first error and degenerate
-// operators are kept for k_side_finish.
-template <bool COUNT>
-__global__ void __launch_bounds__(128) k_side_plan(SideArgs S, int* ntask, const int* task_off, SideTask* tasks,
-                                                   int* ccount, int* bcount, int* ferr, int* ndegs, int32_t* toff,
-                                                   double* tval) {
+// The modified operators.  Whichever of up to nine rows a line belongs to,
+// its operator has the same points and moments, and it is known by the IBI
+// next to its expansion node and by whether it expands about the line's
+// centre: so each is solved once per IBI and kind (2 n_ibi solves instead of
+// about five times as many, 2.5 ms at 513^3 now 0.6), and the rows scale it
+// by their line's weight.  kind 0: the line's centre is the fluid node (masks
+// 1, 4, 5); kind 1: the centre is the solid node (masks 2, 3, 6).
+struct __align__(16) OpRec {
+    double cc[6];  // weights of the ng grid nodes along the walk, then of the nib IBIs
+    int ib2;       // the second IBI (nib = 2)
+    int8_t ng, nib, flags, err;  // flags: kOpDegenerate, kOpSingular; err: the walk's error detail
+};
+enum { kOpDegenerate = 1, kOpSingular = 2 };
+
+// the line through the centre of IBI code's operator of `kind`, and the
+// operator's index on it; false: such a line has another operator there
+__device__ bool op_line(const SideArgs& S, const int idx[3], int dir, int kind, Line& ln, int& k) {
     const int nx = S.a.n[0], ny = S.a.n[1];
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < S.a.n_irr;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t lin = S.a.irr_lin[s];
+    const int64_t st[3] = {1, nx, (int64_t)nx * ny};
+    const int d = dir >> 1, side = (dir & 1) ? 1 : -1;  // the solid neighbour's side
+    ln.d = d;
+    ln.base[0] = idx[0];
+    ln.base[1] = idx[1];
+    ln.base[2] = idx[2];
+    if (kind) ln.base[d] += side;
+    ln.m = ln.base[d];
+    ln.a = S.ax[d].a[ln.m];
+    ln.c = S.ax[d].c[ln.m];
+    ln.w = 1.0;
+    ln.bl = lin3(ln.base[0], ln.base[1], ln.base[2], nx, ny);
+    int mask = 0;
+    for (int s = -1; s <= 1; ++s) mask = (mask << 1) | (S.a.type[ln.bl + s * st[d]] == CFP_SOLID);
+    ln.mask = mask;
+    k = mask == 2 && side < 0 ? 1 : 0;  // the solid middle node's second operator lies on its +1 side
+    return !(mask == 5 && side < 0);    // between two solid nodes: one operator, walking away from the +1 side
+}
+
+__global__ void __launch_bounds__(64) k_side_ops(SideArgs S, const int32_t* __restrict__ src, int64_t n_ibi,
+                                                 OpRec* __restrict__ ops) {
+    const int nx = S.a.n[0], ny = S.a.n[1];
+    const int64_t st[3] = {1, nx, (int64_t)nx * ny};
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 2 * n_ibi;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int kind = t >= n_ibi;  // a warp's operators are of one kind
+        const int64_t m = t - kind * n_ibi;
+        const int32_t code = src[m];
+        const int64_t lin = S.a.irr_lin[code >> 3];
         const int idx[3] = {(int)(lin % nx), (int)((lin / nx) % ny), (int)(lin / ((int64_t)nx * ny))};
-        const int64_t st[3] = {1, nx, (int64_t)nx * ny};
-        int cn = 0, bn = 0, nt = 0, ndeg = 0, err = kSideNoErr;
-        const int t0 = COUNT ? 0 : task_off[s];
-        for (int L = 0; L < 27 && err == kSideNoErr; ++L) {
-            Line ln;
-            line_at(S, idx, st, L, ln);
-            if (ln.mask == 0 || ln.mask == 7) continue;  // regular or dropped line
-            for (int q = -1; q <= 1 && err == kSideNoErr; ++q)
-                if (!((ln.mask >> (1 - q)) & 1)) {
-                    if (cn == kMaxRaw) {
-                        err = side_err(L, 0, 0, DETAIL_OVERFLOW);
-                        break;
-                    }
-                    if (!COUNT) {
-                        toff[s * kMaxRaw + cn] = (int32_t)(ln.bl + q * st[ln.d] - lin);
-                        tval[s * kMaxRaw + cn] = -ln.w * Rc(S.ax[ln.d], ln.m, q);
-                    }
-                    ++cn;
-                }
-            for (int k = 0; k < line_nops(ln.mask) && err == kSideNoErr; ++k) {
-                const OpSpec o = op_spec(ln.mask, k, ln.a, ln.c);
-                OpWalk W;
-                op_walk(S, ln, o, lin, st, W);
-                if (W.err) {
-                    err = side_err(L, k, 1, W.err);
-                    break;
-                }
-                ndeg += W.deg ? 1 : 0;
-                if (!COUNT) tasks[t0 + nt] = SideTask{(int)s, 2 * L + k, cn, bn};
-                ++nt;
-                cn += W.ng;
-                bn += W.nib;
-                // adds past the slice: the operator still runs, for a singular
-                // matrix comes first, but stores nothing
-                if (cn > kMaxRaw || bn > kMaxBib) err = side_err(L, k, 3, DETAIL_OVERFLOW);
+        OpRec R = {};
+        Line ln;
+        int k;
+        if (op_line(S, idx, code & 7, kind, ln, k)) {
+            const OpSpec o = op_spec(ln.mask, k, ln.a, ln.c);
+            OpWalk W;
+            op_walk(S, ln, o, lin, st, W);
+            R.err = (int8_t)W.err;
+            if (!W.err) {
+                const int d = ln.d, ng = W.ng, nib = W.nib, M = ng + nib;
+                R.ng = (int8_t)ng;
+                R.nib = (int8_t)nib;
+                R.ib2 = nib > 1 ? W.ib[1] : -1;
+                if (W.deg) R.flags |= kOpDegenerate;
+                for (int q = 0; q < nib; ++q) W.xi[ng + q] = S.ibi_xyz[3 * (int64_t)W.ib[q] + d];
+                const double xe = S.X[d][ln.base[d] + o.e];
+                double xs[2];
+                for (int q = 0; q < o.ns; ++q) xs[q] = S.X[d][ln.base[d] + o.surv[q]];
+                double hs = 0.0;
+                for (int q = 1; q < M; ++q) hs = fmax(hs, fabs(W.xi[q] - xe));
+                if (!moment_solve(M, W.xi, xe, o.ns, xs, o.Ls, hs, R.cc)) R.flags |= kOpSingular;
             }
         }
-        if (COUNT) {
-            ntask[s] = nt;
-        } else {
-            ccount[s] = cn;
-            bcount[s] = bn;
-            ferr[s] = err;
-            ndegs[s] = ndeg;
-        }
+        ops[2 * m + kind] = R;
     }
 }
 
-// One modified operator per thread: its walk again, the moment matching of
-// Eqs. mat1-mat4 (matrix M of Eq. M), and its correction adds and IBI
-// weights (script B of Eq. bc), scaled by the line's weight, at the places
-// k_side_plan gave them.
-__global__ void __launch_bounds__(64) k_side_solve(SideArgs S, const SideTask* tasks, int64_t ntasks, int* ferr,
-                                                   int32_t* toff, double* tval, int32_t* tbidx, double* tbval) {
-    const int nx = S.a.n[0], ny = S.a.n[1];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ntasks;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const SideTask T = tasks[t];
-        const int64_t s = T.slot;
-        const int L = T.code >> 1, k = T.code & 1;
+// The row of every irregular point, one warp a row and one lane a line (27 of
+// 32): the R subtraction of every line with a solid node (Eq. cor: minus the
+// regular R operator at the line's fluid nodes), then its modified operators'
+// weights times the line's (Eqs. mat1-mat4; script B of Eq. bc), at places
+// that a scan over the lanes gives in the order of lines, operators and nodes.
+// The adds are then merged in shared memory, 32 at a time and in their order:
+// an offset seen before adds its value to that entry, a new one opens the next
+// entry (the order of first appearance), through an open-addressing index
+// (kMergeSlots > kMaxRaw, so an empty slot always exists).
+constexpr int kRowWarps = 4;
+constexpr int kMergeSlots = 512;
+
+__global__ void __launch_bounds__(32 * kRowWarps)
+    k_side_rows(SideArgs S, const OpRec* __restrict__ ops, int* ccount, int* bcount, int* ferr, int* ndegs,
+                int32_t* toff, double* tval, int32_t* tbidx, double* tbval) {
+    __shared__ double sval_[kRowWarps][kMaxRaw];
+    __shared__ int32_t soff_[kRowWarps][kMaxRaw];
+    __shared__ int sslot_[kRowWarps][kMergeSlots];
+    const unsigned all = 0xffffffffu;
+    const int nx = S.a.n[0], ny = S.a.n[1], lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    double* sval = sval_[wl];
+    int32_t* soff = soff_[wl];
+    int* sslot = sslot_[wl];
+    const int64_t st[3] = {1, nx, (int64_t)nx * ny};
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t s = warp; s < S.a.n_irr; s += nwarps) {
         const int64_t lin = S.a.irr_lin[s];
         const int idx[3] = {(int)(lin % nx), (int)((lin / nx) % ny), (int)(lin / ((int64_t)nx * ny))};
-        const int64_t st[3] = {1, nx, (int64_t)nx * ny};
+        for (int q = lane; q < kMergeSlots; q += 32) sslot[q] = 0;
+        // the lane's line: its adds, its operators, its first error
         Line ln;
-        line_at(S, idx, st, L, ln);
-        const OpSpec o = op_spec(ln.mask, k, ln.a, ln.c);
-        OpWalk W;
-        op_walk(S, ln, o, lin, st, W);
-        const int d = ln.d, ng = W.ng, nib = W.nib, M = ng + nib;
-        for (int q = 0; q < nib; ++q) W.xi[ng + q] = S.ibi_xyz[3 * (int64_t)W.ib[q] + d];
-        const double xe = S.X[d][ln.base[d] + o.e];
-        double xs[2];
-        for (int q = 0; q < o.ns; ++q) xs[q] = S.X[d][ln.base[d] + o.surv[q]];
-        double hs = 0.0;
-        for (int q = 1; q < M; ++q) hs = fmax(hs, fabs(W.xi[q] - xe));
-        double cc[7];
-        if (!moment_solve(M, W.xi, xe, o.ns, xs, o.Ls, hs, cc)) {
-            atomicMin(&ferr[s], side_err(L, k, 2, DETAIL_SINGULAR));
-            continue;
+        ln.mask = 0;
+        if (lane < 27) line_at(S, idx, st, lane, ln);
+        const bool mod = ln.mask != 0 && ln.mask != 7;
+        int nr = 0, nop = 0, cn = 0, bn = 0, ndeg = 0, err = kSideNoErr;
+        int ib[2] = {-1, -1}, kind[2] = {0, 0}, ng[2] = {0, 0}, nib[2] = {0, 0};
+        int64_t fl[2] = {0, 0};
+        int sgs[2] = {0, 0};
+        if (mod) {
+            nr = 3 - __popc(ln.mask);
+            cn = nr;
+            for (int k = 0; k < line_nops(ln.mask) && err == kSideNoErr; ++k) {
+                const OpSpec o = op_spec(ln.mask, k, ln.a, ln.c);
+                fl[k] = ln.bl + o.e * st[ln.d];
+                sgs[k] = o.sg;
+                kind[k] = o.e != 0;
+                const uint8_t ft = S.a.type[fl[k]];
+                if (ft != CFP_REGULAR && ft != CFP_IRREGULAR) {
+                    err = side_err(lane, k, 1, DETAIL_BOXIBI);
+                    break;
+                }
+                ib[k] = ibi_index(S, fl[k], 2 * ln.d + (o.sg > 0 ? 0 : 1));
+                if (ib[k] < 0) {
+                    err = side_err(lane, k, 1, DETAIL_MISSINGIBI);
+                    break;
+                }
+                const OpRec& R = ops[2 * (int64_t)ib[k] + kind[k]];
+                if (R.err) err = side_err(lane, k, 1, R.err);
+                else if (R.flags & kOpSingular) err = side_err(lane, k, 2, DETAIL_SINGULAR);
+                if (err != kSideNoErr) break;
+                ng[k] = R.ng;
+                nib[k] = R.nib;
+                ndeg += R.flags & kOpDegenerate;
+                cn += ng[k];
+                bn += nib[k];
+                ++nop;
+            }
         }
-        if (T.cpos + ng > kMaxRaw || T.bpos + nib > kMaxBib) continue;
-        for (int q = 0; q < ng; ++q) {
-            toff[s * kMaxRaw + T.cpos + q] = W.offs[q];
-            tval[s * kMaxRaw + T.cpos + q] = ln.w * cc[q];
+        int c0 = cn, b0 = bn, nd = ndeg;  // inclusive scans
+        for (int o = 1; o < 32; o <<= 1) {
+            const int c = __shfl_up_sync(all, c0, o), b = __shfl_up_sync(all, b0, o);
+            if (lane >= o) {
+                c0 += c;
+                b0 += b;
+            }
         }
-        for (int q = 0; q < nib; ++q) {
-            tbidx[s * kMaxBib + T.bpos + q] = W.ib[q];
-            tbval[s * kMaxBib + T.bpos + q] = ln.w * cc[ng + q];
+        const int nraw = __shfl_sync(all, c0, 31), nbib = __shfl_sync(all, b0, 31);
+        c0 -= cn;
+        b0 -= bn;
+        // overflow of the row's slices, in the order of the steps
+        if (mod) {
+            int c = c0 + nr, b = b0;
+            if (c > kMaxRaw) err = min(err, side_err(lane, 0, 0, DETAIL_OVERFLOW));
+            for (int k = 0; k < nop; ++k) {
+                c += ng[k];
+                b += nib[k];
+                if (c > kMaxRaw || b > kMaxBib) err = min(err, side_err(lane, k, 3, DETAIL_OVERFLOW));
+            }
         }
+        for (int o = 16; o; o >>= 1) {
+            err = min(err, __shfl_xor_sync(all, err, o));
+            nd += __shfl_xor_sync(all, nd, o);
+        }
+        if (lane == 0) {
+            ferr[s] = err;
+            ndegs[s] = nd;
+            bcount[s] = nbib;
+            ccount[s] = 0;
+        }
+        if (err != kSideNoErr) continue;  // the same in every lane
+        if (mod) {
+            int c = c0, b = b0;
+            for (int q = -1; q <= 1; ++q)
+                if (!((ln.mask >> (1 - q)) & 1)) {
+                    soff[c] = (int32_t)(ln.bl + q * st[ln.d] - lin);
+                    sval[c] = -ln.w * Rc(S.ax[ln.d], ln.m, q);
+                    ++c;
+                }
+            for (int k = 0; k < nop; ++k) {
+                const OpRec& R = ops[2 * (int64_t)ib[k] + kind[k]];
+                for (int q = 0; q < ng[k]; ++q, ++c) {
+                    soff[c] = (int32_t)(fl[k] - lin + q * sgs[k] * st[ln.d]);
+                    sval[c] = ln.w * R.cc[q];
+                }
+                for (int q = 0; q < nib[k]; ++q, ++b) {
+                    tbidx[s * kMaxBib + b] = q ? R.ib2 : ib[k];
+                    tbval[s * kMaxBib + b] = ln.w * R.cc[ng[k] + q];
+                }
+            }
+        }
+        __syncwarp();
+        int n = 0;  // merged entries, at the front of soff / sval (never past the adds still to come)
+        for (int base = 0; base < nraw; base += 32) {
+            const bool on = base + lane < nraw;
+            const int o = on ? soff[base + lane] : 0;
+            const double v = on ? sval[base + lane] : 0.0;
+            const unsigned act = __ballot_sync(all, on);
+            unsigned grp = 0;
+            if (on) grp = __match_any_sync(act, o);
+            const bool lead = on && lane == __ffs(grp) - 1;  // the offset's first add in this chunk
+            const unsigned h0 = ((unsigned)o * 2654435761u) >> 23;  // 9 bits
+            int at = -1;  // its entry, if it has one
+            if (lead)
+                for (unsigned h = h0;; h = (h + 1) & (kMergeSlots - 1)) {
+                    const int x = sslot[h];
+                    if (x == 0) break;
+                    if (soff[x - 1] == o) {
+                        at = x - 1;
+                        break;
+                    }
+                }
+            const bool fresh = lead && at < 0;
+            const unsigned fm = __ballot_sync(all, fresh);
+            double acc = v;
+            if (lead && !fresh) acc = sval[at] + v;
+            unsigned rem = lead ? grp & (grp - 1) : 0u;  // the offset's other adds here, in order
+            while (__any_sync(all, rem != 0u)) {
+                const double w = __shfl_sync(all, v, rem ? __ffs(rem) - 1 : 0);
+                if (rem) acc += w;
+                rem &= rem - 1;
+            }
+            if (fresh) at = n + __popc(fm & ((1u << lane) - 1u));
+            __syncwarp();  // every entry of this chunk has been read
+            if (lead) {
+                soff[at] = o;
+                sval[at] = acc;
+            }
+            if (fresh)
+                for (unsigned h = h0; atomicCAS(&sslot[h], 0, at + 1) != 0;) h = (h + 1) & (kMergeSlots - 1);
+            n += __popc(fm);
+            __syncwarp();
+        }
+        for (int q = lane; q < n; q += 32) {
+            toff[s * kMaxRaw + q] = soff[q];
+            tval[s * kMaxRaw + q] = sval[q];
+        }
+        if (lane == 0) ccount[s] = n;
+        __syncwarp();
     }
 }
 
@@ -839,67 +1031,6 @@ __global__ void k_side_finish(SideArgs S, int* ccount, int* bcount, const int* f
             kr[2 + 2 * d] = ip >= 0 ? 0.0 : cc;
         }
         for (int q = 0; q < 7; ++q) krow[7 * s + q] = kr[q];
-    }
-}
-
-// Merges each row's correction adds in place, in their order: an offset
-// seen before adds its value to that entry, a new offset opens the next
-// entry (the order of first appearance).  One warp per row; lane 0 walks the
-// adds through an open-addressing index in shared memory (kMergeSlots >
-// kMaxRaw, so an empty slot always exists), then the warp writes the merged
-// entries back to the front of the row's slice.
-constexpr int kMergeWarps = 4;
-constexpr int kMergeSlots = 512;
-
-__global__ void __launch_bounds__(32 * kMergeWarps) k_side_merge(int64_t n_irr, int* ccount, int32_t* toff,
-                                                                 double* tval) {
-    __shared__ int32_t soff[kMergeWarps][kMaxRaw];
-    __shared__ double sval[kMergeWarps][kMaxRaw];
-    __shared__ int16_t sslot[kMergeWarps][kMergeSlots];
-    __shared__ int smerged[kMergeWarps];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t s = warp; s < n_irr; s += nwarps) {
-        const int nraw = ccount[s];
-        int32_t* off = toff + s * kMaxRaw;
-        double* val = tval + s * kMaxRaw;
-        for (int q = lane; q < kMergeSlots; q += 32) sslot[wl][q] = 0;
-        __syncwarp();
-        if (lane == 0) {
-            int n = 0;
-            for (int e = 0; e < nraw; ++e) {
-                const int o = off[e];
-                const double v = val[e];
-                unsigned h = ((unsigned)o * 2654435761u) >> 23;  // 9 bits
-                bool merged = false;
-                for (int probe = 0; probe < kMergeSlots; ++probe) {
-                    const int x = sslot[wl][h];
-                    if (x == 0) break;
-                    if (soff[wl][x - 1] == o) {
-                        sval[wl][x - 1] += v;
-                        merged = true;
-                        break;
-                    }
-                    h = (h + 1) & (kMergeSlots - 1);
-                }
-                if (!merged) {
-                    soff[wl][n] = o;
-                    sval[wl][n] = v;
-                    sslot[wl][h] = (int16_t)(n + 1);
-                    ++n;
-                }
-            }
-            smerged[wl] = n;
-        }
-        __syncwarp();
-        const int n = smerged[wl];
-        for (int q = lane; q < n; q += 32) {
-            off[q] = soff[wl][q];
-            val[q] = sval[wl][q];
-        }
-        if (lane == 0) ccount[s] = n;
-        __syncwarp();
     }
 }
 
@@ -985,7 +1116,7 @@ cfp_status classify(cfp_ctx* c) {
     g.inside = c->fluid_inside;
 
     launch_metrics(c);  // the 1D grid metrics are rebuilt with every classification
-    k_classify_solid<<<grid_for(N, 256), 256, 0, c->stream>>>(g, c->type, N);
+    k_classify_solid<<<grid_for(32 * (int64_t)ny * nz, 256), 256, 0, c->stream>>>(g, c->type, ny * nz);
     c->launches += 2;
     {
         const int nw = (nx - 2 + 29) / 30;
@@ -1000,23 +1131,22 @@ cfp_status classify(cfp_ctx* c) {
     {
         // size the list first with a counting pass
         long long nirr = 0;
-        const int64_t nb = (N + kScanChunk - 1) / kScanChunk;
+        const int64_t nb = (N + kListChunk - 1) / kListChunk;
         if (nb > c->scan_cap) {
             pool_free_ptr(c, c->scan_bsum);
             CFP_CUDA(pool_malloc(&c->scan_bsum, sizeof(int) * nb, c->stream));
             c->scan_cap = nb;
         }
-        k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, c->stream>>>(FlagIrregular{c->type}, N, c->scan_bsum);
+        CFP_CUDA(cudaMemsetAsync(c->slot, 0xff, sizeof(int32_t) * (size_t)N, c->stream));
+        k_list_count<<<(unsigned)nb, kScanThreads, 0, c->stream>>>(c->type, N, c->scan_bsum);
         k_scan_blocks<<<1, kScanThreads, 0, c->stream>>>(c->scan_bsum, (int)nb, c->dtotal);
-        c->launches += 3;  // with the scatter below
+        c->launches += 3;  // with the stores below
         CFP_CUDA(cudaGetLastError());
         CFP_CUDA(cudaMemcpyAsync(&nirr, c->dtotal, sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
         CFP_CUDA(cudaStreamSynchronize(c->stream));
         c->n_irr = nirr;
         CFP_CUDA(pool_malloc(&c->irr_lin, sizeof(int32_t) * std::max<long long>(nirr, 1), c->stream));
-        k_scan_scatter<<<(unsigned)nb, kScanThreads, 0, c->stream>>>(FlagIrregular{c->type},
-                                                                      SinkSlots{c->slot, c->irr_lin}, N,
-                                                                      c->scan_bsum);
+        if (nirr) k_list_store<<<(unsigned)nb, kScanThreads, 0, c->stream>>>(c->type, N, c->scan_bsum, c->slot, c->irr_lin);
         CFP_CUDA(cudaGetLastError());
     }
     const int64_t nirr = c->n_irr;
@@ -1040,17 +1170,14 @@ cfp_status classify(cfp_ctx* c) {
     c->n_ibi = h;
     CFP_CUDA(cudaMemcpyAsync(c->ibi_off + nirr, c->dtotal, sizeof(int32_t), cudaMemcpyDeviceToDevice, c->stream));
     CFP_CUDA(pool_malloc(&c->ibi_xyz, sizeof(double) * 3 * std::max<int64_t>(c->n_ibi, 1), c->stream));
+    int32_t* isrc = nullptr;
     if (c->n_ibi > 0) {
-        int32_t* isrc = nullptr;
         CFP_CUDA(pool_malloc(&isrc, sizeof(int32_t) * c->n_ibi, c->stream));
         k_ibi_map<<<grid_for(nirr, 256), 256, 0, c->stream>>>(ia, c->ibi_off, isrc);
         k_ibi_roots<<<grid_for(c->n_ibi, 128), 128, 0, c->stream>>>(ia, g, isrc, c->n_ibi, c->ibi_xyz);
         c->launches += 2;
         CFP_CUDA(cudaGetLastError());
-        CFP_CUDA(cudaStreamSynchronize(c->stream));
-        pool_free(isrc, c->stream);
     }
-    CFP_CUDA(cudaGetLastError());
 
     // side list: count, scan, fill
     SideArgs S;
@@ -1083,36 +1210,21 @@ cfp_status classify(cfp_ctx* c) {
     CFP_CUDA(pool_malloc(&c->krow, sizeof(double) * 7 * std::max<int64_t>(nirr, 1), c->stream));
     CFP_CUDA(pool_malloc(&c->krow32, sizeof(float) * 7 * std::max<int64_t>(nirr, 1), c->stream));
     if (nirr) {
-        // plan (count, then place), one thread per operator for the moment
-        // matching, finish; the adds land in the order the row is built in
-        int *ntask = nullptr, *task_off = nullptr, *ferr = nullptr, *ndegs = nullptr;
-        SideTask* tasks = nullptr;
-        CFP_CUDA(pool_malloc(&ntask, sizeof(int) * nirr, c->stream));
-        CFP_CUDA(pool_malloc(&task_off, sizeof(int) * nirr, c->stream));
+        // the operators, then the rows, merged; finish
+        int *ferr = nullptr, *ndegs = nullptr;
+        OpRec* ops = nullptr;
         CFP_CUDA(pool_malloc(&ferr, sizeof(int) * nirr, c->stream));
         CFP_CUDA(pool_malloc(&ndegs, sizeof(int) * nirr, c->stream));
-        k_side_plan<true><<<grid_for(nirr, 128), 128, 0, c->stream>>>(S, ntask, nullptr, nullptr, nullptr, nullptr,
-                                                                      nullptr, nullptr, nullptr, nullptr);
-        c->launches += 1;
-        CFP_CUDA(cudaGetLastError());
-        long long ntasks = 0;
-        CFP_TRY(scan(c, FetchInt{ntask}, SinkOffsets{task_off}, nirr, c->dtotal, &ntasks));
-        CFP_CUDA(pool_malloc(&tasks, sizeof(SideTask) * std::max<long long>(ntasks, 1), c->stream));
-        k_side_plan<false><<<grid_for(nirr, 128), 128, 0, c->stream>>>(S, ntask, task_off, tasks, cnt, cnt2, ferr,
-                                                                       ndegs, toff, tval);
-        if (ntasks)
-            k_side_solve<<<grid_for(ntasks, 64), 64, 0, c->stream>>>(S, tasks, ntasks, ferr, toff, tval, tbidx,
-                                                                    tbval);
+        CFP_CUDA(pool_malloc(&ops, sizeof(OpRec) * 2 * std::max<int64_t>(c->n_ibi, 1), c->stream));
+        if (c->n_ibi) k_side_ops<<<grid_for(2 * c->n_ibi, 64), 64, 0, c->stream>>>(S, isrc, c->n_ibi, ops);
+        k_side_rows<<<grid_for(32 * nirr, 32 * kRowWarps), 32 * kRowWarps, 0, c->stream>>>(
+            S, ops, cnt, cnt2, ferr, ndegs, toff, tval, tbidx, tbval);
         k_side_finish<<<grid_for(nirr, 128), 128, 0, c->stream>>>(S, cnt, cnt2, ferr, ndegs, c->krow, ndeg, c->derr);
-        c->launches += ntasks ? 3 : 2;
+        c->launches += c->n_ibi ? 3 : 2;
         CFP_CUDA(cudaGetLastError());
-        for (void* q : {(void*)ntask, (void*)task_off, (void*)ferr, (void*)ndegs, (void*)tasks}) pool_free(q, c->stream);
+        for (void* q : {(void*)ferr, (void*)ndegs, (void*)ops}) pool_free(q, c->stream);
     }
-    if (nirr) {
-        k_side_merge<<<grid_for(32 * nirr, 32 * kMergeWarps), 32 * kMergeWarps, 0, c->stream>>>(nirr, cnt, toff, tval);
-        c->launches += 1;
-        CFP_CUDA(cudaGetLastError());
-    }
+    pool_free(isrc, c->stream);
     DevError he;
     long long hdeg = 0;
     CFP_CUDA(cudaMemcpyAsync(&he, c->derr, sizeof(DevError), cudaMemcpyDeviceToHost, c->stream));
