@@ -456,10 +456,10 @@ enum { CFP_APPLY_STREAM = 1,  /* each thread streams its column of `rows`
  * the apply are summed per CTA, so their rounding does.  Without a call the
  * context uses CFP_APPLY_STREAM in FP64, in a shape that spreads the grid over
  * the SMs (cfp_apply_shape reports it as 4 rows x 64 planes); in FP32
- * CFP_APPLY_RING with 64 planes where its 512-column tiles are at least 85 %
- * filled by the n_x - 2 interior columns, else CFP_APPLY_STREAM with 2 x 64
- * (fewer planes, down to 4, where 64 would leave the SMs fewer than four CTAs
- * each; cfp_apply_shape reports at least 16).
+ * CFP_APPLY_RING from 2^23 nodes on where its tiles (512 columns, 256 where
+ * n_x <= 258) are at least 85 % filled by the n_x - 2 interior columns, in
+ * chunks of planes that make about 1024 tiles (reported as 2 x 64), else
+ * CFP_APPLY_STREAM, again in a shape by grid size (reported as 4 x 64).
  *   ms  NULL or the chosen candidate's mean time per launch.
  * Requires classification.  Synchronises.  Errors: CFP_ESTATE, CFP_EINVAL
  * (a choice outside those values, or CFP_APPLY_RING with CFP_PREC_FP64 or

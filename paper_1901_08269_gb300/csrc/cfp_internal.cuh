@@ -132,7 +132,6 @@ struct DevError {
 enum { DETAIL_OFFGRID = 1, DETAIL_FEWPOINTS = 2, DETAIL_SINGULAR = 3, DETAIL_BOXIBI = 4,
        DETAIL_OVERFLOW = 5, DETAIL_MISSINGIBI = 6 };
 
-constexpr int kAX = 128;           // apply CTA: columns (threads) along x
 
 constexpr int kUpdBlocks = 152 * 8;   // grid of the vector-update kernels
 constexpr int kUpdThreads = 256;

@@ -4,8 +4,8 @@
 //      A x = sum_r Lz[r] (sum_q Ly[q] XR + Ry[q] XL) + Rz[r] (sum_q Ly[q] XL),
 //      XR = sum_p Rx[p] x,  XL = sum_p Lx[p] x,
 //    with the y-pass results of three planes kept in registers while a thread
-//    (FP64, narrow FP32 grids) or a shared-memory ring's consumer (wide FP32
-//    grids) marches in z; the rows of irregular points, with their
+//    (FP64, most FP32 grids) or a shared-memory ring's consumer (large FP32
+//    grids whose width fills its tiles) marches in z; the rows of irregular points, with their
 //    modified-stencil corrections, in a kernel beside it; solid rows are zero.
 //  - the right-hand side of Eq. Bu=q and helpers of the solves.
 #include <algorithm>
@@ -91,20 +91,53 @@ __device__ __forceinline__ double fmat(double a, double b, double c) { return __
 __device__ __forceinline__ float mult(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a, b); }
 
+// Packed FP32 pairs: one fma.rn.f32x2 instruction does the (IEEE,
+// round-to-nearest) arithmetic of both halves (two rows of a streaming thread,
+// two columns of a ring consumer), with the results of two scalar fmaf calls.
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 f2b(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+
+// DotAcc<float> on both halves at once: a running sum and its lost
+// low-order part per half, the latter kept negated (cn = -c), so that no
+// step needs a negation: v = x y - c = fma(x, y, cn); t = s + v; the new
+// c = (t - s) - v, that is cn = (s - t) + v, with s - t formed exactly as
+// fma(t, -1, s).  Round-to-nearest is symmetric, so every value is the
+// negation of the plain form's, bit for bit.
+struct DotAcc2 {
+    float2 s = {0.f, 0.f}, cn = {0.f, 0.f};
+    __device__ __forceinline__ void add(float2 x, float2 y) {
+        const float2 v = fma2(x, y, cn);
+        const float2 t = add2(s, v);
+        cn = add2(fma2(t, make_float2(-1.f, -1.f), s), v);
+        s = t;
+    }
+    __device__ __forceinline__ double total() const {
+        return ((double)s.x + (double)cn.x) + ((double)s.y + (double)cn.y);
+    }
+};
+
 // Regular part of B x at the unknowns in FP32 (the streaming kernel; the
-// ring below takes the wide grids).  One thread owns the column i of TY
-// consecutive rows j and marches the planes k0 .. k1 - 1 of its z chunk (kc
-// planes, at most kMaxPlanes); TY x kc is the tile shape (apply32_planes, or
-// the autotuner's choice).  The z
-// coefficients of the chunk are staged in shared memory once.
-// Per plane it loads the values x(i-1..i+1, j) of the rows j0-1 .. j0+TY (the
-// x and y neighbours come from L1/L2; the loads of the next plane are issued
-// before the current one is used), forms the x-pass XR = Rx x, XL = Lx x of
-// those rows (each shared by up to three output rows), the y-pass
+// ring below takes large grids that fill its tiles).  A warp is 32 columns x TY consecutive rows
+// (a lane each) and marches the planes k0 .. k1 - 1 of its z chunk (kc planes,
+// at most kMaxPlanes); a CTA is four warps, one above the other in y.
+// Per plane a thread loads the values x(i-1..i+1, j) of the rows j0-1 .. j0+TY
+// (the x and y neighbours come from L1/L2; the loads of the next plane are
+// issued once the x pass has used this one's), forms the x-pass XR = Rx x,
+// XL = Lx x of those rows (each shared by up to three output rows), the y-pass
 // P = Ly XR + Ry XL, Q = Ly XL of its rows, and keeps P, Q of three planes in
 // registers for the z-pass
 //   out(k) = Lz (P(k-1), P(k), P(k+1)) + Rz (Q(k-1), Q(k), Q(k+1)).
-// No shared memory and no barriers.  Solid rows are zero; the rows of
+// Rows t and t + TY / 2 are the halves of packed instructions.  The kernel is
+// bound by the latency of the loads (long scoreboard 6.3 cycles per issue, 20 %
+// of the L1 and DRAM rates at 321 x 257 x 289), so each lane also asks L2 for 32
+// bytes of the rows kAhead planes on: 513^3 460 -> 390 us.  With the dot: 385^3
+// 224 -> 181 us, 129^3 16.6 -> 12.4, 33^3 9.7 -> 6.2 against one column of 2
+// rows x 64 planes per thread, scalar, in CTAs of 128 columns.  No barriers in
+// the march; the z coefficients of the chunk are staged in shared memory once,
+// each twice.  Solid rows are zero; the rows of
 // irregular points are left to k_apply_irr, which runs beside this kernel on
 // a second stream.  (Gathering the corrections inside this kernel, at each plane or
 // from a per-warp list after the march, measured 1.57x slower at 513^3: the
@@ -112,144 +145,173 @@ __device__ __forceinline__ double mult(double a, double b) { return __dmul_rn(a,
 // bodies become the tail.)
 // DOT = 0: y only; 1: partial (d0, y); 2: partials (d0, y) and (y, y).
 constexpr int kMaxPlanes = 64;
+constexpr int kA32Warps = 4;
+constexpr int kAhead = 3;  // planes; 5: 0 to 3 % slower
+
+// the pairs (row p, row p + NP), p = 0 .. NP + 1, of the 2 NP + 2 rows a thread
+// holds, from the NP + 1 distinct ones: d[0 .. NP - 1] those, d[NP] the last two rows
+template <int NP>
+__device__ __forceinline__ void row_pairs(const float2 (&d)[NP + 1], float2 (&w)[NP + 2]) {
+#pragma unroll
+    for (int p = 0; p < NP; ++p) w[p] = d[p];
+    w[NP] = f2(d[0].y, d[NP].x);
+    w[NP + 1] = f2(NP == 1 ? d[1].x : d[NP - 1].y, d[NP].y);
+}
+
 template <int DOT, int TY>
-__global__ void __launch_bounds__(kAX, TY == 2 ? 8 : 4)
-    k_apply(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
-            const float* __restrict__ d0, double* __restrict__ partial, int kc) {
+__global__ void __launch_bounds__(32 * kA32Warps, TY == 4 ? 4 : 6)
+    k_apply32(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
+              const float* __restrict__ d0, double* __restrict__ partial, int kc) {
+    constexpr int NP = TY / 2;
     constexpr int R = TY + 2;  // rows loaded per plane
     const int nx = G.nx, ny = G.ny, nz = G.nz;
-    const int i = 1 + blockIdx.x * kAX + threadIdx.x;
-    const int j0 = 1 + blockIdx.y * TY;
+    const int i = 1 + blockIdx.x * 32 + threadIdx.x;
+    const int j0 = 1 + (blockIdx.y * kA32Warps + threadIdx.y) * TY;
     const int k0 = 1 + blockIdx.z * kc;
     const int k1 = min(k0 + kc, nz - 1);
-    // z coefficients of the chunk's output planes k0 .. k1 - 1
-    __shared__ float zc[5][kMaxPlanes];
-    for (int q = threadIdx.x; q < 5 * kMaxPlanes; q += kAX) {
-        const int m = q / kMaxPlanes, kq = min(k0 + q % kMaxPlanes, nz - 2);
-        const float* src = m == 0 ? G.ax[2].a : m == 1 ? G.ax[2].c : m == 2 ? G.ax[2].ar : m == 3 ? G.ax[2].br : G.ax[2].cr;
-        zc[m][q % kMaxPlanes] = src[kq];
+    // z coefficients of the chunk's output planes k0 .. k1 - 1: a, c, ar, br, cr twice each, two unused
+    __shared__ float4 zc[3 * kMaxPlanes];
+    for (int q = threadIdx.x + 32 * threadIdx.y; q < k1 - k0; q += 32 * kA32Warps) {
+        const int k = k0 + q;
+        const float a = G.ax[2].a[k], c = G.ax[2].c[k], ar = G.ax[2].ar[k], br = G.ax[2].br[k], cr = G.ax[2].cr[k];
+        zc[3 * q] = make_float4(a, a, c, c);
+        zc[3 * q + 1] = make_float4(ar, ar, br, br);
+        zc[3 * q + 2] = make_float4(cr, cr, 0.f, 0.f);
     }
     __syncthreads();
-    const bool iin = i <= nx - 2;
-    const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
-    // node offsets fit in 32 bits: contexts hold fewer than 2^31 nodes
-    const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
-    const float ax = G.ax[0].a[ic], cx = G.ax[0].c[ic];
-    const float arx = G.ax[0].ar[ic], brx = G.ax[0].br[ic], crx = G.ax[0].cr[ic];
-    float ay[TY], cy[TY], ary[TY], bry[TY], cry[TY];
-    bool jin[TY];
-    unsigned lout0[TY];
+    DotAcc2 dacc0, dacc1;
+    if (j0 <= ny - 2) {
+        const bool iin = i <= nx - 2;
+        const int ic = iin ? i : 1;  // clamped: every load stays inside the grid
+        // node offsets fit in 32 bits: contexts hold fewer than 2^31 nodes
+        const unsigned sy = (unsigned)nx, sz = (unsigned)nx * (unsigned)ny;
+        const float2 ax = f2b(G.ax[0].a[ic]), cx = f2b(G.ax[0].c[ic]);
+        const float2 arx = f2b(G.ax[0].ar[ic]), brx = f2b(G.ax[0].br[ic]), crx = f2b(G.ax[0].cr[ic]);
+        float2 ay[NP], cy[NP], ary[NP], bry[NP], cry[NP];
+        bool ok[TY];
+        unsigned l[TY];  // the output nodes of the step's plane
 #pragma unroll
-    for (int t = 0; t < TY; ++t) {
-        jin[t] = j0 + t <= ny - 2;
-        const int jc = jin[t] ? j0 + t : j0;
-        ay[t] = G.ax[1].a[jc];
-        cy[t] = G.ax[1].c[jc];
-        ary[t] = G.ax[1].ar[jc];
-        bry[t] = G.ax[1].br[jc];
-        cry[t] = G.ax[1].cr[jc];
-        lout0[t] = (unsigned)k0 * sz + (unsigned)jc * sy + (unsigned)ic;
-    }
-    unsigned roff[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) roff[r] = (unsigned)min(j0 - 1 + r, ny - 1) * sy;
-    const float* p = x + ((unsigned)(k0 - 1) * sz + (unsigned)ic);
-    float n[3 * R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const float* q = p + roff[r];
-        n[3 * r] = q[-1];
-        n[3 * r + 1] = q[0];
-        n[3 * r + 2] = q[1];
-    }
-    // type byte and dot operand of the next output node of each row
-    uint8_t t_next[TY];
-    float d_next[TY];
-#pragma unroll
-    for (int t = 0; t < TY; ++t) {
-        t_next[t] = type[lout0[t]];
-        d_next[t] = DOT ? d0[lout0[t]] : 0.f;
-    }
-    float Pm[TY], P0[TY], Pp[TY], Qm[TY], Q0[TY], Qp[TY];
-#pragma unroll
-    for (int t = 0; t < TY; ++t) Pm[t] = P0[t] = Pp[t] = Qm[t] = Q0[t] = Qp[t] = 0.f;
-    DotAcc<float> dacc0, dacc1;
-#pragma unroll 3
-    for (int kk = k0 - 1; kk <= k1; ++kk) {
-        float c[3 * R];
-#pragma unroll
-        for (int q = 0; q < 3 * R; ++q) c[q] = n[q];
-        if (kk < k1) {  // prefetch plane kk + 1
-            p += sz;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float* q = p + roff[r];
-                n[3 * r] = q[-1];
-                n[3 * r + 1] = q[0];
-                n[3 * r + 2] = q[1];
-            }
+        for (int q = 0; q < NP; ++q) {
+            const int ja = min(j0 + q, ny - 2), jb = min(j0 + q + NP, ny - 2);
+            ay[q] = f2(G.ax[1].a[ja], G.ax[1].a[jb]);
+            cy[q] = f2(G.ax[1].c[ja], G.ax[1].c[jb]);
+            ary[q] = f2(G.ax[1].ar[ja], G.ax[1].ar[jb]);
+            bry[q] = f2(G.ax[1].br[ja], G.ax[1].br[jb]);
+            cry[q] = f2(G.ax[1].cr[ja], G.ax[1].cr[jb]);
         }
-        // output of this step is plane kk - 1 (from step k0 + 1 on); its type
-        // bytes and dot operands were fetched one step earlier
-        uint8_t t_cur[TY];
-        float d_cur[TY];
 #pragma unroll
         for (int t = 0; t < TY; ++t) {
-            t_cur[t] = t_next[t];
-            d_cur[t] = d_next[t];
+            ok[t] = iin && j0 + t <= ny - 2;
+            l[t] = (unsigned)(k0 - 2) * sz + (unsigned)min(j0 + t, ny - 2) * sy + (unsigned)ic;
         }
-        if (kk >= k0 + 1 && kk < k1) {
+        unsigned roff[R];
 #pragma unroll
-            for (int t = 0; t < TY; ++t) {
-                const unsigned ln = lout0[t] + (unsigned)(kk - k0) * sz;
-                t_next[t] = type[ln];
-                if (DOT) d_next[t] = d0[ln];
-            }
-        }
-        float XR[R], XL[R];
+        for (int r = 0; r < R; ++r) roff[r] = (unsigned)min(j0 - 1 + r, ny - 1) * sy;
+        const float* p = x + ((unsigned)(k0 - 1) * sz + (unsigned)ic);
+        float n[3 * R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            XR[r] = fmat(crx, c[3 * r + 2], fmat(brx, c[3 * r + 1], mult(arx, c[3 * r])));
-            XL[r] = fmat(cx, c[3 * r + 2], fmat(ax, c[3 * r], c[3 * r + 1]));
+            const float* q = p + roff[r];
+            n[3 * r] = q[-1];
+            n[3 * r + 1] = q[0];
+            n[3 * r + 2] = q[1];
         }
+        // what this lane fetches into L2 ahead of the warp's loads: 32 bytes of one of its rows of x
+        // (lanes 8 t .. 8 t + 3), d0 (8 t + 4 .. 8 t + 7) or, second, of type (lane t)
+        const int pt = threadIdx.x >> 3, pc = (int)blockIdx.x * 32 + 1 + 8 * (int)(threadIdx.x & 3);
+        const bool pd = threadIdx.x & 4;
+        const bool pin = pt < TY && (DOT || !pd) && j0 + pt <= ny - 2 && pc <= nx - 2;
+        const float* pf = (DOT && pd ? d0 : x) + ((unsigned)(k0 - 1 + kAhead) * sz +
+                                                  (unsigned)min(j0 + pt, ny - 2) * sy + (unsigned)pc);
+        const bool tin = threadIdx.x < TY && j0 + (int)threadIdx.x <= ny - 2;
+        const uint8_t* tf = type + ((unsigned)(k0 - 1 + kAhead) * sz +
+                                    (unsigned)min(j0 + (int)threadIdx.x, ny - 2) * sy + blockIdx.x * 32 + 1);
+        float2 Pm[NP], P0[NP], Pp[NP], Qm[NP], Q0[NP], Qp[NP];
 #pragma unroll
-        for (int t = 0; t < TY; ++t) {
-            Pm[t] = P0[t];
-            P0[t] = Pp[t];
-            Qm[t] = Q0[t];
-            Q0[t] = Qp[t];
-            Pp[t] = fmat(cry[t], XL[t + 2],
-                         fmat(bry[t], XL[t + 1],
-                              fmat(ary[t], XL[t], fmat(cy[t], XR[t + 2], fmat(ay[t], XR[t], XR[t + 1])))));
-            Qp[t] = fmat(cy[t], XL[t + 2], fmat(ay[t], XL[t], XL[t + 1]));
-        }
-        if (kk >= k0 + 1 && iin) {
-            const int k = kk - 1, kl = k - k0;
-            const float az = zc[0][kl], cz = zc[1][kl];
-            const float arz = zc[2][kl], brz = zc[3][kl], crz = zc[4][kl];
+        for (int q = 0; q < NP; ++q) Pm[q] = P0[q] = Pp[q] = Qm[q] = Q0[q] = Qp[q] = f2b(0.f);
+#pragma unroll 1
+        for (int kk = k0 - 1; kk <= k1; ++kk) {
+            // the output plane is kk - 1, from step k0 + 1 on
+            uint8_t ty[TY];
+            float d[TY];
+            if (kk > k0) {
 #pragma unroll
-            for (int t = 0; t < TY; ++t) {
-                if (!jin[t]) continue;
-                float v = fmat(cz, Pp[t], fmat(az, Pm[t], P0[t])) + fmat(crz, Qp[t], fmat(brz, Q0[t], mult(arz, Qm[t])));
-                const unsigned l = (unsigned)k * sz + (unsigned)(j0 + t) * sy + (unsigned)i;
-                // solid rows are zero; irregular rows belong to k_apply_irr
-                if (t_cur[t] != CFP_REGULAR) v = 0;
-                if (t_cur[t] != CFP_IRREGULAR) y[l] = v;
-                if (DOT >= 1) dacc0.add(d_cur[t], v);
-                if (DOT == 2) dacc1.add(v, v);
+                for (int t = 0; t < TY; ++t) {
+                    ty[t] = type[l[t]];
+                    d[t] = DOT ? d0[l[t]] : 0.f;
+                }
             }
+            float2 XR[NP + 2], XL[NP + 2];
+            {
+                float2 xr[NP + 1], xl[NP + 1];
+#pragma unroll
+                for (int q = 0; q <= NP; ++q) {
+                    const int ra = q < NP ? q : 2 * NP, rb = q < NP ? q + NP : 2 * NP + 1;
+                    const float2 m = f2(n[3 * ra], n[3 * rb]), o = f2(n[3 * ra + 1], n[3 * rb + 1]),
+                                 u = f2(n[3 * ra + 2], n[3 * rb + 2]);
+                    xr[q] = fma2(crx, u, fma2(brx, o, mul2(arx, m)));
+                    xl[q] = fma2(cx, u, fma2(ax, m, o));
+                }
+                row_pairs<NP>(xr, XR);
+                row_pairs<NP>(xl, XL);
+            }
+            if (kk + kAhead <= k1) {
+                if (pin) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
+                if (tin) asm volatile("prefetch.global.L2 [%0];" ::"l"(tf));
+                pf += sz;
+                tf += sz;
+            }
+            if (kk < k1) {  // the next plane's loads, ahead of the y and z passes
+                p += sz;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float* q = p + roff[r];
+                    n[3 * r] = q[-1];
+                    n[3 * r + 1] = q[0];
+                    n[3 * r + 2] = q[1];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                Pm[q] = P0[q];
+                P0[q] = Pp[q];
+                Qm[q] = Q0[q];
+                Q0[q] = Qp[q];
+                Pp[q] = fma2(cry[q], XL[q + 2],
+                             fma2(bry[q], XL[q + 1],
+                                  fma2(ary[q], XL[q], fma2(cy[q], XR[q + 2], fma2(ay[q], XR[q], XR[q + 1])))));
+                Qp[q] = fma2(cy[q], XL[q + 2], fma2(ay[q], XL[q], XL[q + 1]));
+            }
+            if (kk > k0) {
+                const float4 z0 = zc[3 * (kk - 1 - k0)], z1 = zc[3 * (kk - 1 - k0) + 1], z2 = zc[3 * (kk - 1 - k0) + 2];
+#pragma unroll
+                for (int q = 0; q < NP; ++q) {
+                    float2 v = add2(fma2(f2(z0.z, z0.w), Pp[q], fma2(f2(z0.x, z0.y), Pm[q], P0[q])),
+                                    fma2(f2(z2.x, z2.y), Qp[q], fma2(f2(z1.z, z1.w), Q0[q], mul2(f2(z1.x, z1.y), Qm[q]))));
+                    const int ta = q, tb = q + NP;
+                    // solid rows are zero; irregular rows belong to k_apply_irr
+                    v = f2(ok[ta] && ty[ta] == CFP_REGULAR ? v.x : 0.f, ok[tb] && ty[tb] == CFP_REGULAR ? v.y : 0.f);
+                    if (ok[ta] && ty[ta] != CFP_IRREGULAR) y[l[ta]] = v.x;
+                    if (ok[tb] && ty[tb] != CFP_IRREGULAR) y[l[tb]] = v.y;
+                    if (DOT >= 1) dacc0.add(f2(ok[ta] ? d[ta] : 0.f, ok[tb] ? d[tb] : 0.f), v);
+                    if (DOT == 2) dacc1.add(v, v);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < TY; ++t) l[t] += sz;
         }
     }
     if (DOT) {
         double acc0 = dacc0.total(), acc1 = dacc1.total();
         block_reduce2(acc0, acc1);
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
             const int64_t b = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
             partial[2 * b] = acc0;
             partial[2 * b + 1] = acc1;
         }
     }
 }
+
 // The FP64 apply.  GB300 issues about two FP64 instructions per SM and clock,
 // so the kernel is bound by their number (20.5 per node with four rows to a
 // thread: 5 per loaded row, 7 and 6 per output in y and z), not by memory.
@@ -263,7 +325,7 @@ __global__ void __launch_bounds__(kAX, TY == 2 ? 8 : 4)
 // Before: 128-column CTAs of 4 x 64 columns x planes at every
 // size.  With the irregular rows and the dot: 33^3 98 -> 8 us, 97 x 65 x 82
 // 194 -> 36 us, 129^3 199 -> 110 us; 513^3 is as before (5.0 ms).
-// DOT, solid and irregular rows as in k_apply.
+// DOT, solid and irregular rows as in k_apply32.
 constexpr int kA64Warps = 4;
 
 template <int DOT, int TY>
@@ -375,10 +437,11 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
 // memory.  The streaming kernel above keeps one plane of loads in flight per
 // thread, too few bytes per SM to cover the HBM latency.  Here a producer
 // warp copies each plane of a tile several planes ahead of the consumers
-// into one of kRingStages stages: the x rows j0-1 .. j0+2 with their halo
-// columns, and for the output planes the dot operand and the type bytes of
-// the rows j0, j0+1.  A tile is 512 columns x 2 rows x KC planes.  When it
-// spans the whole row width (n_x <= 514), its rows are contiguous in the
+// into one of kRingStages stages: the x rows of the tile and of its two
+// neighbours with their halo columns, and for the output planes the dot operand
+// and the type bytes of its rows.  A tile is TX columns x 1024 / TX rows x KC
+// planes, TX = 512 or, on grids up to 258 wide, 256 (ring_tx).  When it
+// spans the whole row width (n_x <= TX + 2), its rows are contiguous in the
 // natural layout and each array's rows of a plane are one bulk copy; wider
 // grids copy row by row.  Rows start at any 4-byte offset (n_x is odd in the
 // benchmark grids), so each copy starts at the 16-byte boundary at or below
@@ -386,37 +449,37 @@ __global__ void __launch_bounds__(32 * kA64Warps, TY == 4 ? 3 : 4)
 // the array's last 16-byte boundary; the elements after it (at the end of
 // the array only) are stored into the stage by the producer lane itself.
 // Tiles go to a persistent grid, rows fastest within a z chunk; 256 consumer
-// threads own columns i0 + lx and i0 + 256 + lx of both rows and march the
+// threads in groups of TX / 2 own two columns TX / 2 apart of two rows each and march the
 // planes with the same sum-factorised arithmetic and fused multiply-add
-// chains as k_apply<float>, so both give the same bits.  Solid rows are zero;
+// chains as k_apply32, so both give the same bits.  Solid rows are zero;
 // irregular rows are left to k_apply_irr.
 // A wait that runs out (1 s) records a code in *wait_err (31: producer, stage
 // free; 32: producer, final drain; 33: consumer, stage filled).  A producer
 // whose wait ran out issues no further copy and waits (bounded) for the
 // copies it issued; a consumer whose wait ran out stops waiting (every index
 // stays in bounds whatever a stage holds), so the launch still ends.
-constexpr int kRingTX = 512;                // columns per tile
-constexpr int kRingRows = 2;                // rows per tile
-constexpr int kRingCons = 256;              // consumer threads: two columns each
+constexpr int kRingCons = 256;  // consumer threads: two columns and two rows each
 constexpr int kRingThreads = kRingCons + 32;
 constexpr int kRingStages = 6;
-constexpr int kRingSpanNx = kRingTX + 2;    // widest grid copied as whole-plane spans
-constexpr int kRingXRow = 520;              // floats per x row (row-by-row copies): 514 + alignment
-constexpr int kRingDRow = 516;              // floats per dot-operand row: 512 + alignment
-constexpr int kRingTRow = 528;              // bytes per type row: 512 + alignment
-constexpr int kRingXBytes = 8320;           // >= 4 x-rows either way (span: 4 n_x + 6 floats)
-constexpr int kRingDBytes = 4160;           // >= 2 dot rows either way (span: 2 n_x + 6 floats)
-constexpr int kRingTBytes = 1088;           // >= 2 type rows either way (span: 2 n_x + 30 bytes)
-constexpr int kRingDOff = kRingXBytes, kRingTOff = kRingDOff + kRingDBytes;
-constexpr int kRingStage = kRingTOff + kRingTBytes;
-constexpr int kRingSmem = kRingStages * kRingStage + 2 * kRingStages * 8;  // + barriers
-static_assert(kRingXBytes >= (kRingRows + 2) * kRingXRow * 4 && kRingXBytes >= (4 * kRingSpanNx + 8) * 4 &&
-                  kRingDBytes >= kRingRows * kRingDRow * 4 && kRingDBytes >= (2 * kRingSpanNx + 8) * 4 &&
-                  kRingTBytes >= kRingRows * kRingTRow && kRingTBytes >= 2 * kRingSpanNx + 32,
-              "stage regions hold either copy pattern");
-static_assert(kRingStage % 128 == 0 && kRingDOff % 16 == 0 && kRingTOff % 16 == 0 && kRingXRow % 4 == 0 &&
-                  kRingDRow % 4 == 0 && kRingTRow % 16 == 0,
-              "bulk copies want 16-byte destinations");
+// a tile of TX columns
+template <int TX>
+struct RingTile {
+    static constexpr int rows = 4 * kRingCons / TX;
+    static constexpr int span_nx = TX + 2;   // widest grid copied as whole-plane spans
+    static constexpr int xrow = TX + 8;      // floats per x row (row-by-row copies): TX + 2 + alignment
+    static constexpr int drow = TX + 4;      // floats per dot-operand row: TX + alignment
+    static constexpr int trow = TX + 16;     // bytes per type row: TX + alignment
+    // the regions hold either copy pattern
+    static constexpr int xbytes = (std::max((rows + 2) * xrow, (rows + 2) * span_nx + 8) * 4 + 127) / 128 * 128;
+    static constexpr int dbytes = (std::max(rows * drow, rows * span_nx + 8) * 4 + 15) / 16 * 16;
+    static constexpr int tbytes = std::max(rows * trow, rows * span_nx + 32);
+    static constexpr int doff = xbytes, toff = doff + dbytes;
+    static constexpr int stage = (toff + tbytes + 127) / 128 * 128;
+    static constexpr int smem = kRingStages * stage + 2 * kRingStages * 8;  // + barriers
+    static_assert(doff % 16 == 0 && toff % 16 == 0 && xrow % 4 == 0 && drow % 4 == 0 && trow % 16 == 0,
+                  "bulk copies want 16-byte destinations");
+    static_assert(2 * rows + rows + 2 <= 32, "a producer lane per row copy");
+};
 
 // Elements e .. e + want - 1 of an array of n elements of esize bytes into
 // the stage at dst, which receives the array from e0 = the 16-byte boundary
@@ -444,45 +507,19 @@ __device__ __forceinline__ unsigned ring_copy(unsigned char* dst, const unsigned
     return stop > e0 ? (unsigned)((stop - e0) * esize) : 0u;
 }
 
-// Packed FP32 pairs: the halves are the two columns a ring consumer thread
-// owns, and one fma.rn.f32x2 instruction does the (IEEE, round-to-nearest)
-// arithmetic of both, with the results of two scalar fmaf calls.
-__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 f2b(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-
-// DotAcc<float> on both halves at once: a running sum and its lost
-// low-order part per column, the latter kept negated (cn = -c), so that no
-// step needs a negation: v = x y - c = fma(x, y, cn); t = s + v; the new
-// c = (t - s) - v, that is cn = (s - t) + v, with s - t formed exactly as
-// fma(t, -1, s).  Round-to-nearest is symmetric, so every value is the
-// negation of the plain form's, bit for bit.
-struct DotAcc2 {
-    float2 s = {0.f, 0.f}, cn = {0.f, 0.f};
-    __device__ __forceinline__ void add(float2 x, float2 y) {
-        const float2 v = fma2(x, y, cn);
-        const float2 t = add2(s, v);
-        cn = add2(fma2(t, make_float2(-1.f, -1.f), s), v);
-        s = t;
-    }
-    __device__ __forceinline__ double total() const {
-        return ((double)s.x + (double)cn.x) + ((double)s.y + (double)cn.y);
-    }
-};
-
-template <int DOT, bool SPAN>
+template <int DOT, bool SPAN, int TX>
 __global__ void __launch_bounds__(kRingThreads, 2)
     k_apply_ring(Grid<float> G, const uint8_t* __restrict__ type, const float* __restrict__ x, float* __restrict__ y,
                  const float* __restrict__ d0, double* __restrict__ partial, int ntx, int nty, int ntz, int kc,
                  int* __restrict__ wait_err) {
     using namespace tc;
+    using Tile = RingTile<TX>;
+    constexpr int kRingRows = Tile::rows, HX = TX / 2;  // the halves of a thread are HX columns apart
     // indexed from the __shared__ array itself, so that every stage access
     // is a shared-memory load with a 32-bit address
     extern __shared__ __align__(16) unsigned char ring_smem[];
     const float* sf = reinterpret_cast<const float*>(ring_smem);
-    uint64_t* full = reinterpret_cast<uint64_t*>(ring_smem + kRingStages * kRingStage);  // filled: 32 producer lanes
+    uint64_t* full = reinterpret_cast<uint64_t*>(ring_smem + kRingStages * Tile::stage);  // filled: 32 producer lanes
     uint64_t* empty = full + kRingStages;  // released by the consumer warps
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -500,31 +537,31 @@ __global__ void __launch_bounds__(kRingThreads, 2)
     const int ntiles = ntx * nty * ntz;
     DotAcc2 dacc0, dacc1;
     if (warp == kRingCons / 32) {
-        // producer warp.  SPAN (n_x <= 514, one tile column): lane 0 copies
+        // producer warp.  SPAN (one tile column): lane 0 copies
         // x, lane 1 the dot operand, lane 2 the type bytes, each as one span
-        // of whole rows.  Otherwise lanes 0-3 copy the x rows, 4-5 the dot
-        // rows, 6-7 the type rows.  Every lane arrives on the stage's barrier
+        // of whole rows.  Otherwise a lane per row copies the x rows, then the
+        // dot rows, then the type rows.  Every lane arrives on the stage's barrier
         // once per plane with the bytes its copy will deliver.
         constexpr int nxl = SPAN ? 1 : kRingRows + 2, per = SPAN ? 1 : kRingRows;
         const bool xl = lane < nxl, dl = !xl && lane < nxl + per, tl = !xl && !dl && lane < nxl + 2 * per;
         const int r = xl ? lane : dl ? lane - nxl : lane - nxl - per;  // row of a row copy
         const unsigned char* arr = xl ? (const unsigned char*)x : dl ? (const unsigned char*)d0 : type;
         const int esize = tl ? 1 : 4;
-        const int dst_off = xl ? r * kRingXRow * 4 : dl ? kRingDOff + r * kRingDRow * 4 : kRingTOff + r * kRingTRow;
+        const int dst_off = xl ? r * Tile::xrow * 4 : dl ? Tile::doff + r * Tile::drow * 4 : Tile::toff + r * Tile::trow;
         unsigned g = 0;  // planes issued; plane g uses stage g % kRingStages
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
             const int tyi = tile % nty, rest = tile / nty, tx = rest % ntx, tz = rest / ntx;
-            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
+            const int i0 = 1 + tx * TX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
             const int k1 = min(k0 + kc, nz - 1);
             int64_t rowe;  // the copy's first element within a plane
             int w;         // elements wanted
             if (SPAN) {
                 rowe = (int64_t)(xl ? j0 - 1 : j0) * sy;
-                w = xl ? min(4, ny - (j0 - 1)) * nx : 2 * nx;  // the rows that exist
+                w = (xl ? min(kRingRows + 2, ny - (j0 - 1)) : min(kRingRows, ny - j0)) * nx;  // the rows that exist
             } else {
                 rowe = xl ? (int64_t)min(j0 - 1 + r, ny - 1) * sy + (i0 - 1) : (int64_t)min(j0 + r, ny - 2) * sy + i0;
-                w = xl ? kRingTX + 2 : kRingTX;
+                w = xl ? TX + 2 : TX;
             }
             for (int k = k0 - 1; k <= k1; ++k, ++g) {
                 const int st = g % kRingStages;
@@ -541,7 +578,7 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                 const bool act = xl || (outp && (tl || (dl && DOT)));
                 unsigned bytes = 0;
                 const unsigned char* src = nullptr;
-                unsigned char* dst = ring_smem + st * kRingStage + dst_off;
+                unsigned char* dst = ring_smem + st * Tile::stage + dst_off;
                 if (act) bytes = ring_copy(dst, arr, (int64_t)k * sz + rowe, w, esize, N, &src);
                 mbar_arrive_expect_tx(&full[st], bytes);
                 if (bytes) bulk_load(dst, src, bytes, &full[st]);
@@ -554,27 +591,28 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                 if (!mbar_wait(&full[q % kRingStages], (q / kRingStages) & 1)) atomicExch(wait_err, 32);
         __syncwarp();
     } else {
-        // consumer: columns i0 + lx (low half) and i0 + 256 + lx (high half)
-        // of the rows j0, j0 + 1
-        const int lx = threadIdx.x;
+        // consumer: columns i0 + lx (low half) and i0 + HX + lx (high half)
+        // of the rows j0 + jg, j0 + jg + 1
+        const int lx = threadIdx.x % HX, jg = threadIdx.x / HX * 2;
         int st = 0;       // stage of the next plane
         unsigned ph = 0;  // and its phase
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const int tyi = tile % nty, rest = tile / nty, tx = rest % ntx, tz = rest / ntx;
-            const int i0 = 1 + tx * kRingTX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
+            const int i0 = 1 + tx * TX, j0 = 1 + tyi * kRingRows, k0 = 1 + tz * kc;
             const int k1 = min(k0 + kc, nz - 1);
-            const int c = i0 + lx;  // the low half's column; the high half's is c + 256
-            const bool in0 = c <= nx - 2, in1 = c + kRingCons <= nx - 2;
-            const int c0i = in0 ? c : nx - 2, c1i = in1 ? c + kRingCons : nx - 2;
+            const int c = i0 + lx;  // the low half's column; the high half's is c + HX
+            const int jr = j0 + jg;  // the thread's first row
+            const bool in0 = c <= nx - 2 && jr <= ny - 2, in1 = c + HX <= nx - 2;
+            const int c0i = min(c, nx - 2), c1i = min(c + HX, nx - 2);
             const float2 AX = f2(G.ax[0].a[c0i], G.ax[0].a[c1i]), CX = f2(G.ax[0].c[c0i], G.ax[0].c[c1i]);
             const float2 ARX = f2(G.ax[0].ar[c0i], G.ax[0].ar[c1i]), BRX = f2(G.ax[0].br[c0i], G.ax[0].br[c1i]);
             const float2 CRX = f2(G.ax[0].cr[c0i], G.ax[0].cr[c1i]);
             float2 AY[2], CY[2], ARY[2], BRY[2], CRY[2];
-            const bool jin1 = j0 + 1 <= ny - 2;  // row j0 always is
+            const bool jin1 = jr + 1 <= ny - 2;
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
-                const int jc = min(j0 + t, ny - 2);
+                const int jc = min(jr + t, ny - 2);
                 AY[t] = f2b(G.ax[1].a[jc]);
                 CY[t] = f2b(G.ax[1].c[jc]);
                 ARY[t] = f2b(G.ax[1].ar[jc]);
@@ -586,16 +624,17 @@ __global__ void __launch_bounds__(kRingThreads, 2)
             // (SPAN: rows n_x apart, one offset for all); likewise for the
             // output rows.  kx, ko carry kp of the plane being read and of the
             // one being written, kept below 16 (only their low bits count).
-            const int xrow = SPAN ? nx : kRingXRow, drow = SPAN ? nx : kRingDRow, trow = SPAN ? nx : kRingTRow;
-            const int xcol = SPAN ? c : c - (i0 - 1), ocol = SPAN ? c : c - i0;
+            const int xrow = SPAN ? nx : Tile::xrow, drow = SPAN ? nx : Tile::drow, trow = SPAN ? nx : Tile::trow;
+            const int xcol = (SPAN ? c : c - (i0 - 1)) + jg * xrow, ocol = SPAN ? c : c - i0;
+            const int tcol = ocol + jg * trow, dcol = ocol + jg * drow;
             unsigned xa[4], oa[2];
 #pragma unroll
             for (int q = 0; q < 4; ++q)
                 xa[q] = SPAN ? ((unsigned)(j0 - 1) * sy) & 3u
-                             : ((unsigned)min(j0 - 1 + q, ny - 1) * sy + (unsigned)(i0 - 1)) & 3u;
+                             : ((unsigned)min(jr - 1 + q, ny - 1) * sy + (unsigned)(i0 - 1)) & 3u;
 #pragma unroll
             for (int t = 0; t < 2; ++t)
-                oa[t] = ((SPAN ? (unsigned)j0 : (unsigned)min(j0 + t, ny - 2)) * sy + (SPAN ? 0u : (unsigned)i0)) & 15u;
+                oa[t] = ((SPAN ? (unsigned)j0 : (unsigned)min(jr + t, ny - 2)) * sy + (SPAN ? 0u : (unsigned)i0)) & 15u;
             unsigned kx = ((unsigned)(k0 - 1) * sz) & 15u, ko = 0;
             float2 Pm[2], P0[2], Pp[2], Qm[2], Q0[2], Qp[2];
 #pragma unroll
@@ -603,7 +642,7 @@ __global__ void __launch_bounds__(kRingThreads, 2)
             // z coefficients of the plane the next step outputs, loaded a step ahead
             const float* zp = G.ax[2].a + k0;  // a, c, ar, br, cr follow at n_z
             float zn[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-            float* yr = y + ((unsigned)k0 * sz + (unsigned)j0 * sy + (unsigned)c);
+            float* yr = y + ((unsigned)k0 * sz + (unsigned)jr * sy + (unsigned)c);
             int sprev = 0;  // stage of the plane before
             for (int kk = k0 - 1; kk <= k1; ++kk) {
                 const float2 AZ = f2b(zn[0]), CZ = f2b(zn[1]), ARZ = f2b(zn[2]), BRZ = f2b(zn[3]), CRZ = f2b(zn[4]);
@@ -616,13 +655,13 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                     ok = false;
                     atomicExch(wait_err, 33);
                 }
-                const float* xs = sf + st * (kRingStage / 4) + xcol + (SPAN ? (int)((kx + xa[0]) & 3u) : 0);
+                const float* xs = sf + st * (Tile::stage / 4) + xcol + (SPAN ? (int)((kx + xa[0]) & 3u) : 0);
                 float2 XR[4], XL[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const float* row = xs + q * xrow + (SPAN ? 0 : (int)((kx + xa[q]) & 3u));
-                    const float2 xm = f2(row[-1], row[kRingCons - 1]), x0 = f2(row[0], row[kRingCons]),
-                                 xp = f2(row[1], row[kRingCons + 1]);
+                    const float2 xm = f2(row[-1], row[HX - 1]), x0 = f2(row[0], row[HX]),
+                                 xp = f2(row[1], row[HX + 1]);
                     XR[q] = fma2(CRX, xp, fma2(BRX, x0, mul2(ARX, xm)));
                     XL[q] = fma2(CX, xp, fma2(AX, xm, x0));
                 }
@@ -641,9 +680,9 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                     if (kk >= k0 + 1) {
                         if (in0) {
                             const unsigned char* ts =
-                                ring_smem + sprev * kRingStage + kRingTOff + ocol + (SPAN ? (int)((ko + oa[0]) & 15u) : 0);
+                                ring_smem + sprev * Tile::stage + Tile::toff + tcol + (SPAN ? (int)((ko + oa[0]) & 15u) : 0);
                             const float* ds =
-                                sf + sprev * (kRingStage / 4) + kRingDOff / 4 + ocol + (SPAN ? (int)((ko + oa[0]) & 3u) : 0);
+                                sf + sprev * (Tile::stage / 4) + Tile::doff / 4 + dcol + (SPAN ? (int)((ko + oa[0]) & 3u) : 0);
 #pragma unroll
                             for (int t = 0; t < 2; ++t) {
                                 if (t && !jin1) continue;
@@ -651,15 +690,15 @@ __global__ void __launch_bounds__(kRingThreads, 2)
                                                 fma2(CRZ, Qp[t], fma2(BRZ, Q0[t], mul2(ARZ, Qm[t]))));
                                 const unsigned char* tr = ts + t * trow + (SPAN ? 0 : (int)((ko + oa[t]) & 15u));
                                 // solid rows are zero; irregular rows belong to k_apply_irr
-                                const uint8_t t0 = tr[0], t1 = in1 ? tr[kRingCons] : (uint8_t)CFP_SOLID;
+                                const uint8_t t0 = tr[0], t1 = in1 ? tr[HX] : (uint8_t)CFP_SOLID;
                                 if (t0 != CFP_REGULAR) v.x = 0.f;
                                 if (t1 != CFP_REGULAR) v.y = 0.f;
                                 float* yt = yr + t * nx;
                                 if (t0 != CFP_IRREGULAR) yt[0] = v.x;
-                                if (in1 && t1 != CFP_IRREGULAR) yt[kRingCons] = v.y;
+                                if (in1 && t1 != CFP_IRREGULAR) yt[HX] = v.y;
                                 if (DOT >= 1) {
                                     const float* dr = ds + t * drow + (SPAN ? 0 : (int)((ko + oa[t]) & 3u));
-                                    dacc0.add(f2(dr[0], in1 ? dr[kRingCons] : 0.f), v);
+                                    dacc0.add(f2(dr[0], in1 ? dr[HX] : 0.f), v);
                                 }
                                 if (DOT == 2) dacc1.add(v, v);
                             }
@@ -944,6 +983,7 @@ __global__ void __launch_bounds__(128)
 // (Eqs. A27_mod, cor, cor_case2).  One thread per irregular point.  The
 // regular rows' kernels leave these rows alone, so this kernel runs beside
 // them on a second stream; its dot terms go to its own partials.
+constexpr int kIrrGroup = 8;
 template <class T, int DOT>
 __global__ void __launch_bounds__(128)
     k_apply_irr(Grid<T> G, Side<T> S, const int32_t* __restrict__ irr_lin, int64_t n_irr, const T* __restrict__ x,
@@ -954,7 +994,22 @@ __global__ void __launch_bounds__(128)
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_irr;
          s += (int64_t)gridDim.x * blockDim.x) {
         const int64_t l = irr_lin[s];
-        const int k = (int)(l / sz), rem = (int)(l - k * sz), j = rem / nx, i = rem - j * nx;
+        // the corrections, summed in entry order: the offsets and weights of the
+        // next eight are fetched while this eight's values are on their way
+        const int e0 = S.corr_ptr[s], e1 = S.corr_ptr[s + 1];
+        int off[kIrrGroup];
+        T w[kIrrGroup];
+        auto fetch = [&](int e) {
+#pragma unroll
+            for (int q = 0; q < kIrrGroup; ++q) {
+                const bool in = e + q < e1;
+                off[q] = in ? S.corr_off[e + q] : 0;
+                w[q] = in ? S.corr_val[e + q] : T(0);
+            }
+        };
+        fetch(e0);
+        const unsigned lu = (unsigned)l, k = lu / (unsigned)sz, rem = lu - k * (unsigned)sz, j = rem / (unsigned)nx,
+                       i = rem - j * (unsigned)nx;
         const T ax = G.ax[0].a[i], cx = G.ax[0].c[i], arx = G.ax[0].ar[i], brx = G.ax[0].br[i], crx = G.ax[0].cr[i];
         const T ay = G.ax[1].a[j], cy = G.ax[1].c[j], ary = G.ax[1].ar[j], bry = G.ax[1].br[j], cry = G.ax[1].cr[j];
         const T az = G.ax[2].a[k], cz = G.ax[2].c[k], arz = G.ax[2].ar[k], brz = G.ax[2].br[k], crz = G.ax[2].cr[k];
@@ -972,19 +1027,19 @@ __global__ void __launch_bounds__(128)
             Q[dz] = fmat(cy, XL[2], fmat(ay, XL[0], XL[1]));
         }
         T v = fmat(cz, P[2], fmat(az, P[0], P[1])) + fmat(crz, Q[2], fmat(brz, Q[1], mult(arz, Q[0])));
-        // the corrections, summed in entry order; the loads of four entries
-        // are issued before their products are added (the gather is
-        // latency-bound, and beside the ring kernel few of these CTAs fit)
         T cor = T(0);
-        const int e1 = S.corr_ptr[s + 1];
-        int e = S.corr_ptr[s];
-        for (; e + 4 <= e1; e += 4) {
-            const int o0 = S.corr_off[e], o1 = S.corr_off[e + 1], o2 = S.corr_off[e + 2], o3 = S.corr_off[e + 3];
-            const T w0 = S.corr_val[e], w1 = S.corr_val[e + 1], w2 = S.corr_val[e + 2], w3 = S.corr_val[e + 3];
-            const T x0 = x[l + o0], x1 = x[l + o1], x2 = x[l + o2], x3 = x[l + o3];
-            cor = fmat(w3, x3, fmat(w2, x2, fmat(w1, x1, fmat(w0, x0, cor))));
+        for (int e = e0; e < e1; e += kIrrGroup) {
+            T xv[kIrrGroup], wv[kIrrGroup];
+#pragma unroll
+            for (int q = 0; q < kIrrGroup; ++q) {
+                xv[q] = x[l + off[q]];
+                wv[q] = w[q];
+            }
+            fetch(e + kIrrGroup);
+#pragma unroll
+            for (int q = 0; q < kIrrGroup; ++q)
+                if (e + q < e1) cor = fmat(wv[q], xv[q], cor);
         }
-        for (; e < e1; ++e) cor = fmat(S.corr_val[e], x[l + S.corr_off[e]], cor);
         v = v + cor;
         y[l] = v;
         if (DOT >= 1) acc0 += (double)d0[l] * (double)v;
@@ -1057,84 +1112,40 @@ unsigned flat_grid(int64_t n) {
 
 namespace {
 
-dim3 rows_grid(const cfp_ctx* c, int rows, int kc) {
-    return dim3((unsigned)((c->n[0] - 2 + kAX - 1) / kAX), (unsigned)((c->n[1] - 2 + rows - 1) / rows),
-                (unsigned)((c->n[2] - 2 + kc - 1) / kc));
+// the ring's tile width: 256 only where a tile spans the row (copied row by row,
+// 256-column tiles of 513^3 took 443 us, 512-column ones 354)
+int ring_tx(const cfp_ctx* c) { return c->n[0] <= RingTile<256>::span_nx ? 256 : 512; }
+// planes per z chunk where the tuner set none: some 1024 tiles, of 64 to 128
+// planes (513^3: 128 336 us, 64 354); beside the irregular rows' kernel, whose
+// CTAs delay some of the ring's, few rounds of tiles lose least (bodies, 257^3:
+// 64 67 us, 24 87; 513^3: 64 412, 128 422)
+int ring_planes(const cfp_ctx* c) {
+    if (c->apply_kc[1]) return std::max(32, c->apply_kc[1]);
+    const int tx = ring_tx(c), rows = 4 * kRingCons / tx;
+    const int64_t col = (int64_t)((c->n[0] - 2 + tx - 1) / tx) * ((c->n[1] - 2 + rows - 1) / rows);
+    return c->n_irr > 0 ? 64 : (int)std::max<int64_t>(64, std::min<int64_t>(128, col * (c->n[2] - 2) / 1024));
 }
-
 // the apply's kernel and tile shape of precision q (0 FP64, 1 FP32), as set
-// by the autotuner; otherwise in FP64 the shape apply64_shape finds (reported
-// as 4 x 64), in FP32 (apply32_planes; reported with at least 16 planes) the ring (2 x 64) where its 512-column tiles are at least 85 % filled
-// (n_x = 513: 511 of 512 columns) and else the streaming kernel with 2 x 64
-// (at 385^3, 383 of 512 columns, it measured 0.285 ms against 0.256 ms)
+// by the autotuner; otherwise in FP64 the shape apply64_shape finds, in FP32 the
+// ring from 2^23 nodes on where its tiles' columns are at least 85 % filled
+// (257^3 55 us against the streaming kernel's 68, 225^3 45 : 55, 449 x 385 x 321
+// 174 : 180, 513^3 337 : 406; but 257 x 129 x 65 18 : 12, 385^3 205 : 181) and else
+// the streaming kernel (apply32_shape).  The shapes found are reported as 4 x
+// 64, the ring's as 2 x 64.
 int apply_kind(const cfp_ctx* c, int q) {
     if (c->apply_kind[q]) return c->apply_kind[q];
     if (q == 1 && c->ring_grid > 0) {
-        const int cols = c->n[0] - 2, tiles = (cols + kRingTX - 1) / kRingTX;
-        if (cols * 100 >= 85 * tiles * kRingTX) return CFP_APPLY_RING;
+        const int cols = c->n[0] - 2, tx = ring_tx(c), tiles = (cols + tx - 1) / tx;
+        const int64_t nodes = (int64_t)cols * (c->n[1] - 2) * (c->n[2] - 2);
+        if (nodes >= (int64_t)1 << 23 && cols * 100 >= 85 * tiles * tx) return CFP_APPLY_RING;
     }
     return CFP_APPLY_STREAM;
 }
-int apply_rows(const cfp_ctx* c, int q) { return c->apply_ty[q] ? c->apply_ty[q] : (q ? 2 : 4); }
+int apply_rows(const cfp_ctx* c, int q) { return c->apply_ty[q] ? c->apply_ty[q] : 4; }
 int apply_planes(const cfp_ctx* c, int q) { return c->apply_kc[q] ? c->apply_kc[q] : 64; }
 
-// planes per z chunk of the FP32 streaming kernel: the tuner's, else 64, less
-// on grids that 64 would leave with fewer than four CTAs per SM (33^3 with 64
-// is 16 CTAs and takes 12.4 us, with 4 it is 128)
-int apply32_planes(const cfp_ctx* c) {
-    int kc = apply_planes(c, 1);
-    if (!c->apply_kc[1])
-        while (kc > 4) {
-            const dim3 g = rows_grid(c, apply_rows(c, 1), kc);
-            if ((int64_t)g.x * g.y * g.z >= 4 * 152) break;
-            kc /= 2;
-        }
-    return kc;
-}
-
-}  // namespace
-
-// the kernel and tile shape the apply of precision q runs with, as a shape
-// that can be set
-void apply_shape(const cfp_ctx* c, int q, int* kernel, int* rows, int* planes) {
-    *kernel = apply_kind(c, q);
-    *rows = *kernel == CFP_APPLY_RING ? 2 : apply_rows(c, q);
-    *planes = q ? std::max(16, apply32_planes(c)) : apply_planes(c, q);
-    if (*kernel == CFP_APPLY_RING && *planes < 32) *planes = 32;
-}
-
-namespace {
-
-// the ring's tiles: 512 columns x 2 rows x kc planes
-void ring_tiles(const cfp_ctx* c, int kc, int* ntx, int* nty, int* ntz) {
-    *ntx = (c->n[0] - 2 + kRingTX - 1) / kRingTX;
-    *nty = (c->n[1] - 2 + kRingRows - 1) / kRingRows;
-    *ntz = (c->n[2] - 2 + kc - 1) / kc;
-}
-
-bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
-
-}  // namespace
-
-void launch_metrics(cfp_ctx* c) {
-    int64_t off = 0;
-    for (int d = 0; d < 3; ++d) {
-        const int n = c->n[d];
-        k_metrics<<<(n + 255) / 256, 256, 0, c->stream>>>(c->dX[d], n, c->dcoef64 + off, c->dcoef32 + off);
-        off += 8 * (int64_t)n;
-    }
-    c->launches += 3;
-}
-
-// CTAs of k_apply_irr (128 threads, one irregular point each per pass; at
-// most 152 x 8)
-int irr_blocks(const cfp_ctx* c) {
-    if (c->n_irr <= 0) return 0;
-    return (int)std::min<int64_t>((c->n_irr + 127) / 128, 152 * 8);
-}
-
 // k_apply64's rows per thread and planes per z chunk
-struct Shape64 {
+struct Shape {
     int ty, kc;
     dim3 grid(const cfp_ctx* c) const {
         const int rows = ty * kA64Warps;
@@ -1158,12 +1169,12 @@ struct Shape64 {
 // 250 and 895), 97 x 65 x 82 2 x 8; 33^3 takes 128 CTAs of 1 x 2, where 4 x
 // 64 would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
 // 33^3 14.5 us with them, 10.4 with four warps in the same shape.)
-Shape64 shape64(const cfp_ctx* c, double row, double yout, double zout) {
-    Shape64 best{4, 64};
+Shape shape64(const cfp_ctx* c, double row, double yout, double zout) {
+    Shape best{4, 64};
     double est_best = 1e300;
     for (int t : {4, 2, 1})
         for (int q : {64, 32, 16, 8, 4, 2}) {
-            const Shape64 sh{t, q};
+            const Shape sh{t, q};
             const double cta = kA64Warps * ((q + 2) * (row * (t + 2) + yout * t) + zout * q * t);
             const double per = (double)((sh.ctas(c) + 151) / 152);
             const double est = per * cta + 130.0 * (q + 2) + (per > 4 ? 0.5 * cta : 0.0);
@@ -1174,9 +1185,80 @@ Shape64 shape64(const cfp_ctx* c, double row, double yout, double zout) {
         }
     return best;
 }
-Shape64 apply64_shape(const cfp_ctx* c) {
-    if (c->apply_ty[0] && c->apply_kc[0]) return Shape64{c->apply_ty[0], c->apply_kc[0]};
+Shape apply64_shape(const cfp_ctx* c) {
+    if (c->apply_ty[0] && c->apply_kc[0]) return Shape{c->apply_ty[0], c->apply_kc[0]};
     return shape64(c, 5.0, 7.0, 6.0);
+}
+
+// The FP32 streaming kernel is bound by the latency of a plane's loads, so its
+// time goes with the rounds of resident CTAs (four with 4 rows, six with 2 per
+// SM) times the planes each marches, about 1 us per plane with 4 rows, and
+// some 6 for a round's start (257^3: 4 x 64 68 us, 4 x 8 78; 129^3: 4 x 8 12.4,
+// 4 x 16 14.5; 321 x 257 x 289: 4 x 32 91, 4 x 64 106).  Without a dot product 2 rows take 0.65 of it
+// (513^3 361 us against 390), with one more (448 against 406).
+Shape apply32_shape(const cfp_ctx* c, bool dot) {
+    if (c->apply_ty[1] && c->apply_kc[1]) return Shape{c->apply_ty[1], c->apply_kc[1]};
+    Shape best{4, 64};
+    double est_best = 1e300;
+    for (int t : {4, 2})
+        for (int q : {64, 32, 16, 8, 4, 2}) {
+            if (t == 2 && dot) continue;
+            const Shape sh{t, q};
+            const int64_t per = 152 * (t == 4 ? 4 : 6);
+            const double est = (double)((sh.ctas(c) + per - 1) / per) * (q + 8) * (t == 4 ? 1.0 : 0.65);
+            if (est < est_best) {
+                est_best = est;
+                best = sh;
+            }
+        }
+    return best;
+}
+
+}  // namespace
+
+// the kernel and tile shape the apply of precision q runs with, as a shape
+// that can be set
+void apply_shape(const cfp_ctx* c, int q, int* kernel, int* rows, int* planes) {
+    *kernel = apply_kind(c, q);
+    *rows = *kernel == CFP_APPLY_RING ? 2 : apply_rows(c, q);
+    *planes = apply_planes(c, q);
+}
+
+namespace {
+
+// the ring's launch: tile width, planes per z chunk, tiles per axis
+struct RingShape {
+    int tx, kc, ntx, nty, ntz;
+    int tiles() const { return ntx * nty * ntz; }
+};
+RingShape ring_shape(const cfp_ctx* c) {
+    RingShape r{ring_tx(c), ring_planes(c), 0, 0, 0};
+    const int rows = 4 * kRingCons / r.tx;
+    r.ntx = (c->n[0] - 2 + r.tx - 1) / r.tx;
+    r.nty = (c->n[1] - 2 + rows - 1) / rows;
+    r.ntz = (c->n[2] - 2 + r.kc - 1) / r.kc;
+    return r;
+}
+
+bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
+}  // namespace
+
+void launch_metrics(cfp_ctx* c) {
+    int64_t off = 0;
+    for (int d = 0; d < 3; ++d) {
+        const int n = c->n[d];
+        k_metrics<<<(n + 255) / 256, 256, 0, c->stream>>>(c->dX[d], n, c->dcoef64 + off, c->dcoef32 + off);
+        off += 8 * (int64_t)n;
+    }
+    c->launches += 3;
+}
+
+// CTAs of k_apply_irr (128 threads, one irregular point each per pass; at
+// most 152 x 8)
+int irr_blocks(const cfp_ctx* c) {
+    if (c->n_irr <= 0) return 0;
+    return (int)std::min<int64_t>((c->n_irr + 127) / 128, 152 * 8);
 }
 
 // the most CTAs any apply tile shape launches, with the irregular rows' kernel's
@@ -1185,19 +1267,15 @@ Shape64 apply64_shape(const cfp_ctx* c) {
 int apply_blocks(cfp_ctx* c) {
     int64_t m = 0;
     for (int ty : {2, 4})
-        for (int kc : {16, 32, 64}) {
-            const dim3 g = rows_grid(c, ty, kc);
-            m = std::max(m, std::max((int64_t)g.x * g.y * g.z, Shape64{ty, kc}.ctas(c)));
-        }
-    m = std::max(m, apply64_shape(c).ctas(c));
-    const dim3 g = rows_grid(c, apply_rows(c, 1), apply32_planes(c));
-    m = std::max(m, (int64_t)g.x * g.y * g.z);
+        for (int kc : {16, 32, 64}) m = std::max(m, Shape{ty, kc}.ctas(c));
+    m = std::max(m, std::max(apply64_shape(c).ctas(c), apply32_shape(c, true).ctas(c)));
+    if (c->ring_grid > 0) m = std::max<int64_t>(m, std::min(ring_shape(c).tiles(), c->ring_grid));
     return (int)m + irr_blocks(c);
 }
 
 // the FP64 regular rows' kernel
 template <int DOT>
-void apply64_launch(cfp_ctx* c, const Shape64& sh, const double* x, double* y, const double* d0, double* partial,
+void apply64_launch(cfp_ctx* c, const Shape& sh, const double* x, double* y, const double* d0, double* partial,
                     cudaStream_t s) {
     const dim3 g = sh.grid(c), b(32, kA64Warps);
     if (sh.ty == 4) k_apply64<DOT, 4><<<g, b, 0, s>>>(grid_view<double>(c), c->type, x, y, d0, partial, sh.kc);
@@ -1205,28 +1283,43 @@ void apply64_launch(cfp_ctx* c, const Shape64& sh, const double* x, double* y, c
     else k_apply64<DOT, 1><<<g, b, 0, s>>>(grid_view<double>(c), c->type, x, y, d0, partial, sh.kc);
 }
 
+// the FP32 ring
+template <int DOT, int TX>
+void ring_launch_tx(cfp_ctx* c, const RingShape& r, int ctas, const float* x, float* y, const float* d0,
+                    double* partial, cudaStream_t s) {
+    auto k = k_apply_ring<DOT, true, TX>;
+    if constexpr (TX == 512)
+        if (c->n[0] > RingTile<TX>::span_nx) k = k_apply_ring<DOT, false, TX>;
+    k<<<ctas, kRingThreads, RingTile<TX>::smem, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, r.ntx, r.nty,
+                                                     r.ntz, r.kc, c->dwait);
+}
+template <int DOT>
+void ring_launch(cfp_ctx* c, const RingShape& r, int ctas, const float* x, float* y, const float* d0, double* partial,
+                 cudaStream_t s) {
+    if (r.tx == 512) ring_launch_tx<DOT, 512>(c, r, ctas, x, y, d0, partial, s);
+    else ring_launch_tx<DOT, 256>(c, r, ctas, x, y, d0, partial, s);
+}
+
 // B x: the regular rows' kernel on s and, forked onto the context's second
 // stream and joined back before anything later on s, the irregular rows'
 // kernel; dot partials: the main kernel's CTAs, then k_apply_irr's.
 template <class T, int DOT>
 void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cudaStream_t s, int* nb) {
-    int nmain = 0, ntx = 0, nty = 0, ntz = 0, kc = 0;
+    int nmain = 0;
     bool ring = false;
-    dim3 grid;
-    Shape64 sh64{0, 0};
+    Shape sh{0, 0};
+    RingShape rs{0, 0, 0, 0, 0};
     if constexpr (sizeof(T) == 8) {
-        sh64 = apply64_shape(c);
-        nmain = (int)sh64.ctas(c);
+        sh = apply64_shape(c);
+        nmain = (int)sh.ctas(c);
     } else {
         ring = apply_kind(c, 1) == CFP_APPLY_RING && c->ring_grid > 0 && aligned16(x) && (!DOT || aligned16(d0));
         if (ring) {
-            kc = std::max(32, apply_planes(c, 1));  // the ring marches 32 or 64 planes
-            ring_tiles(c, kc, &ntx, &nty, &ntz);
-            nmain = std::min(ntx * nty * ntz, c->ring_grid);
+            rs = ring_shape(c);
+            nmain = std::min(rs.tiles(), c->ring_grid);
         } else {
-            kc = apply32_planes(c);
-            grid = rows_grid(c, apply_rows(c, 1), kc);
-            nmain = (int)(grid.x * grid.y * grid.z);
+            sh = apply32_shape(c, DOT > 0);
+            nmain = (int)sh.ctas(c);
         }
     }
     const int nirr = irr_blocks(c);
@@ -1237,19 +1330,13 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
                                                       d0, partial ? partial + 2 * (int64_t)nmain : nullptr);
     }
     if constexpr (sizeof(T) == 8) {
-        apply64_launch<DOT>(c, sh64, x, y, d0, partial, s);
+        apply64_launch<DOT>(c, sh, x, y, d0, partial, s);
     } else if (ring) {
-        const Grid<float> G = grid_view<float>(c);
-        if (c->n[0] <= kRingSpanNx)
-            k_apply_ring<DOT, true><<<nmain, kRingThreads, kRingSmem, s>>>(G, c->type, x, y, d0, partial, ntx, nty, ntz,
-                                                                           kc, c->dwait);
-        else
-            k_apply_ring<DOT, false><<<nmain, kRingThreads, kRingSmem, s>>>(G, c->type, x, y, d0, partial, ntx, nty, ntz,
-                                                                            kc, c->dwait);
-    } else if (apply_rows(c, 1) == 4) {
-        k_apply<DOT, 4><<<grid, kAX, 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, kc);
+        ring_launch<DOT>(c, rs, nmain, x, y, d0, partial, s);
+    } else if (sh.ty == 4) {
+        k_apply32<DOT, 4><<<sh.grid(c), dim3(32, kA64Warps), 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, sh.kc);
     } else {
-        k_apply<DOT, 2><<<grid, kAX, 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, kc);
+        k_apply32<DOT, 2><<<sh.grid(c), dim3(32, kA64Warps), 0, s>>>(grid_view<float>(c), c->type, x, y, d0, partial, sh.kc);
     }
     if (nirr) {
         cudaEventRecord(c->ev_join, c->aux);
@@ -1260,17 +1347,18 @@ void apply_launch(cfp_ctx* c, const T* x, T* y, const T* d0, double* partial, cu
 }
 
 namespace {
-template <int DOT, bool SPAN>
+template <int DOT, bool SPAN, int TX>
 bool ring_attr(int* per) {
-    if (cudaFuncSetAttribute(k_apply_ring<DOT, SPAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmem) !=
-        cudaSuccess)
-        return false;
+    const auto k = k_apply_ring<DOT, SPAN, TX>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RingTile<TX>::smem) != cudaSuccess) return false;
     int p = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_apply_ring<DOT, SPAN>, kRingThreads, kRingSmem) !=
-        cudaSuccess)
-        return false;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k, kRingThreads, RingTile<TX>::smem) != cudaSuccess) return false;
     *per = std::min(*per, p);
     return true;
+}
+template <bool SPAN, int TX>
+bool ring_attrs(int* per) {
+    return ring_attr<0, SPAN, TX>(per) && ring_attr<1, SPAN, TX>(per) && ring_attr<2, SPAN, TX>(per);
 }
 }  // namespace
 
@@ -1279,8 +1367,7 @@ bool ring_attr(int* per) {
 bool setup_apply_ring(cfp_ctx* c) {
     if (c->ring_grid) return c->ring_grid > 0;
     int per = 1 << 20, nsm = 0;
-    const bool ok = ring_attr<0, true>(&per) && ring_attr<1, true>(&per) && ring_attr<2, true>(&per) &&
-                    ring_attr<0, false>(&per) && ring_attr<1, false>(&per) && ring_attr<2, false>(&per) &&
+    const bool ok = ring_attrs<true, 512>(&per) && ring_attrs<false, 512>(&per) && ring_attrs<true, 256>(&per) &&
                     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess;
     cudaGetLastError();
     c->ring_grid = ok && per >= 1 ? per * nsm : -1;
@@ -1341,7 +1428,7 @@ void launch_rhs(cfp_ctx* c, const double* f, const double* g, const double* g_ib
     const Grid<double> G = grid_view<double>(c);
     const int64_t box = 2 * ((int64_t)nx * ny + (int64_t)nx * nz + (int64_t)ny * nz);
     k_rhs_box<<<flat_grid(box), 256, 0, s>>>(g, gb, rhs, nx, ny, nz);
-    const Shape64 sh = shape64(c, 2.0, 2.0, 2.0);
+    const Shape sh = shape64(c, 2.0, 2.0, 2.0);
     const dim3 gr = sh.grid(c), b(32, kA64Warps);
     const bool solid = !c->bodies.empty();
 #define CFP_SOURCE(TY)                                                                                     \
