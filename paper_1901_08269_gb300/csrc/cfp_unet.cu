@@ -103,10 +103,33 @@ cfp_status prep_conv() {
             cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, W::SMEM) !=
                 cudaSuccess)
             return CFP_ECUDA;
+        if constexpr (MarchCfg<CIN, COUT>::fits)
+            if (cudaFuncSetAttribute(k_conv_march<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     MarchCfg<CIN, COUT>::SMEM) != cudaSuccess)
+                return CFP_ECUDA;
         return CFP_OK;
     }();
     if (st != CFP_OK) return fail(st, "cudaFuncSetAttribute failed for a convolution kernel");
     return CFP_OK;
+}
+
+// k_conv_march's split for cap resident CTAs: the chunk with the least rounds x
+// (planes + the two it reads beyond); tiles = 0 where a plane leaves more than
+// 15 % of its tiles' rows empty (k_conv_tc's tiles run on across planes)
+March march_split(const Pad& P, int cap) {
+    const int plane = P.nxp * P.nyp;
+    March M{(plane + 127) / 128, 1, P.nzp};
+    if ((int64_t)plane * 100 < (int64_t)M.tiles * 128 * 85) return March{0, 0, 0};
+    int64_t best = INT64_MAX;
+    for (int z = P.nzp; z >= 1; --z) {
+        const int64_t chunks = (P.nzp + z - 1) / z, est = ((int64_t)M.tiles * chunks + cap - 1) / cap * (z + 2);
+        if (est < best) {
+            best = est;
+            M.planes = z;
+            M.chunks = (int)chunks;
+        }
+    }
+    return M;
 }
 
 template <int CIN, int COUT>
@@ -124,9 +147,20 @@ cfp_status conv_t(cudaStream_t s, const uint16_t* in, const uint16_t* wsrc, bool
     const int nw = COUT * 27 * CIN;
     if (flip) k_wpack<CIN, COUT, true><<<blocks(nw), 256, 0, s>>>(wsrc, wpk);
     else k_wpack<CIN, COUT, false><<<blocks(nw), 256, 0, s>>>(wsrc, wpk);
+    uint16_t* const out_bf = (flags & F_OUT_F32) ? nullptr : (uint16_t*)out;
+    float* const out_f = (flags & F_OUT_F32) ? (float*)out : nullptr;
+    if constexpr (MarchCfg<CIN, COUT>::fits) {
+        using C = MarchCfg<CIN, COUT>;
+        const March M = march_split(P, C::PER * num_sms());
+        if (M.tiles > 0) {
+            k_conv_march<CIN, COUT><<<M.tiles * M.chunks, kConvThreads, C::SMEM, s>>>(in, wpk, bias, act, P, M, flags,
+                                                                                      out_bf, out_f, err);
+            CFP_CUDA(cudaGetLastError());
+            return CFP_OK;
+        }
+    }
     k_conv_tc<CIN, COUT><<<conv_grid<CIN, COUT>(P), kConvThreads, C::SMEM, s>>>(
-        in, wpk, bias, act, P, flags, (flags & F_OUT_F32) ? nullptr : (uint16_t*)out,
-        (flags & F_OUT_F32) ? (float*)out : nullptr, err);
+        in, wpk, bias, act, P, flags, out_bf, out_f, err);
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
 }

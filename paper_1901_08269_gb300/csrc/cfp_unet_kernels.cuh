@@ -12,7 +12,7 @@
 // (t/3)%3 - 1, t%3 - 1):
 //     out[v][co] = bias[co] + sum_t sum_ci W[co][t][ci] in[v + off(t)][ci].
 //
-// Forward convolution (k_conv_tc): the implicit GEMM D (128 voxels x Cout) =
+// Forward convolution (k_conv_tc; k_conv_march up to 32 input channels): the implicit GEMM D (128 voxels x Cout) =
 // sum over taps of A_t (128 x Cin) B_t^T.  For each (dy, dz) pair one window
 // of 130 rows (the 128 outputs and one row either side) serves the three taps
 // dx = -1, 0, 1, whose A operands start 0, 16 and 32 bytes into it (K-major,
@@ -156,6 +156,68 @@ __global__ void k_wpack(const uint16_t* __restrict__ w, uint16_t* __restrict__ o
     }
 }
 
+// The epilogue of one warp's 32 rows (this lane's: row), accumulated at acc: bias,
+// RELU, MASK, ACCUM as below; rows that are not valid are left alone.
+template <int COUT>
+__device__ __forceinline__ void conv_rows(unsigned acc, int row, bool valid, const Pad& P, const float* __restrict__ bias,
+                                          const uint16_t* __restrict__ act, int flags, uint16_t* __restrict__ out_bf,
+                                          float* __restrict__ out_f) {
+                const bool in = valid && interior(P, row);
+    #pragma unroll 1
+                for (int c16 = 0; c16 < COUT / 16; ++c16) {
+                    float v[16];
+                    tc::tmem_ld16(acc + 16 * c16, v);
+                    if (!valid) continue;
+                    const int c0 = 16 * c16;
+                    if (!in) {
+    #pragma unroll
+                        for (int q = 0; q < 16; ++q) v[q] = 0.f;
+                    } else {
+                        uint16_t am[16], ac[16];
+                        if (flags & F_MASK) {
+                            const uint4* ap = reinterpret_cast<const uint4*>(act + (size_t)row * COUT + c0);
+                            *reinterpret_cast<uint4*>(am) = ap[0];
+                            *reinterpret_cast<uint4*>(am + 8) = ap[1];
+                        }
+                        if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) {
+                            const uint4* op = reinterpret_cast<const uint4*>(out_bf + (size_t)row * COUT + c0);
+                            *reinterpret_cast<uint4*>(ac) = op[0];
+                            *reinterpret_cast<uint4*>(ac + 8) = op[1];
+                        }
+    #pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            float x = v[q] + (bias ? __ldg(bias + c0 + q) : 0.f);
+                            if (flags & F_RELU) x = fmaxf(x, 0.f);
+                            if ((flags & F_MASK) && !bf_pos(am[q])) x = 0.f;
+                            if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) x += bf2f(ac[q]);
+                            v[q] = x;
+                        }
+                    }
+                    if (flags & F_OUT_F32) {
+                        float4* op = reinterpret_cast<float4*>(out_f + (size_t)row * COUT + c0);
+    #pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float4 o = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                            if (flags & F_ACCUM) {
+                                const float4 p = op[q];
+                                o.x += p.x;
+                                o.y += p.y;
+                                o.z += p.z;
+                                o.w += p.w;
+                            }
+                            op[q] = o;
+                        }
+                    } else {
+                        uint16_t h[16];
+    #pragma unroll
+                        for (int q = 0; q < 16; ++q) h[q] = f2bf(v[q]);
+                        uint4* op = reinterpret_cast<uint4*>(out_bf + (size_t)row * COUT + c0);
+                        op[0] = *reinterpret_cast<uint4*>(h);
+                        op[1] = *reinterpret_cast<uint4*>(h + 8);
+                    }
+                }
+}
+
 // out (Np x COUT) = epilogue(conv(in, W) + bias): RELU max(., 0); MASK times
 // [act > 0]; ACCUM adds the values already in out (BF16); OUT_F32 FP32
 // output.  Padding rows get 0.  Bounded waits: a wait that runs out records
@@ -275,61 +337,173 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
             if (!ok) break;
             tc::fence_after();
             const int row = tile * 128 + 32 * warp + lane;
-            const bool valid = row < P.Np;
-            const bool in = valid && interior(P, row);
-#pragma unroll 1
-            for (int c16 = 0; c16 < COUT / 16; ++c16) {
-                float v[16];
-                tc::tmem_ld16(tmem + ((unsigned)(32 * warp) << 16) + b * COUT + 16 * c16, v);
-                if (!valid) continue;
-                const int c0 = 16 * c16;
-                if (!in) {
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) v[q] = 0.f;
-                } else {
-                    uint16_t am[16], ac[16];
-                    if (flags & F_MASK) {
-                        const uint4* ap = reinterpret_cast<const uint4*>(act + (size_t)row * COUT + c0);
-                        *reinterpret_cast<uint4*>(am) = ap[0];
-                        *reinterpret_cast<uint4*>(am + 8) = ap[1];
-                    }
-                    if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) {
-                        const uint4* op = reinterpret_cast<const uint4*>(out_bf + (size_t)row * COUT + c0);
-                        *reinterpret_cast<uint4*>(ac) = op[0];
-                        *reinterpret_cast<uint4*>(ac + 8) = op[1];
-                    }
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        float x = v[q] + (bias ? __ldg(bias + c0 + q) : 0.f);
-                        if (flags & F_RELU) x = fmaxf(x, 0.f);
-                        if ((flags & F_MASK) && !bf_pos(am[q])) x = 0.f;
-                        if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) x += bf2f(ac[q]);
-                        v[q] = x;
-                    }
-                }
-                if (flags & F_OUT_F32) {
-                    float4* op = reinterpret_cast<float4*>(out_f + (size_t)row * COUT + c0);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float4 o = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                        if (flags & F_ACCUM) {
-                            const float4 p = op[q];
-                            o.x += p.x;
-                            o.y += p.y;
-                            o.z += p.z;
-                            o.w += p.w;
-                        }
-                        op[q] = o;
-                    }
-                } else {
-                    uint16_t h[16];
-#pragma unroll
-                    for (int q = 0; q < 16; ++q) h[q] = f2bf(v[q]);
-                    uint4* op = reinterpret_cast<uint4*>(out_bf + (size_t)row * COUT + c0);
-                    op[0] = *reinterpret_cast<uint4*>(h);
-                    op[1] = *reinterpret_cast<uint4*>(h + 8);
-                }
+            conv_rows<COUT>(tmem + ((unsigned)(32 * warp) << 16) + b * COUT, row, row < P.Np, P, bias, act, flags, out_bf,
+                            out_f);
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&acce[b]);
+        }
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc::fence_after();
+        tc::tmem_free<C::TCOLS>(tmem);
+    }
+}
+
+// The same convolution for few input channels, marching planes: a tile is 128
+// consecutive voxels of a plane and a CTA takes it through a chunk of planes,
+// so that a plane's three windows (dy = -1, 0, 1) are copied once and serve the
+// outputs of three planes, and the 27 taps' weights stay in shared memory.
+// k_conv_tc copies nine windows and the weights per tile, and those copies'
+// issue bounds it (129 x 97 x 65, 16 -> 16: 58 % of the issue slots, 7 % of the tensor
+// pipe, 76 us).  Here it takes 58 us (32 -> 32 194 with the call against 206),
+// bound by a plane's chain of copy, 27 small MMAs and epilogue: two CTAs per SM
+// instead of three take a third longer.  The products are added in the same
+// order: the same bits.
+template <int CIN, int COUT>
+struct MarchCfg {
+    static constexpr int NCH = CIN / 8;
+    static constexpr int STAGE = rup(NCH * kPlane, 128);  // a window
+    static constexpr int W_TAP = NCH * COUT * 16;
+    static constexpr int W_BYTES = 27 * W_TAP;
+    static constexpr int FIXED = W_BYTES + 128 + (2 * 18 + 6) * 8 + 16;
+    static constexpr int TCOLS = pow2ceil(2 * COUT);
+    // nine windows serve an output; CTAs per SM while twelve fit
+    static constexpr int PER = 3 * (FIXED + 12 * STAGE) <= 220 * 1024   ? 3
+                               : 2 * (FIXED + 12 * STAGE) <= 220 * 1024 ? 2
+                                                                        : 1;
+    static constexpr int S0 = (220 * 1024 / PER - FIXED) / STAGE;
+    static constexpr int STAGES = S0 > 18 ? 18 : S0;
+    static constexpr int SMEM = FIXED + STAGES * STAGE;
+    // one CTA per SM only where k_conv_tc has one too (32 -> 16, two there: 157 us against 194)
+    static constexpr bool fits = CIN <= 32 && STAGES >= 12 && (PER > 1 || ConvCfg<CIN, COUT>::PER == 1);
+};
+
+struct March {
+    int tiles;   // 128-voxel tiles of a plane
+    int planes;  // of a chunk
+    int chunks;
+};
+
+// as k_conv_tc; one CTA per unit (tile, chunk), tile fastest
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(kConvThreads, MarchCfg<CIN, COUT>::PER)
+    k_conv_march(const uint16_t* __restrict__ in, const uint16_t* __restrict__ wpk, const float* __restrict__ bias,
+                 const uint16_t* __restrict__ act, Pad P, March M, int flags, uint16_t* __restrict__ out_bf,
+                 float* __restrict__ out_f, int* __restrict__ err) {
+    using C = MarchCfg<CIN, COUT>;
+    constexpr unsigned S = C::STAGES;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    unsigned char* wsm = base + S * C::STAGE;
+    uint64_t* full = (uint64_t*)(wsm + C::W_BYTES);
+    uint64_t* empty = full + S;
+    uint64_t* accf = empty + S;  // accumulator b filled
+    uint64_t* acce = accf + 2;   // accumulator b read out by the four epilogue warps
+    uint64_t* wful = acce + 2;   // the weights
+    uint64_t* fin = wful + 1;    // every MMA of this CTA completed
+    unsigned* tslot = (unsigned*)(fin + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (unsigned q = 0; q < S; ++q) {
+            tc::mbar_init(&full[q], kProd);
+            tc::mbar_init(&empty[q], 1);
+        }
+        for (int q = 0; q < 2; ++q) {
+            tc::mbar_init(&accf[q], 1);
+            tc::mbar_init(&acce[q], 4);
+        }
+        tc::mbar_init(wful, 1);
+        tc::mbar_init(fin, 1);
+        tc::mbar_fence_init();
+    }
+    if (warp == 0) tc::tmem_alloc<C::TCOLS>(tslot);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const unsigned tmem = *tslot;
+    const int plane = P.nxp * P.nyp;
+    const int v0 = (int)(blockIdx.x % M.tiles) * 128;
+    const int k0 = (int)(blockIdx.x / M.tiles) * M.planes, k1 = min(k0 + M.planes, P.nzp);
+
+    if (warp >= 4 && warp < 8) {  // producers: windows (plane k0 - 1, dy = -1), (k0 - 1, 0), ...
+        const int p = threadIdx.x - 128;
+        if (p == 0) {
+            tc::mbar_arrive_expect_tx(wful, C::W_BYTES);
+            tc::bulk_load(wsm, wpk, C::W_BYTES, wful);
+        }
+        const unsigned nw = 3 * (k1 - k0 + 2);
+        for (unsigned g = 0; g < nw; ++g) {
+            const unsigned st = g % S;
+            int free = 1;
+            if (g >= S && lane == 0 && !tc::mbar_wait(&empty[st], ((g / S) - 1) & 1)) {
+                free = 0;
+                atomicExch(err, 17);
             }
+            if (!__shfl_sync(0xffffffffu, free, 0)) break;
+            const int row0 = (k0 - 1 + (int)(g / 3)) * plane + v0 + ((int)(g % 3) - 1) * P.nxp - 1;
+            copy_rows<C::NCH, kPlane>(tc::smem_u32(base + st * C::STAGE), in, CIN, 0, row0, kWin, P.Np, p);
+            copy_arrive(&full[st]);
+        }
+        copy_wait_all();
+        if (p == 0 && !tc::mbar_wait(wful, 0)) atomicExch(err, 12);  // landed before the CTA may end
+    } else if (warp == 8 && lane == 0) {  // MMA issuer
+        constexpr unsigned idesc = tc::idesc_bf16(128, COUT, 0, 0);
+        bool ok = tc::mbar_wait(wful, 0);
+        if (!ok) atomicExch(err, 18);
+        const unsigned wb = tc::smem_u32(wsm);
+        unsigned got = 0;  // windows waited for
+        for (int k = k0; k < k1 && ok; ++k) {
+            const unsigned tl = k - k0, b = tl & 1;
+            if (tl >= 2 && !tc::mbar_wait(&acce[b], ((tl / 2) - 1) & 1)) {
+                atomicExch(err, 13);
+                break;
+            }
+            tc::fence_after();
+            const unsigned d = tmem + b * COUT;
+            for (unsigned s = 0; s < 9; ++s) {  // 3 (dz + 1) + (dy + 1)
+                const unsigned g = 3 * tl + s, st = g % S;
+                if (g == got) {
+                    if (!tc::mbar_wait(&full[st], (g / S) & 1)) {
+                        ok = false;
+                        atomicExch(err, 14);
+                        break;
+                    }
+                    async_after();
+                    tc::fence_after();
+                    ++got;
+                }
+                const unsigned ab = tc::smem_u32(base + st * C::STAGE);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                    for (int q = 0; q < C::NCH / 2; ++q) {
+                        const uint64_t da = tc::sdesc(ab + dx * 16 + q * 2 * kPlane, kPlane, 128);
+                        const uint64_t db = tc::sdesc(wb + (3 * s + dx) * C::W_TAP + q * 2 * COUT * 16, COUT * 16, 128);
+                        tc::mma_bf16(d, da, db, idesc, (s | dx | q) != 0);
+                    }
+            }
+            if (!ok) break;
+            tc::mma_commit(&accf[b]);
+            for (unsigned s = 0; s < 3; ++s) tc::mma_commit(&empty[(3 * tl + s) % S]);  // plane k - 1 has served
+        }
+        tc::mma_commit(fin);
+        if (!tc::mbar_wait(fin, 0)) atomicExch(err, 15);
+    } else if (warp < 4) {  // epilogue: warp w reads tensor-memory lanes 32w .. 32w + 31
+        for (int k = k0; k < k1; ++k) {
+            const unsigned tl = k - k0, b = tl & 1;
+            int ok = 1;
+            if (lane == 0 && !tc::mbar_wait(&accf[b], (tl / 2) & 1)) {
+                ok = 0;
+                atomicExch(err, 16);
+            }
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+            tc::fence_after();
+            const int v = v0 + 32 * warp + lane;
+            conv_rows<COUT>(tmem + ((unsigned)(32 * warp) << 16) + b * COUT, k * plane + v, v < plane, P, bias, act, flags,
+                            out_bf, out_f);
             tc::fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&acce[b]);

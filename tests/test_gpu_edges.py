@@ -114,9 +114,11 @@ def test_vcycle_sizes(n, nu, post):
     ctx.close()
 
 
-# fewer rows than a tile of 128, and a remainder past one and several tiles
-@pytest.mark.parametrize("cin,cout", [(16, 16), (64, 32), (128, 128)])
-@pytest.mark.parametrize("d", [(5, 3, 3), (17, 9, 3), (40, 7, 11)])
+# fewer rows than a tile of 128, a remainder past one and several tiles, planes
+# marched one by one (40 x 7 x 11) and in chunks (the last one short)
+@pytest.mark.parametrize("d,cin,cout", [((5, 3, 3), 16, 16), ((5, 3, 3), 128, 128), ((17, 9, 3), 64, 32),
+                                        ((40, 7, 11), 16, 16), ((40, 7, 11), 32, 64), ((40, 7, 11), 128, 128),
+                                        ((126, 30, 21), 16, 16), ((126, 30, 21), 16, 32), ((62, 61, 21), 32, 32)])
 def test_layer_sizes(d, cin, cout):
     axis = np.linspace(-1.0, 1.0, 9)
     ctx = cfp.Context(axis, axis, axis)
