@@ -250,7 +250,8 @@ struct cfp_ctx {
 
     // side-list build scratch (per-slot slices), kept across classifications
     void* side_scratch = nullptr;
-    void* nn_wflip = nullptr;      // learned part: mirrored, transposed weights of a layer
+    void* nn_work = nullptr;       // learned part: work space of the single-layer calls
+    size_t nn_work_bytes = 0;
     size_t side_scratch_bytes = 0;
 
     // scan scratch
