@@ -433,8 +433,9 @@ enum { CFP_APPLY_STREAM = 1,  /* each thread streams its column of `rows`
                                  rows through the z planes of its chunk with
                                  plain loads, one plane ahead (FP64, FP32)  */
        CFP_APPLY_RING = 2     /* FP32: a producer warp copies the planes of a
-                                 512-column x 2-row tile with bulk (TMA)
-                                 copies into a ring of shared-memory stages
+                                 512-column x 2-row (n_x <= 258: 256 x 4)
+                                 tile with bulk (TMA) copies into a ring of
+                                 shared-memory stages
                                  ahead of 256 consumer threads; persistent
                                  grid.  Needs 16-byte aligned x and dot
                                  operand (otherwise the streaming kernel
