@@ -100,22 +100,30 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// The .sync.aligned instructions below need the whole warp, converged: each
+// wrapper first brings its lanes together again (__syncwarp), whatever branches
+// they took since the last one.
+
 // tensor-memory columns (a power of two >= 32), by one whole warp
 template <int COLS>
 __device__ __forceinline__ void tmem_alloc(unsigned* slot) {
     static_assert(COLS >= 32 && COLS <= 512 && (COLS & (COLS - 1)) == 0, "tensor-memory columns");
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "n"(COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 template <int COLS>
 __device__ __forceinline__ void tmem_free(unsigned base) {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "n"(COLS) : "memory");
 }
 // 16 consecutive FP32 columns of the warp's 32 lanes (lane = row); taddr
-// carries the warp's lane base in bits 16..31
+// carries the warp's lane base in bits 16..31.  Every lane calls it, those whose
+// row is not wanted too.
 __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     unsigned r[16];
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),

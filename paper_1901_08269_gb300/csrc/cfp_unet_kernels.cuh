@@ -156,66 +156,74 @@ __global__ void k_wpack(const uint16_t* __restrict__ w, uint16_t* __restrict__ o
     }
 }
 
-// The epilogue of one warp's 32 rows (this lane's: row), accumulated at acc: bias,
-// RELU, MASK, ACCUM as below; rows that are not valid are left alone.
+// The epilogue of channels c0 .. c0 + 15 of one row, accumulated in v: bias,
+// RELU, MASK, ACCUM as below; a padding row (in false) gets zeros.
+template <int COUT>
+__device__ __forceinline__ void conv_row16(float (&v)[16], int c0, int row, bool in, const float* __restrict__ bias,
+                                           const uint16_t* __restrict__ act, int flags,
+                                           uint16_t* __restrict__ out_bf, float* __restrict__ out_f) {
+    if (!in) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = 0.f;
+    } else {
+        uint16_t am[16], ac[16];
+        if (flags & F_MASK) {
+            const uint4* ap = reinterpret_cast<const uint4*>(act + (size_t)row * COUT + c0);
+            *reinterpret_cast<uint4*>(am) = ap[0];
+            *reinterpret_cast<uint4*>(am + 8) = ap[1];
+        }
+        if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) {
+            const uint4* op = reinterpret_cast<const uint4*>(out_bf + (size_t)row * COUT + c0);
+            *reinterpret_cast<uint4*>(ac) = op[0];
+            *reinterpret_cast<uint4*>(ac + 8) = op[1];
+        }
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            float x = v[q] + (bias ? __ldg(bias + c0 + q) : 0.f);
+            if (flags & F_RELU) x = fmaxf(x, 0.f);
+            if ((flags & F_MASK) && !bf_pos(am[q])) x = 0.f;
+            if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) x += bf2f(ac[q]);
+            v[q] = x;
+        }
+    }
+    if (flags & F_OUT_F32) {
+        float4* op = reinterpret_cast<float4*>(out_f + (size_t)row * COUT + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float4 o = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            if (flags & F_ACCUM) {
+                const float4 p = op[q];
+                o.x += p.x;
+                o.y += p.y;
+                o.z += p.z;
+                o.w += p.w;
+            }
+            op[q] = o;
+        }
+    } else {
+        uint16_t h[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) h[q] = f2bf(v[q]);
+        uint4* op = reinterpret_cast<uint4*>(out_bf + (size_t)row * COUT + c0);
+        op[0] = *reinterpret_cast<uint4*>(h);
+        op[1] = *reinterpret_cast<uint4*>(h + 8);
+    }
+}
+
+// The epilogue of one warp's 32 rows (this lane's: row), accumulated at acc;
+// rows that are not valid are left alone (their lanes still take part in the
+// tensor-memory loads, which are the whole warp's).
 template <int COUT>
 __device__ __forceinline__ void conv_rows(unsigned acc, int row, bool valid, const Pad& P, const float* __restrict__ bias,
                                           const uint16_t* __restrict__ act, int flags, uint16_t* __restrict__ out_bf,
                                           float* __restrict__ out_f) {
-                const bool in = valid && interior(P, row);
-    #pragma unroll 1
-                for (int c16 = 0; c16 < COUT / 16; ++c16) {
-                    float v[16];
-                    tc::tmem_ld16(acc + 16 * c16, v);
-                    if (!valid) continue;
-                    const int c0 = 16 * c16;
-                    if (!in) {
-    #pragma unroll
-                        for (int q = 0; q < 16; ++q) v[q] = 0.f;
-                    } else {
-                        uint16_t am[16], ac[16];
-                        if (flags & F_MASK) {
-                            const uint4* ap = reinterpret_cast<const uint4*>(act + (size_t)row * COUT + c0);
-                            *reinterpret_cast<uint4*>(am) = ap[0];
-                            *reinterpret_cast<uint4*>(am + 8) = ap[1];
-                        }
-                        if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) {
-                            const uint4* op = reinterpret_cast<const uint4*>(out_bf + (size_t)row * COUT + c0);
-                            *reinterpret_cast<uint4*>(ac) = op[0];
-                            *reinterpret_cast<uint4*>(ac + 8) = op[1];
-                        }
-    #pragma unroll
-                        for (int q = 0; q < 16; ++q) {
-                            float x = v[q] + (bias ? __ldg(bias + c0 + q) : 0.f);
-                            if (flags & F_RELU) x = fmaxf(x, 0.f);
-                            if ((flags & F_MASK) && !bf_pos(am[q])) x = 0.f;
-                            if ((flags & F_ACCUM) && !(flags & F_OUT_F32)) x += bf2f(ac[q]);
-                            v[q] = x;
-                        }
-                    }
-                    if (flags & F_OUT_F32) {
-                        float4* op = reinterpret_cast<float4*>(out_f + (size_t)row * COUT + c0);
-    #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            float4 o = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                            if (flags & F_ACCUM) {
-                                const float4 p = op[q];
-                                o.x += p.x;
-                                o.y += p.y;
-                                o.z += p.z;
-                                o.w += p.w;
-                            }
-                            op[q] = o;
-                        }
-                    } else {
-                        uint16_t h[16];
-    #pragma unroll
-                        for (int q = 0; q < 16; ++q) h[q] = f2bf(v[q]);
-                        uint4* op = reinterpret_cast<uint4*>(out_bf + (size_t)row * COUT + c0);
-                        op[0] = *reinterpret_cast<uint4*>(h);
-                        op[1] = *reinterpret_cast<uint4*>(h + 8);
-                    }
-                }
+    const bool in = valid && interior(P, row);
+#pragma unroll 1
+    for (int c16 = 0; c16 < COUT / 16; ++c16) {
+        float v[16];
+        tc::tmem_ld16(acc + 16 * c16, v);
+        if (valid) conv_row16<COUT>(v, 16 * c16, row, in, bias, act, flags, out_bf, out_f);
+    }
 }
 
 // out (Np x COUT) = epilogue(conv(in, W) + bias): RELU max(., 0); MASK times
