@@ -775,7 +775,7 @@ __global__ void k_zero_box(T* __restrict__ y, int nx, int ny, int nz) {
 
 // The source term of Eq. q with the weights of solid points set to zero
 // (Q-bar): the tensor product Q = Lx Ly Lz applied to f with its solid
-// entries replaced by zero (SOLID: there are bodies), sum-factorised and
+// entries replaced by zero (SOLID: there may be some), sum-factorised and
 // marched in z like k_apply64, whose launch shape it shares: 7 FP64
 // instructions per node with four rows per thread, which is what bounds it
 // (265 us at 321 x 257 x 289).  Interior solid nodes get 0.
@@ -1430,7 +1430,9 @@ void launch_rhs(cfp_ctx* c, const double* f, const double* g, const double* g_ib
     k_rhs_box<<<flat_grid(box), 256, 0, s>>>(g, gb, rhs, nx, ny, nz);
     const Shape sh = shape64(c, 2.0, 2.0, 2.0);
     const dim3 gr = sh.grid(c), b(32, kA64Warps);
-    const bool solid = !c->bodies.empty();
+    // no solid points: no bodies, and the fluid outside them (the inside of no
+    // body is no fluid at all)
+    const bool solid = !c->bodies.empty() || c->fluid_inside;
 #define CFP_SOURCE(TY)                                                                                     \
     (solid ? k_rhs_source<TY, true><<<gr, b, 0, s>>>(G, c->type, f, rhs, sh.kc)                            \
            : k_rhs_source<TY, false><<<gr, b, 0, s>>>(G, c->type, f, rhs, sh.kc))
