@@ -1,6 +1,6 @@
 """The right-hand side where there is no fluid at all (the inside of no body):
 zero at every node, whatever f and g hold there, like the row-by-row form of
-cfp_assemble_rhs_noalloc."""
+cfp_assemble_rhs_noalloc; and where it shares memory with an input."""
 import numpy as np
 import pytest
 
@@ -37,4 +37,35 @@ def test_interior_of_no_body(n):
         rhs = torch.full((ctx.N,), float("nan"), dtype=torch.float64, device="cuda")
         entry(f, g, None, rhs)
         assert torch.equal(rhs, torch.zeros_like(rhs)), entry
+    ctx.close()
+
+
+BALL = W.sphere((0.05, -0.03, 0.02), 0.3)
+
+
+@pytest.mark.parametrize("which", ["f", "g", "g_ibi", "shifted"])
+def test_rhs_may_share_memory_with_an_input(which):
+    """The same bits as with memory of its own: rhs in the place of f, of g,
+    over g_ibi, and beginning in the middle of f."""
+    n = (41, 35, 38)
+    axes = [W.tanh_grid(-1, 1, q, 0.7) for q in n]
+    ctx = cfp.Context(*axes, [BALL])
+    ctx.classify_points()
+    gen = torch.Generator("cuda").manual_seed(3)
+
+    def field(m):
+        return torch.randn(m, dtype=torch.float64, device="cuda", generator=gen)
+
+    f, g, gi = field(ctx.N), field(ctx.N), field(ctx.n_ibi)
+    want = torch.empty(ctx.N, dtype=torch.float64, device="cuda")
+    ctx.assemble_rhs(f, g, gi, want)
+    room = torch.zeros(2 * ctx.N, dtype=torch.float64, device="cuda")
+    start = 0 if which != "shifted" else ctx.N // 2 + 1
+    src = {"f": f, "g": g, "g_ibi": gi, "shifted": f}[which]
+    inp, rhs = room[:src.numel()], room[start:start + ctx.N]
+    inp.copy_(src)
+    a = {"f": f, "g": g, "g_ibi": gi}
+    a["f" if which == "shifted" else which] = inp
+    ctx.assemble_rhs(a["f"], a["g"], a["g_ibi"], rhs)
+    assert torch.equal(rhs, want)
     ctx.close()
