@@ -300,6 +300,7 @@ struct cfp_ctx {
     int mg_fuse = 0;           // 1: and the fused black-then-red passes (opts.mg_tma == 2)
     int* dwait = nullptr;      // device word: nonzero once a bounded pipeline wait timed out
     int ring_grid = 0;         // CTAs of the apply ring's persistent grid (0: not set up)
+    int coarse_cl[2] = {0, 0}; // CTAs of the coarse levels' cluster, FP64 and FP32 (0: not used)
     std::vector<cfp::MgLevel> mg;
     // ILU(0) of K (CFP_PRECOND_ILU): [pivots | work field], FP64 and FP32
     double* ilu64 = nullptr;

@@ -1556,37 +1556,35 @@ void half_sweep(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colou
     }
 }
 
-// The cluster of k_coarse with shared levels: 16 CTAs where the device
-// schedules such a cluster (a non-portable size) with kCoarseSmem bytes each,
-// else 8, else 0 (not used); found once.
+// The cluster of k_coarse with shared levels: 16 CTAs where the context's
+// device schedules such a cluster (a non-portable size) with kCoarseSmem bytes
+// each, else 8, else 0 (not used).  Function attributes belong to a device, so
+// every context sets them and asks for itself (ensure_mg, before any capture).
 template <class T>
 int coarse_cluster_size() {
-    static const int size = []() {
-        int found = 0;
-        if (cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem) == cudaSuccess)
-            for (int cl : {16, 8}) {
-                cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3((unsigned)cl);
-                cfg.blockDim = dim3(kCoarseThreads);
-                cfg.dynamicSmemBytes = kCoarseSmem;
-                cudaLaunchAttribute at[1];
-                at[0].id = cudaLaunchAttributeClusterDimension;
-                at[0].val.clusterDim.x = (unsigned)cl;
-                at[0].val.clusterDim.y = 1;
-                at[0].val.clusterDim.z = 1;
-                cfg.attrs = at;
-                cfg.numAttrs = 1;
-                int n = 0;
-                if (cudaOccupancyMaxActiveClusters(&n, k_coarse<T>, &cfg) == cudaSuccess && n >= 1) {
-                    found = cl;
-                    break;
-                }
+    int found = 0;
+    if (cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCoarseSmem) == cudaSuccess)
+        for (int cl : {16, 8}) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)cl);
+            cfg.blockDim = dim3(kCoarseThreads);
+            cfg.dynamicSmemBytes = kCoarseSmem;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)cl;
+            at[0].val.clusterDim.y = 1;
+            at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, k_coarse<T>, &cfg) == cudaSuccess && n >= 1) {
+                found = cl;
+                break;
             }
-        cudaGetLastError();
-        return found;
-    }();
-    return size;
+        }
+    cudaGetLastError();
+    return found;
 }
 
 // k_coarse's arguments with level `first` as its first level; false where
@@ -1595,7 +1593,7 @@ int coarse_cluster_size() {
 template <class T>
 bool coarse_args(cfp_ctx* c, int first, CoarseArgs<T>* A, size_t* smem, int* cl) {
     const int nl = (int)c->mg.size() - first;
-    const int size = coarse_cluster_size<T>();
+    const int size = c->coarse_cl[sizeof(T) == 4];
     if (size == 0 || nl < 1 || nl > kCoarseLevels || c->mg[first].N > kCoarseMaxNodes) return false;
     A->nl = nl;
     A->ndist = 0;
@@ -1976,6 +1974,8 @@ cfp_status ensure_mg(cfp_ctx* c, int prec) {
         }
     }
     bool fresh32 = false;
+    if (prec == 0 && !c->mg[0].s64) c->coarse_cl[0] = coarse_cluster_size<double>();
+    if (prec == 1 && !c->mg[0].s32) c->coarse_cl[1] = coarse_cluster_size<float>();
     for (MgLevel& L : c->mg) {
         const size_t n = (size_t)kSplitVecs * L.Nh;
         if (prec == 0 && !L.s64) {

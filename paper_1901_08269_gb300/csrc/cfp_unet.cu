@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "cfp_internal.cuh"
+#include "cfp_device.cuh"
 #include "cfp_unet_kernels.cuh"
 #include "../../include/cfp_nn.h"
 
@@ -93,24 +94,22 @@ cfp_status aligned_act(const void* p) {
 }
 
 // ------------------------------------------------------ launch dispatch
+// the kernels' shared-memory attributes, on each device a call is made for
 template <int CIN, int COUT>
 cfp_status prep_conv() {
     using C = ConvCfg<CIN, COUT>;
     using W = WgCfg<CIN, COUT>;
-    static cfp_status st = []() {
-        if (cudaFuncSetAttribute(k_conv_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) !=
-                cudaSuccess ||
-            cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, W::SMEM) !=
-                cudaSuccess)
-            return CFP_ECUDA;
+    static OncePerDevice done;
+    int dev = 0;
+    CFP_CUDA(cudaGetDevice(&dev));
+    return done.run(dev, []() -> cfp_status {
+        CFP_CUDA(cudaFuncSetAttribute(k_conv_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+        CFP_CUDA(cudaFuncSetAttribute(k_wgrad_tc<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, W::SMEM));
         if constexpr (MarchCfg<CIN, COUT>::fits)
-            if (cudaFuncSetAttribute(k_conv_march<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     MarchCfg<CIN, COUT>::SMEM) != cudaSuccess)
-                return CFP_ECUDA;
+            CFP_CUDA(cudaFuncSetAttribute(k_conv_march<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          MarchCfg<CIN, COUT>::SMEM));
         return CFP_OK;
-    }();
-    if (st != CFP_OK) return fail(st, "cudaFuncSetAttribute failed for a convolution kernel");
-    return CFP_OK;
+    });
 }
 
 // k_conv_march's split for cap resident CTAs: the chunk with the least rounds x
