@@ -210,11 +210,12 @@ constexpr int kSweepPlanes = sizeof(T) == 8 ? 2 : 3;
 
 template <class T, int MODE, bool FINE>
 __global__ void __launch_bounds__(kSplitThreads)
-    k_sweep_split(SLev<T> L, Half<T> H, Side<T> S, int colour, const T* __restrict__ rho, T* __restrict__ phi) {
+    k_sweep_split(SLev<T> L, Half<T> H, Side<T> S, int colour, const T* __restrict__ rho, T* __restrict__ phi,
+                  unsigned z0) {
     constexpr bool F64 = sizeof(T) == 8, READ = MODE == 0 || MODE == 3;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
@@ -1026,10 +1027,10 @@ __global__ void __launch_bounds__(kPairThreads, 4)
 // loads first, and the fine level's Shortley-Weller rows, as in the
 // half-sweep.
 template <class T, bool FINE>
-__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S) {
+__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S, unsigned z0) {
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
@@ -1157,10 +1158,11 @@ __global__ void k_restrict_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
 // e1 += P e_c at the fine black unknowns (the red values are overwritten by
 // the next red half-sweep without being read); three planes per thread.
 template <class T>
-__global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
+__global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C,
+                                                                  unsigned z0) {
     const int nx = F.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
     if (2 * m > nx - 2 || j > F.ny - 2) return;
     const unsigned hc = (unsigned)C.hp;
     const IpPk<T> py = X.ip[1][j];
@@ -1322,11 +1324,21 @@ dim3 plane_block(const int n[3]) {
     const int bx = std::min(kSplitThreads, (n[0] / 2 + 31) / 32 * 32);
     return dim3((unsigned)bx, (unsigned)(kSplitThreads / bx));
 }
-template <class T>
-dim3 plane_grid(const int n[3]) {
+// launch(grid, block, z0) for the block rows z0 .. z0 + grid.z - 1 of a pass that
+// takes kSweepPlanes planes per block row: one launch up to 65535 block rows
+// (131072 planes in FP64, 196607 in FP32), as many as it takes above.  Returns
+// the launches.
+constexpr unsigned kMaxGridZ = 65535;
+template <class T, class F>
+int by_planes(const int n[3], F launch) {
     const dim3 b = plane_block(n);
-    return dim3((unsigned)((n[0] / 2 + b.x - 1) / b.x), (unsigned)((n[1] - 2 + b.y - 1) / b.y),
-                (unsigned)((n[2] - 2 + kSweepPlanes<T> - 1) / kSweepPlanes<T>));
+    const unsigned rows = (unsigned)((n[2] - 2 + kSweepPlanes<T> - 1) / kSweepPlanes<T>);
+    int count = 0;
+    for (unsigned z0 = 0; z0 < rows; z0 += kMaxGridZ, ++count)
+        launch(dim3((unsigned)((n[0] / 2 + b.x - 1) / b.x), (unsigned)((n[1] - 2 + b.y - 1) / b.y),
+                    std::min(rows - z0, kMaxGridZ)),
+               b, z0);
+    return count;
 }
 
 template <class T>
@@ -1521,13 +1533,13 @@ void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, co
 template <class T, int MODE>
 void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Half<T>& H, const Side<T>& S, int colour,
                         const T* rho, T* phi, cudaStream_t s) {
-    const dim3 g = plane_grid<T>(c->mg[l].n), blk = plane_block(c->mg[l].n);
     const bool after = MODE == 2 && sizeof(T) == 4 && c->mg[l].tma;
-    if (l == 0 && c->n_irr > 0 && !after) {
-        k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
-        return;
-    }
-    k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi);
+    const bool fine = l == 0 && c->n_irr > 0 && !after;
+    c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
+        if (fine) k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi, z0);
+        else k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi, z0);
+    });
+    if (fine) return;
     if constexpr (MODE == 2 && sizeof(T) == 4)
         if (l == 0) launch_sweep_fix<2>(c, L, H, S, colour, phi, s);
 }
@@ -1537,10 +1549,10 @@ void half_sweep(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colou
                 cudaStream_t s) {
     const Half<T> H{L.ty[colour], L.e[colour], L.e[1 - colour], L.b[colour], L.b[1 - colour], L.ty[1 - colour],
                     L.rd[colour]};
-    c->launches += 1;
     // the TMA-fed pass: plain, or the last black half-sweep of the fine level
     if (mode == 0 || (mode == 3 && colour == 1)) {
         if (sweep_tma(c, l, L, mode == 0 ? 0 : 2, colour, phi, s)) {
+            c->launches += 1;
             if constexpr (sizeof(T) == 4) {
                 if (l == 0 && mode == 0) launch_sweep_fix<0>(c, L, H, S, colour, phi, s);
                 else if (l == 0) launch_sweep_fix<3>(c, L, H, S, colour, phi, s);
@@ -2011,7 +2023,9 @@ void launch_prolong(cfp_ctx* c, int l, const SLev<T>& F, const SLev<T>& C, cudaS
         const dim3 g((unsigned)((Cn.n[0] - 1 + 127) / 128), (unsigned)(Cn.n[1] - 1), (unsigned)(Cn.n[2] - 1));
         k_prolong_cell<T><<<g, 128, 0, s>>>(transfer<T>(c->mg[l]), F, C);
     } else {
-        k_prolong_split<T><<<plane_grid<T>(c->mg[l].n), plane_block(c->mg[l].n), 0, s>>>(transfer<T>(c->mg[l]), F, C);
+        c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
+            k_prolong_split<T><<<g, blk, 0, s>>>(transfer<T>(c->mg[l]), F, C, z0);
+        }) - 1;  // the caller counts one
     }
 }
 
@@ -2044,9 +2058,10 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
                 }
             }
         } else {
-            const dim3 g = plane_grid<T>(c->mg[l].n), blk = plane_block(c->mg[l].n);
-            if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(F, S);
-            else k_resid_split<T, false><<<g, blk, 0, s>>>(F, S);
+            c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
+                if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(F, S, z0);
+                else k_resid_split<T, false><<<g, blk, 0, s>>>(F, S, z0);
+            }) - 1;  // counted below with the restriction
         }
         const MgLevel& Cn = c->mg[l + 1];
         const dim3 gr((unsigned)((Cn.n[0] - 2 + 127) / 128), (unsigned)(Cn.n[1] - 2), (unsigned)(Cn.n[2] - 2));
