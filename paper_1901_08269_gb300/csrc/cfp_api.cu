@@ -368,7 +368,7 @@ cfp_status cfp_precondition_ex(cfp_ctx* c, const cfp_opts* o, const double* rho,
     c->mg_fuse = opts.mg_tma == 2;
     cfp_status st = CFP_OK;
     if (c->precond_kind == CFP_PRECOND_MG || (c->precond_kind == CFP_PRECOND_RBGS && opts.sweeps > 0))
-        st = ensure_mg(c, prec);
+        st = ensure_mg(c, prec, c->precond_kind == CFP_PRECOND_MG);
     if (st == CFP_OK && c->precond_kind == CFP_PRECOND_ILU) st = ensure_ilu(c, prec);
     if (st == CFP_OK) {
         if (prec == 1) {

@@ -429,7 +429,7 @@ extern "C" cfp_status cfp_solve_fgmres(cfp_ctx* c, cfp_unet* net, const double* 
     c->mg_tma = opts.mg_tma != 0;
     c->mg_fuse = opts.mg_tma == 2;
     const bool mixed = opts.precision == CFP_PREC_MIXED;
-    if (c->precond_kind == CFP_PRECOND_MG || opts.sweeps > 0) CFP_TRY(ensure_mg(c, mixed ? 1 : 0));
+    if (c->precond_kind == CFP_PRECOND_MG || opts.sweeps > 0) CFP_TRY(ensure_mg(c, mixed ? 1 : 0, c->precond_kind == CFP_PRECOND_MG));
     CFP_TRY(ensure_work(c, mixed));
     const int64_t N = c->N;
     Fgm F;

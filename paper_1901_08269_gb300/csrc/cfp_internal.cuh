@@ -371,7 +371,8 @@ template <class T>
 void launch_precond(cfp_ctx* c, int sweeps, const T* rho, T* phi, cudaStream_t s);
 
 // multigrid (cfp_mg.cu)
-cfp_status ensure_mg(cfp_ctx* c, int prec);  // prec: 0 FP64 vectors, 1 FP32 vectors
+// prec: 0 FP64 vectors, 1 FP32 vectors; vcycle: for V-cycles, not only the fine level's sweeps
+cfp_status ensure_mg(cfp_ctx* c, int prec, bool vcycle = false);
 void free_mg(cfp_ctx* c);
 template <class T>
 void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s);

@@ -611,7 +611,7 @@ cfp_status cfp::solve_impl(cfp_ctx* c, const double* f, const double* g, const d
     const bool mixed = opts.precision == CFP_PREC_MIXED;
     // the multigrid option and the red-black sweeps (on the fine level's split arrays)
     if (c->precond_kind == CFP_PRECOND_MG || (c->precond_kind == CFP_PRECOND_RBGS && opts.sweeps > 0))
-        CFP_TRY(ensure_mg(c, mixed ? 1 : 0));
+        CFP_TRY(ensure_mg(c, mixed ? 1 : 0, c->precond_kind == CFP_PRECOND_MG));
     if (c->precond_kind == CFP_PRECOND_ILU) CFP_TRY(ensure_ilu(c, mixed ? 1 : 0));
     CFP_TRY(ensure_work(c, mixed));
     const int64_t N = c->N;
@@ -1002,7 +1002,7 @@ cfp_status prepare_device_solve(cfp_ctx* c, const cfp_opts& opts) {
     c->mg_tma = opts.mg_tma != 0;
     c->mg_fuse = opts.mg_tma == 2;
     if (c->precond_kind == CFP_PRECOND_MG || (c->precond_kind == CFP_PRECOND_RBGS && opts.sweeps > 0))
-        CFP_TRY(ensure_mg(c, 1));
+        CFP_TRY(ensure_mg(c, 1, c->precond_kind == CFP_PRECOND_MG));
     if (c->precond_kind == CFP_PRECOND_ILU) CFP_TRY(ensure_ilu(c, 1));
     CFP_TRY(ensure_work(c, true));
     return CFP_OK;

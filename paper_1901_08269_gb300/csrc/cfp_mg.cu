@@ -1977,7 +1977,7 @@ cfp_status setup_tma(cfp_ctx* c) {
 // Build the hierarchy if needed and the split vectors of precision `prec`
 // (0: FP64, 1: FP32), zero-filled: entries that are never written (the
 // non-unknowns, the box, the black residuals) must read as zero.
-cfp_status ensure_mg(cfp_ctx* c, int prec) {
+cfp_status ensure_mg(cfp_ctx* c, int prec, bool vcycle) {
     if (c->mg.empty()) {
         const cfp_status st = build_levels(c);
         if (st != CFP_OK) {
@@ -1985,6 +1985,13 @@ cfp_status ensure_mg(cfp_ctx* c, int prec) {
             return st;
         }
     }
+    // The V-cycle's transfers take a block row per coarse row and plane.  Refused
+    // here, before a solve captures its loop: refused by CUDA within the capture,
+    // they brought the process down.
+    if (vcycle && c->mg.size() > 1)
+        for (int d = 1; d < 3; ++d)
+            if (c->mg[1].n[d] - (c->mg_tma ? 1 : 2) > (int)kMaxGridZ)
+                return fail(CFP_ECUDA, "grid too long in y or z for the multigrid transfers (65536 coarse nodes)");
     bool fresh32 = false;
     if (prec == 0 && !c->mg[0].s64) c->coarse_cl[0] = coarse_cluster_size<double>();
     if (prec == 1 && !c->mg[0].s32) c->coarse_cl[1] = coarse_cluster_size<float>();

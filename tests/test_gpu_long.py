@@ -40,3 +40,25 @@ def test_red_black_sweeps_along_a_long_axis(precision, nz, unit):
         ctx.close()
     assert np.max(np.abs(out["z"])) > 0 and np.all(np.isfinite(out["z"]))
     assert np.max(np.abs(out["z"] - out["x"])) <= 512 * unit * np.max(np.abs(out["x"]))
+
+
+def test_multigrid_on_too_long_a_grid_is_refused():
+    """The V-cycle's transfers take one block row per coarse plane: 70001 of
+    them are refused, by the solve (whose loop is captured) as by the
+    preconditioner, every time, and the context goes on."""
+    axes = [W.uniform_grid(-1, 1, n) for n in (17, 17, 140001)]
+    ctx = cfp.Context(*axes)
+    ctx.classify_points()
+    f = torch.ones(ctx.N, dtype=torch.float64, device="cuda")
+    g = torch.zeros_like(f)
+    for _ in range(2):
+        u = torch.zeros_like(f)
+        with pytest.raises(cfp.CfpError) as e:
+            ctx.solve(f, g, None, u, tol=1e-10, precond=cfp.PRECOND_MG, maxit=2)
+        assert e.value.status == cfp.ECUDA
+        with pytest.raises(cfp.CfpError) as e:
+            ctx.precondition_ex(f, u, precond=cfp.PRECOND_MG)
+        assert e.value.status == cfp.ECUDA
+    ctx.precondition(f, u, sweeps=1)
+    assert float(u.abs().max()) > 0.0
+    ctx.close()
