@@ -448,19 +448,20 @@ enum { CFP_APPLY_STREAM = 1,  /* each thread streams its column of `rows`
  * precision (CFP_PREC_FP64, or CFP_PREC_MIXED for the FP32 apply of the
  * mixed solve's inner iterations): the kernel (CFP_APPLY_STREAM with 2 or 4
  * rows per thread and 16, 32 or 64 planes a CTA marches in z;
- * CFP_APPLY_RING, FP32 only, 2 rows per tile and 32 or 64 planes).
- * kernel = rows = planes = 0: every candidate (the context's own shape by grid
- * size, 6 others in FP64, 8 in FP32) is timed (CUDA events, 5 launches after
- * two untimed, on the context's work vectors) and the fastest is kept by the context for its later solves;
- * otherwise that choice is set and timed.  The rows of B x do not depend on the choice (the same fused
- * multiply-add chain per row in every kernel); the dot products fused into
- * the apply are summed per CTA, so their rounding does.  Without a call the
- * context uses CFP_APPLY_STREAM in FP64, in a shape that spreads the grid over
- * the SMs (cfp_apply_shape reports it as 4 rows x 64 planes); in FP32
- * CFP_APPLY_RING from 2^23 nodes on where its tiles (512 columns, 256 where
- * n_x <= 258) are at least 85 % filled by the n_x - 2 interior columns, in
- * chunks of planes that make about 1024 tiles (reported as 2 x 64), else
- * CFP_APPLY_STREAM, again in a shape by grid size (reported as 4 x 64).
+ * CFP_APPLY_RING, FP32 only, 2 rows per tile and 32 or 64 planes), or the
+ * shape by grid size that contexts use without a call.
+ * kernel = rows = planes = 0: every candidate (the shape by grid size, 6
+ * others in FP64, 8 in FP32) is timed (CUDA events, 5 launches after two
+ * untimed, on the context's work vectors) and the fastest is kept by the
+ * context for its later solves; otherwise that choice is set and timed.  The
+ * rows of B x do not depend on the choice (the same fused multiply-add chain
+ * per row in every kernel); the dot products fused into the apply are summed
+ * per CTA, so their rounding does.  By grid size: in FP64 CFP_APPLY_STREAM
+ * with 1, 2 or 4 rows and 2 to 64 planes that spread the grid over the SMs;
+ * in FP32 CFP_APPLY_RING from 2^23 nodes on where its tiles (512 columns, 256
+ * where n_x <= 258) are at least 85 % filled by the n_x - 2 interior columns,
+ * in chunks of 64 to 128 planes that make about 1024 tiles (64 beside
+ * irregular points), else CFP_APPLY_STREAM with 2 to 64 planes.
  *   ms  NULL or the chosen candidate's mean time per launch.
  * Requires classification.  Synchronises.  Errors: CFP_ESTATE, CFP_EINVAL
  * (a choice outside those values, or CFP_APPLY_RING with CFP_PREC_FP64 or
@@ -470,8 +471,8 @@ cfp_status cfp_tune_apply(cfp_ctx* ctx, int precision, int kernel, int rows, int
 
 /*
  * The apply's kernel and tile shape the context uses for `precision` (set
- * by cfp_tune_apply or the default), as cfp_tune_apply takes them: for
- * instance to give contexts of one grid size the shape tuned on one of them.
+ * by cfp_tune_apply or by grid size), as cfp_tune_apply takes them on contexts
+ * of that grid size: for instance to give them the shape tuned on one of them.
  * Outputs may be NULL.  Errors: CFP_EINVAL.
  */
 cfp_status cfp_apply_shape(const cfp_ctx* ctx, int precision, int* kernel, int* rows, int* planes);

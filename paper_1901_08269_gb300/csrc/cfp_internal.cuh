@@ -410,6 +410,7 @@ cfp_status assemble_rhs(cfp_ctx* c, const double* f, const double* g, const doub
 bool setup_apply_ring(cfp_ctx* c);
 // the kernel and tile shape the apply of precision q (0 FP64, 1 FP32) runs with
 void apply_shape(const cfp_ctx* c, int q, int* kernel, int* rows, int* planes);
+bool shape_by_size(const cfp_ctx* c, int q, int kernel, int rows, int planes, bool* own);
 // phi = P(rho) in FP32 (the mixed solve's inner preconditioner) for FP64
 // fields: rho rounded to FP32, phi widened back; phi zeroed first
 cfp_status precondition32(cfp_ctx* c, int sweeps, const double* rho, double* phi);

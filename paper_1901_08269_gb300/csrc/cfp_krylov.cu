@@ -489,7 +489,7 @@ cfp_status time_kernel_t(cfp_ctx* c, int prec, int kernel, int reps, double* ms,
 // the FP32 ring with 2 rows per tile) x planes per z chunk, each candidate
 // timed over `reps` launches (after two untimed) with the fused (r_hat0, v)
 // dot, the fastest kept in the context.  kind, rows, planes > 0: that choice
-// is set and timed only.
+// (one of these, or the shape by grid size) is set and timed only.
 cfp_status tune_apply(cfp_ctx* c, int prec, int kind, int rows, int planes, int reps, double* best_ms) {
     const int q = prec == CFP_PREC_MIXED ? 1 : 0;
     struct Choice {
@@ -500,9 +500,10 @@ cfp_status tune_apply(cfp_ctx* c, int prec, int kind, int rows, int planes, int 
     if (kind > 0 || rows > 0 || planes > 0) {
         const bool shape = kind == CFP_APPLY_STREAM ? (rows == 2 || rows == 4) && (planes == 16 || planes == 32 || planes == 64)
                                                     : kind == CFP_APPLY_RING && rows == 2 && (planes == 32 || planes == 64);
-        if (!shape)
+        bool own;
+        if (!shape && !shape_by_size(c, q, kind, rows, planes, &own))  // as taken over from another context
             return fail(CFP_EINVAL, "apply: kernel 1 with rows 2 or 4 and planes 16, 32 or 64, or kernel 2 with "
-                                    "rows 2 and planes 32 or 64");
+                                    "rows 2 and planes 32 or 64, or the shape by grid size");
         if (kind == CFP_APPLY_RING && !ring)
             return fail(CFP_EINVAL, "apply ring: FP32 only, and its launch could not be set up");
         cand.push_back({kind, rows, planes});
@@ -526,6 +527,11 @@ cfp_status tune_apply(cfp_ctx* c, int prec, int kind, int rows, int planes, int 
             bs = ch;
         }
     }
+    // what the context would run with anyway is left to go by size, so that it
+    // is the same here and where it is taken over to (by size, the FP32 apply
+    // without a dot product has a shape of its own)
+    bool own = false;
+    if (bs.kind && shape_by_size(c, q, bs.kind, bs.ty, bs.kc, &own) && own) bs = Choice{0, 0, 0};
     c->apply_kind[q] = bs.kind;
     c->apply_ty[q] = bs.ty;
     c->apply_kc[q] = bs.kc;

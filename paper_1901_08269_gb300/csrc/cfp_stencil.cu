@@ -1115,25 +1115,24 @@ namespace {
 // the ring's tile width: 256 only where a tile spans the row (copied row by row,
 // 256-column tiles of 513^3 took 443 us, 512-column ones 354)
 int ring_tx(const cfp_ctx* c) { return c->n[0] <= RingTile<256>::span_nx ? 256 : 512; }
-// planes per z chunk where the tuner set none: some 1024 tiles, of 64 to 128
-// planes (513^3: 128 336 us, 64 354); beside the irregular rows' kernel, whose
-// CTAs delay some of the ring's, few rounds of tiles lose least (bodies, 257^3:
-// 64 67 us, 24 87; 513^3: 64 412, 128 422)
-int ring_planes(const cfp_ctx* c) {
-    if (c->apply_kc[1]) return std::max(32, c->apply_kc[1]);
+// planes per z chunk by grid size: some 1024 tiles, of 64 to 128 planes (513^3:
+// 128 336 us, 64 354); beside the irregular rows' kernel, whose CTAs delay some
+// of the ring's, few rounds of tiles lose least (bodies, 257^3: 64 67 us, 24 87;
+// 513^3: 64 412, 128 422)
+int ring_planes_by_size(const cfp_ctx* c, bool irregular) {
     const int tx = ring_tx(c), rows = 4 * kRingCons / tx;
     const int64_t col = (int64_t)((c->n[0] - 2 + tx - 1) / tx) * ((c->n[1] - 2 + rows - 1) / rows);
-    return c->n_irr > 0 ? 64 : (int)std::max<int64_t>(64, std::min<int64_t>(128, col * (c->n[2] - 2) / 1024));
+    return irregular ? 64 : (int)std::max<int64_t>(64, std::min<int64_t>(128, col * (c->n[2] - 2) / 1024));
 }
-// the apply's kernel and tile shape of precision q (0 FP64, 1 FP32), as set
-// by the autotuner; otherwise in FP64 the shape apply64_shape finds, in FP32 the
-// ring from 2^23 nodes on where its tiles' columns are at least 85 % filled
-// (257^3 55 us against the streaming kernel's 68, 225^3 45 : 55, 449 x 385 x 321
-// 174 : 180, 513^3 337 : 406; but 257 x 129 x 65 18 : 12, 385^3 205 : 181) and else
-// the streaming kernel (apply32_shape).  The shapes found are reported as 4 x
-// 64, the ring's as 2 x 64.
-int apply_kind(const cfp_ctx* c, int q) {
-    if (c->apply_kind[q]) return c->apply_kind[q];
+int ring_planes(const cfp_ctx* c) {
+    return c->apply_kc[1] ? std::max(32, c->apply_kc[1]) : ring_planes_by_size(c, c->n_irr > 0);
+}
+// the apply's kernel of precision q (0 FP64, 1 FP32) by grid size: in FP64 the
+// streaming kernel, in FP32 the ring from 2^23 nodes on where its tiles' columns
+// are at least 85 % filled (257^3 55 us against the streaming kernel's 68, 225^3
+// 45 : 55, 449 x 385 x 321 174 : 180, 513^3 337 : 406; but 257 x 129 x 65 18 : 12,
+// 385^3 205 : 181) and else the streaming kernel
+int kind_by_size(const cfp_ctx* c, int q) {
     if (q == 1 && c->ring_grid > 0) {
         const int cols = c->n[0] - 2, tx = ring_tx(c), tiles = (cols + tx - 1) / tx;
         const int64_t nodes = (int64_t)cols * (c->n[1] - 2) * (c->n[2] - 2);
@@ -1141,8 +1140,7 @@ int apply_kind(const cfp_ctx* c, int q) {
     }
     return CFP_APPLY_STREAM;
 }
-int apply_rows(const cfp_ctx* c, int q) { return c->apply_ty[q] ? c->apply_ty[q] : 4; }
-int apply_planes(const cfp_ctx* c, int q) { return c->apply_kc[q] ? c->apply_kc[q] : 64; }
+int apply_kind(const cfp_ctx* c, int q) { return c->apply_kind[q] ? c->apply_kind[q] : kind_by_size(c, q); }
 
 // k_apply64's rows per thread and planes per z chunk
 struct Shape {
@@ -1158,8 +1156,8 @@ struct Shape {
     }
 };
 
-// The launch shape of k_apply64 (where the tuner set none) and k_rhs_source:
-// the one with the smallest estimate.  A warp issues w = (kc + 2) (row (ty +
+// The launch shape of k_apply64 (where the tuner set none) and k_rhs_source
+// by grid size: the one with the smallest estimate.  A warp issues w = (kc + 2) (row (ty +
 // 2) + yout ty) + zout kc ty FP64 instructions (row per loaded row, yout and
 // zout per output row in y and z: 5, 7, 6 in the apply; its two halo planes do
 // the x and y passes only), a CTA 4 w; the estimate is the busiest of 152 SMs, the latency of a plane's loads
@@ -1185,9 +1183,10 @@ Shape shape64(const cfp_ctx* c, double row, double yout, double zout) {
         }
     return best;
 }
+Shape apply64_by_size(const cfp_ctx* c) { return shape64(c, 5.0, 7.0, 6.0); }
 Shape apply64_shape(const cfp_ctx* c) {
     if (c->apply_ty[0] && c->apply_kc[0]) return Shape{c->apply_ty[0], c->apply_kc[0]};
-    return shape64(c, 5.0, 7.0, 6.0);
+    return apply64_by_size(c);
 }
 
 // The FP32 streaming kernel is bound by the latency of a plane's loads, so its
@@ -1196,8 +1195,7 @@ Shape apply64_shape(const cfp_ctx* c) {
 // some 6 for a round's start (257^3: 4 x 64 68 us, 4 x 8 78; 129^3: 4 x 8 12.4,
 // 4 x 16 14.5; 321 x 257 x 289: 4 x 32 91, 4 x 64 106).  Without a dot product 2 rows take 0.65 of it
 // (513^3 361 us against 390), with one more (448 against 406).
-Shape apply32_shape(const cfp_ctx* c, bool dot) {
-    if (c->apply_ty[1] && c->apply_kc[1]) return Shape{c->apply_ty[1], c->apply_kc[1]};
+Shape apply32_by_size(const cfp_ctx* c, bool dot) {
     Shape best{4, 64};
     double est_best = 1e300;
     for (int t : {4, 2})
@@ -1214,14 +1212,43 @@ Shape apply32_shape(const cfp_ctx* c, bool dot) {
     return best;
 }
 
+Shape apply32_shape(const cfp_ctx* c, bool dot) {
+    // (a ring's planes, where the streaming kernel takes its place, may be more
+    // than it stages coefficients for)
+    if (c->apply_ty[1] && c->apply_kc[1]) return Shape{c->apply_ty[1], std::min(c->apply_kc[1], kMaxPlanes)};
+    return apply32_by_size(c, dot);
+}
+
 }  // namespace
 
-// the kernel and tile shape the apply of precision q runs with, as a shape
-// that can be set
+// the kernel and tile shape the apply of precision q runs with (FP32: with a
+// dot product, as in a solve)
 void apply_shape(const cfp_ctx* c, int q, int* kernel, int* rows, int* planes) {
     *kernel = apply_kind(c, q);
-    *rows = *kernel == CFP_APPLY_RING ? 2 : apply_rows(c, q);
-    *planes = apply_planes(c, q);
+    if (*kernel == CFP_APPLY_RING) {
+        *rows = 2;
+        *planes = ring_planes(c);
+        return;
+    }
+    const Shape sh = q == 0 ? apply64_shape(c) : apply32_shape(c, true);
+    *rows = sh.ty;
+    *planes = sh.kc;
+}
+
+// Whether a shape is one that apply_shape reports for contexts of this grid
+// size that no tuner touched, with or without irregular points, before and
+// after their ring is set up.  *own: it is what this context would run with.
+bool shape_by_size(const cfp_ctx* c, int q, int kernel, int rows, int planes, bool* own) {
+    *own = false;
+    if (kernel == CFP_APPLY_RING) {
+        if (q == 0 || rows != 2) return false;
+        *own = kind_by_size(c, q) == CFP_APPLY_RING && planes == ring_planes_by_size(c, c->n_irr > 0);
+        return planes == ring_planes_by_size(c, false) || planes == ring_planes_by_size(c, true);
+    }
+    const Shape sh = q == 0 ? apply64_by_size(c) : apply32_by_size(c, true);
+    const bool same = kernel == CFP_APPLY_STREAM && rows == sh.ty && planes == sh.kc;
+    *own = same && kind_by_size(c, q) == CFP_APPLY_STREAM;
+    return same;
 }
 
 namespace {
