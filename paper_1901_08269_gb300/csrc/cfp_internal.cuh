@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda.h>  // CUtensorMap (types only; the encoder is fetched from the CUDA driver at run time)
+#include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -426,6 +427,8 @@ cfp_status diag_bounded_wait(cfp_ctx* c);
 cudaStream_t unet_use_stream(cfp_unet* u, cudaStream_t s);
 int64_t unet_launches(const cfp_unet* u);
 cfp_ctx* unet_owner(const cfp_unet* u);
+// cuTensorMapEncodeTiled (NULL: the driver has none)
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 // FP64 vector helpers over all N nodes: dot (synchronises), y = alpha x + beta y
 cfp_status vec_dot(cfp_ctx* c, const double* a, const double* b, double* out);
 cfp_status vec_axpby(cfp_ctx* c, double alpha, const double* x, double beta, double* y);

@@ -39,7 +39,6 @@
 #include <vector>
 
 #include <cooperative_groups.h>
-#include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 
 #include "cfp_internal.cuh"
 
@@ -1885,6 +1884,8 @@ cfp_status build_levels(cfp_ctx* c) {
 
 namespace {
 
+}  // namespace
+
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
 // (the library does not link libcuda)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
@@ -1899,6 +1900,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     }();
     return fn;
 }
+
+namespace {
 
 // 3D map (x = entry in a row of hp, y = row, z = plane) of one colour array
 // with a box of bx x by x 1 elements; out-of-array elements read as zero

@@ -1,5 +1,5 @@
 // Blackwell (sm_103a) building blocks of the learned part's tensor-core
-// kernels, as inline PTX: mbarriers with bounded waits, bulk copies
+// kernels, as inline PTX: mbarriers with bounded waits, TMA tiled and bulk copies
 // into shared memory, tcgen05 shared-memory descriptors, MMA issue,
 // commit, tensor-memory allocation and loads.
 //
@@ -62,6 +62,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
     }
 }
 
+// 2D tiled copy global -> shared, completion counted on bar (bytes)
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+            smem_u32(dst)),
+        "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+        : "memory");
+}
 // contiguous copy global -> shared (16-byte aligned ends, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
     asm volatile(

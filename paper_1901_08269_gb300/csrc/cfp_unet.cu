@@ -87,6 +87,22 @@ unsigned blocks(int64_t n, int per = 256) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 152 * 32));
 }
 
+// Activation (Np x C BF16) as a 2D tensor (channels innermost) with a box of
+// 8 channels x one window's rows; rows outside [0, Np) read as zero.
+cfp_status act_map(CUtensorMap* m, const void* base, int C, int Np) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc) return fail(CFP_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    const cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)Np};
+    const cuuint64_t strides[1] = {(cuuint64_t)C * 2};
+    const cuuint32_t box[2] = {8, (cuuint32_t)kWin};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(CFP_ECUDA, "cuTensorMapEncodeTiled failed for an activation");
+    return CFP_OK;
+}
+
 // the producers copy 16 bytes at a time
 cfp_status aligned_act(const void* p) {
     if (((uintptr_t)p & 15) != 0) return fail(CFP_EINVAL, "activation arrays must be 16-byte aligned");
@@ -117,13 +133,12 @@ cfp_status prep_conv() {
 // 15 % of its tiles' rows empty (k_conv_tc's tiles run on across planes)
 March march_split(const Pad& P, int cap) {
     const int plane = P.nxp * P.nyp;
-    March M{(plane + 127) / 128, 1, P.nzp};
-    if ((int64_t)plane * 100 < (int64_t)M.tiles * 128 * 85) return March{0, 0, 0};
-    int64_t best = INT64_MAX;
+    March M{(plane + 127) / 128, 1, P.nzp, INT64_MAX};
+    if ((int64_t)plane * 100 < (int64_t)M.tiles * 128 * 85) return March{0, 0, 0, 0};
     for (int z = P.nzp; z >= 1; --z) {
         const int64_t chunks = (P.nzp + z - 1) / z, est = ((int64_t)M.tiles * chunks + cap - 1) / cap * (z + 2);
-        if (est < best) {
-            best = est;
+        if (est < M.cost) {
+            M.cost = est;
             M.planes = z;
             M.chunks = (int)chunks;
         }
@@ -151,15 +166,22 @@ cfp_status conv_t(cudaStream_t s, const uint16_t* in, const uint16_t* wsrc, bool
     if constexpr (MarchCfg<CIN, COUT>::fits) {
         using C = MarchCfg<CIN, COUT>;
         const March M = march_split(P, C::PER * num_sms());
-        if (M.tiles > 0) {
+        // 32 -> 64, where k_conv_tc has its windows by TMA: a plane here takes
+        // about 4/5 of a tile there (100 x 90 x 30, 18 planes : 16 tiles 59.5 us
+        // against 61; 129 x 97 x 65, 57 : 45 179 against 163)
+        const int64_t tiles = ((P.Np + 127) / 128 + num_sms() - 1) / num_sms();
+        if (M.tiles > 0 && (!ConvCfg<CIN, COUT>::TMA || 4 * M.cost <= 5 * tiles)) {
             k_conv_march<CIN, COUT><<<M.tiles * M.chunks, kConvThreads, C::SMEM, s>>>(in, wpk, bias, act, P, M, flags,
                                                                                       out_bf, out_f, err);
             CFP_CUDA(cudaGetLastError());
             return CFP_OK;
         }
     }
-    k_conv_tc<CIN, COUT><<<conv_grid<CIN, COUT>(P), kConvThreads, C::SMEM, s>>>(
-        in, wpk, bias, act, P, flags, out_bf, out_f, err);
+    typename C::In src;
+    if constexpr (C::TMA) CFP_TRY(act_map(&src, in, CIN, P.Np));
+    else src = in;
+    k_conv_tc<CIN, COUT><<<conv_grid<CIN, COUT>(P), C::THREADS, C::SMEM, s>>>(src, wpk, bias, act, P, flags, out_bf,
+                                                                              out_f, err);
     CFP_CUDA(cudaGetLastError());
     return CFP_OK;
 }

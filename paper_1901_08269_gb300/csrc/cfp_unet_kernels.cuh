@@ -12,21 +12,24 @@
 // (t/3)%3 - 1, t%3 - 1):
 //     out[v][co] = bias[co] + sum_t sum_ci W[co][t][ci] in[v + off(t)][ci].
 //
-// Forward convolution (k_conv_tc; k_conv_march up to 32 input channels): the implicit GEMM D (128 voxels x Cout) =
+// Forward convolution (k_conv_tc; k_conv_march for 16 -> 16 and 16 -> 32
+// channels and some 32 -> 64 ones): the implicit GEMM D (128 voxels x Cout) =
 // sum over taps of A_t (128 x Cin) B_t^T.  For each (dy, dz) pair one window
 // of 130 rows (the 128 outputs and one row either side) serves the three taps
 // dx = -1, 0, 1, whose A operands start 0, 16 and 32 bytes into it (K-major,
 // no swizzle).  The weights of the three taps come with it, in the operand
 // layout (k_wpack), as one bulk copy.  The input gradient is the same kernel
 // on flipped, transposed weights.
-// The windows are copied by four producer warps with 16-byte cp.async: the
-// operand layout scatters a row's 8-channel pieces over planes, which the TMA
-// engine does 16 bytes at a time (about two cycles each: 2340 pieces per tile
-// bound the 16-channel layers to 5 % of the tensor pipe), while the copies of
-// 128 threads run at the shared-memory write rate.  Weight gradient (k_wgrad_tc): D_t (Cin x
-// Cout) = sum over voxels of X(v + off_t)^T G(v), both operands MN-major, the
-// voxel shift again a start-address offset.  The windows of 128 / Cin (dy, dz)
-// pairs lie one after the other in a stage, so one MMA's 128 rows are that
+// The operand layout scatters a row's 8-channel pieces over planes.  With 32
+// channels or more in and out the windows come by TMA, a box per plane.  With
+// fewer the MMAs of a window are over before the TMA engine has placed it 16
+// bytes at a time (2340 pieces per tile bound the 16-channel layers to 5 % of
+// the tensor pipe), and four producer warps copy the windows with 16-byte
+// cp.async at the shared-memory write rate instead.
+// Weight gradient (k_wgrad_tc): D_t (Cin x Cout) = sum over voxels of
+// X(v + off_t)^T G(v), both operands MN-major, the voxel shift again a
+// start-address offset, windows by cp.async.  The windows of 128 / Cin (dy,
+// dz) pairs lie one after the other in a stage, so one MMA's 128 rows are that
 // many pairs' channels (with 16 channels a single pair would leave seven of
 // eight rows idle, and reading the operand is what an MMA of 16 columns
 // costs).  Per-chunk partials are summed in a fixed order (deterministic).
@@ -53,6 +56,7 @@ constexpr int kWin = 130;             // rows of a window: 128 outputs + one eit
 // together, fall into different banks
 constexpr int kPlane = 137 * 16;
 constexpr int kGPlane = 129 * 16;
+constexpr int kTmaPlane = 136 * 16;   // of a window copied by TMA (destinations on 128-byte boundaries)
 constexpr int kConvThreads = 288;     // warps 0-3 epilogue, 4-7 producers, 8 MMA issuer
 constexpr int kProd = 128;            // producer threads
 
@@ -110,9 +114,22 @@ struct ConvCfg {
     static constexpr int KB = CIN < 64 ? CIN : 64;  // input channels per stage
     static constexpr int NKB = CIN / KB;
     static constexpr int NCH = KB / 8;              // 8-channel planes per stage
-    static constexpr int A_BYTES = NCH * kPlane;
+    // The windows by TMA (one producer thread), or by cp.async (four warps) where
+    // a stage has few channels in or out: the TMA engine takes about two cycles
+    // per 16-byte piece whatever the MMAs that wait for it do, the threads'
+    // copies cost issue slots and a fence.  By TMA and by cp.async, us: 32 -> 32
+    // at 129^3 369 : 427 (k_conv_march), 64 -> 64 736 : 807, 64 -> 128 at 65^3
+    // 132 : 146, 128 -> 128 at 129^3 1667 : 1789, at 17^3 19.9 : 21.2; but 32 ->
+    // 16 at 65^3 55 : 52, 16 -> 32 42 : 30 (k_conv_march).
+    static constexpr bool TMA = CIN >= 32 && COUT >= 32;
+    using In = std::conditional_t<TMA, CUtensorMap, const uint16_t*>;
+    static constexpr int PWARPS = TMA ? 1 : kProd / 32;
+    static constexpr int THREADS = 32 * (5 + PWARPS);
+    static constexpr int PLANE = TMA ? kTmaPlane : kPlane;
+    static constexpr int A_BYTES = NCH * PLANE;
     static constexpr int W_TAP = NCH * COUT * 16;   // one tap's weights for the stage's channels
     static constexpr int W_BYTES = 3 * W_TAP;
+    static constexpr unsigned TX = W_BYTES + (TMA ? NCH * kWin * 16 : 0);  // bytes counted on a stage's barrier
     static constexpr int STAGE = rup(A_BYTES + W_BYTES, 128);
     static constexpr int S0 = (196 * 1024) / STAGE;
     static constexpr int STAGES = S0 > 8 ? 8 : S0;
@@ -232,8 +249,8 @@ __device__ __forceinline__ void conv_rows(unsigned acc, int row, bool valid, con
 // a code in *err and that role stops issuing; every issued copy and MMA is
 // waited for (bounded) before the tensor memory is released.
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
-    k_conv_tc(const uint16_t* __restrict__ in, const uint16_t* __restrict__ wpk,
+__global__ void __launch_bounds__(ConvCfg<CIN, COUT>::THREADS, ConvCfg<CIN, COUT>::PER)
+    k_conv_tc(const __grid_constant__ typename ConvCfg<CIN, COUT>::In in, const uint16_t* __restrict__ wpk,
               const float* __restrict__ bias, const uint16_t* __restrict__ act, Pad P, int flags,
               uint16_t* __restrict__ out_bf, float* __restrict__ out_f, int* __restrict__ err) {
     using C = ConvCfg<CIN, COUT>;
@@ -249,7 +266,7 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int q = 0; q < S; ++q) {
-            tc::mbar_init(&full[q], 1 + kProd);  // the weights' bytes; the producer threads
+            tc::mbar_init(&full[q], C::TMA ? 1 : 1 + kProd);  // the bytes counted; the copying threads
             tc::mbar_init(&empty[q], 1);
         }
         for (int q = 0; q < 2; ++q) {
@@ -266,7 +283,7 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
     const unsigned tmem = *tslot;
     const int ntiles = (P.Np + 127) / 128;
 
-    if (warp >= 4 && warp < 8) {  // producers
+    if (warp >= 4 && warp < 4 + C::PWARPS && (!C::TMA || lane == 0)) {  // producers
         const int p = threadIdx.x - 128;
         unsigned g = 0;
         bool ok = true;
@@ -278,23 +295,29 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
                     free = 0;
                     atomicExch(err, 11);
                 }
-                ok = __shfl_sync(0xffffffffu, free, 0);
+                ok = C::TMA ? free : __shfl_sync(0xffffffffu, free, 0);
                 if (!ok) break;
                 unsigned char* buf = base + st * C::STAGE;
+                const int row0 = tile * 128 + ((gi / 3 - 1) * P.nyp + (gi % 3 - 1)) * P.nxp - 1;
                 if (p == 0) {
-                    tc::mbar_arrive_expect_tx(&full[st], C::W_BYTES);
+                    tc::mbar_arrive_expect_tx(&full[st], C::TX);
+                    if constexpr (C::TMA)
+#pragma unroll
+                        for (int c = 0; c < C::NCH; ++c)
+                            tc::tma_load_2d(buf + c * C::PLANE, &in, &full[st], (kb * C::NCH + c) * 8, row0);
                     tc::bulk_load(buf + C::A_BYTES, wpk + (size_t)(kb * 9 + gi) * (C::W_BYTES / 2), C::W_BYTES, &full[st]);
                 }
-                const int row0 = tile * 128 + ((gi / 3 - 1) * P.nyp + (gi % 3 - 1)) * P.nxp - 1;
-                copy_rows<C::NCH, kPlane>(tc::smem_u32(buf), in, CIN, kb * C::NCH, row0, kWin, P.Np, p);
-                copy_arrive(&full[st]);
+                if constexpr (!C::TMA) {
+                    copy_rows<C::NCH, C::PLANE>(tc::smem_u32(buf), in, CIN, kb * C::NCH, row0, kWin, P.Np, p);
+                    copy_arrive(&full[st]);
+                }
             }
         }
-        copy_wait_all();
+        if constexpr (!C::TMA) copy_wait_all();
         if (p == 0)  // every bulk copy issued has landed before the CTA may end
             for (unsigned q = g > (unsigned)S ? g - S : 0; q < g; ++q)
                 if (!tc::mbar_wait(&full[q % S], (q / S) & 1)) atomicExch(err, 12);
-    } else if (warp == 8 && lane == 0) {  // MMA issuer
+    } else if (warp == 4 + C::PWARPS && lane == 0) {  // MMA issuer
         constexpr unsigned idesc = tc::idesc_bf16(128, COUT, 0, 0);
         unsigned g = 0, tl = 0;
         bool ok = true;
@@ -314,14 +337,14 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
                     atomicExch(err, 14);
                     break;
                 }
-                async_after();
+                if constexpr (!C::TMA) async_after();
                 tc::fence_after();
                 const unsigned ab = tc::smem_u32(base + st * C::STAGE), wb = ab + C::A_BYTES;
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
                     for (int q = 0; q < C::NCH / 2; ++q) {
-                        const uint64_t da = tc::sdesc(ab + dx * 16 + q * 2 * kPlane, kPlane, 128);
+                        const uint64_t da = tc::sdesc(ab + dx * 16 + q * 2 * C::PLANE, C::PLANE, 128);
                         const uint64_t db = tc::sdesc(wb + dx * C::W_TAP + q * 2 * COUT * 16, COUT * 16, 128);
                         tc::mma_bf16(d, da, db, idesc, (s | dx | q) != 0);
                     }
@@ -364,12 +387,12 @@ __global__ void __launch_bounds__(kConvThreads, ConvCfg<CIN, COUT>::PER)
 // consecutive voxels of a plane and a CTA takes it through a chunk of planes,
 // so that a plane's three windows (dy = -1, 0, 1) are copied once and serve the
 // outputs of three planes, and the 27 taps' weights stay in shared memory.
-// k_conv_tc copies nine windows and the weights per tile, and those copies'
-// issue bounds it (129 x 97 x 65, 16 -> 16: 58 % of the issue slots, 7 % of the tensor
-// pipe, 76 us).  Here it takes 58 us (32 -> 32 194 with the call against 206),
-// bound by a plane's chain of copy, 27 small MMAs and epilogue: two CTAs per SM
-// instead of three take a third longer.  The products are added in the same
-// order: the same bits.
+// k_conv_tc copies nine windows and the weights per tile, and with 16 channels
+// those copies' issue bounds it (129 x 97 x 65, 16 -> 16: 58 % of the issue
+// slots, 7 % of the tensor pipe, 76 us).  Here it takes 58 us, bound by a
+// plane's chain of copy, 27 small MMAs and epilogue: two CTAs per SM instead of
+// three take a third longer.  The products are added in the same order: the
+// same bits.
 template <int CIN, int COUT>
 struct MarchCfg {
     static constexpr int NCH = CIN / 8;
@@ -385,14 +408,14 @@ struct MarchCfg {
     static constexpr int S0 = (220 * 1024 / PER - FIXED) / STAGE;
     static constexpr int STAGES = S0 > 18 ? 18 : S0;
     static constexpr int SMEM = FIXED + STAGES * STAGE;
-    // one CTA per SM only where k_conv_tc has one too (32 -> 16, two there: 157 us against 194)
-    static constexpr bool fits = CIN <= 32 && STAGES >= 12 && (PER > 1 || ConvCfg<CIN, COUT>::PER == 1);
+    static constexpr bool fits = (CIN == 16 || (CIN == 32 && COUT == 64)) && STAGES >= 12;
 };
 
 struct March {
-    int tiles;   // 128-voxel tiles of a plane
-    int planes;  // of a chunk
+    int tiles;     // 128-voxel tiles of a plane
+    int planes;    // of a chunk
     int chunks;
+    int64_t cost;  // planes that the SM with the most works through, one after the other
 };
 
 // as k_conv_tc; one CTA per unit (tile, chunk), tile fastest
