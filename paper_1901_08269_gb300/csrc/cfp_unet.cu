@@ -1088,26 +1088,25 @@ constexpr size_t kNnKeep = size_t(32) << 20;
 struct NnWork {
     cfp_ctx* c;
     void* p = nullptr;
-    bool own;
-    NnWork(cfp_ctx* ctx, size_t bytes) : c(ctx), own(bytes > kNnKeep) {
-        cudaError_t e = cudaSuccess;
-        if (own) {
-            e = pool_malloc(&p, bytes, c->stream);
-        } else {
-            if (c->nn_work_bytes < bytes) {
-                pool_free(c->nn_work, c->stream);
-                c->nn_work = nullptr;
-                c->nn_work_bytes = 0;
-                e = pool_malloc(&c->nn_work, bytes, c->stream);
-                if (e == cudaSuccess) c->nn_work_bytes = bytes;
-                else c->nn_work = nullptr;
-            }
-            p = c->nn_work;
+    bool own = false;
+    explicit NnWork(cfp_ctx* ctx) : c(ctx) {}
+    cfp_status get(size_t bytes) {
+        if (bytes > kNnKeep) {
+            CFP_CUDA(pool_malloc(&p, bytes, c->stream));
+            own = true;  // from here on the destructor gives it back
+            return CFP_OK;
         }
-        if (e != cudaSuccess) {
-            p = nullptr;
-            cuda_fail(e, "allocating a layer's work space");
+        if (c->nn_work_bytes < bytes) {
+            pool_free(c->nn_work, c->stream);
+            c->nn_work = nullptr;
+            c->nn_work_bytes = 0;
+            void* q = nullptr;
+            CFP_CUDA(pool_malloc(&q, bytes, c->stream));
+            c->nn_work = q;
+            c->nn_work_bytes = bytes;
         }
+        p = c->nn_work;
+        return CFP_OK;
     }
     ~NnWork() {
         if (own) pool_free(p, c->stream);
@@ -1139,8 +1138,8 @@ cfp_status cfp_nn_conv3d(cfp_ctx* ctx, int nx, int ny, int nz, int cin, int cout
         CFP_CUDA(cudaMalloc(&ctx->dwait, sizeof(int)));
         CFP_CUDA(cudaMemsetAsync(ctx->dwait, 0, sizeof(int), ctx->stream));
     }
-    NnWork wpk(ctx, (size_t)27 * cin * cout * 2);
-    if (!wpk.p) return CFP_ENOMEM;
+    NnWork wpk(ctx);
+    CFP_TRY(wpk.get((size_t)27 * cin * cout * 2));
     const int f = (flags & CFP_NN_RELU ? F_RELU : 0) | (flags & CFP_NN_MASK ? F_MASK : 0) |
                   (flags & CFP_NN_OUT_F32 ? F_OUT_F32 : 0) | (flags & CFP_NN_ACCUM ? F_ACCUM : 0);
     cfp_status st = conv_any(ctx->stream, cin, cout, in_dev, w_dev, (flags & CFP_NN_DGRAD) != 0, (uint16_t*)wpk.p,
@@ -1161,8 +1160,8 @@ cfp_status cfp_nn_conv3d_wgrad(cfp_ctx* ctx, int nx, int ny, int nz, int cin, in
         CFP_CUDA(cudaMemsetAsync(ctx->dwait, 0, sizeof(int), ctx->stream));
     }
     const int64_t cap = (int64_t)num_sms() * 27 * cin * cout;
-    NnWork work(ctx, (cap + kColBlocks * 128) * 4);  // the chunks' partials, the bias gradient's
-    if (!work.p) return CFP_ENOMEM;
+    NnWork work(ctx);
+    CFP_TRY(work.get((cap + kColBlocks * 128) * 4));  // the chunks' partials, the bias gradient's
     cfp_status st = wgrad_any(ctx->stream, cin, cout, in_dev, gout_dev, P, (float*)work.p, cap, dw_dev, db_dev,
                               (float*)work.p + cap, ctx->dwait);
     ctx->launches += db_dev ? 4 : 2;
