@@ -92,8 +92,12 @@ typedef struct {
     int max_refine;    /* CFP_PREC_MIXED: cap on refinement steps (default 40) */
     int use_graph;     /* 1 (default): the iteration runs as one CUDA graph
                           with a device-side while loop; 0: plain launches   */
-    int precond;       /* CFP_PRECOND_RBGS (default), CFP_PRECOND_MG or
-                          CFP_PRECOND_ILU                                    */
+    int precond;       /* CFP_PRECOND_RBGS (default), CFP_PRECOND_MG (at most
+                          131071 nodes in y and in z) or CFP_PRECOND_ILU.
+                          The first two keep work arrays with the context:
+                          per two nodes of a level seven FP64 values (two of
+                          them reciprocal diagonals: 1.1 of 4 GB at 513^3),
+                          in CFP_PREC_MIXED six FP32 values                  */
     int mg_smooth;     /* CFP_PRECOND_MG: sweeps before the coarse correction
                           on each level, and after it unless mg_post is set
                           (default 2)                                       */
@@ -103,9 +107,11 @@ typedef struct {
                           multigrid levels (and of the fine level's sweeps)
                           with at least 192 nodes per row stream their tiles
                           through shared memory with TMA bulk-tensor copies,
-                          the coarse levels from the first of at most 2^16
-                          nodes down run as one launch of a thread-block
-                          cluster that holds them in shared memory,
+                          the coarse levels run as one launch of a
+                          thread-block cluster that holds them in shared
+                          memory, from the first of at most 2^16 nodes
+                          that fits there down (some flat FP64 levels do
+                          not: they run one launch per pass),
                           and the prolongation runs one thread per coarse
                           cell; 0: plain loads, one launch per half-sweep,
                           one prolongation thread per fine pair; 2: as 1,

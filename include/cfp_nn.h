@@ -58,7 +58,9 @@ enum { CFP_NN_RELU = 1,     /* max(., 0) after the bias                        *
  * of (16,16) (16,32) (32,16) (32,32) (32,64) (64,32) (64,64) (64,128)
  * (128,64) (128,128).  bias (cout FP32) may be NULL; act (Np x cout BF16) is
  * read with CFP_NN_MASK.  Tensor-core implicit GEMM (tcgen05, operands staged
- * by TMA).  Synchronises.  Errors: CFP_EINVAL, CFP_ECUDA.
+ * by TMA, with 16 channels in or out by the threads).  Up to 32 MB of work
+ * space, of this call and of cfp_nn_conv3d_wgrad, stays with the context until
+ * it is destroyed.  Synchronises.  Errors: CFP_EINVAL, CFP_ENOMEM, CFP_ECUDA.
  */
 cfp_status cfp_nn_conv3d(cfp_ctx* ctx, int nx, int ny, int nz, int cin, int cout, const uint16_t* in_dev,
                          const uint16_t* w_dev, const float* bias_dev, const uint16_t* act_dev, int flags,

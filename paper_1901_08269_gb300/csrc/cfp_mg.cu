@@ -193,7 +193,7 @@ struct Off {
 // first test (rows j, k and the pair are interior, entry m - 1 exists for
 // m = 0 because the row is not the first; planes past the last interior one
 // repeat plane k0 and store nothing), so the loads of all kSweepPlanes nodes
-// are issued before any value is stored: three independent nodes per thread
+// are issued before any value is stored: several independent nodes per thread
 // keep more loads in flight.  FINE: the fine level, whose irregular nodes
 // take their Shortley-Weller rows (Eq. A7_mod) from the side list: few
 // nodes (0.3 % at 513^3), whose dependent loads other warps cover, for one
@@ -1022,7 +1022,7 @@ __global__ void __launch_bounds__(kPairThreads, 4)
 
 // r0 = b0 - K e at the red unknowns (black residuals are zero after a black
 // half-sweep; r0 stays zero at the other red entries): the half-sweep's chain
-// and one more product with the diagonal; three planes per thread with all
+// and one more product with the diagonal; kSweepPlanes per thread with all
 // loads first, and the fine level's Shortley-Weller rows, as in the
 // half-sweep.
 template <class T, bool FINE>
@@ -1155,7 +1155,7 @@ __global__ void k_restrict_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
 }
 
 // e1 += P e_c at the fine black unknowns (the red values are overwritten by
-// the next red half-sweep without being read); three planes per thread.
+// the next red half-sweep without being read); kSweepPlanes per thread.
 template <class T>
 __global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C,
                                                                   unsigned z0) {

@@ -3,6 +3,11 @@
 // down to the coarsest and back up -- smoothing, red residual, restriction,
 // the coarsest level's 16 sweeps, prolongation, smoothing -- on one
 // thread-block cluster, with the levels in shared memory.
+// Where a level's share, with the rows copied from either side, is more than
+// kCoarseSmem (FP64, some flat levels: 68 x 54 x 17, 87 x 65 x 9; 0.5 % of the
+// grids of 33 to 449 nodes per axis) the list begins one level further down and
+// that level runs one launch per pass (V(2,2) of 135 x 107 x 33 217 us, 345 x
+// 254 x 33 551; 757 and 1010 when only its smoothing was a cluster's).
 //
 // These levels hold too few nodes to fill the GPU: a pass over one costs its
 // latency, one launch per pass or a CTA working in L2 alike.  Shared memory

@@ -5,8 +5,9 @@
 //      XR = sum_p Rx[p] x,  XL = sum_p Lx[p] x,
 //    with the y-pass results of three planes kept in registers while a thread
 //    (FP64, most FP32 grids) or a shared-memory ring's consumer (large FP32
-//    grids whose width fills its tiles) marches in z; the rows of irregular points, with their
-//    modified-stencil corrections, in a kernel beside it; solid rows are zero.
+//    grids whose width fills its tiles) marches in z; the rows of irregular
+//    points, with their modified-stencil corrections, in a kernel beside it;
+//    solid rows are zero.
 //  - the right-hand side of Eq. Bu=q and helpers of the solves.
 #include <algorithm>
 
@@ -119,10 +120,11 @@ struct DotAcc2 {
     }
 };
 
-// Regular part of B x at the unknowns in FP32 (the streaming kernel; the
-// ring below takes large grids that fill its tiles).  A warp is 32 columns x TY consecutive rows
-// (a lane each) and marches the planes k0 .. k1 - 1 of its z chunk (kc planes,
-// at most kMaxPlanes); a CTA is four warps, one above the other in y.
+// Regular part of B x at the unknowns in FP32 (the streaming kernel; the ring
+// below takes large grids that fill its tiles).  A warp is 32 columns x TY
+// consecutive rows (a lane each) and marches the planes k0 .. k1 - 1 of its z
+// chunk (kc planes, at most kMaxPlanes); a CTA is four warps, one above the
+// other in y.
 // Per plane a thread loads the values x(i-1..i+1, j) of the rows j0-1 .. j0+TY
 // (the x and y neighbours come from L1/L2; the loads of the next plane are
 // issued once the x pass has used this one's), forms the x-pass XR = Rx x,
@@ -1156,17 +1158,18 @@ struct Shape {
     }
 };
 
-// The launch shape of k_apply64 (where the tuner set none) and k_rhs_source
-// by grid size: the one with the smallest estimate.  A warp issues w = (kc + 2) (row (ty +
-// 2) + yout ty) + zout kc ty FP64 instructions (row per loaded row, yout and
-// zout per output row in y and z: 5, 7, 6 in the apply; its two halo planes do
-// the x and y passes only), a CTA 4 w; the estimate is the busiest of 152 SMs, the latency of a plane's loads
-// (about 130 slots per plane), which counts where few CTAs share an SM, and,
-// past four CTAs per SM, half of a last one that runs alone.  Large grids
-// take 4 rows and 64 planes, 129^3 and 257^3 4 x 16 (109 and 712 us; 4 x 64
-// 250 and 895), 97 x 65 x 82 2 x 8; 33^3 takes 128 CTAs of 1 x 2, where 4 x
-// 64 would leave the work to 8 SMs.  (CTAs of one warp share a scheduler:
-// 33^3 14.5 us with them, 10.4 with four warps in the same shape.)
+// The launch shape of k_apply64 (where the tuner set none) and k_rhs_source by
+// grid size: the one with the smallest estimate.  A warp issues w = (kc + 2)
+// (row (ty + 2) + yout ty) + zout kc ty FP64 instructions (row per loaded row,
+// yout and zout per output row in y and z: 5, 7, 6 in the apply; its two halo
+// planes do the x and y passes only), a CTA 4 w; the estimate is the busiest of
+// 152 SMs, the latency of a plane's loads (about 130 slots per plane), which
+// counts where few CTAs share an SM, and, past four CTAs per SM, half of a last
+// one that runs alone.  Large grids take 4 rows and 64 planes, 129^3 and 257^3
+// 4 x 16 (109 and 712 us; 4 x 64 250 and 895), 97 x 65 x 82 2 x 8; 33^3 takes
+// 128 CTAs of 1 x 2, where 4 x 64 would leave the work to 8 SMs.  (CTAs of one
+// warp share a scheduler: 33^3 14.5 us with them, 10.4 with four warps in the
+// same shape.)
 Shape shape64(const cfp_ctx* c, double row, double yout, double zout) {
     Shape best{4, 64};
     double est_best = 1e300;
@@ -1191,10 +1194,11 @@ Shape apply64_shape(const cfp_ctx* c) {
 
 // The FP32 streaming kernel is bound by the latency of a plane's loads, so its
 // time goes with the rounds of resident CTAs (four with 4 rows, six with 2 per
-// SM) times the planes each marches, about 1 us per plane with 4 rows, and
-// some 6 for a round's start (257^3: 4 x 64 68 us, 4 x 8 78; 129^3: 4 x 8 12.4,
-// 4 x 16 14.5; 321 x 257 x 289: 4 x 32 91, 4 x 64 106).  Without a dot product 2 rows take 0.65 of it
-// (513^3 361 us against 390), with one more (448 against 406).
+// SM) times the planes each marches, about 1 us per plane with 4 rows, and some
+// 6 for a round's start (257^3: 4 x 64 68 us, 4 x 8 78; 129^3: 4 x 8 12.4, 4 x
+// 16 14.5; 321 x 257 x 289: 4 x 32 91, 4 x 64 106).  Without a dot product 2
+// rows take 0.65 of it (513^3 361 us against 390), with one more (448 against
+// 406).
 Shape apply32_by_size(const cfp_ctx* c, bool dot) {
     Shape best{4, 64};
     double est_best = 1e300;
