@@ -209,12 +209,11 @@ constexpr int kSweepPlanes = sizeof(T) == 8 ? 2 : 3;
 
 template <class T, int MODE, bool FINE>
 __global__ void __launch_bounds__(kSplitThreads)
-    k_sweep_split(SLev<T> L, Half<T> H, Side<T> S, int colour, const T* __restrict__ rho, T* __restrict__ phi,
-                  unsigned z0) {
+    k_sweep_split(SLev<T> L, Half<T> H, Side<T> S, int colour, const T* __restrict__ rho, T* __restrict__ phi) {
     constexpr bool F64 = sizeof(T) == 8, READ = MODE == 0 || MODE == 3;
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
@@ -1026,10 +1025,10 @@ __global__ void __launch_bounds__(kPairThreads, 4)
 // loads first, and the fine level's Shortley-Weller rows, as in the
 // half-sweep.
 template <class T, bool FINE>
-__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S, unsigned z0) {
+__global__ void __launch_bounds__(kSplitThreads) k_resid_split(SLev<T> L, Side<T> S) {
     const int nx = L.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > L.ny - 2) return;
     const int hp = L.hp;
     const unsigned hs = L.hs;
@@ -1157,11 +1156,10 @@ __global__ void k_restrict_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
 // e1 += P e_c at the fine black unknowns (the red values are overwritten by
 // the next red half-sweep without being read); kSweepPlanes per thread.
 template <class T>
-__global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C,
-                                                                  unsigned z0) {
+__global__ void __launch_bounds__(kSplitThreads) k_prolong_split(Transfer<T> X, SLev<T> F, SLev<T> C) {
     const int nx = F.nx;
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * (z0 + blockIdx.z);
+    const int j = 1 + blockIdx.y * blockDim.y + threadIdx.y, k0 = 1 + kSweepPlanes<T> * blockIdx.z;
     if (2 * m > nx - 2 || j > F.ny - 2) return;
     const unsigned hc = (unsigned)C.hp;
     const IpPk<T> py = X.ip[1][j];
@@ -1323,20 +1321,42 @@ dim3 plane_block(const int n[3]) {
     const int bx = std::min(kSplitThreads, (n[0] / 2 + 31) / 32 * 32);
     return dim3((unsigned)bx, (unsigned)(kSplitThreads / bx));
 }
-// launch(grid, block, z0) for the block rows z0 .. z0 + grid.z - 1 of a pass that
-// takes kSweepPlanes planes per block row: one launch up to 65535 block rows
-// (131072 planes in FP64, 196607 in FP32), as many as it takes above.  Returns
-// the launches.
-constexpr unsigned kMaxGridZ = 65535;
+// The part of a level from plane z on (z even, so that colours stay), as a
+// level of its own.
+template <class T>
+SLev<T> from_plane(SLev<T> L, int z) {
+    const int64_t o = (int64_t)z * L.hs;
+    for (int c = 0; c < 2; ++c) {
+        L.ty[c] += o;
+        L.e[c] += o;
+        L.b[c] += o;
+        if (L.rd[c]) L.rd[c] += o;
+    }
+    L.r0 += o;
+    L.cz += z;
+    L.nz -= z;
+    return L;
+}
+template <class T>
+Side<T> from_plane(Side<T> S, const SLev<T>& L, int z) {
+    if (S.slot) S.slot += (int64_t)z * L.nx * L.ny;
+    return S;
+}
+
+// launch(grid, block, z) for a pass that takes kSweepPlanes planes per block
+// row, over the part of the level from plane z on: once, z = 0, for up to
+// kMaxRows block rows (131070 planes in FP64, 196604 in FP32), and for each
+// such number of them above.  Returns the launches.
+constexpr int kMaxGridZ = 65535, kMaxRows = kMaxGridZ - 1;  // even
 template <class T, class F>
 int by_planes(const int n[3], F launch) {
     const dim3 b = plane_block(n);
-    const unsigned rows = (unsigned)((n[2] - 2 + kSweepPlanes<T> - 1) / kSweepPlanes<T>);
+    const int rows = (n[2] - 2 + kSweepPlanes<T> - 1) / kSweepPlanes<T>;
     int count = 0;
-    for (unsigned z0 = 0; z0 < rows; z0 += kMaxGridZ, ++count)
+    for (int r = 0; r < rows; r += kMaxRows, ++count)
         launch(dim3((unsigned)((n[0] / 2 + b.x - 1) / b.x), (unsigned)((n[1] - 2 + b.y - 1) / b.y),
-                    std::min(rows - z0, kMaxGridZ)),
-               b, z0);
+                    (unsigned)std::min(rows - r, kMaxRows)),
+               b, r * kSweepPlanes<T>);
     return count;
 }
 
@@ -1513,6 +1533,12 @@ void reset_red(cfp_ctx* c) {
     for (MgLevel& M : c->mg) M.red_cur = 0;
 }
 
+// the arrays of a half-sweep of colour c
+template <class T>
+Half<T> half(const SLev<T>& L, int c) {
+    return Half<T>{L.ty[c], L.e[c], L.e[1 - c], L.b[c], L.b[1 - c], L.ty[1 - c], L.rd[c]};
+}
+
 // the fine level's Shortley-Weller rows after a half-sweep of a large FP32 grid
 template <int MODE>
 void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, const Side<float>& S, int colour,
@@ -1530,40 +1556,43 @@ void launch_sweep_fix(cfp_ctx* c, const SLev<float>& L, const Half<float>& H, co
 // which is bound by HBM and pays more for the branch (513^3: 289 us against
 // 233 and a follow-up of 5).
 template <class T, int MODE>
-void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Half<T>& H, const Side<T>& S, int colour,
-                        const T* rho, T* phi, cudaStream_t s) {
+void launch_sweep_split(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colour, const T* rho, T* phi,
+                        cudaStream_t s) {
     const bool after = MODE == 2 && sizeof(T) == 4 && c->mg[l].tma;
     const bool fine = l == 0 && c->n_irr > 0 && !after;
-    c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
-        if (fine) k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi, z0);
-        else k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(L, H, S, colour, rho, phi, z0);
+    c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, int z) {
+        const SLev<T> P = from_plane(L, z);
+        const Half<T> H = half(P, colour);
+        const int64_t o = (int64_t)z * L.nx * L.ny;
+        const T* r = rho ? rho + o : nullptr;
+        T* f = phi ? phi + o : nullptr;
+        if (fine) k_sweep_split<T, MODE, true><<<g, blk, 0, s>>>(P, H, from_plane(S, L, z), colour, r, f);
+        else k_sweep_split<T, MODE, false><<<g, blk, 0, s>>>(P, H, S, colour, r, f);
     });
     if (fine) return;
     if constexpr (MODE == 2 && sizeof(T) == 4)
-        if (l == 0) launch_sweep_fix<2>(c, L, H, S, colour, phi, s);
+        if (l == 0) launch_sweep_fix<2>(c, L, half(L, colour), S, colour, phi, s);
 }
 
 template <class T>
 void half_sweep(cfp_ctx* c, int l, const SLev<T>& L, const Side<T>& S, int colour, int mode, const T* rho, T* phi,
                 cudaStream_t s) {
-    const Half<T> H{L.ty[colour], L.e[colour], L.e[1 - colour], L.b[colour], L.b[1 - colour], L.ty[1 - colour],
-                    L.rd[colour]};
     // the TMA-fed pass: plain, or the last black half-sweep of the fine level
     if (mode == 0 || (mode == 3 && colour == 1)) {
         if (sweep_tma(c, l, L, mode == 0 ? 0 : 2, colour, phi, s)) {
             c->launches += 1;
             if constexpr (sizeof(T) == 4) {
-                if (l == 0 && mode == 0) launch_sweep_fix<0>(c, L, H, S, colour, phi, s);
-                else if (l == 0) launch_sweep_fix<3>(c, L, H, S, colour, phi, s);
+                if (l == 0 && mode == 0) launch_sweep_fix<0>(c, L, half(L, colour), S, colour, phi, s);
+                else if (l == 0) launch_sweep_fix<3>(c, L, half(L, colour), S, colour, phi, s);
             }
             return;
         }
     }
     switch (mode) {
-        case 0: launch_sweep_split<T, 0>(c, l, L, H, S, colour, rho, phi, s); break;
-        case 1: launch_sweep_split<T, 1>(c, l, L, H, S, colour, rho, phi, s); break;
-        case 2: launch_sweep_split<T, 2>(c, l, L, H, S, colour, rho, phi, s); break;
-        default: launch_sweep_split<T, 3>(c, l, L, H, S, colour, rho, phi, s); break;
+        case 0: launch_sweep_split<T, 0>(c, l, L, S, colour, rho, phi, s); break;
+        case 1: launch_sweep_split<T, 1>(c, l, L, S, colour, rho, phi, s); break;
+        case 2: launch_sweep_split<T, 2>(c, l, L, S, colour, rho, phi, s); break;
+        default: launch_sweep_split<T, 3>(c, l, L, S, colour, rho, phi, s); break;
     }
 }
 
@@ -1993,7 +2022,7 @@ cfp_status ensure_mg(cfp_ctx* c, int prec, bool vcycle) {
     // they brought the process down.
     if (vcycle && c->mg.size() > 1)
         for (int d = 1; d < 3; ++d)
-            if (c->mg[1].n[d] - (c->mg_tma ? 1 : 2) > (int)kMaxGridZ)
+            if (c->mg[1].n[d] - (c->mg_tma ? 1 : 2) > kMaxGridZ)
                 return fail(CFP_ECUDA, "grid too long in y or z for the multigrid transfers (65536 coarse nodes)");
     bool fresh32 = false;
     if (prec == 0 && !c->mg[0].s64) c->coarse_cl[0] = coarse_cluster_size<double>();
@@ -2033,8 +2062,10 @@ void launch_prolong(cfp_ctx* c, int l, const SLev<T>& F, const SLev<T>& C, cudaS
         const dim3 g((unsigned)((Cn.n[0] - 1 + 127) / 128), (unsigned)(Cn.n[1] - 1), (unsigned)(Cn.n[2] - 1));
         k_prolong_cell<T><<<g, 128, 0, s>>>(transfer<T>(c->mg[l]), F, C);
     } else {
-        c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
-            k_prolong_split<T><<<g, blk, 0, s>>>(transfer<T>(c->mg[l]), F, C, z0);
+        c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, int z) {
+            Transfer<T> X = transfer<T>(c->mg[l]);
+            X.ip[2] += z;
+            k_prolong_split<T><<<g, blk, 0, s>>>(X, from_plane(F, z), C);
         }) - 1;  // the caller counts one
     }
 }
@@ -2068,9 +2099,10 @@ void launch_precond_mg(cfp_ctx* c, const T* rho, T* phi, cudaStream_t s) {
                 }
             }
         } else {
-            c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, unsigned z0) {
-                if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(F, S, z0);
-                else k_resid_split<T, false><<<g, blk, 0, s>>>(F, S, z0);
+            c->launches += by_planes<T>(c->mg[l].n, [&](dim3 g, dim3 blk, int z) {
+                const SLev<T> P = from_plane(F, z);
+                if (l == 0 && c->n_irr > 0) k_resid_split<T, true><<<g, blk, 0, s>>>(P, from_plane(S, F, z));
+                else k_resid_split<T, false><<<g, blk, 0, s>>>(P, S);
             }) - 1;  // counted below with the restriction
         }
         const MgLevel& Cn = c->mg[l + 1];
