@@ -1911,10 +1911,6 @@ cfp_status build_levels(cfp_ctx* c) {
 
 }  // namespace
 
-namespace {
-
-}  // namespace
-
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
 // (the library does not link libcuda)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
